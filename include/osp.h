@@ -360,7 +360,8 @@ int64_t osp_device_bytes(const osp_ctx *ctx);
 osp_status osp_get_seed_stats(osp_ctx *ctx, int32_t *iterations, double *qoff_l1,
                               double *last_l1, int32_t cap, int32_t *count);
 
-/* The pull-step schedule in force (host array of 4): items per warp task,
+/* The pull-step schedule in force (host array of 4): items per warp task (at
+ * most; a graph too small to give every warp a few such tasks is cut finer),
  * in-list length above which lists are summed in pieces, the piece length, and
  * the items a node counts for in task planning. */
 osp_status osp_get_schedule(osp_ctx *ctx, int32_t *out);

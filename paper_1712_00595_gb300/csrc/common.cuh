@@ -27,12 +27,19 @@ constexpr int kAbsParts = 1024;  // CTAs of the L1-norm reduction (per-CTA parti
 constexpr int kMaxGrid = 4096;           // CTAs of the persistent kernel (partials array size)
 constexpr int kPropThreads = 256;
 constexpr int kPropWarps = kPropThreads / 32;
+// The one-seed kernel runs one CTA of 32 warps per SM: as many warps as four
+// CTAs of eight at its 64 registers, and a quarter of the arrivals at each
+// grid barrier.
+constexpr int kOneThreads = 1024;
+constexpr int kOneWarps = kOneThreads / 32;
+constexpr int kPushPiece = 256;  // push step: longer rows are scattered in pieces of this size
 constexpr int kHubThreshold = 1024;  // pull step: in-lists longer than this are summed in pieces
 constexpr int kHubPiece = 1024;      // pull step: edges per hub piece
 constexpr int kMultiHub = 256;       // seed block: in-lists longer than this, in pieces of this size
 constexpr int kMultiNodeItems = 4;   // seed block: task items per node (a node's score row costs more)
 constexpr int kTaskItems = 1024;     // pull step: default items (edges + nodes) per warp task
 constexpr int kMinTaskItems = 256;   // smallest task size a schedule may choose (sizes the plan)
+constexpr int kMaxSmallTasks = 1 << 16;  // most tasks a small graph is cut into below that size
 constexpr double kPushAlpha = 14.0;  // push step while frontier out-edges <= m / alpha
 constexpr double kPushBeta = 24.0;   // ... and frontier size <= n / beta
 
@@ -63,7 +70,8 @@ struct Ctl {
   int epoch;                   // frontier mark of x(0); step i uses epoch + i
   int q_size[2];               // frontier queue lengths
   unsigned int bar_count, bar_gen;
-  int ctr[4];                  // dynamic work counters, reset at every barrier
+  int ctr[4];                  // dynamic work counters (one seed: by step number mod 4)
+  int n_big;                   // push step: pieces of the long rows
   int iter, mode, push_iters, stop, pull_used, noconv;
   long long visited;
   long long ef;                // out-edges of the current frontier
@@ -155,9 +163,11 @@ struct Dev {
   int* piece_hub;  // [2 pool cap / kMultiHub + 4] the long in-list each piece belongs to
   double* piece_part;  // [as piece_hub] deterministic mode: per-piece partial sums
   double* hub_l1;      // [as hubs] deterministic mode: |x_v| of each long in-list's node
-  int* big_u; double* big_y;  // push step: rows longer than kHubThreshold [pool cap / kHubThreshold + 2]
+  // push step: pieces of the rows longer than kPushPiece [2 pool cap / kPushPiece + 2]
+  unsigned* big_off; int* big_len; double* big_y;
+  unsigned* bar;  // grid barrier of the one-seed kernel: arrivals of the call, on a line of its own
   // reductions and history
-  double* part_l1; long long* part_ef;  // [kMaxGrid]
+  double* part_l1; long long* part_ef;  // [2 kMaxGrid] by step parity
   double* l1_hist;                      // [kMaxHist]
   unsigned long long* step_ns;          // [kMaxHist + 1] device clock at kernel start and after each step
   Ctl* ctl;

@@ -476,7 +476,15 @@ osp_status plan_pull(osp_ctx* ctx, int64_t n_bound, int64_t m_bound) {
   k_scan_add<<<(ns + 255) / 256, 256, 0, st>>>(ctx->d.pc, ctx->scan_bsum, ns);
   ++ctx->launches;
   const int* sc = schedule(ctx);
-  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0]);
+  // A graph whose tasks of sc[0] items would leave warps idle is cut finer:
+  // two tasks a warp with one seed (down to 32 items: 10,000 nodes and 100,000
+  // edges in double ran 82 us a step in 107 tasks of 1,024, 9.6 us in 3,437 of
+  // 32, 12.9 us in 430 of 256), four with several (65,537 nodes, 10^6 edges,
+  // 17 seeds in double: 160 -> 110 us a step).
+  const bool many = ctx->S > 1;
+  const int want = many ? ctx->grid_multi * kPropWarps * 4 : ctx->grid_prop * kOneWarps * 2;
+  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], many ? 64 : 32,
+                                                std::min(kMaxSmallTasks, want));
   ++ctx->launches;
   k_hub_prefix<<<1, 1024, 0, st>>>(ctx->d, sc[2], ctx->opt.deterministic != 0);
   ++ctx->launches;
@@ -1150,7 +1158,7 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     AL(d.piece_base, npc, 0);
   }
   AL(d.pc, nc + 1, 0);
-  AL(d.task_first, (int64_t)(kMultiNodeItems * nc + (int64_t)cap) / kMinTaskItems + 2, 0);
+  AL(d.task_first, (int64_t)(kMultiNodeItems * nc + (int64_t)cap) / kMinTaskItems + kMaxSmallTasks + 2, 0);
   {
     // lists longer than a threshold t number at most (live edges) / t <= cap / t;
     // the pull plan uses t = kMultiHub for the seed block, kHubThreshold otherwise
@@ -1163,12 +1171,15 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     AL(d.hub_l1, nh, 0);
     AL(d.hub_acc, nh, 0);
     AL(d.hub_cnt, nh, 0);
-    const int64_t nb = (int64_t)(cap / kHubThreshold) + 2;  // push: rows above kHubThreshold
-    AL(d.big_u, nb, 0);
+    // push: a row above kPushPiece entries has at most 2 len / kPushPiece pieces
+    const int64_t nb = 2 * (int64_t)(cap / kPushPiece) + 2;
+    AL(d.big_off, nb, 0);
+    AL(d.big_len, nb, 0);
     AL(d.big_y, nb, 0);
   }
-  AL(d.part_l1, kMaxGrid, 0);
-  AL(d.part_ef, kMaxGrid, 0);
+  AL(d.part_l1, 2 * kMaxGrid, 0);
+  AL(d.part_ef, 2 * kMaxGrid, 0);
+  AL(d.bar, 64, 0);
   AL(d.l1_hist, kMaxHist, 0);
   AL(d.step_ns, kMaxHist + 1, 0);
   AL(d.ctl, 1, 0);

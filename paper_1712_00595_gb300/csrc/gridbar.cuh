@@ -61,4 +61,28 @@ static __device__ __forceinline__ bool bar_release(Ctl* ctl, BarShared& sh) {
   return sh.ok;
 }
 
+// Arrive at a barrier whose arrivals only count up and wait until `target`
+// have come (one thread per CTA, after a __syncthreads; the caller broadcasts
+// the result). What any thread of an arrived CTA wrote is visible afterwards.
+// Bounded like bar_release; false after a timeout.
+static __device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, Ctl* ctl) {
+  bool ok = true;
+  __threadfence();
+  atomicAdd(bar, 1u);
+  unsigned long long t0 = 0;
+  unsigned spins = 0;
+  while ((int)(*(volatile unsigned*)bar - target) < 0) {
+    if ((++spins & 1023u) == 0) {
+      if (t0 == 0) t0 = global_ns();
+      if (spins >= kBarrierMaxSpins || global_ns() - t0 > kBarrierTimeoutNs) {
+        atomicCAS(&ctl->status, 0, (int)OSP_ETIMEOUT);
+        ok = false;
+        break;
+      }
+    }
+  }
+  __threadfence();
+  return ok;
+}
+
 }  // namespace osp

@@ -176,7 +176,9 @@ __global__ void k_reset_batch(Dev d, int cont) {
   c->n_dst_nz = 0;
   c->n_src_nz = 0;
   for (int i = 0; i < 4; ++i) c->ctr[i] = 0;
+  c->n_big = 0;
   c->bar_count = 0;
+  d.bar[0] = 0;
   c->iter = 0;
   c->mode = kPush;
   c->push_iters = 0;

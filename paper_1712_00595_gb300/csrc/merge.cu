@@ -338,11 +338,14 @@ __global__ void k_merge_finish(Dev d) {
 // pc[v] + node_w v >= t * task_items (so a task holds about task_items items,
 // an edge counting 1 and a node node_w, and never splits a list); in-lists
 // longer than hub_thr are listed for piecewise summation.
-__global__ void k_pull_plan(Dev d, int hub_thr, int node_w, int task_items) {
+// Small graphs get shorter tasks, down to task_min items, so that `want` warps
+// have one each.
+__global__ void k_pull_plan(Dev d, int hub_thr, int node_w, int task_items, int task_min, int want) {
   Ctl* ctl = d.ctl;
   if (*(volatile int*)&ctl->status) return;
   const int n = ctl->n;
   const long long W = (long long)node_w * n + ctl->m;
+  task_items = (int)min((long long)task_items, max((long long)task_min, (W + want - 1) / want));
   const int nt = (int)((W + task_items - 1) / task_items);
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;

@@ -651,10 +651,15 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
   double l1n[W];
 #pragma unroll
   for (int c = 0; c < W; ++c) l1n[c] = 0.0;
-  for (;;) {
-    int t = 0;
-    if (lane == 0) t = atomicAdd(&ctl->ctr[1], 1);
-    t = __shfl_sync(0xffffffffu, t, 0);
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int k = 0;; ++k) {
+    int t = gw;  // the first item is the warp's own number, later ones come from the counter
+    if (k > 0) {
+      if (n_items <= nw) break;
+      if (lane == 0) t = nw + atomicAdd(&ctl->ctr[1], 1);
+      t = __shfl_sync(0xffffffffu, t, 0);
+    }
     if (t >= n_items) break;
     if (t < n_pieces) {
       // a piece of a long in-list; the piece that completes the list finishes it
@@ -1549,10 +1554,13 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
     }
     prev_narrow = narrow;
     if (!narrow)
-    for (;;) {
-      int t = 0;
-      if (lane == 0) t = atomicAdd(&ctl->ctr[1], 1);
-      t = __shfl_sync(0xffffffffu, t, 0);
+    for (int k = 0;; ++k) {
+      int t = gw;  // the first item is the warp's own number, later ones come from the counter
+      if (k > 0) {
+        if (total <= nw) break;
+        if (lane == 0) t = nw + atomicAdd(&ctl->ctr[1], 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+      }
       if (t >= total) break;
       // task-major: a work item's groups come one after the other, so its
       // in-list ids and node headers are read from DRAM once for all groups

@@ -1,0 +1,77 @@
+"""The one-seed kernel at the sizes where its step forms change hands, against
+the oracle: in-lists around the stream, block and piece lengths, rows around
+the push piece, frontiers of one node and of more nodes than warps, and pool
+offsets in any order (lists rewritten by batches).
+
+Tolerances are those of the parity tests (FP64 L1 1e-10; FP32 products 1e-5,
+the oracle replaying the same step counts).
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1712_00595_gb300 import native as N
+from paper_1712_00595_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+C_RESTART = 0.15
+TOL = {N.OSP_PREC_FP64: 1e-10, N.OSP_PREC_FP32_ACC64: 1e-5}
+LENGTHS = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 513, 1023, 1024,
+           1025, 1300, 2049]
+
+
+def edge_graph(rng, n, chain):
+    """Nodes 0.. have in-lists (chain = 0) or out-lists (1) of every length of
+    LENGTHS, between others of 0..9 entries."""
+    src, dst = [], []
+    for v in range(n):
+        k = LENGTHS[v // 3] if v % 3 == 0 and v // 3 < len(LENGTHS) else int(rng.integers(0, 10))
+        u = rng.choice(n, min(k, n), replace=False)
+        src += list(u) if not chain else [v] * u.size
+        dst += [v] * u.size if not chain else list(u)
+    return np.array(src, np.int32), np.array(dst, np.int32)
+
+
+@pytest.mark.parametrize("prec", [N.OSP_PREC_FP64, N.OSP_PREC_FP32_ACC64])
+@pytest.mark.parametrize("chain", [0, 1])
+@pytest.mark.parametrize("n", [2300, 40011])
+def test_list_lengths_at_the_edges_of_the_step_forms(prec, chain, n):
+    rng = np.random.default_rng(n + chain)
+    src, dst = edge_graph(rng, n, chain)
+    seed = 3 * (len(LENGTHS) - 1)  # the longest row of the out-list graph
+    eng = N.Engine(precision=prec, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds([seed], C_RESTART)
+    st = eng.init_scores(1e-13)
+    g = O.Graph(n, src, dst)
+    r, _, _ = O.cpi(*g.csr(), seed, C_RESTART, 1e-13, force_iters=st["iterations"])
+    assert np.abs(eng.query() - r).sum() <= TOL[prec]
+    # one op (a frontier of one row), then rewrites of many lists
+    batches = W.edge_update_stream(src, dst, n, 1, 1, 0, seed=5)
+    batches += W.edge_update_stream(np.concatenate([src, batches[0]["u"]]),
+                                    np.concatenate([dst, batches[0]["v"]]), n, 2, 400, 400, seed=6)
+    for ops in batches:
+        st = eng.apply_updates(ops, 1e-12)
+        old = g.csr()
+        assert g.apply(ops) == -1
+        r, _, _, _ = O.osp(old, g.csr(), r, C_RESTART, 1e-12, force_iters=st["iterations"])
+        assert np.abs(eng.query() - r).sum() <= TOL[prec]
+    eng.close()
+
+
+def test_push_only_steps_reach_every_row_length():
+    """push_alpha so small that every step pushes: frontiers from one node to
+    all of them, rows of every length."""
+    n = 9000
+    rng = np.random.default_rng(8)
+    src, dst = edge_graph(rng, n, 1)
+    eng = N.Engine(precision=N.OSP_PREC_FP64, device=0, push_alpha=1e-9, push_beta=1e-9)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds([3 * (len(LENGTHS) - 1)], C_RESTART)
+    st = eng.init_scores(1e-12)
+    assert st["push_iterations"] == st["iterations"]
+    r, _, _ = O.cpi(*O.Graph(n, src, dst).csr(), 3 * (len(LENGTHS) - 1), C_RESTART, 1e-12,
+                    force_iters=st["iterations"])
+    assert np.abs(eng.query() - r).sum() <= 1e-10
+    eng.close()
