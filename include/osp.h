@@ -122,15 +122,17 @@ typedef struct {
                             0 = by row size (2 for rows of at most 256 bytes, i.e. 32 K x the
                             element size, else 1), 1 = each lane loads its columns of up to eight
                             rows into registers, 2 = whole rows are copied into a shared-memory
-                            ring by bulk asynchronous copies (cp.async.bulk, mbarrier). Results
+                            ring by bulk asynchronous copies (cp.async.bulk, mbarrier). bf16 rows
+                            of groups of up to 128 columns are staged in shared memory and
+                            summed by the tensor cores with 0 and 1. Results
                             are the same up to rounding order. */
     int32_t seed_group;  /* seed block: columns per column group of the pull steps (32, 64, 128
-                            or 256, at most Sp; 0 = 32 for bf16 gather rows, else Sp, one
-                            group). A pull step walks the graph
+                            or 256, at most Sp; 0 = 128 for bf16 gather rows of a graph of 2^19
+                            nodes or more, 64 of a smaller one, else Sp, one group). A pull step walks the graph
                             once per group that still has a running column, so groups whose
                             seeds have all stopped cost nothing; inside a group, a lane whose
                             columns have all stopped loads and stores nothing. With bf16 rows
-                            in 32-column groups (and more than 32 seeds) each call also orders
+                            in groups of up to 128 columns each call also orders
                             the columns into groups by offset size, largest first, and once
                             only the first 8 (4) of that order run, steps read compact 8 (4)
                             column rows. Results are the same up to rounding order. */

@@ -69,7 +69,6 @@ struct Ctl {
   long long n_dst_nz, n_src_nz;  // nodes with a nonempty in-list / out-list (pull plan)
   int epoch;                   // frontier mark of x(0); step i uses epoch + i
   int q_size[2];               // frontier queue lengths
-  unsigned int bar_count, bar_gen;
   int ctr[4];                  // dynamic work counters (one seed: by step number mod 4)
   int n_big;                   // push step: pieces of the long rows
   int iter, mode, push_iters, stop, pull_used, noconv;
@@ -82,6 +81,9 @@ struct Ctl {
   int grp[8];                  // ... and their indices, for the next pull step
   int narrow;                  // bf16 seed block: the next step runs on 4-column rows (see multi.cu)
   double c;
+  // grid barrier of the seed block, on lines of their own (every CTA polls bar_gen)
+  alignas(128) unsigned int bar_count;
+  alignas(128) unsigned int bar_gen;
 };
 
 constexpr int kMaxSeeds = 256;
@@ -105,7 +107,7 @@ struct Multi {
   void* y0; void* y1;  // [nc Sp] gather blocks (double, float or bf16), group-major
   void* e;             // [nc Sp] bf16 rounding residuals of the gather block (bf16 only)
   void* yn0; void* yn1;  // [nc 4] bf16 narrow gather rows: group slots 0..3 (packed bf16 blocks)
-  double* part;        // [kMaxGrid Sp] per-CTA |x| partials
+  double* part;        // [2 Sp] ||x||_1 per column of the current step, by step parity
   int* active;         // [Sp] 1 while the column still propagates
   int* touched;        // [Sp] 1: the column has a nonzero offset entry in this call
   int* col_iters;      // [Sp] steps run per column

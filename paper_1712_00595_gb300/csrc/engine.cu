@@ -450,13 +450,20 @@ osp_status finish_call(osp_ctx* ctx, int64_t m_before, osp_batch_stats* st) {
   return OSP_OK;
 }
 
+bool seed_mma(const osp_ctx* ctx, int precision, int KG);
+
 // The pull-step schedule in force: {task items, long-list threshold, piece,
 // node weight}; unset entries take the defaults of the seed count.
 const int* schedule(osp_ctx* ctx) {
   static const int single[4] = {kTaskItems, kHubThreshold, kHubPiece, 1};
   static const int multi[4] = {kTaskItems, kMultiHub, kMultiHub, kMultiNodeItems};
+  // tensor-core gathers: a piece costs atomics, a fence and a dozen dependent
+  // loads, so long ones (2^21 nodes, 256 seeds: 45.4 ms a batch with 256
+  // entries, 40.6 with 1,024); a node's finish weighs as much as 8 edges
+  static const int mma[4] = {kTaskItems, 1024, 1024, 8};
   if (ctx->sched[0] > 0) return ctx->sched;
-  return ctx->S > 1 ? multi : single;
+  if (ctx->S > 1) return seed_mma(ctx, ctx->opt.precision, ctx->d.mu.KG) ? mma : multi;
+  return single;
 }
 
 // Pull-step plan for the graph as it is after the merge: in-list length prefix
@@ -480,11 +487,13 @@ osp_status plan_pull(osp_ctx* ctx, int64_t n_bound, int64_t m_bound) {
   // two tasks a warp with one seed (down to 32 items: 10,000 nodes and 100,000
   // edges in double ran 82 us a step in 107 tasks of 1,024, 9.6 us in 3,437 of
   // 32, 12.9 us in 430 of 256), four with several (65,537 nodes, 10^6 edges,
-  // 17 seeds in double: 160 -> 110 us a step).
-  const bool many = ctx->S > 1;
-  const int want = many ? ctx->grid_multi * kPropWarps * 4 : ctx->grid_prop * kOneWarps * 2;
-  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], many ? 64 : 32,
-                                                std::min(kMaxSmallTasks, want));
+  // 17 seeds in double: 160 -> 110 us a step), two of at least 256 items where
+  // the tensor cores sum the rows (131,071 nodes, 1.5 M edges, 100 seeds: 456 us
+  // a batch with four of 64, 394 with two of 256).
+  const bool many = ctx->S > 1, mma = many && seed_mma(ctx, ctx->opt.precision, ctx->d.mu.KG);
+  const int warps = many ? ctx->grid_multi * kPropWarps : ctx->grid_prop * kOneWarps;
+  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], mma ? 256 : many ? 64 : 32,
+                                                std::min(kMaxSmallTasks, warps * (many && !mma ? 4 : 2)));
   ++ctx->launches;
   k_hub_prefix<<<1, 1024, 0, st>>>(ctx->d, sc[2], ctx->opt.deterministic != 0);
   ++ctx->launches;
@@ -537,7 +546,14 @@ bool seed_bulk(const osp_ctx* ctx, int precision, int KG) {
   if (ctx->opt.seed_gather != 0) return ctx->opt.seed_gather == 2;
   const int elem = precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
   const int row = 32 * KG * elem;
+  if (precision == OSP_PREC_BF16_ACC64 && KG <= 4) return false;  // tensor cores (seed_mma)
   return row >= 128 && row <= 256;
+}
+
+// bf16 groups of up to 128 columns are summed by the tensor cores unless bulk
+// copies are asked for.
+bool seed_mma(const osp_ctx* ctx, int precision, int KG) {
+  return precision == OSP_PREC_BF16_ACC64 && KG <= 4 && !seed_bulk(ctx, precision, KG);
 }
 
 // The persistent propagation kernel of one call.
@@ -552,10 +568,10 @@ osp_status enqueue_propagate(osp_ctx* ctx, const PropParams& pp, bool init) {
     p.hot_n = hot_rows(ctx, prec, KG);
     const bool bulk = seed_bulk(ctx, prec, KG);
     Dev d = ctx->d;
-    // bf16 32-column groups gathered by teams: the columns are packed into
-    // groups per call, largest offsets first, so that the columns still running
+    // groups summed by the tensor cores: the columns are packed into groups
+    // per call, largest offsets first, so that the columns still running
     // after the first steps share few groups
-    d.mu.pack = prec == OSP_PREC_BF16_ACC64 && KG == 1 && !bulk && d.mu.Sp > 32;
+    d.mu.pack = seed_mma(ctx, prec, KG);
     CK(launch_propagate_multi(d, p, prec, KG, as_init ? ctx->grid_multi_init : ctx->grid_multi,
                               bulk, ctx->stream));
   }
@@ -1319,7 +1335,7 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
       ML(yn0, (size_t)ctx->nc * 16);
       ML(yn1, (size_t)ctx->nc * 16);
     }
-    ML(M.part, (size_t)kMaxGrid * 32 * K);
+    ML(M.part, 2 * 32 * K);
     ML(M.active, 32 * K);
     ML(M.touched, 32 * K);
     ML(M.col_iters, 32 * K);
@@ -1341,11 +1357,15 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
     M.yn0 = yn0;
     M.yn1 = yn1;
     M.hub_acc = hub;
-    // column groups: 32 columns for bf16 gather rows (64-byte slices; measured
-    // 8 ms per pass at R-MAT 2^24 against 28.7 ms for one masked 256-column
-    // pass), else one group of all Sp columns, unless the options say
+    // column groups: one group of all Sp columns, but for bf16 gather rows 128
+    // columns from 2^19 nodes on and 64 below (steps over 128 columns share the
+    // ids and memberships of an edge among more values, but keep only two row
+    // stages in flight a warp: 2^21 nodes, 256 seeds 1,624 against 1,930 us a
+    // step, 2^20 nodes, 128 seeds 634 against 727; 131,071 nodes, 100 seeds 60
+    // against 48), unless the options say
     const int g = ctx->opt.seed_group > 0 ? ctx->opt.seed_group
-                  : ctx->opt.precision == OSP_PREC_BF16_ACC64 ? 32 : 32 * K;
+                  : ctx->opt.precision == OSP_PREC_BF16_ACC64 ? (ctx->n >= (1 << 19) ? 128 : 64)
+                                                              : 32 * K;
     M.KG = std::max(1, std::min(K, g / 32));
     M.KG_init = ctx->opt.seed_group > 0 ? M.KG : K;
     CK(cudaMemcpyAsync(M.seeds, by_col.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, ctx->stream));

@@ -187,8 +187,6 @@ template <> struct Feedback<__nv_bfloat16> { static constexpr bool on = true; };
 // Registers of one warp lane: KG columns of one column group.
 template <typename TY, int KG>
 struct ColGroup {
-  static constexpr int G = 32 * KG;                      // columns of a group
-  static constexpr int kRowBytes = G * (int)sizeof(TY);  // a group's slice of a gather row
   // rows gathered per batch of loads (more when a lane's share is small)
   static constexpr int kDepth = KG * (int)sizeof(TY) <= 8 ? 16 : 8;
 };
@@ -300,101 +298,206 @@ __device__ __forceinline__ A scale_of(const Dev& d, int v) {
   return std::is_same<A, double>::value ? (A)__ldg(d.scale_d + v) : (A)__ldg(d.scale_f + v);
 }
 
+__device__ __forceinline__ void bf16x4(uint2 x, float* f) {
+  f[0] = __uint_as_float(x.x << 16);
+  f[1] = __uint_as_float(x.x & 0xFFFF0000u);
+  f[2] = __uint_as_float(x.y << 16);
+  f[3] = __uint_as_float(x.y & 0xFFFF0000u);
+}
+
+__device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
+  return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
+         ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+}
+
+// (double)x for a normal x in four integer operations: the conversion itself
+// runs at the double rate, 16 cycles of the SM per warp. Step values are finite
+// (|x| <= 2); a subnormal one (below 2^-126) comes out below 2^-125.
+__device__ __forceinline__ double widen(float x) {
+  const int b = __float_as_int(x);
+  return __hiloint2double(((b >> 3) & 0x8FFFFFFF) + 0x38000000, b << 29);
+}
+
 // ---------------------------------------------------------------------------
-// Team gather for bf16 rows of a 32-column group (64 bytes). The warp works as
-// 4 teams of 8 lanes; lane (team t, sub s) loads columns [4 s, 4 s + 4) of a
-// row (8 bytes), so one load instruction brings 4 rows. A window is 32
-// consecutive positions of an edge stream (the in-lists of a run of nodes, or
-// one piece of a long in-list); team t takes positions 8 t .. 8 t + 7 of it.
-// Ids are loaded two windows ahead and rows one window ahead, so that up to
-// 64 rows per warp are in flight whatever the list lengths.
+// Tensor-core gather for bf16 rows of a group of G = 32 KG columns (64 KG
+// bytes). Summing the gathered rows of each node is the product of the rows with
+// a 0/1 matrix "edge belongs to node": for 16 edges and 8 nodes, mma.m16n8k16
+//   A = rows transposed (m = columns, G / 16 tiles; k = edges),
+//   B = membership      (k = edges, n = nodes, entries 1.0 or 0.0),
+//   D = sums            (m = columns, n = nodes, float accumulation).
+// Products with 1.0 and 0.0 are exact, the sums are float sums. A warp keeps a
+// ring of kStages stages of 16 rows in shared memory: cp.async brings the rows
+// in (16 bytes a lane, no registers held), ldmatrix.trans takes them out as A
+// fragments, and a membership entry is one comparison of the edge's node number.
+// Adding the rows in lanes took 13 warp instructions per edge and 32 columns
+// (four conversions and two packed additions a row and lane, a node test, a
+// flush per run); this form takes about 2. The kernel had been bound by
+// instruction issue: with all memory traffic cut out it ran 25% faster only.
+// tcgen05.mma reads both operands from shared memory and its sums from tensor
+// memory; at 8 nodes a tile the membership operand alone would cost more stores
+// than the rows, so the register-fed form is used.
+// Rows of running columns are finite (|x| <= 2), so a zero entry never makes one
+// NaN; whatever a stopped column holds stays in its own row of D, unused.
 // ---------------------------------------------------------------------------
-struct TeamWin {
-  uint2 v[8];  // this lane's 4 columns of its team's 8 rows (bf16 pairs)
+__device__ __forceinline__ void cp_async16(unsigned smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Shared memory of one warp.
+template <int KG>
+struct MmaWarp {
+  static constexpr int G = 32 * KG;
+  static constexpr int kRow = 2 * G;                    // bytes of a row
+  static constexpr int kChunks = kRow / 16;             // 16-byte chunks of a row
+  // 16 warps an SM (registers), with the ring that leaves room for: 227 KB
+  static constexpr int kStages = KG == 4 ? 2 : 4;
+  static constexpr int kWarps = 8;  // of a CTA
+  static constexpr int kCtas = 2;   // per SM
+  static constexpr int kStageBytes = 16 * kRow;
+  alignas(128) unsigned char rows[kStages * kStageBytes];
+  alignas(16) float acc[8][G + 4];  // sums of eight nodes, by node and slot
+  alignas(16) unsigned words[4][32];  // edges of four windows: row | node of the run << 25
+  alignas(8) uint2 lists[32];       // nonempty lists of a run: pool offset - position, node << 25
 };
 
-__device__ __forceinline__ void team_load(TeamWin& w, int idx, const __nv_bfloat16* ysg, bool on,
-                                          const L2Pol& pol, unsigned long long cold, int hot_n) {
-  const int lane = threadIdx.x & 31;
-  const int base = lane & 24, sub = lane & 7;
+// Byte offset of 16-byte chunk ch of row r in a stage, swizzled so that eight
+// consecutive rows' chunks lie in different banks.
+template <int KG>
+__device__ __forceinline__ int row_chunk(int r, int ch) {
+  const int sw = KG == 1 ? ch ^ ((r >> 1) & 3) : (ch & 8) | ((ch ^ r) & 7);
+  return r * (64 * KG) + 16 * sw;
+}
+
+// 32-slot parts of a group up to its last running column (am: running slots).
+template <int KG>
+__device__ __forceinline__ int running_parts(const unsigned* am) {
+  int p = 1;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int u = __shfl_sync(0xffffffffu, idx, base + k);
-    w.v[k] = make_uint2(0u, 0u);
-    if (on && u >= 0) {
-      const unsigned long long pp = u < hot_n ? pol.keep : cold;
-      asm volatile("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
-                   : "=r"(w.v[k].x), "=r"(w.v[k].y)
-                   : "l"(ysg + (size_t)u * 32 + 4 * sub), "l"(pp));
+  for (int k = 1; k < KG; ++k)
+    if (am[k]) p = k + 1;
+  return p;
+}
+
+// Copy the rows of words w[0 .. 16) into a stage (chunks with a running column).
+template <int KG>
+__device__ __forceinline__ void stage_rows(unsigned stage, const unsigned* w, const char* src,
+                                           bool on) {
+  using W = MmaWarp<KG>;
+  constexpr int kPer = W::kChunks / 2;  // rows a lane copies its chunk of
+  const int lane = threadIdx.x & 31;
+  const int r0 = lane / W::kChunks * kPer, ch = lane % W::kChunks;
+  if (on) {
+    const char* from = src + 16 * ch;
+#pragma unroll
+    for (int i = 0; i < kPer; i += 2) {
+      const uint2 u = *reinterpret_cast<const uint2*>(w + r0 + i);
+      cp_async16(stage + row_chunk<KG>(r0 + i, ch), from + (size_t)(u.x & 0x1FFFFFFu) * W::kRow);
+      cp_async16(stage + row_chunk<KG>(r0 + i + 1, ch), from + (size_t)(u.y & 0x1FFFFFFu) * W::kRow);
     }
   }
 }
 
-// acc (4 columns) += one row slice of 4 bf16 values (the low half of each
-// 32-bit word is the lower column); two packed f32x2 additions.
-__device__ __forceinline__ void team_add(float (&acc)[4], uint2 x) {
-  unsigned long long a01, a23, v01, v23;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(a01) : "f"(acc[0]), "f"(acc[1]));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(a23) : "f"(acc[2]), "f"(acc[3]));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v01) : "r"(x.x << 16), "r"(x.x & 0xFFFF0000u));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v23) : "r"(x.y << 16), "r"(x.y & 0xFFFF0000u));
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a01) : "l"(v01));
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a23) : "l"(v23));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[0]), "=f"(acc[1]) : "l"(a01));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2]), "=f"(acc[3]) : "l"(a23));
+// Membership of two edges in a node: two bf16 ones or zeros.
+__device__ __forceinline__ unsigned member2(uint2 u, unsigned node) {
+  return ((u.x >> 25) == node ? 0x3F80u : 0u) | ((u.y >> 25) == node ? 0x3F800000u : 0u);
 }
 
-// Sum of the rows of one piece of a long in-list (ids p[0 .. L)). Returns, in
-// the lanes of team 0 (sub s: columns [4 s, 4 s + 4)), the sums over the
-// whole piece; other lanes hold partial sums.
-__device__ __forceinline__ void team_piece(const int* p, int L, const __nv_bfloat16* ysg, bool on,
-                                           const L2Pol& pol, unsigned long long cold, int hot_n,
-                                           float (&acc)[4]) {
+// d += the 16 rows of a stage for membership (b0, b1). Tile f of d: d[4 f],
+// d[4 f + 1] = slot 16 f + g of nodes 2 t, 2 t + 1; d[4 f + 2], d[4 f + 3] = slot
+// 16 f + 8 + g. Only the first `parts` 32-slot parts are summed.
+template <int KG>
+__device__ __forceinline__ void mma_stage(float (&d)[8 * KG], unsigned stage, unsigned b0, unsigned b1,
+                                          int parts) {
   const int lane = threadIdx.x & 31;
-  const int nwin = (L + 31) >> 5;
-  auto id_of = [&](int i) -> int {
-    const int q = i * 32 + lane;
-    return (i < nwin && q < L) ? __ldg(p + q) : -1;
+  const int r = (lane & 7) + 8 * (lane >> 4), c = (lane >> 3) & 1;
+#pragma unroll
+  for (int f = 0; f < 2 * KG; ++f) {
+    if (f >= 2 * parts) break;  // warp-uniform: no column of the later parts runs
+    unsigned a0, a1, a2, a3;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3)
+                 : "r"(stage + row_chunk<KG>(r, 2 * f + c))
+                 : "memory");
+    float* t = d + 4 * f;
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(t[0]), "+f"(t[1]), "+f"(t[2]), "+f"(t[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+}
+
+// A stream of E >= 1 edges, 32 a window, through the ring: word_at(w) gives lane
+// = position of window w its word (any valid row for positions past the end, no
+// node), eat(h, words, stage) consumes half window h.
+template <int KG, typename WordF, typename EatF>
+__device__ __forceinline__ void mma_ring(int E, MmaWarp<KG>& W, const char* src, bool on, WordF word_at,
+                                         EatF eat) {
+  using MW = MmaWarp<KG>;
+  constexpr int S = MW::kStages;
+  const int lane = threadIdx.x & 31;
+  const int nh = (E + 15) >> 4, nwin = (E + 31) >> 5;
+  const unsigned rows = smem_u32(W.rows);
+  unsigned n0 = word_at(0), n1 = nwin > 1 ? word_at(1) : 0u;
+  auto issue = [&](int s) {
+    if (s < nh) {
+      const int w = s >> 1;
+      if (!(s & 1)) {
+        W.words[w & 3][lane] = n0;
+        __syncwarp();
+        n0 = n1;
+        if (w + 2 < nwin) n1 = word_at(w + 2);
+      }
+      stage_rows<KG>(rows + (unsigned)(s % S) * MW::kStageBytes, W.words[w & 3] + 16 * (s & 1), src, on);
+    }
+    cp_async_commit();
   };
+  __syncwarp();  // the last stream's words and rows have been read
 #pragma unroll
-  for (int c = 0; c < 4; ++c) acc[c] = 0.f;
-  // ids run four windows ahead of the rows they name, rows one window ahead
-  // of the additions
-  int i0 = id_of(0), i1 = id_of(1), i2 = id_of(2), i3 = id_of(3);
-  TeamWin A, B;
-  team_load(A, i0, ysg, on, pol, cold, hot_n);
-  for (int i = 0; i < nwin; i += 2) {
-    const int i4 = id_of(i + 4);
-    if (i + 1 < nwin) team_load(B, i1, ysg, on, pol, cold, hot_n);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) team_add(acc, A.v[k]);
-    if (i + 1 >= nwin) break;
-    const int i5 = id_of(i + 5);
-    if (i + 2 < nwin) team_load(A, i2, ysg, on, pol, cold, hot_n);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) team_add(acc, B.v[k]);
-    i1 = i3;
-    i2 = i4;
-    i3 = i5;
+  for (int s = 0; s < S - 1; ++s) issue(s);
+  for (int h = 0; h < nh; ++h) {
+    cp_async_wait<S - 2>();
+    __syncwarp();  // stage h has landed for the whole warp, stage h - 1 has been read
+    issue(h + S - 1);
+    eat(h, W.words[(h >> 1) & 3] + 16 * (h & 1), rows + (unsigned)(h % S) * MW::kStageBytes);
   }
-  // the 4 teams' partial sums, combined in a fixed order
+}
+
+// Sum of the rows of one piece of a long in-list (ids p[0 .. L), L >= 1): in
+// the lanes with t = 0, d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
+template <int KG>
+__device__ __forceinline__ void mma_piece(const int* p, int L, const char* src, bool on, int parts,
+                                          MmaWarp<KG>& W, float (&d)[8 * KG]) {
+  const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 8);
-    acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 16);
-  }
+  for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
+  mma_ring<KG>(
+      L, W, src, on,
+      [&](int w) {  // the list is node 0 of the fragments
+        const int q = 32 * w + lane;
+        return (unsigned)__ldg(p + min(q, L - 1)) | (q < L ? 0u : 127u << 25);
+      },
+      [&](int, const unsigned* w, unsigned stage) {
+        const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
+        const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
+        mma_stage<KG>(d, stage, member2(u0, (unsigned)(lane >> 2)), member2(u1, (unsigned)(lane >> 2)),
+                      parts);
+      });
 }
 
 // The in-lists of a run of up to 32 nodes as one edge stream: lane j holds
-// node j's list length ll (0 to leave it out) and pool offset off; the sums
-// per node and column land in acc_s[j * 32 + column] (shared memory of this
-// warp, zeroed by the caller) through shared-memory atomics, one per column
-// and run of a node's rows inside a team.
-__device__ __forceinline__ void team_stream(const int* pool, int ll, unsigned off,
-                                            const __nv_bfloat16* ysg, bool on, const L2Pol& pol,
-                                            unsigned long long cold, int hot_n, float* acc_s) {
-  const int lane = threadIdx.x & 31;
-  const int base = lane & 24, sub = lane & 7;
+// node j's list length ll (0 to leave it out) and pool offset off. The run's
+// nodes are taken eight at a time: finish(c, d) gets the sums of nodes 8 c ..
+// 8 c + 7 (fragments as in mma_stage), in order, once each.
+template <int KG, typename F>
+__device__ __forceinline__ void mma_stream(const int* pool, int ll, unsigned off, const char* src,
+                                           bool on, int parts, MmaWarp<KG>& W, F finish) {
+  const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
   int incl = ll;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -403,80 +506,48 @@ __device__ __forceinline__ void team_stream(const int* pool, int ll, unsigned of
   }
   const int P = incl - ll;
   const int E = __shfl_sync(0xffffffffu, incl, 31);
-  if (E == 0) return;
-  const int nwin = (E + 31) >> 5;
-  // position q of the stream: node j = the last lane with P_j <= q, id from its list
-  auto at = [&](int i, int& node) -> int {
-    const int q = i * 32 + lane;
-    int j = 0;
+  float d[8 * KG];
 #pragma unroll
-    for (int b = 16; b >= 1; b >>= 1) {
-      const int Pc = __shfl_sync(0xffffffffu, P, j + b);
-      if (Pc <= q) j += b;
-    }
-    const int Pj = __shfl_sync(0xffffffffu, P, j);
-    const unsigned oj = __shfl_sync(0xffffffffu, off, j);
-    node = -1;
-    if (i >= nwin || q >= E) return -1;
-    node = j;
-    return __ldg(pool + oj + (unsigned)(q - Pj));
-  };
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  int cur = -1;
-  // edge: the current node has rows at the first or last row of one of this
-  // team's runs, so other teams or windows may hold rows of it too (its sum
-  // goes in by atomic additions); a node met only inside one run belongs to
-  // this team alone and its sum is stored once
-  bool edge = false;
-  auto flush = [&]() {
-    if (cur >= 0 && on) {
-      float* a = acc_s + cur * 32 + 4 * sub;
-      if (edge) {
+  for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
+  int c = 0;  // eight nodes being summed, and the stream position after them
+  int Ec = __shfl_sync(0xffffffffu, incl, 7);
+  if (E > 0) {
+    __syncwarp();  // the last run's list table has been read
+    const unsigned full = __ballot_sync(0xffffffffu, ll > 0);
+    if (ll > 0) W.lists[__popc(full & lanemask_lt())] = make_uint2(off - (unsigned)P, (unsigned)lane << 25);
+    __syncwarp();
+    int started = -1;  // rank of the list that runs into the next window
+    mma_ring<KG>(
+        E, W, src, on,
+        [&](int w) -> unsigned {  // windows come in order
+          const unsigned at = (unsigned)(P - 32 * w);
+          const unsigned hm = __reduce_or_sync(0xffffffffu, ll > 0 && at < 32u ? 1u << at : 0u);
+          const int q = 32 * w + lane;
+          const uint2 l = W.lists[started + __popc(hm & (lanemask_lt() | (1u << lane)))];
+          started += __popc(hm);
+          // the sum wraps back; positions past the end repeat the last edge, for no node
+          const unsigned u = (unsigned)__ldg(pool + (l.x + (unsigned)min(q, E - 1)));
+          return u | (q < E ? l.y : 127u << 25);
+        },
+        [&](int h, const unsigned* w, unsigned stage) {
+          const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
+          const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
+          for (;;) {
+            if (Ec > 16 * h) {
+              const unsigned node = (unsigned)(8 * c + (lane >> 2));
+              mma_stage<KG>(d, stage, member2(u0, node), member2(u1, node), parts);
+            }
+            if (Ec > 16 * h + 16) break;  // goes on in the next half window
+            finish(c, d);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) atomicAdd(a + c, acc[c]);
-      } else {
-        *reinterpret_cast<float4*>(a) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[c] = 0.f;
-  };
-  auto eat = [&](const TeamWin& w, int nodes) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int jj = __shfl_sync(0xffffffffu, nodes, base + k);
-      if (jj != cur) {
-        flush();
-        cur = jj;
-        edge = k == 0;
-      }
-      team_add(acc, w.v[k]);
-    }
-    edge = true;  // the run's last node may go on in the next team or window
-  };
-  // ids (and nodes) run four windows ahead of the rows they name, rows one
-  // window ahead of the additions
-  int n0, n1, n2, n3, n4, n5;
-  int i0 = at(0, n0), i1 = at(1, n1), i2 = at(2, n2), i3 = at(3, n3);
-  TeamWin A, B;
-  team_load(A, i0, ysg, on, pol, cold, hot_n);
-  for (int i = 0; i < nwin; i += 2) {
-    const int i4 = at(i + 4, n4);
-    if (i + 1 < nwin) team_load(B, i1, ysg, on, pol, cold, hot_n);
-    eat(A, n0);
-    if (i + 1 >= nwin) break;
-    const int i5 = at(i + 5, n5);
-    if (i + 2 < nwin) team_load(A, i2, ysg, on, pol, cold, hot_n);
-    eat(B, n1);
-    n0 = n2;
-    n1 = n3;
-    n2 = n4;
-    n3 = n5;
-    i1 = i3;
-    i2 = i4;
-    i3 = i5;
+            for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
+            if (++c == 4) break;
+            Ec = __shfl_sync(0xffffffffu, incl, 8 * c + 7);
+          }
+        });
+  } else {
+    for (; c < 4; ++c) finish(c, d);
   }
-  flush();
 }
 
 // ---------------------------------------------------------------------------
@@ -494,19 +565,13 @@ __device__ __forceinline__ void team_stream(const int* pool, int ll, unsigned of
 template <int W>
 struct Narrow {
   const __nv_bfloat16* src;  // gather rows of the previous step (row u at src + u stride)
-  int stride;                // its row length: 32 (group 0 of the group layout), 8 or 4
+  int stride;                // its row length: that of a group (group 0), 8 or 4
   __nv_bfloat16* dst;        // next compact rows ([node][W])
   __nv_bfloat16* e;          // residual rows (group 0 of the group layout, slots 0..W-1 used)
+  int estride;               // ... and their length
   int col[W];                // columns of R held by slots 0..W-1
   unsigned act;              // bit c: column col[c] runs
 };
-
-__device__ __forceinline__ void bf16x4(uint2 x, float* f) {
-  f[0] = __uint_as_float(x.x << 16);
-  f[1] = __uint_as_float(x.x & 0xFFFF0000u);
-  f[2] = __uint_as_float(x.y << 16);
-  f[3] = __uint_as_float(x.y & 0xFFFF0000u);
-}
 
 template <int W>
 struct NRow;
@@ -532,11 +597,6 @@ struct NRow<8> {
   }
 };
 
-__device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
-  return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
-         ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
-}
-
 // Node v's sums x: R += x (running columns), |x| into l1, next compact row and
 // residual w = x s + e_old (when v has out-edges).
 template <int W>
@@ -552,7 +612,7 @@ __device__ __forceinline__ void narrow_finish(const Narrow<W>& N, const Multi& M
       }
   }
   if (s != 0.f) {
-    __nv_bfloat16* ep = N.e + (size_t)v * 32;
+    __nv_bfloat16* ep = N.e + (size_t)v * N.estride;
     NRow<W> eo;
     eo.load(ep);
     float e[W], y[W], r[W];
@@ -749,63 +809,36 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
   }
 }
 
-// 16-byte asynchronous copy global -> shared (L2 only), and the wait for this
-// thread's copies.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-// Whole last CTA: per-column sums of the partials (fixed order over CTAs),
-// per-column stopping, the call's stop, the column groups still running and
+// Whole last CTA: per-column stopping from the step's column sums (added up by
+// the CTAs' atomics: summing per-CTA partials here cost 456 double additions a
+// column, 30 us a step of 256 columns at 16 cycles a warp), the call's stop, the column groups still running and
 // the history entry (max over the columns that ran the step). A column whose
 // x(0) is exactly zero has only zero terms: under the eps rule its one
 // do-while step is counted and it stops at once.
-// s_sum (kPropThreads doubles) and s_key (kMaxSeeds doubles) are shared-memory
-// scratch of the caller (buffers that are idle at the grid barrier).
+// s_key (kMaxSeeds doubles) is shared-memory scratch of the caller (a buffer
+// that is idle at the grid barrier).
 template <int KG>
-__device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long long m, double* s_sum,
+__device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long long m,
                              double* s_key) {
   constexpr int G = 32 * KG;
   const Multi& M = d.mu;
   const int Sp = M.Sp;
   Ctl* ctl = d.ctl;
-  __shared__ double s_max[kPropThreads / 32];
+  __shared__ double s_max[32];
   __shared__ unsigned s_gmask;
   __shared__ int s_maxslot;
   if (threadIdx.x == 0) {
     s_gmask = 0;
     s_maxslot = -1;
   }
-  const bool pack = M.pack != 0 && KG == 1;
-  // thread t sums column t % Sp over the CTAs b = t / Sp (mod Q) with eight
-  // independent accumulators; the Q slices are then added in a fixed order
-  const int Q = (int)blockDim.x / Sp;
-  const int GR = (int)gridDim.x;
-  {
-    const int jc = threadIdx.x % Sp, q = threadIdx.x / Sp;
-    double a[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) a[u] = 0.0;
-    if (q < Q)
-      for (int b = q; b < GR; b += 8 * Q) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int bb = b + u * Q;
-          if (bb < GR) a[u] += __ldcg(M.part + (size_t)bb * Sp + jc);
-        }
-      }
-    s_sum[threadIdx.x] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-  }
+  const bool pack = M.pack != 0;
   __syncthreads();
   double seen = 0.0;
   int live = 0;
   for (int j = threadIdx.x; j < Sp; j += blockDim.x) {
-    double L = 0.0;
-    for (int q = 0; q < Q; ++q) L += s_sum[q * Sp + j];
+    double* tot = M.part + (it & 1) * Sp + j;
+    const double L = __ldcg(tot);
+    *tot = 0.0;
     if (j >= M.S) continue;
     const int f = pp.force_iters > 0 ? pp.force_iters : M.force[j];
     if (it == 0) {
@@ -873,7 +906,7 @@ __device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long lo
   const int any = __syncthreads_or(live);
   if (threadIdx.x == 0) {
     double mx = 0.0;
-    for (int i = 0; i < kPropWarps; ++i) mx = fmax(mx, s_max[i]);
+    for (int i = 0; i < (int)blockDim.x / 32; ++i) mx = fmax(mx, s_max[i]);
     if (it < kMaxHist) {
       d.l1_hist[it] = mx;
       d.step_ns[it + 1] = global_ns();
@@ -1245,18 +1278,11 @@ __global__ void k_gather_col(const double* __restrict__ r, int Sp, int col,
     out[i] = r[(size_t)ext2int[i] * Sp + col];
 }
 
-// CTAs per SM the seed-block kernel is built for: the team gather of bf16
-// 32-column groups is built for OSP_TEAM_OCC (default 3; measured 7.3 ms per
-// group pass at R-MAT 2^24 against 8.8 ms with 2) CTAs; otherwise three when a
-// lane's share of a gather row is at most 4 bytes (few registers), else two.
-#ifndef OSP_TEAM_OCC
-#define OSP_TEAM_OCC 3
-#endif
+// CTAs per SM the generic seed-block kernel is built for: three when a lane's
+// share of a gather row is at most 4 bytes (few registers), else two.
 template <typename TY, int KG>
 struct MultiOcc {
-  static constexpr int value = std::is_same<TY, __nv_bfloat16>::value && KG == 1
-                                   ? OSP_TEAM_OCC
-                                   : (KG * (int)sizeof(TY) <= 4 ? 3 : 2);
+  static constexpr int value = KG * (int)sizeof(TY) <= 4 ? 3 : 2;
 };
 
 // The seed block, one persistent cooperative launch per call: the x(0) pass
@@ -1277,16 +1303,8 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
   using A = typename AccOf<TY>::type;
   constexpr int G = 32 * KG;
   constexpr bool FB = Feedback<TY>::on;
-  // bf16 rows of 32-column groups are gathered by teams of 8 lanes over a flat
-  // edge stream (team_stream / team_piece); the other forms walk node by node
-  constexpr bool kTeam = std::is_same<TY, __nv_bfloat16>::value && KG == 1 && !kBulk;
-  __shared__ __align__(16) float s_team_acc[kTeam ? kPropWarps * 1024 : 1];  // node x column sums
-  __shared__ __align__(16) __nv_bfloat16 s_team_e[kTeam ? kPropWarps * 1024 : 8];  // residual rows
   __shared__ BarShared sh;
   __shared__ double s_part[kMaxSeeds];  // per column |x| sums of the CTA (shared-memory atomics)
-  // the decision's scratch: the team node sums (idle at the grid barrier), else its own
-  __shared__ double s_dec_own[kTeam ? 1 : kPropThreads + kMaxSeeds];
-  double* s_dec = kTeam ? reinterpret_cast<double*>(s_team_acc) : s_dec_own;
   __shared__ int s_grp[8];
   __shared__ int s_ngrp;
   __shared__ unsigned s_tmask;
@@ -1310,15 +1328,10 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
   }
   const Multi& M = d.mu;
   const int Sp = M.Sp;
-  // packed groups (bf16 team path): group slot q holds column slot_col[q],
-  // chosen per call by the x(0) decision so that columns likely to run long
-  // share groups; R, the offsets and the per-column state stay by column
-  const bool pack = kTeam && M.pack != 0;
   const size_t gs = (size_t)d.nc * G;  // gather block: elements per column group
   const int n = ctl->n;
   const long long m = ctl->m;
   const int epoch = ctl->epoch;
-  const int n_hubs = ctl->n_hubs;
   const int n_pieces = ctl->n_pieces;
   const int n_tasks = ctl->n_tasks;
   const int hub_thr = ctl->hub_thr, hub_piece = ctl->hub_piece;
@@ -1327,103 +1340,26 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
   const unsigned long long cold = hot_n > 0 ? pol.once : pol.normal;
   TY* yb[2] = {(TY*)M.y0, (TY*)M.y1};
   TY* eb = (TY*)M.e;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   double* my_part = s_part;
   if (blockIdx.x == 0 && threadIdx.x == 0) d.step_ns[0] = global_ns();
 
-  // per-CTA column sums of the warps' partials (fixed order) into M.part
-  auto column_sums = [&]() {
+  // the CTA's column sums into the step's totals (by step parity; the decision
+  // clears them for the step after next)
+  auto column_sums = [&](int it) {
     __syncthreads();
     for (int j = threadIdx.x; j < Sp; j += blockDim.x) {
-      double a = 0.0;
-      a = s_part[j];
-      M.part[(size_t)blockIdx.x * Sp + j] = a;
+      const double a = s_part[j];
+      if (a != 0.0) atomicAdd(M.part + (it & 1) * Sp + j, a);
     }
-    __threadfence();
   };
 
   // x(0): stamped rows move from xacc into R and, scaled, into y(0); every
   // node with out-edges gets its y(0) row (zero when not stamped) in each
   // column group that has a nonzero offset entry
-  if (pack) {
-    // 1. ||x(0)||_1 per column from the stamped rows; the decision orders the
-    //    columns by it (largest first: a larger offset needs more steps) into
-    //    group slots and picks the groups that hold a running column
-    for (int j = lane; j < Sp; j += 32) my_part[j] = 0.0;
-    unsigned tb = 0;  // bit k: column lane + 32 k has an offset entry
-    for (int k = 0; k < 8 && lane + 32 * k < M.S; ++k)
-      if (*(volatile int*)&M.touched[lane + 32 * k]) tb |= 1u << k;
-    __syncthreads();
-    for (int vb = gw * 32; vb < n && __any_sync(0xffffffffu, tb != 0); vb += nw * 32) {
-      const int vl = vb + lane;
-      unsigned stamped = __ballot_sync(0xffffffffu, vl < n && __ldcg(d.mark + vl) == epoch);
-      while (stamped) {
-        const int v = vb + __ffs(stamped) - 1;
-        stamped &= stamped - 1;
-        for (unsigned t = tb; t; t &= t - 1) {
-          const int j = lane + 32 * (__ffs(t) - 1);
-          atomicAdd(my_part + j, fabs(__ldcg(M.xacc + (size_t)v * Sp + j)));
-        }
-      }
-    }
-    column_sums();
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, s_dec, s_dec + kPropThreads);
-    if (!bar_release(ctl, sh)) return;
-    // 2. R += x(0) and the y(0) rows, in group slots
-    if (threadIdx.x < 8) s_grp[threadIdx.x] = *(volatile int*)&ctl->grp[threadIdx.x];
-    if (threadIdx.x == 0) s_ngrp = *(volatile int*)&ctl->n_grp;
-    __syncthreads();
-    const int ng = s_ngrp;
-    int colg[8];
-    unsigned actg = 0;  // bit gi: this lane's column of group s_grp[gi] runs
-#pragma unroll
-    for (int gi = 0; gi < 8; ++gi) {
-      colg[gi] = 0;
-      if (gi < ng) {
-        colg[gi] = __ldcg(M.slot_col + s_grp[gi] * G + lane);
-        if (*(volatile int*)&M.active[colg[gi]]) actg |= 1u << gi;
-      }
-    }
-    for (int vb = gw * 32; vb < n && ng > 0; vb += nw * 32) {
-      const int vl = vb + lane;
-      const unsigned stamped = __ballot_sync(0xffffffffu, vl < n && __ldcg(d.mark + vl) == epoch);
-      const A s_l = vl < n ? scale_of<A>(d, vl) : (A)0;
-      unsigned work = stamped | __ballot_sync(0xffffffffu, s_l != (A)0);
-      while (work) {
-        const int jj = __ffs(work) - 1;
-        work &= work - 1;
-        const int v = vb + jj;
-        const bool st = (stamped >> jj) & 1u;
-        const A s = __shfl_sync(0xffffffffu, s_l, jj);
-#pragma unroll
-        for (int gi = 0; gi < 8; ++gi) {
-          if (gi >= ng || !((actg >> gi) & 1u)) continue;
-          const size_t ybase = s_grp[gi] * gs + (size_t)v * G + lane;
-          TY yv = from_acc((A)0, (TY*)nullptr), ev = yv;
-          if (st) {
-            const size_t rb = (size_t)v * Sp + colg[gi];
-            const double x = __ldcg(M.xacc + rb);
-            if (x != 0.0) {
-              M.r[rb] += x;
-              M.xacc[rb] = 0.0;
-              const A w = (A)((A)x * s);
-              yv = from_acc(w, (TY*)nullptr);
-              if constexpr (FB) ev = __float2bfloat16_rn(w - __bfloat162float(yv));
-            }
-          }
-          if (s != (A)0) {
-            const TY y1[1] = {yv}, e1[1] = {ev};
-            st_pol(yb[0] + ybase, y1, pol.once);
-            if constexpr (FB) st_pol(eb + ybase, e1, pol.once);
-          }
-        }
-      }
-    }
-    if (bar_arrive(ctl, sh) && threadIdx.x == 0) ctl->ctr[1] = 0;
-    if (!bar_release(ctl, sh)) return;
-  } else {
+  {
     if (threadIdx.x == 0) s_tmask = 0;
     for (int j = lane; j < Sp; j += 32) my_part[j] = 0.0;
     __syncthreads();
@@ -1486,13 +1422,12 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
         }
       }
     }
-    column_sums();
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, s_dec, s_dec + kPropThreads);
+    column_sums(0);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, nullptr);
     if (!bar_release(ctl, sh)) return;
   }
 
   A* hub_acc = (A*)M.hub_acc;
-  int prev_narrow = 0;  // row width of the compact block the last step wrote (0: none)
   for (int it = 1;; ++it) {
     if (*(volatile int*)&ctl->stop) break;
     if (threadIdx.x < 8) s_grp[threadIdx.x] = *(volatile int*)&ctl->grp[threadIdx.x];
@@ -1503,13 +1438,8 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
     TY* yd = yb[it & 1];
     const int n_items = n_pieces + n_tasks;
     const long long total = (long long)s_ngrp * n_items;
-    // the groups of a step are gathered side by side: they share the L2
-    // budget for hot rows
-    const int hot_step = s_ngrp > 1 ? hot_n / s_ngrp : hot_n;
     int cur = -1;  // column group of the items this warp works on now
-    int pcol = -1;  // packed bf16 groups: this lane's column in group cur
     unsigned act = 0;
-    bool on4 = false;
     double l1[KG];
 #pragma unroll
     for (int k = 0; k < KG; ++k) l1[k] = 0.0;
@@ -1517,43 +1447,11 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
       if (cur >= 0) {
 #pragma unroll
         for (int k = 0; k < KG; ++k) {
-          atomicAdd(my_part + (kTeam && pack ? pcol : cur * G + lane * KG) + k, l1[k]);
+          atomicAdd(my_part + cur * G + lane * KG + k, l1[k]);
           l1[k] = 0.0;
         }
       }
     };
-    int narrow = 0;  // row width of a narrow step (0: a step over column groups)
-    if constexpr (kTeam) narrow = *(volatile int*)&ctl->narrow;
-    if constexpr (kTeam) {
-      if (narrow) {
-        __nv_bfloat16* yn[2] = {(__nv_bfloat16*)M.yn0, (__nv_bfloat16*)M.yn1};
-        const __nv_bfloat16* src =
-            prev_narrow ? yn[(it - 1) & 1] : reinterpret_cast<const __nv_bfloat16*>(ys);
-        const int stride = prev_narrow ? prev_narrow : 32;
-        float* acc_s = s_team_acc + wid * 1024;
-        if (narrow == 4) {
-          Narrow<4> N{src, stride, yn[it & 1], reinterpret_cast<__nv_bfloat16*>(eb), {}, 0u};
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            N.col[c] = __ldcg(M.slot_col + c);
-            if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
-          }
-          narrow_step<4>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, (float*)hub_acc, acc_s,
-                         my_part, ctl);
-        } else {
-          Narrow<8> N{src, stride, yn[it & 1], reinterpret_cast<__nv_bfloat16*>(eb), {}, 0u};
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            N.col[c] = __ldcg(M.slot_col + c);
-            if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
-          }
-          narrow_step<8>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, (float*)hub_acc, acc_s,
-                         my_part, ctl);
-        }
-      }
-    }
-    prev_narrow = narrow;
-    if (!narrow)
     for (int k = 0;; ++k) {
       int t = gw;  // the first item is the warp's own number, later ones come from the counter
       if (k > 0) {
@@ -1571,22 +1469,14 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
         flush();
         cur = g;
         act = 0;
-        if constexpr (kTeam) pcol = pack ? __ldcg(M.slot_col + g * G + lane) : g * G + lane;
 #pragma unroll
         for (int k = 0; k < KG; ++k)
-          act |= (unsigned)(*(volatile int*)&M.active[(kTeam ? pcol : g * G + lane * KG) + k] != 0)
-                 << k;
-        if constexpr (kTeam) {
-          // team gathers: lane (t, s) loads columns [4 s, 4 s + 4) of a row
-          const unsigned am = __ballot_sync(0xffffffffu, act != 0);
-          on4 = ((am >> (4 * (lane & 7))) & 0xFu) != 0;
-        }
+          act |= (unsigned)(*(volatile int*)&M.active[g * G + lane * KG + k] != 0) << k;
       }
       const TY* ysg = ys + g * gs;           // the group's gather rows, G elements apart
       const TY* ysl = ysg + lane * KG;       // this lane's columns of them
       const size_t c0 = (size_t)g * G + lane * KG;  // slot: gather rows, residuals, hub sums
-      const size_t rc0 = kTeam ? (size_t)pcol : c0;  // column of R
-      auto rbase_of = [&](int v) { return (size_t)v * Sp + rc0; };
+      auto rbase_of = [&](int v) { return (size_t)v * Sp + c0; };
       auto ybase_of = [&](int v) { return g * gs + (size_t)v * G + lane * KG; };
       if (ti < n_pieces) {
         // a piece of a long in-list; the piece that completes the list finishes it
@@ -1596,41 +1486,6 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
         const int full = __ldg(d.len_c + v);
         const int* p = d.pool_c + __ldg(d.off_c + v) + (unsigned)(piece * hub_piece);
         const int L = min(hub_piece, full - piece * hub_piece);
-        if constexpr (kTeam) {
-          float a4[4];
-          team_piece(p, L, ysg, on4, pol, cold, hot_step, a4);
-          float* ha4 = (float*)hub_acc + (size_t)h * Sp + (size_t)g * G + 4 * lane;
-          if (lane < 8 && on4) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) atomicAdd(ha4 + c, a4[c]);
-          }
-          __threadfence();
-          int last = 0;
-          if (lane == 0) {
-            const int np = (full + hub_piece - 1) / hub_piece;
-            last = atomicAdd(&M.hub_cnt[h * 8 + g], 1) == np - 1;
-          }
-          last = __shfl_sync(0xffffffffu, last, 0);
-          if (last) {
-            __threadfence();
-            float* hx = (float*)hub_acc + (size_t)h * Sp + c0;  // lane = column
-            const float x = __ldcg(hx);
-            *hx = 0.f;
-            if (lane == 0) M.hub_cnt[h * 8 + g] = 0;
-            const float sv = scale_of<float>(d, v);
-            if (act) {
-              red_add_once(M.r + rbase_of(v), (double)x, pol.once);
-              l1[0] += fabs((double)x);
-              if (sv != 0.f) {
-                const float w = x * sv + __bfloat162float(eb[ybase_of(v)]);
-                const __nv_bfloat16 yv = __float2bfloat16_rn(w);
-                yd[ybase_of(v)] = yv;
-                eb[ybase_of(v)] = __float2bfloat16_rn(w - __bfloat162float(yv));
-              }
-            }
-          }
-          continue;
-        }
         A acc[KG];
 #pragma unroll
         for (int k = 0; k < KG; ++k) acc[k] = (A)0;
@@ -1669,75 +1524,6 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
       }
       const int task = ti - n_pieces;
       const int c0t = __ldg(d.task_first + task), c1t = __ldg(d.task_first + task + 1);
-      if constexpr (kTeam) {
-        float* acc_s = s_team_acc + wid * 1024;
-        __nv_bfloat16* e_s = s_team_e + wid * 1024;
-        // list lengths, offsets and scales of the next run of 32 nodes load
-        // while the current run is summed
-        int nx_len = 0;
-        unsigned nx_off = 0;
-        float nx_s = 0.f;
-        auto header = [&](int vb) {
-          const int vl = vb + lane;
-          nx_len = 0;
-          nx_off = 0;
-          nx_s = 0.f;
-          if (vl < c1t) {
-            nx_len = __ldg(d.len_c + vl);
-            nx_off = __ldg(d.off_c + vl);
-            nx_s = scale_of<float>(d, vl);
-          }
-        };
-        header(c0t);
-        for (int vb = c0t; vb < c1t; vb += 32) {
-          const int vl = vb + lane;
-          const int my_len = nx_len;
-          const unsigned my_off = nx_off;
-          const float my_s = nx_s;
-          if (vb + 32 < c1t) header(vb + 32);
-          const bool mine = vl < c1t && my_len <= hub_thr;  // hubs go by pieces
-          const unsigned fin = __ballot_sync(0xffffffffu, mine && (my_len > 0 || my_s != 0.f));
-          if (!fin) continue;
-          // this node's residual row (all 32 columns) into shared memory, in flight
-          // while the stream runs
-          if (((fin >> lane) & 1u) && my_s != 0.f) {
-            const __nv_bfloat16* er = eb + g * gs + (size_t)vl * G;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cp_async16(e_s + lane * 32 + 8 * q, er + 8 * q);
-          }
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            reinterpret_cast<float4*>(acc_s)[lane + 32 * q] = make_float4(0.f, 0.f, 0.f, 0.f);
-          __syncwarp();
-          team_stream(d.pool_c, mine ? my_len : 0, my_off, ysg, on4, pol, cold, hot_step, acc_s);
-          cp_async_wait_all();
-          __syncwarp();
-          // finish: lane = column; |x| of the run summed in float (at most 32
-          // nonnegative terms), then added to the FP64 partial once
-          float l1f = 0.f;
-          for (unsigned fb = fin; fb; fb &= fb - 1) {
-            const int j = __ffs(fb) - 1;
-            const int v = vb + j;
-            const float sj = __shfl_sync(0xffffffffu, my_s, j);
-            const bool has_in = __shfl_sync(0xffffffffu, my_len, j) > 0;
-            if (!act) continue;
-            const float x = acc_s[j * 32 + lane];
-            if (has_in) {
-              red_add_once(M.r + rbase_of(v), (double)x, pol.once);
-              l1f += fabsf(x);
-            }
-            if (sj != 0.f) {
-              const float w = x * sj + __bfloat162float(e_s[j * 32 + lane]);
-              const __nv_bfloat16 yv = __float2bfloat16_rn(w);
-              yd[ybase_of(v)] = yv;
-              eb[ybase_of(v)] = __float2bfloat16_rn(w - __bfloat162float(yv));
-            }
-          }
-          l1[0] += (double)l1f;
-          __syncwarp();
-        }
-        continue;
-      }
       for (int vb = c0t; vb < c1t; vb += 32) {
         // offsets, lengths and scales of up to 32 consecutive nodes, coalesced
         const int vl = vb + lane;
@@ -1912,8 +1698,378 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
       }
     }
     flush();
-    column_sums();
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, s_dec, s_dec + kPropThreads);
+    column_sums(it);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, nullptr);
+    if (!bar_release(ctl, sh)) return;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->epoch = epoch + 1;
+}
+
+
+// The bf16 seed block on the tensor cores, one persistent cooperative launch per
+// call. Columns are packed into groups of G = 32 KG slots: slot q holds column
+// slot_col[q], chosen per call by the x(0) decision so that columns likely to
+// run long share groups; R, the offsets and the per-column state stay by column,
+// gather rows, residuals and partial sums by slot. A work item (a piece of a
+// long in-list, or a task of consecutive nodes) is taken by one warp for all
+// groups with a running column when there are several items a warp, so that its
+// ids and headers come from L1 for the later groups; else for one group.
+template <int KG>
+__global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) k_propagate_mma(Dev d, PropParams pp) {
+  constexpr int G = 32 * KG;
+  __shared__ double s_part[kMaxSeeds];  // |x| of this step per column (shared-memory atomics)
+  __shared__ double s_key[kMaxSeeds];
+  __shared__ int s_col[kMaxSeeds];      // column of each slot
+  __shared__ unsigned s_am[kMaxSeeds / 32];  // running slots
+  __shared__ BarShared sh;
+  __shared__ int s_grp[8];
+  __shared__ int s_ngrp;
+  extern __shared__ __align__(128) unsigned char dsm[];
+  Ctl* ctl = d.ctl;
+  if (*(volatile int*)&ctl->status) return;
+  const Multi& M = d.mu;
+  const int Sp = M.Sp;
+  const size_t gs = (size_t)d.nc * G;  // gather block: elements per column group
+  const int n = ctl->n;
+  const long long m = ctl->m;
+  const int epoch = ctl->epoch;
+  const int n_pieces = ctl->n_pieces;
+  const int n_tasks = ctl->n_tasks;
+  const int hub_thr = ctl->hub_thr, hub_piece = ctl->hub_piece;
+  const L2Pol pol = make_l2pol();
+  __nv_bfloat16* yb[2] = {(__nv_bfloat16*)M.y0, (__nv_bfloat16*)M.y1};
+  __nv_bfloat16* eb = (__nv_bfloat16*)M.e;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  MmaWarp<KG>& W = reinterpret_cast<MmaWarp<KG>*>(dsm)[wid];
+  double* my_part = s_part;
+  for (int j = threadIdx.x; j < Sp; j += blockDim.x) s_part[j] = 0.0;
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) d.step_ns[0] = global_ns();
+
+  // the CTA's column sums into the step's totals (by step parity; the decision
+  // clears them for the step after next)
+  auto column_sums = [&](int it) {
+    __syncthreads();
+    for (int j = threadIdx.x; j < Sp; j += blockDim.x) {
+      const double a = s_part[j];
+      s_part[j] = 0.0;
+      if (a != 0.0) atomicAdd(M.part + (it & 1) * Sp + j, a);
+    }
+  };
+
+  // 1. ||x(0)||_1 per column from the stamped rows; the decision orders the
+  //    columns by it (largest first: a larger offset needs more steps) into
+  //    group slots and picks the groups that hold a running column
+  unsigned tb = 0;  // bit k: column lane + 32 k has an offset entry
+  for (int k = 0; k < 8 && lane + 32 * k < M.S; ++k)
+    if (*(volatile int*)&M.touched[lane + 32 * k]) tb |= 1u << k;
+  __syncthreads();
+  double l0[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) l0[k] = 0.0;
+  for (int vb = gw * 32; vb < n && __any_sync(0xffffffffu, tb != 0); vb += nw * 32) {
+    const int vl = vb + lane;
+    unsigned stamped = __ballot_sync(0xffffffffu, vl < n && __ldcg(d.mark + vl) == epoch);
+    for (; stamped; stamped &= stamped - 1) {
+      const int v = vb + __ffs(stamped) - 1;
+      double x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        x[k] = (tb >> k) & 1u ? __ldcg(M.xacc + (size_t)v * Sp + lane + 32 * k) : 0.0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if ((tb >> k) & 1u) l0[k] += fabs(x[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if ((tb >> k) & 1u) atomicAdd(my_part + lane + 32 * k, l0[k]);
+  column_sums(0);
+  if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, s_key);
+  if (!bar_release(ctl, sh)) return;
+  // 2. R += x(0) and the y(0) rows, in group slots
+  if (threadIdx.x < 8) s_grp[threadIdx.x] = *(volatile int*)&ctl->grp[threadIdx.x];
+  if (threadIdx.x == 0) s_ngrp = *(volatile int*)&ctl->n_grp;
+  __syncthreads();
+  const int ng = s_ngrp;
+  // a lane's slots are lane, lane + 32, ...: 32-slot parts q of the groups
+  int colq[8];
+  unsigned actq = 0;  // bit q: this lane's column of part q runs
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    colq[q] = 0;
+    if (32 * q < Sp) {
+      colq[q] = __ldcg(M.slot_col + 32 * q + lane);
+      if (*(volatile int*)&M.active[colq[q]]) actq |= 1u << q;
+    }
+  }
+  for (int vb = gw * 32; vb < n && ng > 0; vb += nw * 32) {
+    const int vl = vb + lane;
+    const unsigned stamped = __ballot_sync(0xffffffffu, vl < n && __ldcg(d.mark + vl) == epoch);
+    const float s_l = vl < n ? scale_of<float>(d, vl) : 0.f;
+    // rows of nodes without an offset entry start at zero: 16 bytes a lane,
+    // 8 / KG rows a store
+    const unsigned blank = __ballot_sync(0xffffffffu, s_l != 0.f) & ~stamped;
+    constexpr int kLanes = 4 * KG;  // lanes a row
+    for (int gi = 0; gi < ng && blank; ++gi) {
+      const size_t at = s_grp[gi] * gs + (size_t)vb * G + 8 * (lane % kLanes);
+#pragma unroll
+      for (int r = 0; r < kLanes; ++r) {
+        const int j = r * (32 / kLanes) + lane / kLanes;
+        if ((blank >> j) & 1u) {
+          *reinterpret_cast<uint4*>(yb[0] + at + (size_t)j * G) = make_uint4(0u, 0u, 0u, 0u);
+          *reinterpret_cast<uint4*>(eb + at + (size_t)j * G) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+    }
+    for (unsigned work = stamped; work; work &= work - 1) {
+      const int jj = __ffs(work) - 1;
+      const int v = vb + jj;
+      const float s = __shfl_sync(0xffffffffu, s_l, jj);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (!((actq >> q) & 1u)) continue;
+        const size_t ybase = (q / KG) * gs + (size_t)v * G + 32 * (q % KG) + lane;
+        __nv_bfloat16 yv = __float2bfloat16_rn(0.f), ev = yv;
+        const size_t rb = (size_t)v * Sp + colq[q];
+        const double x = __ldcg(M.xacc + rb);
+        if (x != 0.0) {
+          M.r[rb] += x;
+          M.xacc[rb] = 0.0;
+          const float w = (float)x * s;
+          yv = __float2bfloat16_rn(w);
+          ev = __float2bfloat16_rn(w - __bfloat162float(yv));
+        }
+        if (s != 0.f) {
+          const __nv_bfloat16 y1[1] = {yv}, e1[1] = {ev};
+          st_pol(yb[0] + ybase, y1, pol.once);
+          st_pol(eb + ybase, e1, pol.once);
+        }
+      }
+    }
+  }
+  if (bar_arrive(ctl, sh) && threadIdx.x == 0) ctl->ctr[1] = 0;
+  if (!bar_release(ctl, sh)) return;
+
+  float* hub_acc = (float*)M.hub_acc;
+  int prev_narrow = 0;  // row width of the compact block the last step wrote (0: none)
+  for (int it = 1;; ++it) {
+    if (*(volatile int*)&ctl->stop) break;
+    if (threadIdx.x < 8) s_grp[threadIdx.x] = *(volatile int*)&ctl->grp[threadIdx.x];
+    if (threadIdx.x == 0) s_ngrp = *(volatile int*)&ctl->n_grp;
+    for (int q = threadIdx.x; q < Sp; q += blockDim.x) {  // warps whole: Sp is a multiple of 32
+      const int col = __ldcg(M.slot_col + q);
+      const unsigned a = __ballot_sync(0xffffffffu, *(volatile int*)&M.active[col] != 0);
+      s_col[q] = col;
+      if (lane == 0) s_am[q >> 5] = a;
+    }
+    __syncthreads();
+    const __nv_bfloat16* ys = yb[(it - 1) & 1];
+    __nv_bfloat16* yd = yb[it & 1];
+    const int n_items = n_pieces + n_tasks;
+    const int narrow = *(volatile int*)&ctl->narrow;  // row width of a narrow step (0: over groups)
+    if (narrow) {
+      __nv_bfloat16* yn[2] = {(__nv_bfloat16*)M.yn0, (__nv_bfloat16*)M.yn1};
+      const __nv_bfloat16* src =
+          prev_narrow ? yn[(it - 1) & 1] : ys;
+      const int stride = prev_narrow ? prev_narrow : G;
+      float* acc_s = &W.acc[0][0];
+      static_assert(sizeof(W.acc) >= 256 * sizeof(float), "sums of a narrow run");
+      if (narrow == 4) {
+        Narrow<4> N{src, stride, yn[it & 1], eb, G, {}, 0u};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          N.col[c] = __ldcg(M.slot_col + c);
+          if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
+        }
+        narrow_step<4>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
+                       my_part, ctl);
+      } else {
+        Narrow<8> N{src, stride, yn[it & 1], eb, G, {}, 0u};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          N.col[c] = __ldcg(M.slot_col + c);
+          if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
+        }
+        narrow_step<8>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
+                       my_part, ctl);
+      }
+    }
+    prev_narrow = narrow;
+    const int ng = s_ngrp;
+    const bool whole = n_items >= 4 * nw;  // an item's groups by one warp
+    const int total = narrow ? 0 : whole ? n_items : n_items * ng;
+    for (int k = 0;; ++k) {
+      int t = gw;  // the first item is the warp's own number, later ones come from the counter
+      if (k > 0) {
+        if (total <= nw) break;
+        if (lane == 0) t = nw + atomicAdd(&ctl->ctr[1], 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+      }
+      if (t >= total) break;
+      const int ti = whole ? t : t / ng;
+      const int g0 = whole ? 0 : t - ti * ng, g1 = whole ? ng : g0 + 1;
+      if (ti < n_pieces) {
+        // a piece of a long in-list; the piece that completes the list finishes it
+        const int h = __ldg(d.piece_hub + ti);
+        const int v = __ldg(d.hubs + h);
+        const int piece = ti - __ldg(d.hub_pstart + h);
+        const int full = __ldg(d.len_c + v);
+        const int* p = d.pool_c + __ldg(d.off_c + v) + (unsigned)(piece * hub_piece);
+        const int L = min(hub_piece, full - piece * hub_piece);
+        const int np = (full + hub_piece - 1) / hub_piece;
+        for (int gi = g0; gi < g1; ++gi) {
+          const int g = s_grp[gi];
+          const unsigned* am = s_am + g * KG;
+          const int ch = lane % MmaWarp<KG>::kChunks;  // the chunk this lane copies
+          float D[8 * KG];
+          mma_piece<KG>(p, L, reinterpret_cast<const char*>(ys + g * gs),
+                        ((am[ch >> 2] >> (8 * (ch & 3))) & 0xFFu) != 0, running_parts<KG>(am), W, D);
+          float* ha = hub_acc + (size_t)h * Sp + g * G;
+          if ((lane & 3) == 0) {
+            const int fg = lane >> 2;
+#pragma unroll
+            for (int f = 0; f < 4 * KG; ++f)
+              if ((am[f >> 2] >> (8 * (f & 3) + fg)) & 1u) atomicAdd(ha + 8 * f + fg, D[2 * f]);
+          }
+          __threadfence();
+          int last = 0;
+          if (lane == 0) last = atomicAdd(&M.hub_cnt[h * 8 + g], 1) == np - 1;
+          last = __shfl_sync(0xffffffffu, last, 0);
+          if (last) {
+            __threadfence();
+            if (lane == 0) M.hub_cnt[h * 8 + g] = 0;
+            const float sv = scale_of<float>(d, v);
+#pragma unroll
+            for (int k = 0; k < KG; ++k) {  // lane = slot
+              const float x = __ldcg(ha + 32 * k + lane);
+              ha[32 * k + lane] = 0.f;
+              if (!((am[k] >> lane) & 1u)) continue;
+              const int col = s_col[g * G + 32 * k + lane];
+              red_add_once(M.r + (size_t)v * Sp + col, (double)x, pol.once);
+              atomicAdd(my_part + col, fabs((double)x));
+              if (sv != 0.f) {
+                const size_t at = g * gs + (size_t)v * G + 32 * k + lane;
+                const float w = x * sv + __bfloat162float(eb[at]);
+                const __nv_bfloat16 yv = __float2bfloat16_rn(w);
+                yd[at] = yv;
+                eb[at] = __float2bfloat16_rn(w - __bfloat162float(yv));
+              }
+            }
+          }
+        }
+        continue;
+      }
+      const int task = ti - n_pieces;
+      const int c0t = __ldg(d.task_first + task), c1t = __ldg(d.task_first + task + 1);
+      for (int gi = g0; gi < g1; ++gi) {
+        const int g = s_grp[gi];
+        const unsigned* am = s_am + g * KG;
+        const int* scol = s_col + g * G;
+        const char* src = reinterpret_cast<const char*>(ys + g * gs);
+        const int ch = lane % MmaWarp<KG>::kChunks;
+        const bool on = ((am[ch >> 2] >> (8 * (ch & 3))) & 0xFFu) != 0;
+        const int parts = running_parts<KG>(am);
+        // list lengths, offsets and scales of the next run of 32 nodes load
+        // while the current run is summed
+        int nx_len = 0;
+        unsigned nx_off = 0;
+        float nx_s = 0.f;
+        auto header = [&](int vb) {
+          const int vl = vb + lane;
+          nx_len = 0;
+          nx_off = 0;
+          nx_s = 0.f;
+          if (vl < c1t) {
+            nx_len = __ldg(d.len_c + vl);
+            nx_off = __ldg(d.off_c + vl);
+            nx_s = scale_of<float>(d, vl);
+          }
+        };
+        header(c0t);
+        for (int vb = c0t; vb < c1t; vb += 32) {
+          const int my_len = nx_len;
+          const unsigned my_off = nx_off;
+          const float my_s = nx_s;
+          if (vb + 32 < c1t) header(vb + 32);
+          const bool mine = vb + lane < c1t && my_len <= hub_thr;  // hubs go by pieces
+          const unsigned fin = __ballot_sync(0xffffffffu, mine && (my_len > 0 || my_s != 0.f));
+          if (!fin) continue;
+          // |x| of the run summed in float (at most 32 nonnegative terms), then
+          // added to the FP64 partial once
+          float l1f[KG];
+#pragma unroll
+          for (int k = 0; k < KG; ++k) l1f[k] = 0.f;
+          mma_stream<KG>(
+              d.pool_c, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
+                if (!((fin >> (8 * c)) & 0xFFu)) return;  // warp-uniform
+                // the sums by node and slot (conflict-free: banks 8 t + g)
+                const int fg = lane >> 2, t2 = 2 * (lane & 3);
+#pragma unroll
+                for (int f = 0; f < 4 * KG; ++f) {
+                  if (f >= 4 * parts) break;
+                  W.acc[t2][8 * f + fg] = D[2 * f];
+                  W.acc[t2 + 1][8 * f + fg] = D[2 * f + 1];
+                }
+                // next gather row and residual: lane = node, every fourth
+                // chunk of four slots; the old residuals load first
+                const int j = lane >> 2, q = lane & 3;
+                const float sj = __shfl_sync(0xffffffffu, my_s, 8 * c + j);
+                const bool src_node = sj != 0.f && ((fin >> (8 * c + j)) & 1u);
+                const size_t at = g * gs + (size_t)(vb + 8 * c + j) * G + 4 * q;
+                uint2 eo[2 * KG];
+#pragma unroll
+                for (int i = 0; i < 2 * KG; ++i)
+                  eo[i] = src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu)
+                              ? __ldcg(reinterpret_cast<const uint2*>(eb + at + 16 * i))
+                              : make_uint2(0u, 0u);
+                __syncwarp();
+                // R += x: lane = slot (a node without in-list has x = 0)
+                double* rp = M.r + (size_t)(vb + 8 * c) * Sp;
+#pragma unroll
+                for (int k = 0; k < KG; ++k) {
+                  if (k >= parts) break;
+                  const bool run = (am[k] >> lane) & 1u;
+                  double* rk = rp + scol[32 * k + lane];
+#pragma unroll
+                  for (int jj = 0; jj < 8; ++jj) {
+                    const float x = W.acc[jj][32 * k + lane];
+                    if (run && x != 0.f) {
+                      red_add_once(rk, widen(x), pol.once);
+                      l1f[k] += fabsf(x);
+                    }
+                    rk += Sp;
+                  }
+                }
+#pragma unroll
+                for (int i = 0; i < 2 * KG; ++i) {
+                  if (i >= 2 * parts) break;
+                  if (!(src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu))) continue;
+                  const float4 x = *reinterpret_cast<const float4*>(&W.acc[j][16 * i + 4 * q]);
+                  const float w0 = x.x * sj + __uint_as_float(eo[i].x << 16);
+                  const float w1 = x.y * sj + __uint_as_float(eo[i].x & 0xFFFF0000u);
+                  const float w2 = x.z * sj + __uint_as_float(eo[i].y << 16);
+                  const float w3 = x.w * sj + __uint_as_float(eo[i].y & 0xFFFF0000u);
+                  const uint2 y = make_uint2(pack_bf16x2(w0, w1), pack_bf16x2(w2, w3));
+                  *reinterpret_cast<uint2*>(yd + at + 16 * i) = y;
+                  *reinterpret_cast<uint2*>(eb + at + 16 * i) =
+                      make_uint2(pack_bf16x2(w0 - __uint_as_float(y.x << 16),
+                                             w1 - __uint_as_float(y.x & 0xFFFF0000u)),
+                                 pack_bf16x2(w2 - __uint_as_float(y.y << 16),
+                                             w3 - __uint_as_float(y.y & 0xFFFF0000u)));
+                }
+                __syncwarp();  // acc is free again
+              });
+#pragma unroll
+          for (int k = 0; k < KG; ++k)
+            if (l1f[k] != 0.f) atomicAdd(my_part + scol[32 * k + lane], (double)l1f[k]);
+        }
+      }
+    }
+    column_sums(it);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, s_key);
     if (!bar_release(ctl, sh)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->epoch = epoch + 1;
@@ -1924,12 +2080,18 @@ namespace {
 struct MultiFn {
   const void* fn;
   int smem;  // dynamic shared memory bytes
+  int threads = kPropThreads;
 };
 
 template <typename TY, int KG>
 MultiFn multi_fn_k(bool bulk) {
   if (bulk) return {(const void*)k_propagate_multi<TY, KG, true>, RingCfg<TY, KG>::kSmem};
-  return {(const void*)k_propagate_multi<TY, KG, false>, 0};
+  // bf16 groups of up to 128 columns are summed by the tensor cores
+  if constexpr (std::is_same<TY, __nv_bfloat16>::value && KG <= 4)
+    return {(const void*)k_propagate_mma<KG>, MmaWarp<KG>::kWarps * (int)sizeof(MmaWarp<KG>),
+            32 * MmaWarp<KG>::kWarps};
+  else
+    return {(const void*)k_propagate_multi<TY, KG, false>, 0};
 }
 
 template <typename TY>
@@ -1956,7 +2118,7 @@ int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk) {
       cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem) != cudaSuccess)
     return 0;
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f.fn, kPropThreads, f.smem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f.fn, f.threads, f.smem) != cudaSuccess ||
       bps <= 0)
     return 0;
   bps = bps > 4 ? 4 : bps;
@@ -1970,7 +2132,7 @@ cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int preci
   PropParams p = pp;
   void* args[] = {&dd, &p};
   const MultiFn f = pick_multi(precision, KG, bulk);
-  return cudaLaunchCooperativeKernel(f.fn, dim3(grid), dim3(kPropThreads), args, (size_t)f.smem, s);
+  return cudaLaunchCooperativeKernel(f.fn, dim3(grid), dim3(f.threads), args, (size_t)f.smem, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -75,3 +75,40 @@ def test_push_only_steps_reach_every_row_length():
                     force_iters=st["iterations"])
     assert np.abs(eng.query() - r).sum() <= 1e-10
     eng.close()
+
+
+@pytest.mark.parametrize("S,group", [(20, 0), (64, 0), (100, 32), (100, 0), (100, 128), (200, 128),
+                                     (200, 256)])
+def test_bf16_blocks_at_the_edges_of_the_row_stages(S, group):
+    """bf16 seed blocks in every group width (tensor-core sums for 32, 64 and 128
+    columns, 256 by lanes): in-lists around the 16-row stages, the 32-edge
+    windows and the long-list pieces, in the oracle's lock-step, L1 <= 1e-5 a
+    seed (the bound of the seed-block tests)."""
+    n = 2300
+    rng = np.random.default_rng(S + group)
+    src, dst = edge_graph(rng, n, 0)
+    more = rng.integers(0, n, (2, 400))
+    for k, v in ((15, 201), (16, 204), (17, 207), (47, 210), (48, 213), (49, 216)):
+        u = rng.choice(n, k, replace=False)
+        src, dst = np.append(src, u), np.append(dst, np.full(k, v))
+    src, dst = np.append(src, more[0]).astype(np.int32), np.append(dst, more[1]).astype(np.int32)
+    seeds = rng.permutation(n)[:S].astype(np.int32)
+    eng = N.Engine(precision=N.OSP_PREC_BF16_ACC64, device=0, seed_group=group, node_order=S % 3 % 2)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(seeds, C_RESTART)
+    eng.init_scores(1e-11)
+    it0, _, _ = eng.get_seed_stats()
+    g = O.Graph(n, src, dst)
+    old = g.csr()
+    pick = list(range(0, S, max(1, S // 12)))
+    r = {j: O.cpi(*old, int(seeds[j]), C_RESTART, 1e-11, force_iters=int(it0[j]))[0] for j in pick}
+    for ops in W.edge_update_stream(src, dst, n, 2, 300, 300, seed=S):
+        eng.apply_updates(ops, 1e-9)
+        assert g.apply(ops) == -1
+        new = g.csr()
+        it, _, _ = eng.get_seed_stats()
+        for j in pick:
+            r[j], _, _, _ = O.osp(old, new, r[j], C_RESTART, 1e-9, force_iters=int(it[j]))
+            assert np.abs(eng.query(j) - r[j]).sum() <= 1e-5
+        old = new
+    eng.close()
