@@ -186,6 +186,8 @@ struct TopkState {
   int above;                  // keys above the bin (all of them are in the top k)
   int bin_count;              // keys inside the bin
   int keep;                   // bin keys kept (all, or the k_rem smallest ids of one key value)
+  int arrived;                // CTAs of the running histogram pass that are done
+  int ties;                   // the bin is one key value with too many holders: ids decide
   int pad;
   unsigned long long kmin;    // smallest and largest key matching the prefix in the last pass
   unsigned long long kmax;

@@ -861,9 +861,15 @@ osp_status enqueue_gather(osp_ctx* ctx, cudaStream_t st, const int* cols, double
       G.col[i] = cols[i];
       G.dst[i] = dsts[i];
     }
-    k_gather_cols<<<dim3(ctx->num_sms * 4, m), 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp,
-                                                            ctx->d.int2ext, n, G);
-    ++ctx->launches;
+    if (m >= 4) {
+      k_gather_cols<<<ctx->num_sms * 6, 128, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, ctx->d.int2ext, n, m, G);
+      ++ctx->launches;
+    }
+    for (int i = 0; i < m && m < 4; ++i) {
+      k_gather_col<<<ctx->num_sms * 8, 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, cols[i], ctx->d.int2ext,
+                                                     n, dsts[i]);
+      ++ctx->launches;
+    }
   } else {
     for (int i = 0; i < m; ++i) {
       k_gather_ext<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d.r, ctx->d.ext2int, n, dsts[i]);
@@ -1514,7 +1520,7 @@ osp_status scores_in_caller_order(osp_ctx* ctx, int col, int normalize, double* 
   const int n = (int)ctx->n;
   cudaStream_t st = ctx->stream;
   if (ctx->S > 1)
-    k_gather_col<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, col, ctx->d.ext2int, n, dst);
+    k_gather_col<<<ctx->num_sms * 8, 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, col, ctx->d.int2ext, n, dst);
   else
     k_gather_ext<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d.r, ctx->d.ext2int, n, dst);
   if (normalize) {

@@ -30,12 +30,14 @@ __global__ void k_gather_ext(const double* __restrict__ r, const int* __restrict
 __global__ void k_scale_copy(const double* r, int n, const double* __restrict__ sum, double* out);
 
 // Top-k (radix select + ordered compaction + one-CTA bitonic sort) over a job
-// table: enqueue_topk_select runs the selection and compaction (16 launches),
+// table: enqueue_topk_select runs the selection and collection (11 launches),
 // enqueue_topk_sort the final sort (k_topk_sort needs the dynamic shared
 // memory attribute set to kTopkSortSmem). Both return their launch counts.
 __global__ void k_topk_sort(TopkJobs J, int cap);
 __global__ void k_gather_cols(const double* __restrict__ r, int Sp, const int* __restrict__ int2ext,
-                              int n, GatherJobs G);
+                              int n, int m, GatherJobs G);
+__global__ void k_gather_col(const double* __restrict__ r, int Sp, int col,
+                             const int* __restrict__ int2ext, int n, double* out);
 int enqueue_topk_select(const TopkJobs& J, int num_sms, cudaStream_t st);
 int enqueue_topk_sort(const TopkJobs& J, cudaStream_t st);
 constexpr int kTopkMaxK = 4096;
@@ -50,8 +52,6 @@ __global__ void k_propagate(Dev d, PropParams pp);
 // Several seeds (csrc/multi.cu).
 __global__ void k_offset_multi_plan(Dev d);
 __global__ void k_multi_cpi_begin(Dev d);
-__global__ void k_gather_col(const double* __restrict__ r, int Sp, int col,
-                             const int* __restrict__ ext2int, int n, double* out);
 // bulk: the variant that stages source rows in shared memory by bulk copies.
 int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk);
 cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int precision, int KG,

@@ -1271,13 +1271,6 @@ __global__ void k_multi_cpi_begin(Dev d) {
   }
 }
 
-// Column col of R in caller order.
-__global__ void k_gather_col(const double* __restrict__ r, int Sp, int col,
-                             const int* __restrict__ ext2int, int n, double* out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    out[i] = r[(size_t)ext2int[i] * Sp + col];
-}
-
 // CTAs per SM the generic seed-block kernel is built for: three when a lane's
 // share of a gather row is at most 4 bytes (few registers), else two.
 template <typename TY, int KG>

@@ -112,3 +112,30 @@ def test_bf16_blocks_at_the_edges_of_the_row_stages(S, group):
             assert np.abs(eng.query(j) - r[j]).sum() <= 1e-5
         old = new
     eng.close()
+
+
+@pytest.mark.parametrize("n", [1, 255, 4097, 70001])
+def test_topk_of_awkward_vectors(n):
+    """Rankings where the radix passes, the collection and the one-CTA narrowing
+    change hands: ties at the cut (ids decide), more equal keys than a sort
+    holds, keys that differ in the last bits, k around 256 and at its limits."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    few = rng.integers(0, 3, n).astype(np.float64) * 0.25
+    near = 1.0 + rng.integers(0, 7, n) * 2.0 ** -52
+    wide = np.exp(rng.normal(-12, 6, n))
+    zeros = np.zeros(n)
+    zeros[rng.integers(0, n, min(n, 37))] = 0.5
+    for v in (few, near, wide, zeros, np.full(n, 1.0 / n)):
+        dv = torch.from_numpy(v).cuda()
+        for k in (1, 100, 255, 256, 257, 1000, 4096):
+            ids = torch.empty(k, dtype=torch.int32, device="cuda")
+            sc = torch.empty(k, dtype=torch.float64, device="cuda")
+            got = torch.zeros(1, dtype=torch.int32, device="cuda")
+            N.topk_noalloc(dv, n, k, ids, sc, got, stream=torch.cuda.current_stream().cuda_stream)
+            torch.cuda.synchronize()
+            c = int(got)
+            want_ids, want_sc = O.topk(v, k)
+            assert c == min(n, k)
+            assert np.array_equal(ids[:c].cpu().numpy(), want_ids)
+            assert np.array_equal(sc[:c].cpu().numpy(), want_sc)
