@@ -119,23 +119,22 @@ typedef struct {
                            2/4/8 with several seeds) on the first CPI steps and keeps the
                            fastest for every later call (osp_get_schedule reports it). */
     int32_t seed_gather; /* seed block (two or more seeds), how pull steps read source rows:
-                            0 = by row size (2 for rows of at most 256 bytes, i.e. 32 K x the
-                            element size, else 1), 1 = each lane loads its columns of up to eight
-                            rows into registers, 2 = whole rows are copied into a shared-memory
-                            ring by bulk asynchronous copies (cp.async.bulk, mbarrier). bf16 rows
-                            of groups of up to 128 columns are staged in shared memory and
-                            summed by the tensor cores with 0 and 1. Results
+                            2 = whole rows are copied into a shared-memory ring by bulk
+                            asynchronous copies (cp.async.bulk, mbarrier); 0 or 1 = through rings
+                            of 16-byte asynchronous copies where a group's row has 64 to 512 bytes
+                            (bf16 rows are then summed by the tensor cores with 0 and 1), else
+                            each lane loads its columns of up to eight rows into registers. Results
                             are the same up to rounding order. */
     int32_t seed_group;  /* seed block: columns per column group of the pull steps (32, 64, 128
-                            or 256, at most Sp; 0 = 128 for bf16 gather rows of a graph of 2^19
-                            nodes or more, 64 of a smaller one, else Sp, one group). A pull step walks the graph
+                            or 256, at most Sp; 0 = 64 for FP64 gather rows and for bf16 rows of a
+                            graph below 2^19 nodes, else 128). A pull step walks the graph
                             once per group that still has a running column, so groups whose
                             seeds have all stopped cost nothing; inside a group, a lane whose
-                            columns have all stopped loads and stores nothing. With bf16 rows
-                            in groups of up to 128 columns each call also orders
-                            the columns into groups by offset size, largest first, and once
-                            only the first 8 (4) of that order run, steps read compact 8 (4)
-                            column rows. Results are the same up to rounding order. */
+                            columns have all stopped loads and stores nothing. With row rings
+                            (see seed_gather) each call also orders the columns into groups by
+                            offset size, largest first; with bf16 rows and more than 32 seeds,
+                            once only the first 8 (4) of that order run, steps read compact 8
+                            (4) column rows. Results are the same up to rounding order. */
     int32_t deterministic; /* != 0 (one seed; osp_set_seeds with two or more returns
                               OSP_ENOTSUP): every propagation step pulls (no push steps, so
                               each costs a pass over all edges), warps take their work in a
@@ -145,7 +144,8 @@ typedef struct {
                               the same device and options then give the same bits in the
                               scores, the per-step norms and the statistics on every run.
                               autotune is ignored (a timed choice would change the bits). */
-    int64_t l2_hot_bytes; /* seed block with node_order 1: bytes of L2 given to the gather rows
+    int64_t l2_hot_bytes; /* seed block with node_order 1, rows gathered by lanes or bulk copies
+                             (see seed_gather): bytes of L2 given to the gather rows
                              of the highest out-degree nodes (kept in L2 before other lines);
                              0 = 60% of the device's L2, < 0 = none. */
     int64_t hbm_budget_bytes; /* device memory the context may allocate (graph store, score

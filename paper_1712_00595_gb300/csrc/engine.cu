@@ -450,19 +450,24 @@ osp_status finish_call(osp_ctx* ctx, int64_t m_before, osp_batch_stats* st) {
   return OSP_OK;
 }
 
-bool seed_mma(const osp_ctx* ctx, int precision, int KG);
+bool seed_ring(const osp_ctx* ctx, int precision, int KG);
 
 // The pull-step schedule in force: {task items, long-list threshold, piece,
 // node weight}; unset entries take the defaults of the seed count.
 const int* schedule(osp_ctx* ctx) {
   static const int single[4] = {kTaskItems, kHubThreshold, kHubPiece, 1};
   static const int multi[4] = {kTaskItems, kMultiHub, kMultiHub, kMultiNodeItems};
-  // tensor-core gathers: a piece costs atomics, a fence and a dozen dependent
-  // loads, so long ones (2^21 nodes, 256 seeds: 45.4 ms a batch with 256
-  // entries, 40.6 with 1,024); a node's finish weighs as much as 8 edges
+  // row rings: a piece costs atomics, a fence and a dozen dependent loads, so
+  // long ones (bf16, 2^21 nodes, 256 seeds: 45.4 ms a batch with 256 entries,
+  // 40.6 with 1,024; float, 2^18 nodes, 64 seeds: 181 us a step with 256, 173
+  // with 512), but not so long that their chain of double additions is the step
+  // (65,537 nodes, 17 seeds: 97 us with 512, 137 with 1,024). A bf16 node's
+  // finish weighs as much as 8 edges.
+  static const int ring[4] = {kTaskItems, 512, 512, kMultiNodeItems};
   static const int mma[4] = {kTaskItems, 1024, 1024, 8};
   if (ctx->sched[0] > 0) return ctx->sched;
-  if (ctx->S > 1) return seed_mma(ctx, ctx->opt.precision, ctx->d.mu.KG) ? mma : multi;
+  if (ctx->S > 1 && !seed_ring(ctx, ctx->opt.precision, ctx->d.mu.KG)) return multi;
+  if (ctx->S > 1) return ctx->opt.precision == OSP_PREC_BF16_ACC64 ? mma : ring;
   return single;
 }
 
@@ -490,10 +495,10 @@ osp_status plan_pull(osp_ctx* ctx, int64_t n_bound, int64_t m_bound) {
   // 17 seeds in double: 160 -> 110 us a step), two of at least 256 items where
   // the tensor cores sum the rows (131,071 nodes, 1.5 M edges, 100 seeds: 456 us
   // a batch with four of 64, 394 with two of 256).
-  const bool many = ctx->S > 1, mma = many && seed_mma(ctx, ctx->opt.precision, ctx->d.mu.KG);
+  const bool many = ctx->S > 1, bf16 = many && ctx->opt.precision == OSP_PREC_BF16_ACC64;
   const int warps = many ? ctx->grid_multi * kPropWarps : ctx->grid_prop * kOneWarps;
-  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], mma ? 256 : many ? 64 : 32,
-                                                std::min(kMaxSmallTasks, warps * (many && !mma ? 4 : 2)));
+  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], bf16 ? 256 : many ? 64 : 32,
+                                                std::min(kMaxSmallTasks, warps * (many && !bf16 ? 4 : 2)));
   ++ctx->launches;
   k_hub_prefix<<<1, 1024, 0, st>>>(ctx->d, sc[2], ctx->opt.deterministic != 0);
   ++ctx->launches;
@@ -537,23 +542,16 @@ int hot_rows(const osp_ctx* ctx, int precision, int KG) {
   return (int)std::min<int64_t>(rows, ctx->nc);
 }
 
-// Seed block of K column groups computed in `precision`: stage source rows by
-// bulk copies? By default only for rows of at most 256 bytes, where it was
-// measured faster (Chung-Lu 2^22, 64 FP32 seeds: 4.16 vs 6.08 ms per pull
-// step); rows of 512 bytes (R-MAT 2^24, 256 bf16 seeds) ran slower (30.7 vs
-// 26.3 ms) and keep register gathers.
-bool seed_bulk(const osp_ctx* ctx, int precision, int KG) {
-  if (ctx->opt.seed_gather != 0) return ctx->opt.seed_gather == 2;
-  const int elem = precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
-  const int row = 32 * KG * elem;
-  if (precision == OSP_PREC_BF16_ACC64 && KG <= 4) return false;  // tensor cores (seed_mma)
-  return row >= 128 && row <= 256;
+int elem_bytes(int precision) {
+  return precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
 }
 
-// bf16 groups of up to 128 columns are summed by the tensor cores unless bulk
-// copies are asked for.
-bool seed_mma(const osp_ctx* ctx, int precision, int KG) {
-  return precision == OSP_PREC_BF16_ACC64 && KG <= 4 && !seed_bulk(ctx, precision, KG);
+// How a seed block's pull steps read source rows: by bulk copies if the options
+// ask for them; else through row rings where a group's row fits (64 to 512
+// bytes), and by lane gathers where not.
+bool seed_bulk(const osp_ctx* ctx) { return ctx->opt.seed_gather == 2; }
+bool seed_ring(const osp_ctx* ctx, int precision, int KG) {
+  return !seed_bulk(ctx) && seed_ring_fits(elem_bytes(precision), KG);
 }
 
 // The persistent propagation kernel of one call.
@@ -566,12 +564,11 @@ osp_status enqueue_propagate(osp_ctx* ctx, const PropParams& pp, bool init) {
     const int KG = as_init ? ctx->d.mu.KG_init : ctx->d.mu.KG;
     PropParams p = pp;
     p.hot_n = hot_rows(ctx, prec, KG);
-    const bool bulk = seed_bulk(ctx, prec, KG);
+    const bool bulk = seed_bulk(ctx);
     Dev d = ctx->d;
-    // groups summed by the tensor cores: the columns are packed into groups
-    // per call, largest offsets first, so that the columns still running
+    // row rings: the columns are packed into groups per call, largest offsets first, so that the columns still running
     // after the first steps share few groups
-    d.mu.pack = seed_mma(ctx, prec, KG);
+    d.mu.pack = seed_ring(ctx, prec, KG);
     CK(launch_propagate_multi(d, p, prec, KG, as_init ? ctx->grid_multi_init : ctx->grid_multi,
                               bulk, ctx->stream));
   }
@@ -1363,24 +1360,24 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
     M.yn0 = yn0;
     M.yn1 = yn1;
     M.hub_acc = hub;
-    // column groups: one group of all Sp columns, but for bf16 gather rows 128
-    // columns from 2^19 nodes on and 64 below (steps over 128 columns share the
-    // ids and memberships of an edge among more values, but keep only two row
-    // stages in flight a warp: 2^21 nodes, 256 seeds 1,624 against 1,930 us a
-    // step, 2^20 nodes, 128 seeds 634 against 727; 131,071 nodes, 100 seeds 60
-    // against 48), unless the options say
+    // column groups: as many columns as a row of 512 bytes holds (float 128,
+    // double 64), for bf16 rows 128 from 2^19 nodes on and 64 below (steps over
+    // 128 columns share the ids and memberships of an edge among more values, but
+    // keep only two row stages in flight a warp: 2^21 nodes, 256 seeds 1,624
+    // against 1,930 us a step, 2^20 nodes, 128 seeds 634 against 727; 131,071
+    // nodes, 100 seeds 60 against 48), unless the options say
     const int g = ctx->opt.seed_group > 0 ? ctx->opt.seed_group
                   : ctx->opt.precision == OSP_PREC_BF16_ACC64 ? (ctx->n >= (1 << 19) ? 128 : 64)
-                                                              : 32 * K;
+                  : ctx->opt.precision == OSP_PREC_FP32_ACC64 ? 128 : 64;
     M.KG = std::max(1, std::min(K, g / 32));
-    M.KG_init = ctx->opt.seed_group > 0 ? M.KG : K;
+    M.KG_init = ctx->opt.seed_group > 0 ? M.KG : std::min(K, 4);
     CK(cudaMemcpyAsync(M.seeds, by_col.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, ctx->stream));
     const int prec_init =
         ctx->opt.precision == OSP_PREC_FP64 ? OSP_PREC_FP64 : OSP_PREC_FP32_ACC64;
     ctx->grid_multi = propagate_multi_grid(ctx->opt.precision, M.KG, ctx->num_sms,
-                                           seed_bulk(ctx, ctx->opt.precision, M.KG));
+                                           seed_bulk(ctx));
     ctx->grid_multi_init = propagate_multi_grid(prec_init, M.KG_init, ctx->num_sms,
-                                                seed_bulk(ctx, prec_init, M.KG_init));
+                                                seed_bulk(ctx));
     if (ctx->grid_multi <= 0 || ctx->grid_multi_init <= 0) {
       free_multi(ctx);
       return fail(ctx, OSP_ECUDA, "no resident grid for the seed-block kernel");

@@ -52,7 +52,10 @@ __global__ void k_propagate(Dev d, PropParams pp);
 // Several seeds (csrc/multi.cu).
 __global__ void k_offset_multi_plan(Dev d);
 __global__ void k_multi_cpi_begin(Dev d);
-// bulk: the variant that stages source rows in shared memory by bulk copies.
+// Group rows the row-ring kernel is built for (K columns a lane): 64 to 512 bytes.
+constexpr bool seed_ring_fits(int elem, int KG) { return KG <= 4 && 32 * KG * elem <= 512; }
+// bulk: the variant that stages source rows in shared memory by bulk copies;
+// else the row ring where its rows fit, lane gathers into registers where not.
 int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk);
 cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int precision, int KG,
                                    int grid, bool bulk, cudaStream_t s);

@@ -313,9 +313,27 @@ __device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
 // (double)x for a normal x in four integer operations: the conversion itself
 // runs at the double rate, 16 cycles of the SM per warp. Step values are finite
 // (|x| <= 2); a subnormal one (below 2^-126) comes out below 2^-125.
+__device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) {
   const int b = __float_as_int(x);
   return __hiloint2double(((b >> 3) & 0x8FFFFFFF) + 0x38000000, b << 29);
+}
+
+// K-element slice of a staged row (plain loads from shared memory).
+template <typename T, int K>
+__device__ __forceinline__ void load_k(const T* p, T (&out)[K]) {
+  constexpr int B = K * (int)sizeof(T);
+  if constexpr (B >= 16) {
+#pragma unroll
+    for (int i = 0; i < B / 16; ++i)
+      reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(p)[i];
+  } else if constexpr (B == 8) {
+    *reinterpret_cast<uint2*>(out) = *reinterpret_cast<const uint2*>(p);
+  } else if constexpr (B == 4) {
+    *reinterpret_cast<unsigned*>(out) = *reinterpret_cast<const unsigned*>(p);
+  } else {
+    *reinterpret_cast<unsigned short*>(out) = *reinterpret_cast<const unsigned short*>(p);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -348,19 +366,22 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Shared memory of one warp.
-template <int KG>
-struct MmaWarp {
+// Shared memory of one warp. Ring stages of kRs rows; 16 warps an SM
+// (registers), with as many stages as 227 KB then leave room for.
+template <typename TY, int KG>
+struct RingWarp {
+  static constexpr bool kMma = std::is_same<TY, __nv_bfloat16>::value;
   static constexpr int G = 32 * KG;
-  static constexpr int kRow = 2 * G;                    // bytes of a row
+  static constexpr int kRow = G * (int)sizeof(TY);      // bytes of a row
   static constexpr int kChunks = kRow / 16;             // 16-byte chunks of a row
-  // 16 warps an SM (registers), with the ring that leaves room for: 227 KB
-  static constexpr int kStages = KG == 4 ? 2 : 4;
+  static constexpr int kRs = kMma || kRow <= 256 ? 16 : 8;  // rows of a stage
+  static constexpr int kStageBytes = kRs * kRow;        // 1 to 4 KB
+  static constexpr int kStages = kMma ? (KG == 4 ? 2 : 4) : kStageBytes > 2048 ? 3 : 4;
   static constexpr int kWarps = 8;  // of a CTA
   static constexpr int kCtas = 2;   // per SM
-  static constexpr int kStageBytes = 16 * kRow;
+  static_assert(kChunks <= 32 && kRow * kRs <= 4096, "a stage is one chunk a lane, up to eight times");
   alignas(128) unsigned char rows[kStages * kStageBytes];
-  alignas(16) float acc[8][G + 4];  // sums of eight nodes, by node and slot
+  alignas(16) float acc[kMma ? 8 : 1][G + 4];  // bf16: sums of eight nodes, by node and slot
   alignas(16) unsigned words[4][32];  // edges of four windows: row | node of the run << 25
   alignas(8) uint2 lists[32];       // nonempty lists of a run: pool offset - position, node << 25
 };
@@ -383,12 +404,13 @@ __device__ __forceinline__ int running_parts(const unsigned* am) {
   return p;
 }
 
-// Copy the rows of words w[0 .. 16) into a stage (chunks with a running column).
-template <int KG>
+// Copy the rows of words w[0 .. kRs) into a stage (chunks with a running column).
+template <typename TY, int KG>
 __device__ __forceinline__ void stage_rows(unsigned stage, const unsigned* w, const char* src,
                                            bool on) {
-  using W = MmaWarp<KG>;
-  constexpr int kPer = W::kChunks / 2;  // rows a lane copies its chunk of
+  using W = RingWarp<TY, KG>;
+  constexpr int kPer = W::kRs * W::kChunks / 32;  // rows a lane copies its chunk of
+  static_assert(kPer % 2 == 0, "row words are read in pairs");
   const int lane = threadIdx.x & 31;
   const int r0 = lane / W::kChunks * kPer, ch = lane % W::kChunks;
   if (on) {
@@ -396,10 +418,20 @@ __device__ __forceinline__ void stage_rows(unsigned stage, const unsigned* w, co
 #pragma unroll
     for (int i = 0; i < kPer; i += 2) {
       const uint2 u = *reinterpret_cast<const uint2*>(w + r0 + i);
-      cp_async16(stage + row_chunk<KG>(r0 + i, ch), from + (size_t)(u.x & 0x1FFFFFFu) * W::kRow);
-      cp_async16(stage + row_chunk<KG>(r0 + i + 1, ch), from + (size_t)(u.y & 0x1FFFFFFu) * W::kRow);
+      const int c0 = W::kMma ? row_chunk<KG>(r0 + i, ch) : (r0 + i) * W::kRow + 16 * ch;
+      const int c1 = W::kMma ? row_chunk<KG>(r0 + i + 1, ch) : (r0 + i + 1) * W::kRow + 16 * ch;
+      cp_async16(stage + c0, from + (size_t)(u.x & 0x1FFFFFFu) * W::kRow);
+      cp_async16(stage + c1, from + (size_t)(u.y & 0x1FFFFFFu) * W::kRow);
     }
   }
+}
+
+// Does the chunk that this lane copies hold a running slot (am: running slots)?
+template <typename TY, int KG>
+__device__ __forceinline__ bool chunk_runs(const unsigned* am) {
+  constexpr int per = 16 / (int)sizeof(TY);  // slots of a chunk
+  const int q = (threadIdx.x & 31) % RingWarp<TY, KG>::kChunks * per;
+  return ((am[q >> 5] >> (q & 31)) & ((1u << per) - 1u)) != 0;
 }
 
 // Membership of two edges in a node: two bf16 ones or zeros.
@@ -434,54 +466,100 @@ __device__ __forceinline__ void mma_stage(float (&d)[8 * KG], unsigned stage, un
 
 // A stream of E >= 1 edges, 32 a window, through the ring: word_at(w) gives lane
 // = position of window w its word (any valid row for positions past the end, no
-// node), eat(h, words, stage) consumes half window h.
-template <int KG, typename WordF, typename EatF>
-__device__ __forceinline__ void mma_ring(int E, MmaWarp<KG>& W, const char* src, bool on, WordF word_at,
-                                         EatF eat) {
-  using MW = MmaWarp<KG>;
-  constexpr int S = MW::kStages;
+// node), eat(h, words, stage) consumes the kRs edges from h kRs on.
+template <typename TY, int KG, typename WordF, typename EatF>
+__device__ __forceinline__ void ring_stream(int E, RingWarp<TY, KG>& W, const char* src, bool on,
+                                            WordF word_at, EatF eat) {
+  using RW = RingWarp<TY, KG>;
+  constexpr int S = RW::kStages, RS = RW::kRs, PW = 32 / RS;  // stages, rows a stage, stages a window
+  static_assert((S - 1 + PW - 1) / PW + 1 <= 3, "four windows of words are kept");
   const int lane = threadIdx.x & 31;
-  const int nh = (E + 15) >> 4, nwin = (E + 31) >> 5;
+  const int nh = (E + RS - 1) / RS, nwin = (E + 31) >> 5;
   const unsigned rows = smem_u32(W.rows);
   unsigned n0 = word_at(0), n1 = nwin > 1 ? word_at(1) : 0u;
+  int slot = 0;  // ring slot of the stage issued next
   auto issue = [&](int s) {
     if (s < nh) {
-      const int w = s >> 1;
-      if (!(s & 1)) {
+      const int w = s / PW;
+      if (s % PW == 0) {
         W.words[w & 3][lane] = n0;
         __syncwarp();
         n0 = n1;
         if (w + 2 < nwin) n1 = word_at(w + 2);
       }
-      stage_rows<KG>(rows + (unsigned)(s % S) * MW::kStageBytes, W.words[w & 3] + 16 * (s & 1), src, on);
+      stage_rows<TY, KG>(rows + (unsigned)slot * RW::kStageBytes, W.words[w & 3] + RS * (s % PW), src, on);
+      slot = slot + 1 == S ? 0 : slot + 1;
     }
     cp_async_commit();
   };
   __syncwarp();  // the last stream's words and rows have been read
 #pragma unroll
   for (int s = 0; s < S - 1; ++s) issue(s);
+  int from = 0;
   for (int h = 0; h < nh; ++h) {
     cp_async_wait<S - 2>();
     __syncwarp();  // stage h has landed for the whole warp, stage h - 1 has been read
     issue(h + S - 1);
-    eat(h, W.words[(h >> 1) & 3] + 16 * (h & 1), rows + (unsigned)(h % S) * MW::kStageBytes);
+    eat(h, W.words[(h / PW) & 3] + RS * (h % PW), rows + (unsigned)from * RW::kStageBytes);
+    from = from + 1 == S ? 0 : from + 1;
   }
 }
 
-// Sum of the rows of one piece of a long in-list (ids p[0 .. L), L >= 1): in
-// the lanes with t = 0, d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
+// The words of a piece of a long in-list (ids p[0 .. L), L >= 1): node 0.
+__device__ __forceinline__ unsigned piece_word(const int* p, int L, int w) {
+  const int q = 32 * w + (threadIdx.x & 31);
+  return (unsigned)__ldg(p + min(q, L - 1)) | (q < L ? 0u : 127u << 25);
+}
+
+// The in-lists of a run of up to 32 nodes as one edge stream: lane j holds node
+// j's list length ll (0 to leave it out) and pool offset off. word() gives the
+// windows' words, in order.
+template <typename TY, int KG>
+struct RunWords {
+  const int* pool;
+  int P, E, started;  // first position of the lane's list, edges of the run, last list's rank
+  int ll;
+  __device__ __forceinline__ RunWords(const int* pl, int l, unsigned off, int incl, RingWarp<TY, KG>& W)
+      : pool(pl), P(incl - l), E(__shfl_sync(0xffffffffu, incl, 31)), started(-1), ll(l) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();  // the last run's list table has been read
+    const unsigned full = __ballot_sync(0xffffffffu, ll > 0);
+    if (ll > 0) W.lists[__popc(full & lanemask_lt())] = make_uint2(off - (unsigned)P, (unsigned)lane << 25);
+    __syncwarp();
+  }
+  __device__ __forceinline__ unsigned word(int w, const RingWarp<TY, KG>& W) {
+    const int lane = threadIdx.x & 31;
+    const unsigned at = (unsigned)(P - 32 * w);
+    const unsigned hm = __reduce_or_sync(0xffffffffu, ll > 0 && at < 32u ? 1u << at : 0u);
+    const int q = 32 * w + lane;
+    const uint2 l = W.lists[started + __popc(hm & (lanemask_lt() | (1u << lane)))];
+    started += __popc(hm);
+    // the sum wraps back; positions past the end repeat the last edge, for no node
+    const unsigned u = (unsigned)__ldg(pool + (l.x + (unsigned)min(q, E - 1)));
+    return u | (q < E ? l.y : 127u << 25);
+  }
+};
+
+__device__ __forceinline__ int warp_inclusive(int x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// bf16: sum of the rows of one piece of a long in-list: in the lanes with t = 0,
+// d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
 template <int KG>
 __device__ __forceinline__ void mma_piece(const int* p, int L, const char* src, bool on, int parts,
-                                          MmaWarp<KG>& W, float (&d)[8 * KG]) {
+                                          RingWarp<__nv_bfloat16, KG>& W, float (&d)[8 * KG]) {
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
-  mma_ring<KG>(
-      L, W, src, on,
-      [&](int w) {  // the list is node 0 of the fragments
-        const int q = 32 * w + lane;
-        return (unsigned)__ldg(p + min(q, L - 1)) | (q < L ? 0u : 127u << 25);
-      },
+  ring_stream<__nv_bfloat16, KG>(
+      L, W, src, on, [&](int w) { return piece_word(p, L, w); },
       [&](int, const unsigned* w, unsigned stage) {
         const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
         const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
@@ -490,45 +568,22 @@ __device__ __forceinline__ void mma_piece(const int* p, int L, const char* src, 
       });
 }
 
-// The in-lists of a run of up to 32 nodes as one edge stream: lane j holds
-// node j's list length ll (0 to leave it out) and pool offset off. The run's
-// nodes are taken eight at a time: finish(c, d) gets the sums of nodes 8 c ..
-// 8 c + 7 (fragments as in mma_stage), in order, once each.
+// bf16: a run's lists. The nodes are taken eight at a time: finish(c, d) gets the
+// sums of nodes 8 c .. 8 c + 7 (fragments as in mma_stage), in order, once each.
 template <int KG, typename F>
 __device__ __forceinline__ void mma_stream(const int* pool, int ll, unsigned off, const char* src,
-                                           bool on, int parts, MmaWarp<KG>& W, F finish) {
+                                           bool on, int parts, RingWarp<__nv_bfloat16, KG>& W, F finish) {
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
-  int incl = ll;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const int P = incl - ll;
-  const int E = __shfl_sync(0xffffffffu, incl, 31);
+  const int incl = warp_inclusive(ll);
   float d[8 * KG];
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
   int c = 0;  // eight nodes being summed, and the stream position after them
   int Ec = __shfl_sync(0xffffffffu, incl, 7);
-  if (E > 0) {
-    __syncwarp();  // the last run's list table has been read
-    const unsigned full = __ballot_sync(0xffffffffu, ll > 0);
-    if (ll > 0) W.lists[__popc(full & lanemask_lt())] = make_uint2(off - (unsigned)P, (unsigned)lane << 25);
-    __syncwarp();
-    int started = -1;  // rank of the list that runs into the next window
-    mma_ring<KG>(
-        E, W, src, on,
-        [&](int w) -> unsigned {  // windows come in order
-          const unsigned at = (unsigned)(P - 32 * w);
-          const unsigned hm = __reduce_or_sync(0xffffffffu, ll > 0 && at < 32u ? 1u << at : 0u);
-          const int q = 32 * w + lane;
-          const uint2 l = W.lists[started + __popc(hm & (lanemask_lt() | (1u << lane)))];
-          started += __popc(hm);
-          // the sum wraps back; positions past the end repeat the last edge, for no node
-          const unsigned u = (unsigned)__ldg(pool + (l.x + (unsigned)min(q, E - 1)));
-          return u | (q < E ? l.y : 127u << 25);
-        },
+  RunWords<__nv_bfloat16, KG> R(pool, ll, off, incl, W);
+  if (R.E > 0) {
+    ring_stream<__nv_bfloat16, KG>(
+        R.E, W, src, on, [&](int w) { return R.word(w, W); },
         [&](int h, const unsigned* w, unsigned stage) {
           const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
           const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
@@ -548,6 +603,83 @@ __device__ __forceinline__ void mma_stream(const int* pool, int ll, unsigned off
   } else {
     for (; c < 4; ++c) finish(c, d);
   }
+}
+
+// ---------------------------------------------------------------------------
+// float and double rows go through the same ring and are added by the lanes,
+// lane l the slots [KG l, KG (l + 1)) of each row: one shared load and KG (float:
+// KG / 2 packed) additions a row, a node's sum staying in registers from its
+// first row to its last. A stage's rows are summed in two chains of their own and
+// then added to the node's sum, so that a float sum's depth is rows / kRs + kRs / 2.
+// (Double rows are bound by their additions, 16 cycles of the SM per row of 32
+// columns, and take one chain.)
+// ---------------------------------------------------------------------------
+template <int KG>
+__device__ __forceinline__ void add_row(float (&a)[KG], const float (&x)[KG]) {
+  if constexpr (KG == 1) {
+    a[0] += x[0];
+  } else {
+#pragma unroll
+    for (int k = 0; k < KG; k += 2) {
+      unsigned long long u, v;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(a[k]), "f"(a[k + 1]));
+      asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x[k]), "f"(x[k + 1]));
+      asm("add.rn.f32x2 %0, %0, %1;" : "+l"(u) : "l"(v));
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(a[k]), "=f"(a[k + 1]) : "l"(u));
+    }
+  }
+}
+template <int KG>
+__device__ __forceinline__ void add_row(double (&a)[KG], const double (&x)[KG]) {
+#pragma unroll
+  for (int k = 0; k < KG; ++k) a[k] += x[k];
+}
+
+// Rows of a stage, each added to its node's sum acc; done(node) is called after a
+// node's last row (then acc starts again from zero). cur: the node being summed
+// (127: none yet).
+template <typename TY, int KG, typename F>
+__device__ __forceinline__ void add_stage(const unsigned* w, const unsigned char* stage, TY (&acc)[KG],
+                                          unsigned& cur, F done) {
+  using RW = RingWarp<TY, KG>;
+  constexpr int RS = RW::kRs;
+  const int lane = threadIdx.x & 31;
+  const unsigned node = w[lane & (RS - 1)] >> 25;
+  const unsigned prev = __shfl_up_sync(0xffffffffu, node, 1);
+  // bit r: row r begins another node than the row before it
+  const unsigned heads = __ballot_sync(0xffffffffu, lane < RS && node != (lane ? prev : cur));
+  const TY* row = reinterpret_cast<const TY*>(stage) + lane * KG;
+  constexpr int kChains = std::is_same<TY, float>::value ? 2 : 1;
+  TY part[kChains][KG];
+#pragma unroll
+  for (int c = 0; c < kChains; ++c)
+#pragma unroll
+    for (int k = 0; k < KG; ++k) part[c][k] = (TY)0;
+  auto gather = [&]() {  // the chains into the node's sum
+    if constexpr (kChains == 2) {
+      add_row<KG>(part[0], part[1]);
+      add_row<KG>(acc, part[0]);
+#pragma unroll
+      for (int c = 0; c < kChains; ++c)
+#pragma unroll
+        for (int k = 0; k < KG; ++k) part[c][k] = (TY)0;
+    }
+  };
+#pragma unroll
+  for (int r = 0; r < RS; ++r) {
+    if ((heads >> r) & 1u) {  // warp-uniform
+      gather();
+      if (cur != 127u) done(cur);
+#pragma unroll
+      for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
+      cur = __shfl_sync(0xffffffffu, node, r);
+    }
+    alignas(16) TY x[KG];
+    load_k<TY, KG>(row + r * RW::G, x);
+    if constexpr (kChains == 2) add_row<KG>(part[r & 1], x);
+    else add_row<KG>(acc, x);
+  }
+  gather();
 }
 
 // ---------------------------------------------------------------------------
@@ -819,7 +951,7 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
 // that is idle at the grid barrier).
 template <int KG>
 __device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long long m,
-                             double* s_key) {
+                             double* s_key, bool narrow_rows) {
   constexpr int G = 32 * KG;
   const Multi& M = d.mu;
   const int Sp = M.Sp;
@@ -928,7 +1060,7 @@ __device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long lo
     ctl->n_grp = ng;
     // packed bf16 groups with only slots 0..7 (0..3) running: narrow steps of
     // 8 (4) columns from now on
-    ctl->narrow = pack && M.yn0 != nullptr && ng == 1 && ctl->grp[0] == 0 && s_maxslot < 8
+    ctl->narrow = narrow_rows && M.yn0 != nullptr && ng == 1 && ctl->grp[0] == 0 && s_maxslot < 8
                       ? (s_maxslot < 4 ? 4 : 8)
                       : 0;
     ctl->stop = !any;
@@ -1061,23 +1193,6 @@ __device__ __forceinline__ void ring_wait(Ring& rg, int b, Ctl* ctl) {
     }
   }
   rg.phase ^= 1u << b;
-}
-
-// K-element slice of a staged row (plain loads from shared memory).
-template <typename T, int K>
-__device__ __forceinline__ void load_k(const T* p, T (&out)[K]) {
-  constexpr int B = K * (int)sizeof(T);
-  if constexpr (B >= 16) {
-#pragma unroll
-    for (int i = 0; i < B / 16; ++i)
-      reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(p)[i];
-  } else if constexpr (B == 8) {
-    *reinterpret_cast<uint2*>(out) = *reinterpret_cast<const uint2*>(p);
-  } else if constexpr (B == 4) {
-    *reinterpret_cast<unsigned*>(out) = *reinterpret_cast<const unsigned*>(p);
-  } else {
-    *reinterpret_cast<unsigned short*>(out) = *reinterpret_cast<const unsigned short*>(p);
-  }
 }
 
 // acc += the cnt rows staged in buffer b (this lane's K columns).
@@ -1416,7 +1531,7 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
       }
     }
     column_sums(0);
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, nullptr);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, nullptr, false);
     if (!bar_release(ctl, sh)) return;
   }
 
@@ -1692,24 +1807,29 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
     }
     flush();
     column_sums(it);
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, nullptr);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, nullptr, false);
     if (!bar_release(ctl, sh)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->epoch = epoch + 1;
 }
 
 
-// The bf16 seed block on the tensor cores, one persistent cooperative launch per
-// call. Columns are packed into groups of G = 32 KG slots: slot q holds column
+// The seed block through row rings (bf16 rows summed by the tensor cores, float
+// and double rows by the lanes), one persistent cooperative launch per call.
+// Columns are packed into groups of G = 32 KG slots: slot q holds column
 // slot_col[q], chosen per call by the x(0) decision so that columns likely to
 // run long share groups; R, the offsets and the per-column state stay by column,
 // gather rows, residuals and partial sums by slot. A work item (a piece of a
 // long in-list, or a task of consecutive nodes) is taken by one warp for all
 // groups with a running column when there are several items a warp, so that its
 // ids and headers come from L1 for the later groups; else for one group.
-template <int KG>
-__global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) k_propagate_mma(Dev d, PropParams pp) {
+template <typename TY, int KG>
+__global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG>::kCtas)
+    k_propagate_ring(Dev d, PropParams pp) {
+  using A = typename AccOf<TY>::type;
+  using RW = RingWarp<TY, KG>;
   constexpr int G = 32 * KG;
+  constexpr bool kMma = RW::kMma;
   __shared__ double s_part[kMaxSeeds];  // |x| of this step per column (shared-memory atomics)
   __shared__ double s_key[kMaxSeeds];
   __shared__ int s_col[kMaxSeeds];      // column of each slot
@@ -1730,12 +1850,12 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
   const int n_tasks = ctl->n_tasks;
   const int hub_thr = ctl->hub_thr, hub_piece = ctl->hub_piece;
   const L2Pol pol = make_l2pol();
-  __nv_bfloat16* yb[2] = {(__nv_bfloat16*)M.y0, (__nv_bfloat16*)M.y1};
+  TY* yb[2] = {(TY*)M.y0, (TY*)M.y1};
   __nv_bfloat16* eb = (__nv_bfloat16*)M.e;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  MmaWarp<KG>& W = reinterpret_cast<MmaWarp<KG>*>(dsm)[wid];
+  RW& W = reinterpret_cast<RW*>(dsm)[wid];
   double* my_part = s_part;
   for (int j = threadIdx.x; j < Sp; j += blockDim.x) s_part[j] = 0.0;
   __syncthreads();
@@ -1780,7 +1900,7 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
   for (int k = 0; k < 8; ++k)
     if ((tb >> k) & 1u) atomicAdd(my_part + lane + 32 * k, l0[k]);
   column_sums(0);
-  if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, s_key);
+  if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, 0, m, s_key, kMma);
   if (!bar_release(ctl, sh)) return;
   // 2. R += x(0) and the y(0) rows, in group slots
   if (threadIdx.x < 8) s_grp[threadIdx.x] = *(volatile int*)&ctl->grp[threadIdx.x];
@@ -1801,44 +1921,44 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
   for (int vb = gw * 32; vb < n && ng > 0; vb += nw * 32) {
     const int vl = vb + lane;
     const unsigned stamped = __ballot_sync(0xffffffffu, vl < n && __ldcg(d.mark + vl) == epoch);
-    const float s_l = vl < n ? scale_of<float>(d, vl) : 0.f;
-    // rows of nodes without an offset entry start at zero: 16 bytes a lane,
-    // 8 / KG rows a store
-    const unsigned blank = __ballot_sync(0xffffffffu, s_l != 0.f) & ~stamped;
-    constexpr int kLanes = 4 * KG;  // lanes a row
+    const A s_l = vl < n ? scale_of<A>(d, vl) : (A)0;
+    // rows of nodes without an offset entry start at zero: 16 bytes a lane
+    const unsigned blank = __ballot_sync(0xffffffffu, s_l != (A)0) & ~stamped;
+    constexpr int kLanes = RW::kChunks;  // lanes a row
     for (int gi = 0; gi < ng && blank; ++gi) {
-      const size_t at = s_grp[gi] * gs + (size_t)vb * G + 8 * (lane % kLanes);
+      const size_t at = s_grp[gi] * gs + (size_t)vb * G + 16 / sizeof(TY) * (lane % kLanes);
 #pragma unroll
       for (int r = 0; r < kLanes; ++r) {
         const int j = r * (32 / kLanes) + lane / kLanes;
         if ((blank >> j) & 1u) {
           *reinterpret_cast<uint4*>(yb[0] + at + (size_t)j * G) = make_uint4(0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>(eb + at + (size_t)j * G) = make_uint4(0u, 0u, 0u, 0u);
+          if constexpr (kMma)
+            *reinterpret_cast<uint4*>(eb + at + (size_t)j * G) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
     }
     for (unsigned work = stamped; work; work &= work - 1) {
       const int jj = __ffs(work) - 1;
       const int v = vb + jj;
-      const float s = __shfl_sync(0xffffffffu, s_l, jj);
+      const A s = __shfl_sync(0xffffffffu, s_l, jj);
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         if (!((actq >> q) & 1u)) continue;
         const size_t ybase = (q / KG) * gs + (size_t)v * G + 32 * (q % KG) + lane;
-        __nv_bfloat16 yv = __float2bfloat16_rn(0.f), ev = yv;
+        TY yv = from_acc((A)0, (TY*)nullptr), ev = yv;
         const size_t rb = (size_t)v * Sp + colq[q];
         const double x = __ldcg(M.xacc + rb);
         if (x != 0.0) {
           M.r[rb] += x;
           M.xacc[rb] = 0.0;
-          const float w = (float)x * s;
-          yv = __float2bfloat16_rn(w);
-          ev = __float2bfloat16_rn(w - __bfloat162float(yv));
+          const A w = (A)x * s;
+          yv = from_acc(w, (TY*)nullptr);
+          if constexpr (kMma) ev = __float2bfloat16_rn(w - __bfloat162float(yv));
         }
-        if (s != 0.f) {
-          const __nv_bfloat16 y1[1] = {yv}, e1[1] = {ev};
+        if (s != (A)0) {
+          const TY y1[1] = {yv}, e1[1] = {ev};
           st_pol(yb[0] + ybase, y1, pol.once);
-          st_pol(eb + ybase, e1, pol.once);
+          if constexpr (kMma) st_pol(eb + ybase, e1, pol.once);
         }
       }
     }
@@ -1846,7 +1966,7 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
   if (bar_arrive(ctl, sh) && threadIdx.x == 0) ctl->ctr[1] = 0;
   if (!bar_release(ctl, sh)) return;
 
-  float* hub_acc = (float*)M.hub_acc;
+  A* hub_acc = (A*)M.hub_acc;
   int prev_narrow = 0;  // row width of the compact block the last step wrote (0: none)
   for (int it = 1;; ++it) {
     if (*(volatile int*)&ctl->stop) break;
@@ -1859,35 +1979,37 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
       if (lane == 0) s_am[q >> 5] = a;
     }
     __syncthreads();
-    const __nv_bfloat16* ys = yb[(it - 1) & 1];
-    __nv_bfloat16* yd = yb[it & 1];
+    const TY* ys = yb[(it - 1) & 1];
+    TY* yd = yb[it & 1];
     const int n_items = n_pieces + n_tasks;
-    const int narrow = *(volatile int*)&ctl->narrow;  // row width of a narrow step (0: over groups)
-    if (narrow) {
-      __nv_bfloat16* yn[2] = {(__nv_bfloat16*)M.yn0, (__nv_bfloat16*)M.yn1};
-      const __nv_bfloat16* src =
-          prev_narrow ? yn[(it - 1) & 1] : ys;
-      const int stride = prev_narrow ? prev_narrow : G;
-      float* acc_s = &W.acc[0][0];
-      static_assert(sizeof(W.acc) >= 256 * sizeof(float), "sums of a narrow run");
-      if (narrow == 4) {
-        Narrow<4> N{src, stride, yn[it & 1], eb, G, {}, 0u};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          N.col[c] = __ldcg(M.slot_col + c);
-          if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
+    const int narrow = kMma ? *(volatile int*)&ctl->narrow : 0;  // row width of a narrow step (0: over groups)
+    if constexpr (kMma) {
+      if (narrow) {
+        __nv_bfloat16* yn[2] = {(__nv_bfloat16*)M.yn0, (__nv_bfloat16*)M.yn1};
+        const __nv_bfloat16* src =
+            prev_narrow ? yn[(it - 1) & 1] : ys;
+        const int stride = prev_narrow ? prev_narrow : G;
+        float* acc_s = &W.acc[0][0];
+        static_assert(sizeof(W.acc) >= 256 * sizeof(float), "sums of a narrow run");
+        if (narrow == 4) {
+          Narrow<4> N{src, stride, yn[it & 1], eb, G, {}, 0u};
+  #pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            N.col[c] = __ldcg(M.slot_col + c);
+            if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
+          }
+          narrow_step<4>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
+                         my_part, ctl);
+        } else {
+          Narrow<8> N{src, stride, yn[it & 1], eb, G, {}, 0u};
+  #pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            N.col[c] = __ldcg(M.slot_col + c);
+            if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
+          }
+          narrow_step<8>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
+                         my_part, ctl);
         }
-        narrow_step<4>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
-                       my_part, ctl);
-      } else {
-        Narrow<8> N{src, stride, yn[it & 1], eb, G, {}, 0u};
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          N.col[c] = __ldcg(M.slot_col + c);
-          if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
-        }
-        narrow_step<8>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
-                       my_part, ctl);
       }
     }
     prev_narrow = narrow;
@@ -1916,16 +2038,36 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
         for (int gi = g0; gi < g1; ++gi) {
           const int g = s_grp[gi];
           const unsigned* am = s_am + g * KG;
-          const int ch = lane % MmaWarp<KG>::kChunks;  // the chunk this lane copies
-          float D[8 * KG];
-          mma_piece<KG>(p, L, reinterpret_cast<const char*>(ys + g * gs),
-                        ((am[ch >> 2] >> (8 * (ch & 3))) & 0xFFu) != 0, running_parts<KG>(am), W, D);
-          float* ha = hub_acc + (size_t)h * Sp + g * G;
-          if ((lane & 3) == 0) {
-            const int fg = lane >> 2;
+          const bool on = chunk_runs<TY, KG>(am);
+          const char* src = reinterpret_cast<const char*>(ys + g * gs);
+          A* ha = hub_acc + (size_t)h * Sp + g * G;
+          if constexpr (kMma) {
+            float D[8 * KG];
+            mma_piece<KG>(p, L, src, on, running_parts<KG>(am), W, D);
+            if ((lane & 3) == 0) {
+              const int fg = lane >> 2;
 #pragma unroll
-            for (int f = 0; f < 4 * KG; ++f)
-              if ((am[f >> 2] >> (8 * (f & 3) + fg)) & 1u) atomicAdd(ha + 8 * f + fg, D[2 * f]);
+              for (int f = 0; f < 4 * KG; ++f)
+                if ((am[f >> 2] >> (8 * (f & 3) + fg)) & 1u) atomicAdd(ha + 8 * f + fg, D[2 * f]);
+            }
+          } else {
+            A acc[KG];
+#pragma unroll
+            for (int k = 0; k < KG; ++k) acc[k] = (A)0;
+            unsigned cur = 0u;
+            ring_stream<TY, KG>(
+                L, W, src, on, [&](int w) { return piece_word(p, L, w); },
+                [&](int, const unsigned* w, unsigned stage) {
+                  // rows past the end begin "no node": the list's sum is put aside there
+                  add_stage<TY, KG>(w, W.rows + (stage - smem_u32(W.rows)), acc, cur, [&](unsigned) {
+#pragma unroll
+                    for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, acc[k]);
+                  });
+                });
+            if (cur == 0u) {
+#pragma unroll
+              for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, acc[k]);
+            }
           }
           __threadfence();
           int last = 0;
@@ -1934,21 +2076,25 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
           if (last) {
             __threadfence();
             if (lane == 0) M.hub_cnt[h * 8 + g] = 0;
-            const float sv = scale_of<float>(d, v);
+            const A sv = scale_of<A>(d, v);
 #pragma unroll
             for (int k = 0; k < KG; ++k) {  // lane = slot
-              const float x = __ldcg(ha + 32 * k + lane);
-              ha[32 * k + lane] = 0.f;
+              const A x = __ldcg(ha + 32 * k + lane);
+              ha[32 * k + lane] = (A)0;
               if (!((am[k] >> lane) & 1u)) continue;
               const int col = s_col[g * G + 32 * k + lane];
               red_add_once(M.r + (size_t)v * Sp + col, (double)x, pol.once);
               atomicAdd(my_part + col, fabs((double)x));
-              if (sv != 0.f) {
+              if (sv != (A)0) {
                 const size_t at = g * gs + (size_t)v * G + 32 * k + lane;
-                const float w = x * sv + __bfloat162float(eb[at]);
-                const __nv_bfloat16 yv = __float2bfloat16_rn(w);
-                yd[at] = yv;
-                eb[at] = __float2bfloat16_rn(w - __bfloat162float(yv));
+                if constexpr (kMma) {
+                  const float w = x * sv + __bfloat162float(eb[at]);
+                  const __nv_bfloat16 yv = __float2bfloat16_rn(w);
+                  yd[at] = yv;
+                  eb[at] = __float2bfloat16_rn(w - __bfloat162float(yv));
+                } else {
+                  yd[at] = x * sv;
+                }
               }
             }
           }
@@ -1962,107 +2108,155 @@ __global__ void __launch_bounds__(32 * MmaWarp<KG>::kWarps, MmaWarp<KG>::kCtas) 
         const unsigned* am = s_am + g * KG;
         const int* scol = s_col + g * G;
         const char* src = reinterpret_cast<const char*>(ys + g * gs);
-        const int ch = lane % MmaWarp<KG>::kChunks;
-        const bool on = ((am[ch >> 2] >> (8 * (ch & 3))) & 0xFFu) != 0;
+        const bool on = chunk_runs<TY, KG>(am);
         const int parts = running_parts<KG>(am);
+        // float and double rows: this lane's slots lane KG + k, their columns
+        int col[KG];
+        unsigned amk = 0;
+#pragma unroll
+        for (int k = 0; k < KG; ++k) {
+          const int q = lane * KG + k;
+          col[k] = scol[q];
+          amk |= ((am[q >> 5] >> (q & 31)) & 1u) << k;
+        }
         // list lengths, offsets and scales of the next run of 32 nodes load
         // while the current run is summed
         int nx_len = 0;
         unsigned nx_off = 0;
-        float nx_s = 0.f;
+        A nx_s = (A)0;
         auto header = [&](int vb) {
           const int vl = vb + lane;
           nx_len = 0;
           nx_off = 0;
-          nx_s = 0.f;
+          nx_s = (A)0;
           if (vl < c1t) {
             nx_len = __ldg(d.len_c + vl);
             nx_off = __ldg(d.off_c + vl);
-            nx_s = scale_of<float>(d, vl);
+            nx_s = scale_of<A>(d, vl);
           }
         };
         header(c0t);
         for (int vb = c0t; vb < c1t; vb += 32) {
           const int my_len = nx_len;
           const unsigned my_off = nx_off;
-          const float my_s = nx_s;
+          const A my_s = nx_s;
           if (vb + 32 < c1t) header(vb + 32);
           const bool mine = vb + lane < c1t && my_len <= hub_thr;  // hubs go by pieces
-          const unsigned fin = __ballot_sync(0xffffffffu, mine && (my_len > 0 || my_s != 0.f));
+          const unsigned fin = __ballot_sync(0xffffffffu, mine && (my_len > 0 || my_s != (A)0));
           if (!fin) continue;
-          // |x| of the run summed in float (at most 32 nonnegative terms), then
-          // added to the FP64 partial once
-          float l1f[KG];
+          // |x| of the run summed in the rows' accumulation type (at most 32
+          // nonnegative terms), then added to the FP64 partial once
+          A l1f[KG];
 #pragma unroll
-          for (int k = 0; k < KG; ++k) l1f[k] = 0.f;
-          mma_stream<KG>(
-              d.pool_c, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
-                if (!((fin >> (8 * c)) & 0xFFu)) return;  // warp-uniform
-                // the sums by node and slot (conflict-free: banks 8 t + g)
-                const int fg = lane >> 2, t2 = 2 * (lane & 3);
-#pragma unroll
-                for (int f = 0; f < 4 * KG; ++f) {
-                  if (f >= 4 * parts) break;
-                  W.acc[t2][8 * f + fg] = D[2 * f];
-                  W.acc[t2 + 1][8 * f + fg] = D[2 * f + 1];
-                }
-                // next gather row and residual: lane = node, every fourth
-                // chunk of four slots; the old residuals load first
-                const int j = lane >> 2, q = lane & 3;
-                const float sj = __shfl_sync(0xffffffffu, my_s, 8 * c + j);
-                const bool src_node = sj != 0.f && ((fin >> (8 * c + j)) & 1u);
-                const size_t at = g * gs + (size_t)(vb + 8 * c + j) * G + 4 * q;
-                uint2 eo[2 * KG];
-#pragma unroll
-                for (int i = 0; i < 2 * KG; ++i)
-                  eo[i] = src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu)
-                              ? __ldcg(reinterpret_cast<const uint2*>(eb + at + 16 * i))
-                              : make_uint2(0u, 0u);
-                __syncwarp();
-                // R += x: lane = slot (a node without in-list has x = 0)
-                double* rp = M.r + (size_t)(vb + 8 * c) * Sp;
-#pragma unroll
-                for (int k = 0; k < KG; ++k) {
-                  if (k >= parts) break;
-                  const bool run = (am[k] >> lane) & 1u;
-                  double* rk = rp + scol[32 * k + lane];
-#pragma unroll
-                  for (int jj = 0; jj < 8; ++jj) {
-                    const float x = W.acc[jj][32 * k + lane];
-                    if (run && x != 0.f) {
-                      red_add_once(rk, widen(x), pol.once);
-                      l1f[k] += fabsf(x);
-                    }
-                    rk += Sp;
+          for (int k = 0; k < KG; ++k) l1f[k] = (A)0;
+          if constexpr (kMma) {
+            mma_stream<KG>(
+                d.pool_c, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
+                  if (!((fin >> (8 * c)) & 0xFFu)) return;  // warp-uniform
+                  // the sums by node and slot (conflict-free: banks 8 t + g)
+                  const int fg = lane >> 2, t2 = 2 * (lane & 3);
+  #pragma unroll
+                  for (int f = 0; f < 4 * KG; ++f) {
+                    if (f >= 4 * parts) break;
+                    W.acc[t2][8 * f + fg] = D[2 * f];
+                    W.acc[t2 + 1][8 * f + fg] = D[2 * f + 1];
                   }
-                }
+                  // next gather row and residual: lane = node, every fourth
+                  // chunk of four slots; the old residuals load first
+                  const int j = lane >> 2, q = lane & 3;
+                  const float sj = __shfl_sync(0xffffffffu, my_s, 8 * c + j);
+                  const bool src_node = sj != 0.f && ((fin >> (8 * c + j)) & 1u);
+                  const size_t at = g * gs + (size_t)(vb + 8 * c + j) * G + 4 * q;
+                  uint2 eo[2 * KG];
+  #pragma unroll
+                  for (int i = 0; i < 2 * KG; ++i)
+                    eo[i] = src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu)
+                                ? __ldcg(reinterpret_cast<const uint2*>(eb + at + 16 * i))
+                                : make_uint2(0u, 0u);
+                  __syncwarp();
+                  // R += x: lane = slot (a node without in-list has x = 0)
+                  double* rp = M.r + (size_t)(vb + 8 * c) * Sp;
+  #pragma unroll
+                  for (int k = 0; k < KG; ++k) {
+                    if (k >= parts) break;
+                    const bool run = (am[k] >> lane) & 1u;
+                    double* rk = rp + scol[32 * k + lane];
+  #pragma unroll
+                    for (int jj = 0; jj < 8; ++jj) {
+                      const float x = W.acc[jj][32 * k + lane];
+                      if (run && x != 0.f) {
+                        red_add_once(rk, widen(x), pol.once);
+                        l1f[k] += fabsf(x);
+                      }
+                      rk += Sp;
+                    }
+                  }
+  #pragma unroll
+                  for (int i = 0; i < 2 * KG; ++i) {
+                    if (i >= 2 * parts) break;
+                    if (!(src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu))) continue;
+                    const float4 x = *reinterpret_cast<const float4*>(&W.acc[j][16 * i + 4 * q]);
+                    const float w0 = x.x * sj + __uint_as_float(eo[i].x << 16);
+                    const float w1 = x.y * sj + __uint_as_float(eo[i].x & 0xFFFF0000u);
+                    const float w2 = x.z * sj + __uint_as_float(eo[i].y << 16);
+                    const float w3 = x.w * sj + __uint_as_float(eo[i].y & 0xFFFF0000u);
+                    const uint2 y = make_uint2(pack_bf16x2(w0, w1), pack_bf16x2(w2, w3));
+                    *reinterpret_cast<uint2*>(yd + at + 16 * i) = y;
+                    *reinterpret_cast<uint2*>(eb + at + 16 * i) =
+                        make_uint2(pack_bf16x2(w0 - __uint_as_float(y.x << 16),
+                                               w1 - __uint_as_float(y.x & 0xFFFF0000u)),
+                                   pack_bf16x2(w2 - __uint_as_float(y.y << 16),
+                                               w3 - __uint_as_float(y.y & 0xFFFF0000u)));
+                  }
+                  __syncwarp();  // acc is free again
+                });
 #pragma unroll
-                for (int i = 0; i < 2 * KG; ++i) {
-                  if (i >= 2 * parts) break;
-                  if (!(src_node && ((am[i >> 1] >> (16 * (i & 1) + 4 * q)) & 0xFu))) continue;
-                  const float4 x = *reinterpret_cast<const float4*>(&W.acc[j][16 * i + 4 * q]);
-                  const float w0 = x.x * sj + __uint_as_float(eo[i].x << 16);
-                  const float w1 = x.y * sj + __uint_as_float(eo[i].x & 0xFFFF0000u);
-                  const float w2 = x.z * sj + __uint_as_float(eo[i].y << 16);
-                  const float w3 = x.w * sj + __uint_as_float(eo[i].y & 0xFFFF0000u);
-                  const uint2 y = make_uint2(pack_bf16x2(w0, w1), pack_bf16x2(w2, w3));
-                  *reinterpret_cast<uint2*>(yd + at + 16 * i) = y;
-                  *reinterpret_cast<uint2*>(eb + at + 16 * i) =
-                      make_uint2(pack_bf16x2(w0 - __uint_as_float(y.x << 16),
-                                             w1 - __uint_as_float(y.x & 0xFFFF0000u)),
-                                 pack_bf16x2(w2 - __uint_as_float(y.y << 16),
-                                             w3 - __uint_as_float(y.y & 0xFFFF0000u)));
-                }
-                __syncwarp();  // acc is free again
-              });
+            for (int k = 0; k < KG; ++k)
+              if (l1f[k] != 0.f) atomicAdd(my_part + scol[32 * k + lane], (double)l1f[k]);
+          } else {
+            // a node's next gather row; one without in-list writes zeros
+            for (unsigned z = fin & __ballot_sync(0xffffffffu, my_len == 0); z; z &= z - 1) {
+              alignas(16) const TY zero[KG] = {};
+              store_k<TY, KG>(yd + g * gs + (size_t)(vb + __ffs(z) - 1) * G + lane * KG, zero);
+            }
+            const int ll = mine ? my_len : 0;
+            RunWords<TY, KG> R(d.pool_c, ll, my_off, warp_inclusive(ll), W);
+            if (R.E == 0) continue;
+            A acc[KG];
 #pragma unroll
-          for (int k = 0; k < KG; ++k)
-            if (l1f[k] != 0.f) atomicAdd(my_part + scol[32 * k + lane], (double)l1f[k]);
+            for (int k = 0; k < KG; ++k) acc[k] = (A)0;
+            unsigned cur = 127u;
+            auto done = [&](unsigned j) {  // node vb + j: x = acc
+              const A sj = __shfl_sync(0xffffffffu, my_s, (int)j);
+              double* rp = M.r + (size_t)(vb + j) * Sp;
+#pragma unroll
+              for (int k = 0; k < KG; ++k)
+                if (((amk >> k) & 1u) && acc[k] != (A)0) {
+                  red_add_once(rp + col[k], widen(acc[k]), pol.once);
+                  l1f[k] += fabs(acc[k]);
+                }
+              if (sj != (A)0) {
+                alignas(16) TY yv[KG];
+#pragma unroll
+                for (int k = 0; k < KG; ++k) yv[k] = acc[k] * sj;
+                store_k<TY, KG>(yd + g * gs + (size_t)(vb + j) * G + lane * KG, yv);
+              }
+            };
+            ring_stream<TY, KG>(
+                R.E, W, src, on, [&](int w) { return R.word(w, W); },
+                [&](int, const unsigned* w, unsigned stage) {
+                  add_stage<TY, KG>(w, W.rows + (stage - smem_u32(W.rows)), acc, cur, done);
+                });
+            if (cur != 127u) done(cur);
+#pragma unroll
+            for (int k = 0; k < KG; ++k)
+              if (l1f[k] != (A)0) atomicAdd(my_part + col[k], (double)l1f[k]);
+          }
         }
       }
     }
     column_sums(it);
-    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, s_key);
+    if (bar_arrive(ctl, sh)) decide_multi<KG>(d, pp, it, m, s_key, kMma);
     if (!bar_release(ctl, sh)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->epoch = epoch + 1;
@@ -2079,10 +2273,9 @@ struct MultiFn {
 template <typename TY, int KG>
 MultiFn multi_fn_k(bool bulk) {
   if (bulk) return {(const void*)k_propagate_multi<TY, KG, true>, RingCfg<TY, KG>::kSmem};
-  // bf16 groups of up to 128 columns are summed by the tensor cores
-  if constexpr (std::is_same<TY, __nv_bfloat16>::value && KG <= 4)
-    return {(const void*)k_propagate_mma<KG>, MmaWarp<KG>::kWarps * (int)sizeof(MmaWarp<KG>),
-            32 * MmaWarp<KG>::kWarps};
+  if constexpr (seed_ring_fits((int)sizeof(TY), KG))
+    return {(const void*)k_propagate_ring<TY, KG>,
+            RingWarp<TY, KG>::kWarps * (int)sizeof(RingWarp<TY, KG>), 32 * RingWarp<TY, KG>::kWarps};
   else
     return {(const void*)k_propagate_multi<TY, KG, false>, 0};
 }

@@ -77,27 +77,33 @@ def test_push_only_steps_reach_every_row_length():
     eng.close()
 
 
-@pytest.mark.parametrize("S,group", [(20, 0), (64, 0), (100, 32), (100, 0), (100, 128), (200, 128),
-                                     (200, 256)])
-def test_bf16_blocks_at_the_edges_of_the_row_stages(S, group):
-    """bf16 seed blocks in every group width (tensor-core sums for 32, 64 and 128
-    columns, 256 by lanes): in-lists around the 16-row stages, the 32-edge
-    windows and the long-list pieces, in the oracle's lock-step, L1 <= 1e-5 a
-    seed (the bound of the seed-block tests)."""
+BF16, F32, F64 = N.OSP_PREC_BF16_ACC64, N.OSP_PREC_FP32_ACC64, N.OSP_PREC_FP64
+
+
+@pytest.mark.parametrize("prec,S,group", [
+    (BF16, 20, 0), (BF16, 64, 0), (BF16, 100, 32), (BF16, 100, 0), (BF16, 100, 128),
+    (BF16, 200, 128), (BF16, 200, 256), (F32, 20, 0), (F32, 64, 0), (F32, 100, 0), (F32, 200, 64),
+    (F32, 200, 256), (F64, 17, 0), (F64, 60, 32), (F64, 60, 0), (F64, 100, 128)])
+def test_blocks_at_the_edges_of_the_row_stages(prec, S, group):
+    """Seed blocks in every group width of the row rings (and past it, by lanes):
+    in-lists around the 8- and 16-row stages, the 32-edge windows and the
+    long-list pieces, in the oracle's lock-step, L1 <= 1e-10 (double) and 1e-5 a
+    seed (the bounds of the seed-block tests)."""
     n = 2300
     rng = np.random.default_rng(S + group)
     src, dst = edge_graph(rng, n, 0)
     more = rng.integers(0, n, (2, 400))
-    for k, v in ((15, 201), (16, 204), (17, 207), (47, 210), (48, 213), (49, 216)):
+    for k, v in ((7, 198), (8, 201), (15, 204), (16, 207), (17, 210), (47, 213), (48, 216), (49, 219)):
         u = rng.choice(n, k, replace=False)
         src, dst = np.append(src, u), np.append(dst, np.full(k, v))
     src, dst = np.append(src, more[0]).astype(np.int32), np.append(dst, more[1]).astype(np.int32)
     seeds = rng.permutation(n)[:S].astype(np.int32)
-    eng = N.Engine(precision=N.OSP_PREC_BF16_ACC64, device=0, seed_group=group, node_order=S % 3 % 2)
+    eng = N.Engine(precision=prec, device=0, seed_group=group, node_order=S % 3 % 2)
     eng.load_graph(n, src, dst)
     eng.set_seeds(seeds, C_RESTART)
     eng.init_scores(1e-11)
     it0, _, _ = eng.get_seed_stats()
+    tol = 1e-10 if prec == F64 else 1e-5
     g = O.Graph(n, src, dst)
     old = g.csr()
     pick = list(range(0, S, max(1, S // 12)))
@@ -109,7 +115,7 @@ def test_bf16_blocks_at_the_edges_of_the_row_stages(S, group):
         it, _, _ = eng.get_seed_stats()
         for j in pick:
             r[j], _, _, _ = O.osp(old, new, r[j], C_RESTART, 1e-9, force_iters=int(it[j]))
-            assert np.abs(eng.query(j) - r[j]).sum() <= 1e-5
+            assert np.abs(eng.query(j) - r[j]).sum() <= tol
         old = new
     eng.close()
 
