@@ -18,6 +18,7 @@ namespace osp {
 
 constexpr int kMaxBatch = 16384;        // ops per sub-batch (keys pack the op index in 14 bits)
 constexpr long long kMaxLargeBatch = 1ll << 22;  // ops per apply call, in sub-batches of kMaxBatch
+constexpr int kIngestOne = 1024;       // ops that one CTA ingests by itself
 constexpr int kMaxNodes = (1 << 25) - 1; // ids fit in 25 bits
 constexpr int kNoPos = 0x7F7F7F7F;       // del_pos of a node not deleted by the batch (memset 0x7F)
 constexpr int kLight = 32;               // lists up to this length are walked by one lane
@@ -66,6 +67,8 @@ struct Ctl {
   int n_opieces;               // several seeds: offset items (256 entries of a changed row)
   int hub_thr, hub_piece;      // pull step: in-lists longer than hub_thr go in pieces of hub_piece
   int batch_U;                 // ops of the batch, for a k_ingest replayed from a CUDA graph
+  int ing_bad, ing_adds, ing_clr;  // larger batches: first invalid op, node additions, any zeroed row
+  long long ing_reins;             // ... and edges written again after their row was zeroed
   long long n_dst_nz, n_src_nz;  // nodes with a nonempty in-list / out-list (pull plan)
   int epoch;                   // frontier mark of x(0); step i uses epoch + i
   int q_size[2];               // frontier queue lengths
@@ -148,6 +151,8 @@ struct Dev {
   // batch scratch: net edits grouped per changed row / column
   int* ins_r; int* del_r; int* ins_c; int* del_c;   // [kMaxBatch]
   int* gi; int* gd;                                  // [kMaxBatch + 1] prefix counts
+  unsigned long long* ing_key; int* ing_na;          // [kMaxBatch] larger batches: sort keys; node
+                                                     // count before each op, then kind of edit
   int* rec_r_node; int* rec_r_is; int* rec_r_ic; int* rec_r_ds; int* rec_r_dc;  // [nc]
   int* rec_c_node; int* rec_c_is; int* rec_c_ic; int* rec_c_ds; int* rec_c_dc;  // [nc]
   int* del_nodes;  // [kMaxBatch]

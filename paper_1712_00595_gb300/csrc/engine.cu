@@ -20,6 +20,10 @@ using namespace osp;
 namespace {
 
 constexpr int kIngestSmem = kMaxBatch * 8;
+// shared memory of the batch sorts: keys of whole rows of 1024, digit counts by warp
+constexpr size_t ingest_sort_smem(int U) {
+  return (size_t)((U + 1023) / 1024) * 1024 * 8 + 32 * 256 * sizeof(int);
+}
 // pinned staging: host ops of a batch first, then the batch size for graph
 // replays, then the ||x(i)||_1 history read back with the control block
 constexpr size_t kPinnedBytes = 256 * 1024;
@@ -609,10 +613,21 @@ osp_status check_ready(osp_ctx* ctx, bool need_scores) {
 osp_status enqueue_update(osp_ctx* ctx, const osp_update* ops_dev, int U, int Np,
                           bool cont = false) {
   const int g = ctx->num_sms * 4;
-  k_reset_batch<<<1, 1, 0, ctx->stream>>>(ctx->d, cont ? 1 : 0);
+  k_reset_batch<<<1, 256, 0, ctx->stream>>>(ctx->d, cont ? 1 : 0);
   ++ctx->launches;
-  k_ingest<<<1, 1024, (size_t)Np * 8, ctx->stream>>>(ctx->d, ops_dev, U);
-  ++ctx->launches;
+  if (Np <= kIngestOne) {
+    k_ingest<<<1, 1024, (size_t)Np * 8, ctx->stream>>>(ctx->d, ops_dev, U);
+    ++ctx->launches;
+  } else {
+    const int nb = (Np + 255) / 256;
+    const size_t sort = ingest_sort_smem(Np);
+    k_ingest_scan<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_keys<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_sort<<<1, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_edits<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_emit<<<1, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
+    ctx->launches += 5;
+  }
   k_expand<<<g, 256, 0, ctx->stream>>>(ctx->d);
   ++ctx->launches;
   k_merge_pieces<<<1, 1024, 0, ctx->stream>>>(
@@ -1005,6 +1020,12 @@ osp_status osp_create(osp_ctx** out, const osp_options* opt) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_ingest, cudaFuncAttributeMaxDynamicSharedMemorySize, kIngestSmem);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_ingest_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ingest_sort_smem(kMaxBatch));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_ingest_emit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ingest_sort_smem(kMaxBatch));
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_topk_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kTopkSortSmem);
   if (e != cudaSuccess) {
@@ -1152,6 +1173,8 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
   AL(d.del_c, kMaxBatch, 0);
   AL(d.gi, kMaxBatch + 1, 0);
   AL(d.gd, kMaxBatch + 1, 0);
+  AL(d.ing_key, kMaxBatch, 0);
+  AL(d.ing_na, kMaxBatch, 0);
   AL(d.rec_r_node, nc, 0);
   AL(d.rec_r_is, nc, 0);
   AL(d.rec_r_ic, nc, 0);
@@ -1392,7 +1415,7 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
 
 // x(0) = c e_s per seed, with the scores cleared.
 osp_status enqueue_cpi_start(osp_ctx* ctx) {
-  k_reset_batch<<<1, 1, 0, ctx->stream>>>(ctx->d, 0);
+  k_reset_batch<<<1, 256, 0, ctx->stream>>>(ctx->d, 0);
   ++ctx->launches;
   if (ctx->S > 1) {
     const Multi& M = ctx->d.mu;

@@ -157,6 +157,12 @@ __device__ void emit_groups(const unsigned long long* skey, int N, int per, int 
 // counts carry over; only the per-sub-batch records restart.
 __global__ void k_reset_batch(Dev d, int cont) {
   Ctl* c = d.ctl;
+  // rows zeroed by the previous batch (merged by now) lose their mark
+  for (int i = threadIdx.x; i < c->n_clr; i += blockDim.x) d.clr_pos[d.clr_nodes[i]] = -1;
+  if (threadIdx.x != 0) return;
+  c->ing_bad = kNoPos;
+  c->ing_clr = 0;
+  c->ing_reins = 0;
   c->status = 0;
   c->bad_op = -1;
   c->n_old = c->n;
@@ -221,9 +227,6 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest(Dev d, const osp_upda
   if (U < 0) U = ctl->batch_U;  // replayed from a CUDA graph: the size is set per call
   const int tid = threadIdx.x;
   const int n_old = ctl->n;
-  // rows zeroed by the previous batch (merged by now) lose their mark
-  const int n_clr_prev = ctl->n_clr;
-  for (int i = tid; i < n_clr_prev; i += kIngestThreads) d.clr_pos[d.clr_nodes[i]] = -1;
   if (tid == 0) {
     s_bad = kNoPos;
     s_ndel = 0;
@@ -411,6 +414,418 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest(Dev d, const osp_upda
     ctl->n_del = s_ndel;
     ctl->n_clr = s_nclr;
     ctl->n = n_old + tot_adds;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Larger batches (more than kIngestOne ops): the same steps over many CTAs. One
+// CTA spent 760 us on 10,001 ops and 867 us on 15,000: two bitonic sorts (105
+// passes of 16,384 keys through shared memory each), the existence searches
+// (some 14 scattered loads an op from one SM) and 16 ops a thread one after the
+// other. Here the searches and validation run one op a thread, and one CTA sorts
+// by stable 8-bit radix passes over the bits in use.
+//   k_ingest_scan   node count before each op; first deletion, last zeroing
+//   k_ingest_keys   validation; sort keys (u, v, position)
+//   k_ingest_sort   the radix sort (or the report of the first invalid op)
+//   k_ingest_edits  last op of each pair against the current row: net edits
+//   k_ingest_emit   edit lists and records of rows, the same sorted for columns
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int kSortRows = kMaxBatch / kIngestThreads;  // keys a thread
+
+// Bits of a node id among n nodes, so that no id has all of them set.
+__device__ __forceinline__ int id_bits(int n) { return 32 - __clz(n); }
+
+// Stable radix sort of `per` * 1024 keys by bits [lo, hi), eight a pass. Thread
+// (warp w, lane l) holds keys w per 32 + 32 r + l, r < per, before and after.
+// s_key: the keys' buffer; s_cnt: 32 x 256 counts.
+__device__ void radix_sort(unsigned long long (&key)[kSortRows], int per, int lo, int hi,
+                           unsigned long long* s_key, int* s_cnt) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int sh = lo; sh < hi; sh += 8) {
+    const unsigned mask = (1u << min(8, hi - sh)) - 1u;
+    for (int i = tid; i < 32 * 256; i += kIngestThreads) s_cnt[i] = 0;
+    __syncthreads();
+    unsigned rank[kSortRows / 2];  // two 16-bit ranks a register
+#pragma unroll
+    for (int r = 0; r < kSortRows; ++r) {
+      if (r >= per) break;
+      const unsigned dg = (unsigned)(key[r] >> sh) & mask;
+      unsigned peers = 0xffffffffu;  // lanes with this digit, a ballot a bit
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        const unsigned v = __ballot_sync(0xffffffffu, (dg >> b) & 1u);
+        peers &= (dg >> b) & 1u ? v : ~v;
+      }
+      const int leader = __ffs(peers) - 1;
+      int old = 0;
+      if (lane == leader) {
+        old = s_cnt[w * 256 + dg];
+        s_cnt[w * 256 + dg] = old + __popc(peers);
+      }
+      __syncwarp();
+      const unsigned rk = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lanemask_lt());
+      rank[r / 2] = r & 1 ? rank[r / 2] | rk << 16 : rk;
+    }
+    __syncthreads();
+    // exclusive scan, digits first, then warps: thread t owns warps 8 (t % 4) ..
+    // of digit t / 4
+    {
+      const int dg = tid >> 2, w0 = 8 * (tid & 3);
+      int c[8], sum = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        c[q] = s_cnt[(w0 + q) * 256 + dg];
+        sum += c[q];
+      }
+      int tot;
+      int base = block_exscan(sum, &tot);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        s_cnt[(w0 + q) * 256 + dg] = base;
+        base += c[q];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortRows; ++r) {
+      if (r >= per) break;
+      const int at = s_cnt[w * 256 + ((unsigned)(key[r] >> sh) & mask)] +
+                     (int)(r & 1 ? rank[r / 2] >> 16 : rank[r / 2] & 0xFFFFu);
+      s_key[at] = key[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortRows; ++r) {
+      if (r >= per) break;
+      key[r] = s_key[(w * per + r) * 32 + lane];
+    }
+    __syncthreads();
+  }
+}
+
+// Edit lists and records of one direction from `per` * 1024 sorted edits (key[r]
+// as in radix_sort; kind 0 none, 1 insert, 2 delete; group_of(key) the list's
+// node, member_of(key) the entry). s_a, s_b: 1024 per + 1 ints each.
+template <typename GroupF, typename MemberF>
+__device__ void emit_edits(const unsigned long long (&key)[kSortRows], const int (&kind)[kSortRows],
+                           int per, unsigned long long* s_key, int* s_a, int* s_b, GroupF group_of,
+                           MemberF member_of, int* ins_out, int* del_out, int* rec_node, int* rec_is,
+                           int* rec_ic, int* rec_ds, int* rec_dc, int* flag_arr, int* n_rec,
+                           int* n_ins, int* n_del) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int N = per * kIngestThreads;
+  // the three running counts (insertions, deletions, groups) by warp: a warp's
+  // keys are consecutive
+  __shared__ int s_heads;
+  int ci = 0, cd = 0, ch = 0;
+  unsigned bi[kSortRows], bd[kSortRows], bh[kSortRows];
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    bi[r] = bd[r] = bh[r] = 0;
+    if (r >= per) continue;
+    const int i = (w * per + r) * 32 + lane;
+    const bool real = key[r] != kNoKey;
+    const bool head = real && (i == 0 || group_of(s_key[i - 1]) != group_of(key[r]));
+    bi[r] = __ballot_sync(0xffffffffu, kind[r] == 1);
+    bd[r] = __ballot_sync(0xffffffffu, kind[r] == 2);
+    bh[r] = __ballot_sync(0xffffffffu, head);
+    ci += __popc(bi[r]);
+    cd += __popc(bd[r]);
+    ch += __popc(bh[r]);
+  }
+  int ti, td, th;
+  const int one = lane == 0;
+  int pi = block_exscan(one ? ci : 0, &ti), pd = block_exscan(one ? cd : 0, &td),
+      ph = block_exscan(one ? ch : 0, &th);
+  pi = __shfl_sync(0xffffffffu, pi, 0);
+  pd = __shfl_sync(0xffffffffu, pd, 0);
+  ph = __shfl_sync(0xffffffffu, ph, 0);
+  // edits out; for group g: counts before its first edit (s_a, s_b)
+  int* head_at = rec_node;  // scratch until the records are written: the groups' nodes
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    if (r >= per) break;
+    const unsigned lt = lanemask_lt();
+    const int ai = pi + __popc(bi[r] & lt), ad = pd + __popc(bd[r] & lt);
+    if (kind[r] == 1) ins_out[ai] = member_of(key[r]);
+    if (kind[r] == 2) del_out[ad] = member_of(key[r]);
+    if ((bh[r] >> lane) & 1u) {
+      const int g = ph + __popc(bh[r] & lt);
+      s_a[g] = ai;
+      s_b[g] = ad;
+      head_at[g] = group_of(key[r]);
+    }
+    pi += __popc(bi[r]);
+    pd += __popc(bd[r]);
+    ph += __popc(bh[r]);
+  }
+  if (tid == 0) {
+    s_a[th] = ti;
+    s_b[th] = td;
+    s_heads = 0;
+  }
+  __syncthreads();
+  // groups with an edit, in order
+  for (int b = 0; b < th; b += kIngestThreads) {
+    const int g = b + tid;
+    int node = 0, is = 0, ic = 0, ds = 0, dc = 0;
+    if (g < th) {
+      node = head_at[g];
+      is = s_a[g];
+      ic = s_a[g + 1] - is;
+      ds = s_b[g];
+      dc = s_b[g + 1] - ds;
+    }
+    int tot;
+    const int at = s_heads + block_exscan(ic + dc > 0, &tot);
+    if (ic + dc > 0) {  // at <= g: the nodes still to be read lie at or above it
+      rec_node[at] = node;
+      rec_is[at] = is;
+      rec_ic[at] = ic;
+      rec_ds[at] = ds;
+      rec_dc[at] = dc;
+      flag_arr[node] = 1;
+    }
+    __syncthreads();
+    if (tid == 0) s_heads += tot;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    *n_rec = s_heads;
+    *n_ins = ti;
+    *n_del = td;
+  }
+  __syncthreads();
+  (void)N;
+}
+
+__device__ __forceinline__ int batch_size(const Dev& d, int U) { return U < 0 ? d.ctl->batch_U : U; }
+
+// Keys a thread for a batch of U: whole rows of 1024.
+__device__ __forceinline__ int sort_rows(int U) { return max(1, (U + kIngestThreads - 1) / kIngestThreads); }
+
+}  // namespace
+
+__global__ void __launch_bounds__(256) k_ingest_scan(Dev d, const osp_update* __restrict__ ops, int U) {
+  __shared__ int s_w[8];
+  Ctl* ctl = d.ctl;
+  U = batch_size(d, U);
+  const int b0 = blockIdx.x * 256;
+  if (b0 >= U && blockIdx.x) return;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // node additions before this CTA's ops, then before each of them
+  int before = 0;
+  for (int i = tid; i < b0; i += 256) before += ops[i].op == OSP_OP_ADD_NODE;
+  before = warp_sum(before);
+  if (lane == 0) s_w[w] = before;
+  __syncthreads();
+  int base = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) base += s_w[q];
+  __syncthreads();
+  const int p = b0 + tid;
+  const bool add = p < U && ops[p].op == OSP_OP_ADD_NODE;
+  const unsigned m = __ballot_sync(0xffffffffu, add);
+  if (lane == 0) s_w[w] = __popc(m);
+  __syncthreads();
+  for (int q = 0; q < w; ++q) base += s_w[q];
+  const int run = base + __popc(m & lanemask_lt());
+  if (p == U - 1) ctl->ing_adds = run + add;
+  if (U == 0 && tid == 0) ctl->ing_adds = 0;
+  if (p >= U) return;
+  const int na = ctl->n + run;
+  d.ing_na[p] = na;
+  const osp_update o = load_op(ops, p, d);
+  if (o.op == OSP_OP_DELETE_NODE) {
+    if (o.u >= 0 && o.u < na && !d.dead[o.u] && !d.seedflag[o.u]) atomicMin(&d.del_pos[o.u], p);
+    else atomicMin(&ctl->ing_bad, p);
+  } else if (o.op == OSP_OP_ZERO_ROW) {
+    // the last zeroing of a row in the batch voids the row's earlier edge ops
+    ctl->ing_clr = 1;
+    if (o.u >= 0 && o.u < na) atomicMax(&d.clr_pos[o.u], p);
+    else atomicMin(&ctl->ing_bad, p);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_ingest_keys(Dev d, const osp_update* __restrict__ ops, int U) {
+  Ctl* ctl = d.ctl;
+  U = batch_size(d, U);
+  const int p = blockIdx.x * 256 + threadIdx.x;
+  if (p >= U) return;
+  const osp_update o = load_op(ops, p, d);
+  const int na = d.ing_na[p];
+  const int bits = id_bits(ctl->n + ctl->ing_adds);
+  bool ok = false;
+  unsigned long long key = kNoKey;
+  if (o.op == OSP_OP_INSERT_EDGE || o.op == OSP_OP_DELETE_EDGE) {
+    if (o.u >= 0 && o.u < na && o.v >= 0 && o.v < na) {
+      const int du = d.del_pos[o.u], dv = d.del_pos[o.v];
+      ok = !d.dead[o.u] && !d.dead[o.v] && du > p && dv > p;
+      if (du == kNoPos && dv == kNoPos && (!ctl->ing_clr || d.clr_pos[o.u] < p))
+        key = ((unsigned long long)o.u << (14 + bits)) | ((unsigned long long)o.v << 14) | (unsigned)p;
+    }
+  } else if (o.op == OSP_OP_ADD_NODE) {
+    ok = true;
+  } else if (o.op == OSP_OP_DELETE_NODE) {
+    ok = o.u >= 0 && o.u < na && !d.dead[o.u] && !d.seedflag[o.u] && d.del_pos[o.u] == p;
+  } else if (o.op == OSP_OP_ZERO_ROW) {
+    ok = o.u >= 0 && o.u < na && !d.dead[o.u] && d.del_pos[o.u] > p;
+  }
+  if (!ok) atomicMin(&ctl->ing_bad, p);
+  d.ing_key[p] = key;
+}
+
+__global__ void __launch_bounds__(kIngestThreads) k_ingest_sort(Dev d, const osp_update* __restrict__ ops,
+                                                                int U) {
+  extern __shared__ unsigned long long skey[];
+  Ctl* ctl = d.ctl;
+  U = batch_size(d, U);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int bad = ctl->ing_bad;
+  if (bad != kNoPos) {
+    for (int p = tid; p < U; p += kIngestThreads) {
+      const int op = ops[p].op;
+      if (op == OSP_OP_DELETE_NODE || op == OSP_OP_ZERO_ROW) {
+        const osp_update o = load_op(ops, p, d);
+        if (o.u >= 0 && o.u < d.nc) {
+          if (op == OSP_OP_DELETE_NODE) d.del_pos[o.u] = kNoPos;
+          else d.clr_pos[o.u] = -1;
+        }
+      }
+    }
+    if (tid == 0) {
+      ctl->status = OSP_EINVAL;
+      ctl->bad_op = bad;
+      ctl->n_clr = 0;
+    }
+    return;
+  }
+  const int per = sort_rows(U);
+  unsigned long long key[kSortRows];
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    const int i = (w * per + r) * 32 + lane;
+    key[r] = r < per && i < U ? d.ing_key[i] : kNoKey;
+  }
+  __syncthreads();  // all keys are in registers
+  radix_sort(key, per, 14, 14 + 2 * id_bits(ctl->n + ctl->ing_adds), skey,
+             reinterpret_cast<int*>(skey + per * kIngestThreads));
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r)
+    if (r < per && (w * per + r) * 32 + lane < U) d.ing_key[(w * per + r) * 32 + lane] = key[r];
+}
+
+// One thread per sorted op: the last op of each (u, v) against the current row.
+__global__ void __launch_bounds__(256) k_ingest_edits(Dev d, const osp_update* __restrict__ ops, int U) {
+  Ctl* ctl = d.ctl;
+  if (*(volatile int*)&ctl->status) return;
+  U = batch_size(d, U);
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= U) return;
+  const unsigned long long key = d.ing_key[i];
+  const int n_old = ctl->n;
+  const int bits = id_bits(n_old + ctl->ing_adds);
+  int kind = 0;
+  if (key != kNoKey && (i == U - 1 || (d.ing_key[i + 1] >> 14) != (key >> 14))) {
+    const int p = (int)(key & 0x3FFF);
+    const int u = (int)(key >> (14 + bits));
+    const int v = (int)((key >> 14) & ((1ull << bits) - 1));
+    const bool after = ops[p].op == OSP_OP_INSERT_EDGE;
+    bool before = false;
+    if (u < n_old && v < n_old) {
+      // u -> v exists iff v is in u's out-list, or u in v's in-list: search the shorter
+      const int lr = d.len_r[u], lc = d.len_c[v];
+      before = lr <= lc ? contains_i(d.pool_r + d.off_r[u], lr, v)
+                        : contains_i(d.pool_c + d.off_c[v], lc, u);
+    }
+    if (ctl->ing_clr && d.clr_pos[u] >= 0) {
+      // u's row was zeroed before this op: the merge drops every old entry of
+      // the row (and u from the old in-lists), so a surviving edge is written
+      // again as an insertion, but it is not a new edge
+      if (after && before) atomicAdd((unsigned long long*)&ctl->ing_reins, 1ull);
+      before = false;
+    }
+    kind = after && !before ? 1 : !after && before ? 2 : 0;
+  }
+  d.ing_na[i] = kind;
+}
+
+__global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp_update* __restrict__ ops,
+                                                                int U) {
+  extern __shared__ unsigned long long skey[];
+  __shared__ int s_ndel, s_nclr;
+  Ctl* ctl = d.ctl;
+  if (*(volatile int*)&ctl->status) return;
+  U = batch_size(d, U);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int per = sort_rows(U);
+  const int adds = ctl->ing_adds;
+  const int bits = id_bits(ctl->n + adds);
+  int* s_a = reinterpret_cast<int*>(skey + per * kIngestThreads);  // at least 32 x 256 ints
+  int* s_b = d.gi;  // [kMaxBatch + 1]
+  unsigned long long key[kSortRows];
+  int kind[kSortRows];
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    const int i = (w * per + r) * 32 + lane;
+    key[r] = r < per && i < U ? d.ing_key[i] : kNoKey;
+    kind[r] = r < per && i < U ? d.ing_na[i] : 0;
+    if (r < per) skey[i] = key[r];
+  }
+  if (tid == 0) s_ndel = s_nclr = 0;
+  __syncthreads();
+  int n_ins = 0, n_del = 0;
+  emit_edits(
+      key, kind, per, skey, d.gd, s_b, [&](unsigned long long k) { return (int)(k >> (14 + bits)); },
+      [&](unsigned long long k) { return (int)((k >> 14) & ((1ull << bits) - 1)); }, d.ins_r, d.del_r,
+      d.rec_r_node, d.rec_r_is, d.rec_r_ic, d.rec_r_ds, d.rec_r_dc, d.rflag, &ctl->n_rec_r, &n_ins,
+      &n_del);
+  if (tid == 0) {  // summed over the sub-batches of a large batch
+    ctl->net_ins += n_ins - ctl->ing_reins;
+    ctl->net_del += n_del;
+  }
+  // the same edits by (v, u): they come by u, so a stable sort by v is enough
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    if (kind[r]) {
+      const unsigned long long u = key[r] >> (14 + bits), v = (key[r] >> 14) & ((1ull << bits) - 1);
+      key[r] = (v << (bits + 1)) | (u << 1) | (kind[r] == 2);
+    } else {
+      key[r] = kNoKey;
+    }
+  }
+  __syncthreads();
+  radix_sort(key, per, bits + 1, 2 * bits + 1, skey, s_a);
+#pragma unroll
+  for (int r = 0; r < kSortRows; ++r) {
+    if (r < per) skey[(w * per + r) * 32 + lane] = key[r];
+    kind[r] = r >= per || key[r] == kNoKey ? 0 : key[r] & 1 ? 2 : 1;
+  }
+  __syncthreads();
+  emit_edits(
+      key, kind, per, skey, d.gd, s_b, [&](unsigned long long k) { return (int)(k >> (bits + 1)); },
+      [&](unsigned long long k) { return (int)((k >> 1) & ((1ull << bits) - 1)); }, d.ins_c, d.del_c,
+      d.rec_c_node, d.rec_c_is, d.rec_c_ic, d.rec_c_ds, d.rec_c_dc, d.cflag, &ctl->n_rec_c, &n_ins,
+      &n_del);
+  // node deletions and zeroed rows
+  for (int p = tid; p < U; p += kIngestThreads) {
+    const int op = ops[p].op;
+    if (op == OSP_OP_DELETE_NODE) {
+      const int u = load_op(ops, p, d).u;
+      d.del_nodes[atomicAdd(&s_ndel, 1)] = u;
+      d.del_pos[u] = kNoPos;
+    } else if (op == OSP_OP_ZERO_ROW) {
+      const int u = load_op(ops, p, d).u;
+      if (d.clr_pos[u] == p) d.clr_nodes[atomicAdd(&s_nclr, 1)] = u;  // once per row
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    ctl->n_del = s_ndel;
+    ctl->n_clr = s_nclr;
+    ctl->n += adds;
   }
 }
 

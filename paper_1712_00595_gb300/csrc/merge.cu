@@ -87,49 +87,66 @@ __global__ void __launch_bounds__(1024) k_merge_pieces(Dev d, double beta) {
   const int nr = ctl->n_rec_r;
   const int R = nr + ctl->n_rec_c;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int per = (R + 1023) / 1024;
-  const int lo = min(R, tid * per), hi = min(R, lo + per);
-  int mine = 0;
+  // lists in rows of 1024, four rows' loads in flight (consecutive lists a thread
+  // had cost 55 us for 10,000 lists, each thread's loads one after the other)
+  __shared__ int s_base;
   long long touch = 0;  // out-list entries old and new of the changed rows
-  for (int c = lo; c < hi; ++c) {
-    const bool rows = c < nr;
-    const int node = rows ? d.rec_r_node[c] : d.rec_c_node[c - nr];
-    const unsigned o = rows ? d.off_r[node] : d.off_c[node];
-    const int L = rows ? d.len_r[node] : d.len_c[node];
-    d.rec_old_off[c] = o;
-    d.rec_old_len[c] = L;
-    mine += L > 0 ? (L + kPiece - 1) / kPiece : 1;
-    if (rows) touch += L + d.rec_r_ic[c];
+  if (tid == 0) s_base = 0;
+  __syncthreads();
+  for (int c0 = 0; c0 < R; c0 += 4 * 1024) {
+    int node[4], L[4];
+    unsigned o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = c0 + 1024 * q + tid;
+      node[q] = c < nr ? d.rec_r_node[c] : c < R ? d.rec_c_node[c - nr] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = c0 + 1024 * q + tid;
+      L[q] = c < nr ? d.len_r[node[q]] : c < R ? d.len_c[node[q]] : 0;
+      o[q] = c < nr ? d.off_r[node[q]] : c < R ? d.off_c[node[q]] : 0u;
+      if (c < nr) touch += L[q] + d.rec_r_ic[c];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = c0 + 1024 * q + tid;
+      if (c0 + 1024 * q >= R) break;  // uniform
+      const int np = c < R ? (L[q] > 0 ? (L[q] + kPiece - 1) / kPiece : 1) : 0;
+      int x = np;
+      for (int k = 1; k < 32; k <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, k);
+        if (lane >= k) x += y;
+      }
+      if (lane == 31) s_w[w] = x;
+      __syncthreads();
+      if (w == 0) {
+        int t = s_w[lane];
+        for (int k = 1; k < 32; k <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, t, k);
+          if (lane >= k) t += y;
+        }
+        s_w[lane] = t;
+      }
+      __syncthreads();
+      const int base = s_base + (w ? s_w[w - 1] : 0) + x - np;
+      if (c < R) {
+        d.rec_old_off[c] = o[q];
+        d.rec_old_len[c] = L[q];
+        d.rec_pstart[c] = base;
+        for (int k = 0; k < np; ++k) d.piece_rec[base + k] = c;
+      }
+      __syncthreads();
+      if (tid == 0) s_base += s_w[31];
+      __syncthreads();
+    }
   }
   touch = warp_sum(touch);
   if (lane == 0) s_b[w] = touch;
-  int x = mine;
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_w[w] = x;
   __syncthreads();
-  if (w == 0) {
-    int t = s_w[lane];
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += y;
-    }
-    s_w[lane] = t;
-  }
-  __syncthreads();
-  int base = (w ? s_w[w - 1] : 0) + x - mine;
-  for (int c = lo; c < hi; ++c) {
-    const int L = d.rec_old_len[c];
-    const int np = L > 0 ? (L + kPiece - 1) / kPiece : 1;
-    d.rec_pstart[c] = base;
-    for (int q = 0; q < np; ++q) d.piece_rec[base + q] = c;
-    base += np;
-  }
   if (tid == 0) {
-    ctl->n_mpieces = s_w[31];
-    d.rec_pstart[R] = s_w[31];
+    ctl->n_mpieces = s_base;
+    d.rec_pstart[R] = s_base;
     long long t = 0;
     for (int i = 0; i < 32; ++i) t += s_b[i];
     // the offset reaches at most `t` nodes; above n/beta the first step is
@@ -553,16 +570,56 @@ __global__ void k_scan_add(unsigned* out, const unsigned* __restrict__ bsum, int
   if (i < n) out[i] += bsum[i / kScanTile];
 }
 
-__global__ void k_compact_copy(const unsigned* __restrict__ off_old, const int* __restrict__ len,
-                               const int* __restrict__ pool_old, const unsigned* __restrict__ off_new,
-                               int* pool_new, int n) {
+// A warp copies kCopyChunk entries of the new pool, whichever lists they belong
+// to (a warp per list had the longest list's copy as its time: 225 us for 3 M
+// entries): the first list by binary search, then 32 lists at a time as one
+// stream of entries, four rounds of 32 in flight.
+constexpr int kCopyChunk = 1024;
+__global__ void __launch_bounds__(256) k_compact_copy(const unsigned* __restrict__ off_old,
+                                                      const int* __restrict__ len,
+                                                      const int* __restrict__ pool_old,
+                                                      const unsigned* __restrict__ off_new,
+                                                      int* pool_new, int n) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int u = gw; u < n; u += nw) {
-    const unsigned a = off_old[u], b = off_new[u];
-    const int l = len[u];
-    for (int j = lane; j < l; j += 32) pool_new[b + j] = pool_old[a + j];
+  const unsigned m = off_new[n - 1] + (unsigned)len[n - 1];
+  for (long long c0 = (long long)gw * kCopyChunk; c0 < (long long)m; c0 += (long long)nw * kCopyChunk) {
+    const unsigned p0 = (unsigned)c0, p1 = min(m, p0 + kCopyChunk);
+    int lo = 0, hi = n - 1;  // the last list that starts at or before p0
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (off_new[mid] <= p0) lo = mid;
+      else hi = mid - 1;
+    }
+    unsigned p = p0;
+    for (int u0 = lo; p < p1; u0 += 32) {
+      const int u = u0 + lane;
+      const unsigned b = u < n ? off_new[u] : m;       // ascending over the lanes
+      const unsigned a = u < n ? off_old[u] : 0u;
+      const unsigned end = min(p1, u0 + 32 < n ? off_new[u0 + 32] : m);
+      for (; p < end; p += 128) {
+        unsigned from[4];
+        int v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const unsigned e = p + 32 * r + lane;
+          int l = 0;  // the last lane whose list starts at or before e
+#pragma unroll
+          for (int q = 16; q > 0; q >>= 1) {
+            const unsigned bm = __shfl_sync(0xffffffffu, b, l + q);
+            if (bm <= e) l += q;
+          }
+          from[r] = __shfl_sync(0xffffffffu, a, l) + (e - __shfl_sync(0xffffffffu, b, l));
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = p + 32 * r + lane < end ? pool_old[from[r]] : 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (p + 32 * r + lane < end) pool_new[p + 32 * r + lane] = v[r];
+      }
+      p = end;
+    }
   }
 }
 

@@ -188,12 +188,12 @@ __global__ void __launch_bounds__(256) k_topk_collect(TopkJobs J, int cap) {
   bin_range(st, &lo, &hi);
   const int stride = gridDim.x * blockDim.x;
   // whole warps stay in the loop: the append below is warp-wide
-  for (int b = blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < n; b += 4 * stride) {
-    unsigned long long key[4];
-    unsigned m[4];
+  for (int b = blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < n; b += 8 * stride) {
+    unsigned long long key[8];
+    unsigned m[8];
     int tot = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 8; ++q) {
       const long long i = (long long)b + (threadIdx.x & 31) + (long long)q * stride;
       key[q] = i < n ? order_key(__ldg(r + i)) : 0ull;
       m[q] = __ballot_sync(0xffffffffu, i < n && key[q] >= lo);
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256) k_topk_collect(TopkJobs J, int cap) {
     if ((threadIdx.x & 31) == 0) at = atomicAdd(&st->count, tot);
     at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 8; ++q) {
       const int p = at + __popc(m[q] & lanemask_lt());
       if ((m[q] >> (threadIdx.x & 31)) & 1u && p < cap) {
         jb.keys[p] = key[q];
@@ -422,9 +422,20 @@ __global__ void __launch_bounds__(1024) k_topk_sort(TopkJobs J, int cap) {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hist[i] = 0;
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kPer; ++q)
-      if (threadIdx.x + 1024 * q < cnt && place(key[q], id[q], p) == 0)
-        atomicAdd(&s_hist[digit(key[q], id[q], p)], 1u);
+    for (int q = 0; q < kPer; ++q) {
+      if (1024 * q >= cnt) break;
+      // survivors of one bin share their leading digits: one addition a warp then
+      const bool in = threadIdx.x + 1024 * q < cnt && place(key[q], id[q], p) == 0;
+      const unsigned dg = digit(key[q], id[q], p);
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (!m) continue;
+      const unsigned d0 = __shfl_sync(0xffffffffu, dg, __ffs(m) - 1);
+      if (__all_sync(0xffffffffu, !in || dg == d0)) {
+        if ((threadIdx.x & 31) == 0) atomicAdd(&s_hist[d0], (unsigned)__popc(m));
+      } else if (in) {
+        atomicAdd(&s_hist[dg], 1u);
+      }
+    }
     __syncthreads();
     if (threadIdx.x < 32) {  // suffix sums from the largest digit; lane l owns digits 255 - 8 l ..
       unsigned c[8], sum = 0;

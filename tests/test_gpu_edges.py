@@ -145,3 +145,54 @@ def test_topk_of_awkward_vectors(n):
             assert c == min(n, k)
             assert np.array_equal(ids[:c].cpu().numpy(), want_ids)
             assert np.array_equal(sc[:c].cpu().numpy(), want_sc)
+
+
+@pytest.mark.parametrize("n_ops", [511, 1024, 1025, 2500, 9000])
+def test_batches_of_every_op_kind_across_the_ingest_sizes(n_ops):
+    """Edge and node ops, row zeroings, repeated and contradicting ops, on both
+    sides of the one-CTA ingest: the graph equals the oracle's, and an invalid op
+    anywhere leaves it unchanged and is the one reported."""
+    rng = np.random.default_rng(n_ops)
+    n = 700
+    src, dst = W.er_graph(n, 6000, 3)
+    seed = 5
+    eng = N.Engine(precision=N.OSP_PREC_FP64, device=0, max_nodes=n + 40000, use_graphs=n_ops % 2 == 0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds([seed], C_RESTART)
+    eng.init_scores(1e-10)
+    g = O.Graph(n, src, dst)
+    nn, dead = n, set()
+    for rep in range(3):
+        kind = rng.choice(5, n_ops, p=[0.46, 0.46, 0.04, 0.02, 0.02])
+        ops = np.zeros(n_ops, W.UPDATE_DTYPE)
+        gone = set(dead)
+        count = nn
+        for i, k in enumerate(kind):
+            live = [x for x in rng.integers(0, count, 40) if x not in gone]
+            u, v = int(live[0]), int(live[1])
+            if k <= 1 and rng.random() < 0.3:  # a few rows get many ops
+                u = int(rng.integers(0, 12))
+                u = u if u not in gone else int(live[0])
+            if k == 3 and u == seed:
+                k = 4
+            ops[i] = (u, v, k) if k != 2 else (0, 0, 2)
+            count += k == 2
+            if k == 3:
+                gone.add(u)
+        bad = ops.copy()
+        at = int(rng.integers(0, n_ops))
+        bad[at] = [(count + 5, 0, 0), (0, -1, 1), (seed, 0, 3), (0, 0, 9)][rep % 4]
+        before = eng.export_graph(0)
+        st = eng.apply_updates(bad, 1e-8, allow=(N.OSP_EINVAL,))
+        assert eng.last_status == N.OSP_EINVAL and st["bad_op"] == at
+        assert all(np.array_equal(a, b) for a, b in zip(before, eng.export_graph(0)))
+        eng.apply_updates(ops, 1e-8)
+        assert g.apply(ops, protect=(seed,)) == -1
+        nn, dead = count, gone
+        ptr, idx = eng.export_graph(0)
+        rp, col = g.csr()
+        assert np.array_equal(ptr, rp) and np.array_equal(idx, col)
+        ptr, idx = eng.export_graph(1)
+        cp, row = g.csc()
+        assert np.array_equal(ptr, cp) and np.array_equal(idx, row)
+    eng.close()
