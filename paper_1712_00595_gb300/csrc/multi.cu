@@ -1305,7 +1305,13 @@ __global__ void __launch_bounds__(1024) k_offset_multi_plan(Dev d) {
 // out-list entries, times +(1-c)/d'_u over the new ones (one combined term
 // for an entry in both lists); stamps the targets. Lane l owns columns
 // l, l + 32, ..., so each atomic instruction of the warp covers 32
-// consecutive columns (8 sectors) of the target's row.
+// consecutive columns (8 sectors) of the target's row. An item has three
+// weights (kept, removed, new), so the products are formed once an item: one
+// double multiplication per entry and 32 columns, at 16 cycles of the SM, and a
+// walk entry by entry through the unchanged ones bound the kernel before (2^18
+// nodes, 64 seeds, 1,000 edge ops: 258 -> 69 us; 131,071 nodes, 100 seeds: 152 ->
+// 60 us). The binary searches run on the part of the other list that the item's
+// first and last entry bound.
 template <int K>
 __global__ void __launch_bounds__(256) k_offset_multi(Dev d) {
   constexpr int Sp = 32 * K;
@@ -1324,46 +1330,65 @@ __global__ void __launch_bounds__(256) k_offset_multi(Dev d) {
     const int u = d.rec_r_node[c];
     const int L = d.rec_old_len[c], dp = d.rec_dp[c];
     double ru[K];
+    unsigned nz = 0;  // bit k: some column of part k has a score
+    unsigned mine = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) ru[k] = __ldcg(d.mu.r + (size_t)u * Sp + lane + 32 * k);
-    bool nz = false;
 #pragma unroll
-    for (int k = 0; k < K; ++k) nz |= ru[k] != 0.0;
-    if (!__any_sync(0xffffffffu, nz)) continue;
+    for (int k = 0; k < K; ++k) {
+      nz |= (unsigned)__any_sync(0xffffffffu, ru[k] != 0.0) << k;
+      mine |= (unsigned)(ru[k] != 0.0) << k;
+    }
+    if (!nz) continue;
     const double wa = L ? c1 / (double)L : 0.0;
     const double wb = dp ? c1 / (double)dp : 0.0;
     const int* oldl = d.pool_r + d.rec_old_off[c];
     const int* newl = d.pool_r + d.rec_fbase[c];
     const int e0 = q * kPiece, e1 = min(e0 + kPiece, L + dp);
+    // the other list's part that can hold this item's entries (both ascend):
+    // lanes 0 and 1 bound the old entries' part of the new list, 2 and 3 the new
+    // entries' part of the old list
+    int bound = 0;
+    {
+      const int o0 = min(e0, L), o1 = min(e1, L), n0 = max(e0 - L, 0), n1 = max(e1 - L, 0);
+      if (lane == 0 && o0 < o1) bound = lower_bound_i(newl, dp, oldl[o0]);
+      if (lane == 1 && o0 < o1) bound = lower_bound_i(newl, dp, oldl[o1 - 1] + 1);
+      if (lane == 2 && n0 < n1) bound = lower_bound_i(oldl, L, newl[n0]);
+      if (lane == 3 && n0 < n1) bound = lower_bound_i(oldl, L, newl[n1 - 1] + 1);
+    }
+    const int nb0 = __shfl_sync(0xffffffffu, bound, 0), nb1 = __shfl_sync(0xffffffffu, bound, 1);
+    const int ob0 = __shfl_sync(0xffffffffu, bound, 2), ob1 = __shfl_sync(0xffffffffu, bound, 3);
+    // one pass an entry kind: 0 kept, (1-c)(1/d' - 1/d), nothing when the degree
+    // did not change; 1 removed; 2 new
     for (int eb = e0; eb < e1; eb += 32) {
       const int e = eb + lane;
-      int a = 0;
-      double wgt = 0.0;
+      int a = 0, kind = 3;
       if (e < e1) {
-        // an entry kept in the new list carries both terms at once:
-        // (1-c)(1/d' - 1/d), zero when the degree did not change
         if (e < L) {
           a = oldl[e];
-          wgt = contains_i(newl, dp, a) ? wb - wa : -wa;
+          kind = contains_i(newl + nb0, nb1 - nb0, a) ? 0 : 1;
         } else {
           a = newl[e - L];
-          wgt = contains_i(oldl, L, a) ? 0.0 : wb;
+          kind = contains_i(oldl + ob0, ob1 - ob0, a) ? 3 : 2;
         }
       }
-      if (!OSP_GUARD(ctl, a >= 0 && a < d.nc, "multi offset target", c, e, a)) a = 0;
-      const int cnt = min(32, e1 - eb);
-      for (int j = 0; j < cnt; ++j) {
-        const double wj = __shfl_sync(0xffffffffu, wgt, j);
-        if (wj == 0.0) continue;  // warp-uniform
-        const int aj = __shfl_sync(0xffffffffu, a, j);
-        double* row = d.mu.xacc + (size_t)aj * Sp + lane;
+      if (!OSP_GUARD(ctl, a >= 0 && a < d.nc, "multi offset target", c, e, a)) kind = 3;
+      for (int t = 0; t < 3; ++t) {
+        const double w = t == 0 ? wb - wa : t == 1 ? -wa : wb;
+        unsigned m = __ballot_sync(0xffffffffu, kind == t);
+        if (!m || w == 0.0) continue;  // warp-uniform
+        double x[K];
 #pragma unroll
-        for (int k = 0; k < K; ++k)
-          if (ru[k] != 0.0) {
-            atomicAdd(row + 32 * k, wj * ru[k]);
-            hit |= 1u << k;
-          }
-        if (lane == 0) d.mark[aj] = epoch;
+        for (int k = 0; k < K; ++k) x[k] = (nz >> k) & 1u ? w * ru[k] : 0.0;
+        hit |= mine;
+        if ((m >> lane) & 1u) d.mark[a] = epoch;
+        for (; m; m &= m - 1) {
+          const int aj = __shfl_sync(0xffffffffu, a, __ffs(m) - 1);
+          double* row = d.mu.xacc + (size_t)aj * Sp + lane;
+#pragma unroll
+          for (int k = 0; k < K; ++k)
+            if ((mine >> k) & 1u) atomicAdd(row + 32 * k, x[k]);
+        }
       }
     }
   }

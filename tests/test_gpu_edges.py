@@ -196,3 +196,45 @@ def test_batches_of_every_op_kind_across_the_ingest_sizes(n_ops):
         cp, row = g.csc()
         assert np.array_equal(ptr, cp) and np.array_equal(idx, row)
     eng.close()
+
+
+@pytest.mark.parametrize("prec,S", [(F64, 20), (F64, 40), (F32, 100), (BF16, 200)])
+def test_block_offsets_of_rows_that_grow_shrink_and_keep_their_length(prec, S):
+    """Changed rows of every length around the offset piece: entries added,
+    removed, exchanged one for one, and all taken out, in the oracle's lock-step,
+    L1 <= 1e-10 (double) and 1e-5 a seed (the bounds of the seed-block tests)."""
+    n = 2300
+    rng = np.random.default_rng(S)
+    src, dst = edge_graph(rng, n, 1)
+    seeds = rng.permutation(n)[:S].astype(np.int32)
+    eng = N.Engine(precision=prec, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(seeds, C_RESTART)
+    eng.init_scores(1e-11)
+    it0, _, _ = eng.get_seed_stats()
+    g = O.Graph(n, src, dst)
+    old = g.csr()
+    pick = list(range(0, S, max(1, S // 10)))
+    r = {j: O.cpi(*old, int(seeds[j]), C_RESTART, 1e-11, force_iters=int(it0[j]))[0] for j in pick}
+    for turn in range(4):
+        ptr, idx = (np.asarray(x) for x in old)
+        ops = []
+        for i in range(len(LENGTHS)):
+            u = 3 * i
+            has = idx[ptr[u]:ptr[u + 1]]
+            lacks = np.setdiff1d(np.arange(n), has)
+            k = {0: 3, 1: 1, 2: 40, 3: has.size}[(turn + i) % 4]
+            if (turn + i) % 4 != 3:
+                ops += [(u, int(v), 0) for v in rng.choice(lacks, min(k, lacks.size), replace=False)]
+            if (turn + i) % 4 != 0:
+                ops += [(u, int(v), 1) for v in rng.choice(has, min(k, has.size), replace=False)]
+        ops = np.array(ops, W.UPDATE_DTYPE)
+        eng.apply_updates(ops, 1e-9)
+        assert g.apply(ops) == -1
+        new = g.csr()
+        it, _, _ = eng.get_seed_stats()
+        for j in pick:
+            r[j], _, _, _ = O.osp(old, new, r[j], C_RESTART, 1e-9, force_iters=int(it[j]))
+            assert np.abs(eng.query(j) - r[j]).sum() <= (1e-10 if prec == F64 else 1e-5)
+        old = new
+    eng.close()
