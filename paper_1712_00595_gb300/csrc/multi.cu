@@ -648,7 +648,13 @@ __device__ __forceinline__ void add_stage(const unsigned* w, const unsigned char
   const unsigned prev = __shfl_up_sync(0xffffffffu, node, 1);
   // bit r: row r begins another node than the row before it
   const unsigned heads = __ballot_sync(0xffffffffu, lane < RS && node != (lane ? prev : cur));
+  // the lane's slots of every row first: between the rows' additions a node may
+  // end, and each load would come after what that stores and be waited for (the
+  // wait for shared memory was the largest stall)
   const TY* row = reinterpret_cast<const TY*>(stage) + lane * KG;
+  alignas(16) TY x[RS][KG];
+#pragma unroll
+  for (int r = 0; r < RS; ++r) load_k<TY, KG>(row + r * RW::G, x[r]);
   constexpr int kChains = std::is_same<TY, float>::value ? 2 : 1;
   TY part[kChains][KG];
 #pragma unroll
@@ -674,10 +680,8 @@ __device__ __forceinline__ void add_stage(const unsigned* w, const unsigned char
       for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
       cur = __shfl_sync(0xffffffffu, node, r);
     }
-    alignas(16) TY x[KG];
-    load_k<TY, KG>(row + r * RW::G, x);
-    if constexpr (kChains == 2) add_row<KG>(part[r & 1], x);
-    else add_row<KG>(acc, x);
+    if constexpr (kChains == 2) add_row<KG>(part[r & 1], x[r]);
+    else add_row<KG>(acc, x[r]);
   }
   gather();
 }
