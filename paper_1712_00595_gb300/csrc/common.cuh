@@ -62,6 +62,7 @@ struct Ctl {
   int n_clr;                   // rows zeroed by the last ingested batch (clr_nodes)
   int n_hubs, n_pieces;        // pull step: long in-lists and their pieces
   int n_tasks;                 // pull step: warp tasks
+  int plan_done;               // CTAs that have planned their nodes
   int n_mpieces;               // merge pieces of the current batch
   int dense0;                  // 1: x(0) is found by a dense scan of xacc (no queue from the merge)
   int n_opieces;               // several seeds: offset items (256 entries of a changed row)
@@ -164,7 +165,6 @@ struct Dev {
   // pull-step plan: prefix of in-list lengths, warp tasks of about
   // kTaskItems items (edges + nodes, lists never split), and the long in-lists
   // summed in pieces
-  unsigned* pc;                       // [nc + 1]  pc[v] = sum of in-list lengths below v
   int* task_first;                    // [(kMultiNodeItems nc + pool cap) / kMinTaskItems + 2] first node of each warp task
   int* hubs; int* hub_pstart; double* hub_acc; int* hub_cnt;  // [pool cap / kHubThreshold + 2]
   int* piece_hub;  // [2 pool cap / kMultiHub + 4] the long in-list each piece belongs to

@@ -475,21 +475,10 @@ const int* schedule(osp_ctx* ctx) {
   return single;
 }
 
-// Pull-step plan for the graph as it is after the merge: in-list length prefix
-// over the first n_bound + 1 ids (ids at or above n have empty lists) and the
-// merge-path tile starts.
-osp_status plan_pull(osp_ctx* ctx, int64_t n_bound, int64_t m_bound) {
-  (void)m_bound;
-  const int ns = (int)std::min<int64_t>(n_bound + 1, ctx->nc);
-  const int nb = (ns + 4095) / 4096;
+// Pull-step plan for the graph as it is after the merge.
+osp_status plan_pull(osp_ctx* ctx) {
   cudaStream_t st = ctx->stream;
-  k_merge_finish<<<1, 1, 0, st>>>(ctx->d);
-  ++ctx->launches;
-  k_scan_local<<<nb, 1024, 0, st>>>(ctx->d.len_c, ctx->d.pc, ctx->scan_bsum, ns);
-  ++ctx->launches;
-  k_scan_top<<<1, 1024, 0, st>>>(ctx->scan_bsum, nb);
-  ++ctx->launches;
-  k_scan_add<<<(ns + 255) / 256, 256, 0, st>>>(ctx->d.pc, ctx->scan_bsum, ns);
+  k_plan_sums<<<ctx->num_sms, 1024, 0, st>>>(ctx->d, ctx->scan_bsum);
   ++ctx->launches;
   const int* sc = schedule(ctx);
   // A graph whose tasks of sc[0] items would leave warps idle is cut finer:
@@ -501,10 +490,9 @@ osp_status plan_pull(osp_ctx* ctx, int64_t n_bound, int64_t m_bound) {
   // a batch with four of 64, 394 with two of 256).
   const bool many = ctx->S > 1, bf16 = many && ctx->opt.precision == OSP_PREC_BF16_ACC64;
   const int warps = many ? ctx->grid_multi * kPropWarps : ctx->grid_prop * kOneWarps;
-  k_pull_plan<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d, sc[1], sc[3], sc[0], bf16 ? 256 : many ? 64 : 32,
-                                                std::min(kMaxSmallTasks, warps * (many && !bf16 ? 4 : 2)));
-  ++ctx->launches;
-  k_hub_prefix<<<1, 1024, 0, st>>>(ctx->d, sc[2], ctx->opt.deterministic != 0);
+  k_pull_plan<<<ctx->num_sms, 1024, 0, st>>>(
+      ctx->d, ctx->scan_bsum, sc[1], sc[2], sc[3], sc[0], bf16 ? 256 : many ? 64 : 32,
+      std::min(kMaxSmallTasks, warps * (many && !bf16 ? 4 : 2)), ctx->opt.deterministic != 0);
   ++ctx->launches;
   CK(cudaGetLastError());
   return OSP_OK;
@@ -582,10 +570,9 @@ osp_status enqueue_propagate(osp_ctx* ctx, const PropParams& pp, bool init) {
   return OSP_OK;
 }
 
-osp_status run_propagation(osp_ctx* ctx, double eps, int64_t n_bound, int64_t m_bound,
-                           bool init = false) {
+osp_status run_propagation(osp_ctx* ctx, double eps, bool init = false) {
   const PropParams pp = prop_params(ctx, eps);
-  osp_status s = plan_pull(ctx, n_bound, m_bound);
+  osp_status s = plan_pull(ctx);
   if (s != OSP_OK) return s;
   // queries in flight read the scores this kernel changes
   if (!ctx->qslots.empty()) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_queries, 0));
@@ -660,7 +647,7 @@ osp_status capture_graphs(osp_ctx* ctx, int Np, double eps, osp_ctx::GraphPair* 
     osp_status s = OSP_OK;
     if (part == 0) {
       s = enqueue_update(ctx, ctx->ops_stage, -1, Np);
-      if (s == OSP_OK) s = plan_pull(ctx, ctx->nc - 1, 0);  // every node slot: fixed grids
+      if (s == OSP_OK) s = plan_pull(ctx);
     } else {
       s = enqueue_propagate(ctx, pp, false);
     }
@@ -802,7 +789,7 @@ osp_status apply_large(osp_ctx* ctx, const osp_update* ops, bool host, int64_t U
     ctx->top_r = h.pool_top_r;
     ctx->top_c = h.pool_top_c;
   }
-  osp_status s = run_propagation(ctx, eps, ctx->nc - 1, ctx->m);
+  osp_status s = run_propagation(ctx, eps);
   if (s != OSP_OK) return s;
   s = finish_call(ctx, m_before, st);
   if (bad >= 0) {
@@ -855,7 +842,7 @@ osp_status apply_common(osp_ctx* ctx, const osp_update* ops_dev, int64_t U, doub
   CK(cudaEventRecord(ctx->ev[0], ctx->stream));
   s = enqueue_update(ctx, ops_dev, (int)U, Np);
   if (s != OSP_OK) return s;
-  s = run_propagation(ctx, eps, std::min<int64_t>(ctx->n + U, ctx->nc - 1), ctx->m + U);
+  s = run_propagation(ctx, eps);
   if (s != OSP_OK) return s;
   return finish_call(ctx, m_before, st);
 }
@@ -1199,7 +1186,6 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     AL(d.piece_cnt, npc, 0);
     AL(d.piece_base, npc, 0);
   }
-  AL(d.pc, nc + 1, 0);
   AL(d.task_first, (int64_t)(kMultiNodeItems * nc + (int64_t)cap) / kMinTaskItems + kMaxSmallTasks + 2, 0);
   {
     // lists longer than a threshold t number at most (live edges) / t <= cap / t;
@@ -1229,7 +1215,7 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
   AL(ctx->dsum, kAbsParts + 2, 0);  // the norm, its per-CTA partials, the CTA count
   AL(ctx->dtmp, nc, 0);
   AL(ctx->scan_off, nc, 0);
-  AL(ctx->scan_bsum, nc / 4096 + 2, 0);
+  AL(ctx->scan_bsum, std::max<int64_t>(nc / 4096 + 2, ctx->num_sms), 0);
   AL(ctx->tk_state, 1, 0);
   AL(ctx->tk_hist, 4096, 0);
   AL(ctx->tk_blk_a, nc / kTopkChunk + 2, 0);
@@ -1459,7 +1445,7 @@ osp_status autotune(osp_ctx* ctx, double eps) {
     const auto& cd = cands[trial < 0 ? 0 : trial];
     for (int i = 0; i < 4; ++i) ctx->sched[i] = cd[i];
     osp_status s = enqueue_cpi_start(ctx);
-    if (s == OSP_OK) s = plan_pull(ctx, ctx->n, ctx->m);
+    if (s == OSP_OK) s = plan_pull(ctx);
     if (s != OSP_OK) return s;
     CK(cudaEventRecord(ctx->ev[1], ctx->stream));
     // time the kernel the batches will run (bf16 gather rows included; the
@@ -1502,7 +1488,7 @@ osp_status osp_init_scores(osp_ctx* ctx, double eps, osp_batch_stats* stats) {
   ctx->res_bound = 0.0;
   s = enqueue_cpi_start(ctx);
   if (s != OSP_OK) return s;
-  s = run_propagation(ctx, eps, ctx->n, ctx->m, true);
+  s = run_propagation(ctx, eps, true);
   if (s != OSP_OK) return s;
   s = finish_call(ctx, ctx->m, stats);
   if (s == OSP_OK || s == OSP_ENOCONV) ctx->scored = true;

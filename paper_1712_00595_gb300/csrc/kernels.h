@@ -18,10 +18,9 @@ __global__ void k_merge_pieces(Dev d, double beta);
 __global__ void k_merge_count(Dev d);
 __global__ void k_merge_plan(Dev d);
 __global__ void k_merge_write(Dev d);
-__global__ void k_merge_finish(Dev d);
-__global__ void k_pull_plan(Dev d, int hub_thr, int node_w, int task_items, int task_min,
-                            int want);
-__global__ void k_hub_prefix(Dev d, int hub_piece, int det);
+__global__ void k_plan_sums(Dev d, unsigned* part);
+__global__ void k_pull_plan(Dev d, const unsigned* __restrict__ part, int hub_thr, int hub_piece,
+                            int node_w, int task_items, int task_min, int want, int det);
 __global__ void k_set_scale(Dev d, int n, double c);
 __global__ void k_scan_local(const int* __restrict__ len, unsigned* out, unsigned* bsum, int n);
 __global__ void k_scan_top(unsigned* bsum, int nb);

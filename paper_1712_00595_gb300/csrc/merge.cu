@@ -23,22 +23,59 @@
 namespace osp {
 namespace {
 
-// queue == false: the batch may touch more than n/beta nodes, and x(0) will be
-// found by a dense scan of xacc, so no mark or queue entry is made here.
-__device__ __forceinline__ void offset_add(const Dev& d, bool want, int v, double val, int epoch,
-                                           bool queue) {
-  if (want && !OSP_GUARD(d.ctl, v >= 0 && v < d.nc, "offset target", v, 0, 0)) want = false;
+// Adds val to the offset of the targets a[r] of this lane whose bit of want[r] is
+// set. queue == false: the batch may touch more than n/beta nodes, and x(0) will
+// be found by a dense scan of xacc, so no mark or queue entry is made here.
+// All rounds of a piece at once: each mark exchange and each append to the queue
+// returns a value, and one after the other for eight rounds they were the time
+// of the kernels that form the offset (one edge at a hub of 100,003 nodes: 20 ->
+// 11 us to write the lists; 1,000 ops at 2^20 nodes: 21 -> 13 us to count them).
+template <int R>
+__device__ __forceinline__ void offset_add(const Dev& d, const unsigned (&want)[R], int (&a)[R],
+                                           double val, int epoch, bool queue) {
+  const int lane = threadIdx.x & 31;
+  unsigned mine = 0;  // bit r: a[r] is wanted
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    mine |= (OSP_GUARD(d.ctl, !((want[r] >> lane) & 1u) || (a[r] >= 0 && a[r] < d.nc), "offset target",
+                       a[r], 0, 0)
+                 ? (want[r] >> lane) & 1u
+                 : 0u)
+            << r;
   if (d.xfix) {
     // deterministic mode: exact integer sums in units of 2^-62 (|q_offset_v| <=
     // (1-c) ||r_old||_1 < 2, and two's-complement wrap-around leaves partial
     // sums harmless), collected by the x(0) scan, so no queue either
-    if (want) atomicAdd(d.xfix + v, (unsigned long long)__double2ll_rn(val * 0x1p62));
+    const unsigned long long q = (unsigned long long)__double2ll_rn(val * 0x1p62);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if ((mine >> r) & 1u) atomicAdd(d.xfix + a[r], q);
     return;
   }
-  if (want) atomicAdd(&d.xacc[v], val);
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if ((mine >> r) & 1u) atomicAdd(&d.xacc[a[r]], val);
   if (!queue) return;
-  bool need = want && (d.mark[v] != epoch) && (atomicExch(&d.mark[v], epoch) != epoch);
-  warp_append(need, v, d.q0, &d.ctl->q_size[0]);
+  int old[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) old[r] = (mine >> r) & 1u ? d.mark[a[r]] : epoch;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (old[r] != epoch) old[r] = atomicExch(&d.mark[a[r]], epoch);
+  int total = 0, at[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const unsigned b = __ballot_sync(0xffffffffu, old[r] != epoch);
+    at[r] = total + __popc(b & lanemask_lt());
+    total += __popc(b);
+  }
+  if (!total) return;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(&d.ctl->q_size[0], total);
+  base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (old[r] != epoch) d.q0[base + at[r]] = a[r];
 }
 
 // One changed list, seen through the combined record index c (out-lists first).
@@ -181,18 +218,25 @@ __global__ void __launch_bounds__(256) k_merge_count(Dev d) {
     const double ru = R.rows && !multi ? d.r[R.node] : 0.0;  // the seed block has its own offset kernel
     const bool contrib = R.rows && ru != 0.0;
     const double wa = L ? 1.0 / (double)L : 0.0;
-    int cnt = 0;
+    int cnt = 0, a[kPiece / 32];
+    unsigned gone[kPiece / 32];
+#pragma unroll
+    for (int r = 0; r < kPiece / 32; ++r) {
+      const int i = q * kPiece + r * 32 + lane;
+      a[r] = i < L ? R.pool[o + i] : 0;
+    }
 #pragma unroll
     for (int r = 0; r < kPiece / 32; ++r) {
       const int i = q * kPiece + r * 32 + lane;
       const bool in = i < L;
-      int a = in ? R.pool[o + i] : 0;
-      if (in && !OSP_GUARD(d.ctl, a >= 0 && a < d.nc, "merge count entry", c, i, a)) a = 0;
-      const bool keep = in && !cleared && !(any_dead && d.dead[a]) &&
-                        !(drop_clr && d.clr_pos[a] >= 0) && !contains_i(R.del + R.ds, R.dc, a);
+      if (in && !OSP_GUARD(d.ctl, a[r] >= 0 && a[r] < d.nc, "merge count entry", c, i, a[r])) a[r] = 0;
+      const bool keep = in && !cleared && !(any_dead && d.dead[a[r]]) &&
+                        !(drop_clr && d.clr_pos[a[r]] >= 0) && !contains_i(R.del + R.ds, R.dc, a[r]);
       cnt += __popc(__ballot_sync(0xffffffffu, keep));
-      if (contrib) offset_add(d, in && !keep, a, c1 * ru * (0.0 - wa), epoch, queue);
+      gone[r] = __ballot_sync(0xffffffffu, in && !keep);
     }
+    if (contrib && cnt != min(kPiece, L - q * kPiece))
+      offset_add(d, gone, a, c1 * ru * (0.0 - wa), epoch, queue);
     if (lane == 0) d.piece_cnt[p] = cnt;
   }
 }
@@ -290,24 +334,28 @@ __global__ void __launch_bounds__(256) k_merge_write(Dev d) {
     const double wb = dp ? 1.0 / (double)dp : 0.0;
     const bool shift = contrib && dp != L;
     unsigned masks[kPiece / 32];
-    int run = 0;
+    int run = 0, a[kPiece / 32];
+#pragma unroll
+    for (int r = 0; r < kPiece / 32; ++r) {
+      const int i = q * kPiece + r * 32 + lane;
+      a[r] = i < L ? R.pool[o + i] : 0;
+    }
 #pragma unroll
     for (int r = 0; r < kPiece / 32; ++r) {
       const int i = q * kPiece + r * 32 + lane;
       const bool in = i < L;
-      int a = in ? R.pool[o + i] : 0;
-      if (in && !OSP_GUARD(d.ctl, a >= 0 && a < d.nc, "merge write entry", c, i, a)) a = 0;
-      const bool keep = in && !cleared && !(any_dead && d.dead[a]) &&
-                        !(drop_clr && d.clr_pos[a] >= 0) && !contains_i(R.del + R.ds, R.dc, a);
+      if (in && !OSP_GUARD(d.ctl, a[r] >= 0 && a[r] < d.nc, "merge write entry", c, i, a[r])) a[r] = 0;
+      const bool keep = in && !cleared && !(any_dead && d.dead[a[r]]) &&
+                        !(drop_clr && d.clr_pos[a[r]] >= 0) && !contains_i(R.del + R.ds, R.dc, a[r]);
       const unsigned m = __ballot_sync(0xffffffffu, keep);
       masks[r] = m;
       if (keep) {
-        const int pos = base + run + __popc(m & lanemask_lt()) + lower_bound_i(I, ic, a);
-        if (OSP_GUARD(d.ctl, pos >= 0 && pos < dp, "merge write position", c, pos, dp)) F[pos] = a;
+        const int pos = base + run + __popc(m & lanemask_lt()) + lower_bound_i(I, ic, a[r]);
+        if (OSP_GUARD(d.ctl, pos >= 0 && pos < dp, "merge write position", c, pos, dp)) F[pos] = a[r];
       }
       run += __popc(m);
-      if (shift) offset_add(d, keep, a, c1 * ru * (wb - wa), epoch, queue);
     }
+    if (shift && run) offset_add(d, masks, a, c1 * ru * (wb - wa), epoch, queue);
     // insertions that fall inside this piece of the old list
     if (ic > 0) {
       const int* A = R.pool + o;
@@ -333,99 +381,179 @@ __global__ void __launch_bounds__(256) k_merge_write(Dev d) {
           if (OSP_GUARD(d.ctl, j + base + kept < dp, "merge insert position", c, j + base + kept, dp))
             F[j + base + kept] = e;
         }
-        if (contrib) offset_add(d, in, e, c1 * ru * (wb - 0.0), epoch, queue);
+        if (contrib) {
+          const unsigned want[1] = {__ballot_sync(0xffffffffu, in)};
+          int to[1] = {e};
+          offset_add(d, want, to, c1 * ru * (wb - 0.0), epoch, queue);
+        }
       }
     }
   }
 }
 
-// Fold the batch's edge-count change into m.
-__global__ void k_merge_finish(Dev d) {
-  Ctl* ctl = d.ctl;
-  if (*(volatile int*)&ctl->status) return;
-  ctl->m += ctl->m_delta;
-  ctl->m_delta = 0;
-  ctl->n_hubs = 0;
-  // a dense first frontier is rebuilt by the x(0) scan: drop entries queued by
-  // earlier sub-batches of the same batch
-  if (ctl->dense0) ctl->q_size[0] = 0;
+// ---------------------------------------------------------------------------
+// Pull-step plan. Warp task t starts at the first node v with
+// f(v) = (in-list entries below v) + node_w v >= t task_items (so a task holds
+// about task_items items, an edge counting 1 and a node node_w, and never
+// splits a list); in-lists longer than hub_thr are listed and cut into pieces.
+// Two launches over kPlanCtas consecutive ranges of nodes: sums of the ranges,
+// then every CTA scans its own range from the sum of those before it. A prefix
+// over all nodes in memory, the task starts from it and the pieces were six
+// launches, with two 64-bit divisions a node; an update phase of 1,000 edge ops
+// at 2^20 nodes took 142 us with them and 126 so, of 100 at 10,000 nodes 85 and
+// 73 (with the offset above).
+// ---------------------------------------------------------------------------
+namespace {
+constexpr int kPlanThreads = 1024;
+
+// Nodes [lo, hi) of CTA b of nb: a multiple of four each, but for the last.
+__device__ __forceinline__ void plan_range(int n, int& lo, int& hi) {
+  const long long per = (((long long)n + gridDim.x - 1) / gridDim.x + 3) & ~3ll;
+  lo = (int)min((long long)n, per * blockIdx.x);
+  hi = (int)min((long long)n, per * (blockIdx.x + 1));
 }
 
-// Pull-step plan, part 1: warp task t starts at the first node v with
-// pc[v] + node_w v >= t * task_items (so a task holds about task_items items,
-// an edge counting 1 and a node node_w, and never splits a list); in-lists
-// longer than hub_thr are listed for piecewise summation.
-// Small graphs get shorter tasks, down to task_min items, so that `want` warps
-// have one each.
-__global__ void k_pull_plan(Dev d, int hub_thr, int node_w, int task_items, int task_min, int want) {
+// a[v .. v + 4), zero from hi on (v a multiple of four)
+__device__ __forceinline__ int4 load4(const int* a, int v, int hi) {
+  if (v + 4 <= hi) return *reinterpret_cast<const int4*>(a + v);
+  return make_int4(v < hi ? a[v] : 0, v + 1 < hi ? a[v + 1] : 0, v + 2 < hi ? a[v + 2] : 0, 0);
+}
+}  // namespace
+
+// In-list entries of each CTA's nodes; nodes with a nonempty list of either kind
+// (byte accounting). Folds the batch's edge-count change into m.
+__global__ void __launch_bounds__(kPlanThreads) k_plan_sums(Dev d, unsigned* part) {
   Ctl* ctl = d.ctl;
   if (*(volatile int*)&ctl->status) return;
-  const int n = ctl->n;
-  const long long W = (long long)node_w * n + ctl->m;
-  task_items = (int)min((long long)task_items, max((long long)task_min, (W + want - 1) / want));
-  const int nt = (int)((W + task_items - 1) / task_items);
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nth = gridDim.x * blockDim.x;
-  if (tid == 0) {
-    ctl->n_tasks = nt;
-    ctl->hub_thr = hub_thr;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ctl->m += ctl->m_delta;
+    ctl->m_delta = 0;
+    ctl->n_hubs = 0;
+    ctl->plan_done = 0;
+    // a dense first frontier is rebuilt by the x(0) scan: drop entries queued by
+    // earlier sub-batches of the same batch
+    if (ctl->dense0) ctl->q_size[0] = 0;
   }
-  // f(v) = pc[v] + node_w v is nondecreasing with f(0) = 0, so the tasks t with
-  // f(v-1) < t * task_items <= f(v) are exactly those starting at node v: one
-  // coalesced pass over the nodes writes every task start.
-  if (tid == 0) {
-    d.task_first[0] = 0;
-    d.task_first[nt] = n;
+  int lo, hi;
+  plan_range(ctl->n, lo, hi);
+  unsigned sum = 0, nd = 0, ns = 0;
+  for (int v = lo + 4 * (int)threadIdx.x; v < hi; v += 4 * kPlanThreads) {
+    const int4 a = load4(d.len_c, v, hi), b = load4(d.len_r, v, hi);
+    sum += (unsigned)a.x + (unsigned)a.y + (unsigned)a.z + (unsigned)a.w;
+    nd += (a.x > 0) + (a.y > 0) + (a.z > 0) + (a.w > 0);
+    ns += (b.x > 0) + (b.y > 0) + (b.z > 0) + (b.w > 0);
   }
-  for (int v = tid + 1; v <= n; v += nth) {
-    const long long f0 = (long long)d.pc[v - 1] + (long long)node_w * (v - 1);
-    const long long f1 = (long long)d.pc[v] + (long long)node_w * v;
-    const long long t0 = f0 / task_items + 1;
-    const long long t1 = min(f1 / task_items, (long long)nt - 1);
-    for (long long t = t0; t <= t1; ++t) d.task_first[t] = v;
-  }
-  const int lane = threadIdx.x & 31;
-  __shared__ unsigned long long s_cnt[2];
-  if (threadIdx.x == 0) s_cnt[0] = s_cnt[1] = 0;
+  __shared__ unsigned s_sum[3];
+  if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
   __syncthreads();
-  unsigned nd = 0, ns = 0;  // destinations and sources of the pull steps (byte accounting)
-  for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += nth) {
-    const int v = base + lane;
-    const int lc = v < n ? d.len_c[v] : 0;
-    const bool h = lc > hub_thr;
-    warp_append(h, v, d.hubs, &ctl->n_hubs);
-    nd += __popc(__ballot_sync(0xffffffffu, lc > 0));
-    ns += __popc(__ballot_sync(0xffffffffu, v < n && d.len_r[v] > 0));
-  }
-  if (lane == 0) {
-    atomicAdd(&s_cnt[0], (unsigned long long)nd);
-    atomicAdd(&s_cnt[1], (unsigned long long)ns);
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  nd = __reduce_add_sync(0xffffffffu, nd);
+  ns = __reduce_add_sync(0xffffffffu, ns);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_sum[0], sum);
+    atomicAdd(&s_sum[1], nd);
+    atomicAdd(&s_sum[2], ns);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (s_cnt[0]) atomicAdd((unsigned long long*)&ctl->n_dst_nz, s_cnt[0]);
-    if (s_cnt[1]) atomicAdd((unsigned long long*)&ctl->n_src_nz, s_cnt[1]);
-  }
+  if (threadIdx.x != 0) return;
+  part[blockIdx.x] = s_sum[0];
+  if (s_sum[1]) atomicAdd((unsigned long long*)&ctl->n_dst_nz, (unsigned long long)s_sum[1]);
+  if (s_sum[2]) atomicAdd((unsigned long long*)&ctl->n_src_nz, (unsigned long long)s_sum[2]);
 }
 
-// Pull-step plan, part 2 (one CTA): piece prefix over the long in-lists.
-// det != 0: the list of long in-lists, appended in whatever order the warps of
-// k_pull_plan ran, is first rebuilt in ascending node order (one ordered
-// compaction over all nodes), so that the pieces and the per-list norm slots
-// have the same positions on every run.
-__global__ void __launch_bounds__(1024) k_hub_prefix(Dev d, int hub_piece, int det) {
+// Task starts and long lists of each CTA's nodes; the CTA that finishes last cuts
+// the long lists into pieces. Small graphs get shorter tasks, down to task_min
+// items, so that `want` warps have one each.
+// det: the long lists, listed in whatever order the CTAs ran, are rebuilt in
+// ascending node order (one ordered compaction over all nodes), so that the
+// pieces and the per-list norm slots have the same positions on every run.
+__global__ void __launch_bounds__(kPlanThreads)
+    k_pull_plan(Dev d, const unsigned* __restrict__ part, int hub_thr, int hub_piece, int node_w,
+                int task_items, int task_min, int want, int det) {
   __shared__ int s_w[32];
   __shared__ int s_base;
+  __shared__ long long s_f;
   Ctl* ctl = d.ctl;
   if (*(volatile int*)&ctl->status) return;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  {
+    const int n = ctl->n;
+    const long long W = (long long)node_w * n + ctl->m;
+    task_items = (int)min((long long)task_items, max((long long)task_min, (W + want - 1) / want));
+    const int nt = (int)((W + task_items - 1) / task_items);
+    if (blockIdx.x == 0 && tid == 0) {
+      ctl->n_tasks = nt;
+      ctl->hub_thr = hub_thr;
+      ctl->hub_piece = hub_piece;
+      d.task_first[0] = 0;
+      d.task_first[nt] = n;
+    }
+    int lo, hi;
+    plan_range(n, lo, hi);
+    unsigned before = 0;
+    for (int b = tid; b < (int)blockIdx.x; b += kPlanThreads) before += part[b];
+    int4 a = load4(d.len_c, lo + 4 * tid, hi);
+    if (tid == 0) s_f = (long long)node_w * lo;
+    __syncthreads();
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (before && lane == 0) atomicAdd((unsigned long long*)&s_f, (unsigned long long)before);
+    for (int v0 = lo; v0 < hi; v0 += 4 * kPlanThreads) {
+      const int v = v0 + 4 * tid;
+      if (v0 > lo) a = load4(d.len_c, v, hi);
+      const int len[4] = {a.x, a.y, a.z, a.w};
+      const unsigned mine = (unsigned)a.x + (unsigned)a.y + (unsigned)a.z + (unsigned)a.w;
+      unsigned x = mine;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) s_w[w] = (int)x;
+      __syncthreads();
+      if (w == 0) {
+        unsigned t = (unsigned)s_w[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned y = __shfl_up_sync(0xffffffffu, t, o);
+          if (lane >= o) t += y;
+        }
+        s_w[lane] = (int)t;
+      }
+      __syncthreads();
+      // f at this thread's first node; the nodes of the tile before it count node_w each
+      long long f = s_f + (w ? (unsigned)s_w[w - 1] : 0u) + (x - mine) + (long long)node_w * (4 * tid);
+      const unsigned total = (unsigned)s_w[31];
+      if (v < hi) {
+        // boundaries t task_items in (f(u), f(u + 1)] start at node u + 1
+        long long t = W <= 0xffffffffll ? (long long)((unsigned)f / (unsigned)task_items) : f / task_items;
+        long long at = (t + 1) * task_items;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (v + q >= hi) break;
+          f += len[q] + node_w;
+          for (; at <= f && t + 1 < nt; at += task_items) d.task_first[++t] = v + q + 1;
+          if (len[q] > hub_thr) d.hubs[atomicAdd(&ctl->n_hubs, 1)] = v + q;
+        }
+      }
+      if (v0 + 4 * kPlanThreads >= hi) break;
+      __syncthreads();
+      if (tid == 0) s_f += total + (long long)node_w * (4 * kPlanThreads);
+      __syncthreads();
+    }
+  }
+  // the last CTA has every long list
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_base = atomicAdd(&ctl->plan_done, 1);
+  __syncthreads();
+  if (s_base != (int)gridDim.x - 1) return;
+  __threadfence();
+  __syncthreads();
   if (det) {
-    const int n = ctl->n, thr = ctl->hub_thr;
+    const int n = ctl->n;
     if (tid == 0) s_base = 0;
     __syncthreads();
     for (int b0 = 0; b0 < n; b0 += 1024) {
       const int v = b0 + tid;
-      const bool h = v < n && d.len_c[v] > thr;
+      const bool h = v < n && d.len_c[v] > hub_thr;
       const unsigned bm = __ballot_sync(0xffffffffu, h);
       if (lane == 0) s_w[w] = __popc(bm);
       __syncthreads();
@@ -444,7 +572,7 @@ __global__ void __launch_bounds__(1024) k_hub_prefix(Dev d, int hub_piece, int d
       __syncthreads();
     }
   }
-  const int nh = ctl->n_hubs;
+  const int nh = *(volatile int*)&ctl->n_hubs;
   const int per = (nh + 1023) / 1024;
   const int lo = min(nh, tid * per), hi = min(nh, lo + per);
   int mine = 0;
@@ -477,7 +605,6 @@ __global__ void __launch_bounds__(1024) k_hub_prefix(Dev d, int hub_piece, int d
   if (tid == 0) {
     d.hub_pstart[nh] = s_w[31];
     ctl->n_pieces = s_w[31];
-    ctl->hub_piece = hub_piece;
   }
 }
 

@@ -238,3 +238,31 @@ def test_block_offsets_of_rows_that_grow_shrink_and_keep_their_length(prec, S):
             assert np.abs(eng.query(j) - r[j]).sum() <= (1e-10 if prec == F64 else 1e-5)
         old = new
     eng.close()
+
+
+@pytest.mark.parametrize("det", [0, 1])
+@pytest.mark.parametrize("n", [2, 607, 609, 4097, 622_591, 700_001])
+def test_pull_plan_over_node_counts_around_its_ranges(n, det):
+    """Every node in one task whatever the split of the nodes over the planning
+    CTAs: few and many nodes a CTA, counts off the multiples of four, long lists
+    first and last, against the oracle (L1 <= 1e-10)."""
+    rng = np.random.default_rng(n)
+    k = min(n, 3000)
+    src = [rng.integers(0, n, 2 * n), rng.choice(n, k, replace=False), rng.choice(n, k, replace=False)]
+    dst = [rng.integers(0, n, 2 * n), np.zeros(k, np.int64), np.full(k, n - 1)]
+    e = np.unique(np.stack([np.concatenate(src), np.concatenate(dst)], 1), axis=0).astype(np.int32)
+    src, dst = np.ascontiguousarray(e[:, 0]), np.ascontiguousarray(e[:, 1])
+    eng = N.Engine(precision=N.OSP_PREC_FP64, device=0, deterministic=det)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds([n // 2], C_RESTART)
+    st = eng.init_scores(1e-9)
+    g = O.Graph(n, src, dst)
+    old = g.csr()
+    r, _, _ = O.cpi(*old, n // 2, C_RESTART, 1e-9, force_iters=st["iterations"])
+    assert np.abs(eng.query() - r).sum() <= 1e-10
+    ops = np.array([(n - 1, 0, 1), (n // 2, n - 1, 0), (0, n // 3, 0)], W.UPDATE_DTYPE)
+    st = eng.apply_updates(ops, 1e-9)
+    assert g.apply(ops) == -1
+    r, _, _, _ = O.osp(old, g.csr(), r, C_RESTART, 1e-9, force_iters=st["iterations"])
+    assert np.abs(eng.query() - r).sum() <= 1e-10
+    eng.close()
