@@ -66,23 +66,21 @@ static __device__ __forceinline__ bool bar_release(Ctl* ctl, BarShared& sh) {
 // the result). What any thread of an arrived CTA wrote is visible afterwards.
 // Bounded like bar_release; false after a timeout.
 static __device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, Ctl* ctl) {
-  bool ok = true;
-  __threadfence();
-  atomicAdd(bar, 1u);
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
   unsigned long long t0 = 0;
   unsigned spins = 0;
-  while ((int)(*(volatile unsigned*)bar - target) < 0) {
+  for (;;) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+    if ((int)(v - target) >= 0) return true;
     if ((++spins & 1023u) == 0) {
       if (t0 == 0) t0 = global_ns();
       if (spins >= kBarrierMaxSpins || global_ns() - t0 > kBarrierTimeoutNs) {
         atomicCAS(&ctl->status, 0, (int)OSP_ETIMEOUT);
-        ok = false;
-        break;
+        return false;
       }
     }
   }
-  __threadfence();
-  return ok;
 }
 
 }  // namespace osp
