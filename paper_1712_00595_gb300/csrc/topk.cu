@@ -12,6 +12,9 @@
 // Every kernel serves a table of independent jobs (one score vector and its
 // scratch each): blockIdx.y is the job, so the top-k of many seeds costs one
 // launch sequence.
+#include <algorithm>
+#include <climits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -24,6 +27,44 @@ constexpr int kBins = 1 << kDigitBits;
 __device__ __forceinline__ unsigned long long order_key(double x) {
   unsigned long long b = (unsigned long long)__double_as_longlong(x);
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+
+// The order of keys as signed numbers: three 32-bit instructions a score.
+__device__ __forceinline__ long long signed_key(long long bits) {
+  return bits ^ ((bits >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ unsigned long long key_of(long long s) {
+  return (unsigned long long)s ^ 0x8000000000000000ull;
+}
+
+// Signed keys of eight of the n scores: pairs p, p + stride, .. p + 3 stride (score
+// 2 p is x[0]). Returns bit q for x[q] being one of the n. Whole pairs of an aligned
+// vector load 16 bytes each, past the L2's set of lines to keep, and without a test
+// of each index: a pass over 32 vectors of 2^21 scores 157 us with guarded 8-byte
+// loads, 88 so.
+__device__ __forceinline__ unsigned load_keys(const double* __restrict__ r, long long p, int stride,
+                                              int n, long long (&x)[8]) {
+  const bool whole = 2 * (p + 3ll * stride) + 1 < n && ((uintptr_t)r & 15) == 0;
+  if (__all_sync(0xffffffffu, whole)) {
+    longlong2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = __ldcs(reinterpret_cast<const longlong2*>(r) + p + q * stride);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      x[2 * q] = signed_key(v[q].x);
+      x[2 * q + 1] = signed_key(v[q].y);
+    }
+    return 0xFFu;
+  }
+  unsigned have = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const long long i = 2 * (p + (long long)(q >> 1) * stride) + (q & 1);
+    const bool in = i < n;
+    have |= (unsigned)in << q;
+    x[q] = in ? signed_key(__double_as_longlong(__ldg(r + i))) : 0ll;
+  }
+  return have;
 }
 
 __device__ __forceinline__ void bin_range(const TopkState* st, unsigned long long* lo,
@@ -77,33 +118,40 @@ __global__ void __launch_bounds__(256) k_topk_hist(TopkJobs J, int width, int ca
   const int bits = st->bits;
   const unsigned long long prefix = st->prefix;
   const int shift = 64 - bits - width;
-  unsigned long long kmin = ~0ull, kmax = 0ull;
   const int stride = gridDim.x * blockDim.x;
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n; b += 4 * stride) {
-    double x[4];
+  const long long pairs = ((long long)n + 1) >> 1;
+  const unsigned mask = (1u << width) - 1u;
+  unsigned long long lo, hi;
+  bin_range(st, &lo, &hi);
+  const long long slo = (long long)key_of((long long)lo), shi = (long long)key_of((long long)hi);
+  // smallest and largest key from the second digit on (in the first they would tell
+  // a vector of equal scores only)
+  long long kmin = LLONG_MAX, kmax = LLONG_MIN;
+  for (long long b = blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < pairs; b += 4ll * stride) {
+    long long x[8];
+    const unsigned have = load_keys(r, b + (threadIdx.x & 31), stride, n, x);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) x[q] = (long long)b + (long long)q * stride < n ? __ldg(r + b + q * stride) : 0.0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if ((long long)b + (long long)q * stride >= n) break;
-      const unsigned long long key = order_key(x[q]);
-      if (bits == 0 || (key >> (64 - bits)) == prefix) {
-        atomicAdd(&sh[(key >> shift) & ((1ull << width) - 1)], 1u);
-        kmin = key < kmin ? key : kmin;
-        kmax = key > kmax ? key : kmax;
+    for (int q = 0; q < 8; ++q) {
+      if (!((have >> q) & 1u) || (bits != 0 && (x[q] < slo || x[q] > shi))) continue;
+      atomicAdd(&sh[(unsigned)(key_of(x[q]) >> shift) & mask], 1u);
+      if (bits != 0) {
+        kmin = x[q] < kmin ? x[q] : kmin;
+        kmax = x[q] > kmax ? x[q] : kmax;
       }
     }
   }
+  if (bits != 0) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long a = __shfl_xor_sync(0xffffffffu, kmin, o);
-    const unsigned long long b = __shfl_xor_sync(0xffffffffu, kmax, o);
-    kmin = a < kmin ? a : kmin;
-    kmax = b > kmax ? b : kmax;
-  }
-  if ((threadIdx.x & 31) == 0 && kmin <= kmax) {
-    atomicMin(&st->kmin, kmin);
-    atomicMax(&st->kmax, kmax);
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long a = __shfl_xor_sync(0xffffffffu, kmin, o);
+      const long long b = __shfl_xor_sync(0xffffffffu, kmax, o);
+      kmin = a < kmin ? a : kmin;
+      kmax = b > kmax ? b : kmax;
+    }
+    if ((threadIdx.x & 31) == 0 && kmin <= kmax) {
+      atomicMin(&st->kmin, key_of(kmin));
+      atomicMax(&st->kmax, key_of(kmax));
+    }
   }
   __syncthreads();
   const int nb = 1 << width;
@@ -186,29 +234,35 @@ __global__ void __launch_bounds__(256) k_topk_collect(TopkJobs J, int cap) {
   const int n = J.n;
   unsigned long long lo, hi;
   bin_range(st, &lo, &hi);
+  const int lane = threadIdx.x & 31;
   const int stride = gridDim.x * blockDim.x;
+  const long long pairs = ((long long)n + 1) >> 1;
+  const long long slo = (long long)key_of((long long)lo);
   // whole warps stay in the loop: the append below is warp-wide
-  for (int b = blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < n; b += 8 * stride) {
-    unsigned long long key[8];
+  for (long long b = blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < pairs; b += 4ll * stride) {
+    long long x[8];
+    const unsigned have = load_keys(r, b + lane, stride, n, x);
+    unsigned in = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) in |= (unsigned)(x[q] >= slo) << q;
+    in &= have;
+    if (!__any_sync(0xffffffffu, in)) continue;  // survivors are rare
     unsigned m[8];
     int tot = 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const long long i = (long long)b + (threadIdx.x & 31) + (long long)q * stride;
-      key[q] = i < n ? order_key(__ldg(r + i)) : 0ull;
-      m[q] = __ballot_sync(0xffffffffu, i < n && key[q] >= lo);
+      m[q] = __ballot_sync(0xffffffffu, (in >> q) & 1u);
       tot += __popc(m[q]);
     }
-    if (!tot) continue;
     int at = 0;
-    if ((threadIdx.x & 31) == 0) at = atomicAdd(&st->count, tot);
+    if (lane == 0) at = atomicAdd(&st->count, tot);
     at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int p = at + __popc(m[q] & lanemask_lt());
-      if ((m[q] >> (threadIdx.x & 31)) & 1u && p < cap) {
-        jb.keys[p] = key[q];
-        jb.ids[p] = b + (threadIdx.x & 31) + q * stride;
+      if ((in >> q) & 1u && p < cap) {
+        jb.keys[p] = key_of(x[q]);
+        jb.ids[p] = (int)(2 * (b + lane + (long long)(q >> 1) * stride) + (q & 1));
       }
       at += __popc(m[q]);
     }
@@ -216,8 +270,9 @@ __global__ void __launch_bounds__(256) k_topk_collect(TopkJobs J, int cap) {
 }
 
 // Per chunk of kTopkChunk ids: how many keys lie above the selected bin and
-// how many inside it.
-__global__ void __launch_bounds__(1024) k_topk_count(TopkJobs J) {
+// how many inside it. (A CTA takes many chunks: with one each, the CTAs of the
+// jobs without ties took 27 us to start and leave, 32 jobs of 2^21 scores.)
+__global__ void __launch_bounds__(1024) k_topk_count(TopkJobs J, int nb) {
   __shared__ int s_a, s_b;
   const TopkJob& jb = J.j[blockIdx.y];
   if (!jb.st->ties) return;
@@ -225,27 +280,30 @@ __global__ void __launch_bounds__(1024) k_topk_count(TopkJobs J) {
   const int n = J.n;
   unsigned long long lo, hi;
   bin_range(jb.st, &lo, &hi);
-  if (threadIdx.x == 0) s_a = s_b = 0;
-  __syncthreads();
-  int a = 0, b = 0;
-  const int base = blockIdx.x * kTopkChunk;
-  for (int j = threadIdx.x; j < kTopkChunk; j += blockDim.x) {
-    const int i = base + j;
-    if (i >= n) break;
-    const unsigned long long key = order_key(r[i]);
-    a += key > hi;
-    b += key >= lo && key <= hi;
-  }
-  a = warp_sum(a);
-  b = warp_sum(b);
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&s_a, a);
-    atomicAdd(&s_b, b);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    jb.blk_a[blockIdx.x] = s_a;
-    jb.blk_b[blockIdx.x] = s_b;
+  for (int c = blockIdx.x; c < nb; c += gridDim.x) {
+    if (threadIdx.x == 0) s_a = s_b = 0;
+    __syncthreads();
+    int a = 0, b = 0;
+    const int base = c * kTopkChunk;
+    for (int j = threadIdx.x; j < kTopkChunk; j += blockDim.x) {
+      const int i = base + j;
+      if (i >= n) break;
+      const unsigned long long key = order_key(r[i]);
+      a += key > hi;
+      b += key >= lo && key <= hi;
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(&s_a, a);
+      atomicAdd(&s_b, b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      jb.blk_a[c] = s_a;
+      jb.blk_b[c] = s_b;
+    }
+    __syncthreads();
   }
 }
 
@@ -316,7 +374,7 @@ __global__ void __launch_bounds__(1024) k_topk_scan(TopkJobs J, int nb, int cand
 
 // Ordered compaction: chunk by chunk in id order, keys above the bin go first,
 // then the first `keep` keys of the bin.
-__global__ void __launch_bounds__(1024) k_topk_emit(TopkJobs J) {
+__global__ void __launch_bounds__(1024) k_topk_emit(TopkJobs J, int nb) {
   __shared__ int s_w[2][32];
   __shared__ int s_run[2];
   const TopkJob& jb = J.j[blockIdx.y];
@@ -327,54 +385,56 @@ __global__ void __launch_bounds__(1024) k_topk_emit(TopkJobs J) {
   unsigned long long lo, hi;
   bin_range(st, &lo, &hi);
   const int above_total = st->above, keep = st->keep;
-  int ra = jb.blk_a[blockIdx.x], rb = jb.blk_b[blockIdx.x];
   unsigned long long* keys = jb.keys;
   int* ids = jb.ids;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int base = blockIdx.x * kTopkChunk;
-  for (int round = 0; round < kTopkChunk / 1024; ++round) {
-    const int i = base + round * 1024 + threadIdx.x;
-    unsigned long long key = 0;
-    int fa = 0, fb = 0;
-    if (i < n) {
-      key = order_key(r[i]);
-      fa = key > hi;
-      fb = key >= lo && key <= hi;
-    }
-    const unsigned ba = __ballot_sync(0xffffffffu, fa), bb = __ballot_sync(0xffffffffu, fb);
-    if (lane == 0) {
-      s_w[0][w] = __popc(ba);
-      s_w[1][w] = __popc(bb);
-    }
-    __syncthreads();
-    int pa = 0, pb = 0;
-    for (int q = 0; q < w; ++q) {
-      pa += s_w[0][q];
-      pb += s_w[1][q];
-    }
-    pa += __popc(ba & lanemask_lt());
-    pb += __popc(bb & lanemask_lt());
-    if (fa) {
-      keys[ra + pa] = key;
-      ids[ra + pa] = i;
-    }
-    if (fb && rb + pb < keep) {
-      keys[above_total + rb + pb] = key;
-      ids[above_total + rb + pb] = i;
-    }
-    if (threadIdx.x == 0) {
-      int ta = 0, tb = 0;
-      for (int q = 0; q < 32; ++q) {
-        ta += s_w[0][q];
-        tb += s_w[1][q];
+  for (int c = blockIdx.x; c < nb; c += gridDim.x) {
+    int ra = jb.blk_a[c], rb = jb.blk_b[c];
+    const int base = c * kTopkChunk;
+    for (int round = 0; round < kTopkChunk / 1024; ++round) {
+      const int i = base + round * 1024 + threadIdx.x;
+      unsigned long long key = 0;
+      int fa = 0, fb = 0;
+      if (i < n) {
+        key = order_key(r[i]);
+        fa = key > hi;
+        fb = key >= lo && key <= hi;
       }
-      s_run[0] = ta;
-      s_run[1] = tb;
+      const unsigned ba = __ballot_sync(0xffffffffu, fa), bb = __ballot_sync(0xffffffffu, fb);
+      if (lane == 0) {
+        s_w[0][w] = __popc(ba);
+        s_w[1][w] = __popc(bb);
+      }
+      __syncthreads();
+      int pa = 0, pb = 0;
+      for (int q = 0; q < w; ++q) {
+        pa += s_w[0][q];
+        pb += s_w[1][q];
+      }
+      pa += __popc(ba & lanemask_lt());
+      pb += __popc(bb & lanemask_lt());
+      if (fa) {
+        keys[ra + pa] = key;
+        ids[ra + pa] = i;
+      }
+      if (fb && rb + pb < keep) {
+        keys[above_total + rb + pb] = key;
+        ids[above_total + rb + pb] = i;
+      }
+      if (threadIdx.x == 0) {
+        int ta = 0, tb = 0;
+        for (int q = 0; q < 32; ++q) {
+          ta += s_w[0][q];
+          tb += s_w[1][q];
+        }
+        s_run[0] = ta;
+        s_run[1] = tb;
+      }
+      __syncthreads();
+      ra += s_run[0];
+      rb += s_run[1];
+      __syncthreads();
     }
-    __syncthreads();
-    ra += s_run[0];
-    rb += s_run[1];
-    __syncthreads();
   }
 }
 
@@ -591,9 +651,10 @@ int enqueue_topk_select(const TopkJobs& J, int num_sms, cudaStream_t st) {
   for (int w : widths) k_topk_hist<<<dim3(gx, m), 256, 0, st>>>(J, w, kTopkCand);
   k_topk_collect<<<dim3(gx, m), 256, 0, st>>>(J, kTopkMaxK + kTopkCand);
   const int nb = (J.n + kTopkChunk - 1) / kTopkChunk;
-  k_topk_count<<<dim3(nb, m), 1024, 0, st>>>(J);
+  const int gc = std::min(nb, std::max(1, num_sms * 2 / m));
+  k_topk_count<<<dim3(gc, m), 1024, 0, st>>>(J, nb);
   k_topk_scan<<<dim3(1, m), 1024, 0, st>>>(J, nb, kTopkCand);
-  k_topk_emit<<<dim3(nb, m), 1024, 0, st>>>(J);
+  k_topk_emit<<<dim3(gc, m), 1024, 0, st>>>(J, nb);
   return 11;
 }
 

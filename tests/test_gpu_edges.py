@@ -266,3 +266,30 @@ def test_pull_plan_over_node_counts_around_its_ranges(n, det):
     r, _, _, _ = O.osp(old, g.csr(), r, C_RESTART, 1e-9, force_iters=st["iterations"])
     assert np.abs(eng.query() - r).sum() <= 1e-10
     eng.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 1023, 65536, 311_297])
+@pytest.mark.parametrize("start", [0, 1])
+def test_topk_of_a_vector_at_any_element(start, n):
+    """Vectors that start at an even and at an odd element, whole and ragged passes
+    of the paired loads, negative and infinite scores: exact."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n + start)
+    v = rng.normal(0, 1, n)
+    v[rng.integers(0, n, 1 + n // 50)] = -0.0
+    v[rng.integers(0, n)] = np.inf
+    v[rng.integers(0, n)] = -np.inf
+    buf = torch.zeros(n + 1, dtype=torch.float64, device="cuda")
+    buf[start:start + n] = torch.from_numpy(v).cuda()
+    for k in (1, 77, 3000):
+        ids = torch.empty(k, dtype=torch.int32, device="cuda")
+        sc = torch.empty(k, dtype=torch.float64, device="cuda")
+        got = torch.zeros(1, dtype=torch.int32, device="cuda")
+        N.topk_noalloc(buf[start:], n, k, ids, sc, got, stream=torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        c = int(got)
+        assert c == min(n, k)
+        key = np.where(np.signbit(v), ~v.view(np.uint64), v.view(np.uint64) | np.uint64(1 << 63))
+        want = np.lexsort((np.arange(n), ~key))[:c]
+        assert np.array_equal(ids[:c].cpu().numpy(), want)
+        assert np.array_equal(sc[:c].cpu().numpy(), v[want])
