@@ -21,11 +21,10 @@ constexpr long long kMaxLargeBatch = 1ll << 22;  // ops per apply call, in sub-b
 constexpr int kIngestOne = 1024;       // ops that one CTA ingests by itself
 constexpr int kMaxNodes = (1 << 25) - 1; // ids fit in 25 bits
 constexpr int kNoPos = 0x7F7F7F7F;       // del_pos of a node not deleted by the batch (memset 0x7F)
-constexpr int kLight = 32;               // lists up to this length are walked by one lane
 constexpr int kPiece = 256;              // old entries per warp task in the list merge
 constexpr int kMaxHist = 4096;           // per-step ||x||_1 history entries
 constexpr int kAbsParts = 1024;  // CTAs of the L1-norm reduction (per-CTA partials, summed in order)
-constexpr int kMaxGrid = 4096;           // CTAs of the persistent kernel (partials array size)
+constexpr int kMaxGrid = 2000;           // CTAs of the persistent kernels (partials array size)
 constexpr int kPropThreads = 256;
 constexpr int kPropWarps = kPropThreads / 32;
 // The one-seed kernel runs one CTA of 32 warps per SM: as many warps as four
@@ -40,7 +39,7 @@ constexpr int kMultiHub = 256;       // seed block: in-lists longer than this, i
 constexpr int kMultiNodeItems = 4;   // seed block: task items per node (a node's score row costs more)
 constexpr int kTaskItems = 1024;     // pull step: default items (edges + nodes) per warp task
 constexpr int kMinTaskItems = 256;   // smallest task size a schedule may choose (sizes the plan)
-constexpr int kMaxSmallTasks = 1 << 16;  // most tasks a small graph is cut into below that size
+constexpr int kMaxSmallTasks = 1 << 14;  // most tasks a small graph is cut into below that size
 constexpr double kPushAlpha = 14.0;  // push step while frontier out-edges <= m / alpha
 constexpr double kPushBeta = 24.0;   // ... and frontier size <= n / beta
 
@@ -152,8 +151,9 @@ struct Dev {
   // batch scratch: net edits grouped per changed row / column
   int* ins_r; int* del_r; int* ins_c; int* del_c;   // [kMaxBatch]
   int* gi; int* gd;                                  // [kMaxBatch + 1] prefix counts
-  unsigned long long* ing_key; int* ing_na;          // [kMaxBatch] larger batches: sort keys; node
-                                                     // count before each op, then kind of edit
+  // [kMaxBatch] larger batches: sort keys (in ins_r and del_r, contiguous); node count
+  // before each op, then kind of edit (in ins_c)
+  unsigned long long* ing_key; int* ing_na;
   int* rec_r_node; int* rec_r_is; int* rec_r_ic; int* rec_r_ds; int* rec_r_dc;  // [nc]
   int* rec_c_node; int* rec_c_is; int* rec_c_ic; int* rec_c_ds; int* rec_c_dc;  // [nc]
   int* del_nodes;  // [kMaxBatch]
@@ -162,15 +162,16 @@ struct Dev {
   unsigned* rec_old_off; int* rec_old_len; int* rec_pstart;  // [2 nc + 1]
   unsigned* rec_fbase; int* rec_dp;                          // [2 nc]
   int* piece_rec; int* piece_cnt; int* piece_base;           // [2 nc + 2 pool cap / kPiece + 2]
-  // pull-step plan: prefix of in-list lengths, warp tasks of about
+  // pull-step plan: warp tasks of about
   // kTaskItems items (edges + nodes, lists never split), and the long in-lists
   // summed in pieces
-  int* task_first;                    // [(kMultiNodeItems nc + pool cap) / kMinTaskItems + 2] first node of each warp task
+  int* task_first;                    // [(kMultiNodeItems nc + pool cap) / kMinTaskItems + small tasks + 2] first node of each warp task
   int* hubs; int* hub_pstart; double* hub_acc; int* hub_cnt;  // [pool cap / kHubThreshold + 2]
   int* piece_hub;  // [2 pool cap / kMultiHub + 4] the long in-list each piece belongs to
   double* piece_part;  // [as piece_hub] deterministic mode: per-piece partial sums
   double* hub_l1;      // [as hubs] deterministic mode: |x_v| of each long in-list's node
-  // push step: pieces of the rows longer than kPushPiece [2 pool cap / kPushPiece + 2]
+  // push step: pieces of the rows longer than kPushPiece [2 pool cap / kPushPiece + 2],
+  // in piece_rec, piece_cnt and piece_part
   unsigned* big_off; int* big_len; double* big_y;
   unsigned* bar;  // grid barrier of the one-seed kernel: arrivals of the call, on a line of its own
   // reductions and history
@@ -288,19 +289,6 @@ __device__ __forceinline__ int lower_bound_i(const int* a, int n, int x) {
 __device__ __forceinline__ bool contains_i(const int* a, int n, int x) {
   int p = lower_bound_i(a, n, x);
   return p < n && a[p] == x;
-}
-
-// Warp-aggregated append of `want` lanes' values to a queue (all lanes of the
-// warp must call this together).
-__device__ __forceinline__ void warp_append(bool want, int val, int* queue, int* counter) {
-  unsigned b = __ballot_sync(0xffffffffu, want);
-  if (!b) return;
-  int leader = __ffs(b) - 1;
-  int lane = threadIdx.x & 31;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(counter, __popc(b));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (want) queue[base + __popc(b & lanemask_lt())] = val;
 }
 
 }  // namespace osp

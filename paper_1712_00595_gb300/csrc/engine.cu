@@ -475,10 +475,16 @@ const int* schedule(osp_ctx* ctx) {
   return single;
 }
 
+// Most tasks that a small graph is cut into (the plan has room for as many more).
+int64_t small_tasks(const osp_ctx* ctx) { return std::min<int64_t>(kMaxSmallTasks, ctx->nc); }
+
 // Pull-step plan for the graph as it is after the merge.
 osp_status plan_pull(osp_ctx* ctx) {
   cudaStream_t st = ctx->stream;
-  k_plan_sums<<<ctx->num_sms, 1024, 0, st>>>(ctx->d, ctx->scan_bsum);
+  static_assert(kMaxBatch * sizeof(osp_update) >= kMaxGrid * sizeof(unsigned), "a sum per CTA");
+  unsigned* sums = reinterpret_cast<unsigned*>(ctx->ops_stage);  // the batch has been merged
+  const int plan_grid = std::min(ctx->num_sms, kMaxGrid);
+  k_plan_sums<<<plan_grid, 1024, 0, st>>>(ctx->d, sums);
   ++ctx->launches;
   const int* sc = schedule(ctx);
   // A graph whose tasks of sc[0] items would leave warps idle is cut finer:
@@ -490,9 +496,9 @@ osp_status plan_pull(osp_ctx* ctx) {
   // a batch with four of 64, 394 with two of 256).
   const bool many = ctx->S > 1, bf16 = many && ctx->opt.precision == OSP_PREC_BF16_ACC64;
   const int warps = many ? ctx->grid_multi * kPropWarps : ctx->grid_prop * kOneWarps;
-  k_pull_plan<<<ctx->num_sms, 1024, 0, st>>>(
-      ctx->d, ctx->scan_bsum, sc[1], sc[2], sc[3], sc[0], bf16 ? 256 : many ? 64 : 32,
-      std::min(kMaxSmallTasks, warps * (many && !bf16 ? 4 : 2)), ctx->opt.deterministic != 0);
+  k_pull_plan<<<plan_grid, 1024, 0, st>>>(
+      ctx->d, sums, sc[1], sc[2], sc[3], sc[0], bf16 ? 256 : many ? 64 : 32,
+      (int)std::min<int64_t>(small_tasks(ctx), warps * (many && !bf16 ? 4 : 2)), ctx->opt.deterministic != 0);
   ++ctx->launches;
   CK(cudaGetLastError());
   return OSP_OK;
@@ -1160,14 +1166,16 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
   AL(d.clr_pos, nc, 0xFF);
   AL(d.rflag, nc, 0);
   AL(d.cflag, nc, 0);
-  AL(d.ins_r, kMaxBatch, 0);
-  AL(d.del_r, kMaxBatch, 0);
+  AL(d.ins_r, 2 * kMaxBatch, 0);
+  d.del_r = d.ins_r + kMaxBatch;
   AL(d.ins_c, kMaxBatch, 0);
   AL(d.del_c, kMaxBatch, 0);
   AL(d.gi, kMaxBatch + 1, 0);
   AL(d.gd, kMaxBatch + 1, 0);
-  AL(d.ing_key, kMaxBatch, 0);
-  AL(d.ing_na, kMaxBatch, 0);
+  // larger batches: the sort's keys and kinds lie where k_ingest_emit, once it has
+  // read them, writes the edits
+  d.ing_key = reinterpret_cast<unsigned long long*>(d.ins_r);
+  d.ing_na = d.ins_c;
   AL(d.rec_r_node, nc, 0);
   AL(d.rec_r_is, nc, 0);
   AL(d.rec_r_ic, nc, 0);
@@ -1192,7 +1200,8 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     AL(d.piece_cnt, npc, 0);
     AL(d.piece_base, npc, 0);
   }
-  AL(d.task_first, (int64_t)(kMultiNodeItems * nc + (int64_t)cap) / kMinTaskItems + kMaxSmallTasks + 2, 0);
+  AL(d.task_first,
+     (int64_t)(kMultiNodeItems * nc + (int64_t)cap) / kMinTaskItems + small_tasks(ctx) + 2, 0);
   {
     // lists longer than a threshold t number at most (live edges) / t <= cap / t;
     // the pull plan uses t = kMultiHub for the seed block, kHubThreshold otherwise
@@ -1205,11 +1214,13 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     AL(d.hub_l1, nh, 0);
     AL(d.hub_acc, nh, 0);
     AL(d.hub_cnt, nh, 0);
-    // push: a row above kPushPiece entries has at most 2 len / kPushPiece pieces
-    const int64_t nb = 2 * (int64_t)(cap / kPushPiece) + 2;
-    AL(d.big_off, nb, 0);
-    AL(d.big_len, nb, 0);
-    AL(d.big_y, nb, 0);
+    // push: a row above kPushPiece entries has at most 2 len / kPushPiece pieces, and
+    // the arrays of the merge's pieces and of the pull-only deterministic sums are
+    // idle then
+    static_assert(kPushPiece >= kPiece && kPushPiece >= kMultiHub, "big rows fit those arrays");
+    d.big_off = reinterpret_cast<unsigned*>(d.piece_rec);
+    d.big_len = d.piece_cnt;
+    d.big_y = d.piece_part;
   }
   AL(d.part_l1, 2 * kMaxGrid, 0);
   AL(d.part_ef, 2 * kMaxGrid, 0);
@@ -1221,7 +1232,7 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
   AL(ctx->dsum, kAbsParts + 2, 0);  // the norm, its per-CTA partials, the CTA count
   AL(ctx->dtmp, nc, 0);
   AL(ctx->scan_off, nc, 0);
-  AL(ctx->scan_bsum, std::max<int64_t>(nc / 4096 + 2, ctx->num_sms), 0);
+  AL(ctx->scan_bsum, nc / 4096 + 2, 0);
   AL(ctx->tk_state, 1, 0);
   AL(ctx->tk_hist, 4096, 0);
   AL(ctx->tk_blk_a, nc / kTopkChunk + 2, 0);

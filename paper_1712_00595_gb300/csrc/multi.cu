@@ -38,23 +38,7 @@ __device__ __forceinline__ __nv_bfloat16 from_acc(float v, __nv_bfloat16*) { ret
 __device__ __forceinline__ float from_acc(float v, float*) { return v; }
 __device__ __forceinline__ double from_acc(double v, double*) { return v; }
 
-// K contiguous elements (K * sizeof(T) bytes, naturally aligned) through L2.
-template <typename T, int K>
-__device__ __forceinline__ void load_cg(const T* p, T (&out)[K]) {
-  constexpr int B = K * (int)sizeof(T);
-  if constexpr (B >= 16) {
-#pragma unroll
-    for (int i = 0; i < B / 16; ++i)
-      reinterpret_cast<uint4*>(out)[i] = __ldcg(reinterpret_cast<const uint4*>(p) + i);
-  } else if constexpr (B == 8) {
-    *reinterpret_cast<uint2*>(out) = __ldcg(reinterpret_cast<const uint2*>(p));
-  } else if constexpr (B == 4) {
-    *reinterpret_cast<unsigned*>(out) = __ldcg(reinterpret_cast<const unsigned*>(p));
-  } else {
-    *reinterpret_cast<unsigned short*>(out) = __ldcg(reinterpret_cast<const unsigned short*>(p));
-  }
-}
-
+// K contiguous elements (K * sizeof(T) bytes, naturally aligned).
 template <typename T, int K>
 __device__ __forceinline__ void store_k(T* p, const T (&v)[K]) {
   constexpr int B = K * (int)sizeof(T);
