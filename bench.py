@@ -586,6 +586,9 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
     achieved = ab / (prop_ms / 1e3) / 1e9
     dense_step = multi_alg_bytes(dict(stats[-1], iterations=1), stats[-1]["m_edges"], S, by)
     hist = np.bincount(np.concatenate(counts[Wm + 1:]).astype(np.int64))
+    # columns per group of the gather rows (the engine's default when not given)
+    group = args.seed_group or (64 if by == 2 and n < 1 << 19 else 128)
+    group = min(group, next(32 * k for k in (1, 2, 4, 8) if 32 * k >= S))
     rec = traffic_record("k_propagate_multi")
     traffic = None
     if rec and config["workload"] == HEADLINE:
@@ -599,16 +602,15 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
         "data": "synthetic",
         "config": dict(config, seed_gather=args.seed_gather, autotune=bool(args.autotune),
                        schedule=list(eng.get_schedule()), node_order="descending out-degree",
-                       seed_group=args.seed_group or (32 if cfg["precision"] == "bf16"
-                                                      else 32 * ((S + 31) // 32)),
-                       column_groups="packed per batch by offset size" if cfg["precision"] == "bf16"
-                       and S > 32 and args.seed_group in (0, 32) else "fixed"),
+                       seed_group=group,
+                       column_groups="packed per batch by offset size" if args.seed_gather != "bulk"
+                       and S > group and group * by <= 512 else "fixed"),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_per_alg_byte": float(rec["dram_bytes_per_alg_byte"])
                      if traffic is not None else None,
                      "traffic_source": rec.get("source") if traffic is not None else None,
-                     "kernel": "k_propagate_multi", "peak_kind": peak_kind + " (hbm_gbs copy)",
+                     "kernel": "k_propagate_ring", "peak_kind": peak_kind + " (hbm_gbs copy)",
                      "alg_bytes_per_launch": ab / K, "ms_per_launch": prop_ms / K,
                      "dense_step_alg_bytes": dense_step},
         "phases_ms_per_step": {"update_merge_offset": sum(s["ms_update"] for s in stats) / K,
