@@ -151,9 +151,9 @@ struct Dev {
   // batch scratch: net edits grouped per changed row / column
   int* ins_r; int* del_r; int* ins_c; int* del_c;   // [kMaxBatch]
   int* gi; int* gd;                                  // [kMaxBatch + 1] prefix counts
-  // [kMaxBatch] larger batches: sort keys (in ins_r and del_r, contiguous); node count
-  // before each op, then kind of edit (in ins_c)
-  unsigned long long* ing_key; int* ing_na;
+  // [kMaxBatch] larger batches: sort keys (in ins_r and del_r, contiguous), sorted
+  // (in ins_c and del_c); node count before each op, then kind of edit (in gi)
+  unsigned long long* ing_key; unsigned long long* ing_sorted; int* ing_na;
   int* rec_r_node; int* rec_r_is; int* rec_r_ic; int* rec_r_ds; int* rec_r_dc;  // [nc]
   int* rec_c_node; int* rec_c_is; int* rec_c_ic; int* rec_c_ds; int* rec_c_dc;  // [nc]
   int* del_nodes;  // [kMaxBatch]

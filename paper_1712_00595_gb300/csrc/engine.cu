@@ -616,7 +616,7 @@ osp_status enqueue_update(osp_ctx* ctx, const osp_update* ops_dev, int U, int Np
     const size_t sort = ingest_sort_smem(Np);
     k_ingest_scan<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
     k_ingest_keys<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
-    k_ingest_sort<<<1, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_rank<<<(Np + 31) / 32, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
     k_ingest_edits<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
     k_ingest_emit<<<1, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
     ctx->launches += 5;
@@ -1019,9 +1019,6 @@ osp_status osp_create(osp_ctx** out, const osp_options* opt) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_ingest, cudaFuncAttributeMaxDynamicSharedMemorySize, kIngestSmem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ingest_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)ingest_sort_smem(kMaxBatch));
-  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_ingest_emit, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)ingest_sort_smem(kMaxBatch));
   if (e == cudaSuccess)
@@ -1168,14 +1165,15 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
   AL(d.cflag, nc, 0);
   AL(d.ins_r, 2 * kMaxBatch, 0);
   d.del_r = d.ins_r + kMaxBatch;
-  AL(d.ins_c, kMaxBatch, 0);
-  AL(d.del_c, kMaxBatch, 0);
+  AL(d.ins_c, 2 * kMaxBatch, 0);
+  d.del_c = d.ins_c + kMaxBatch;
   AL(d.gi, kMaxBatch + 1, 0);
   AL(d.gd, kMaxBatch + 1, 0);
-  // larger batches: the sort's keys and kinds lie where k_ingest_emit, once it has
-  // read them, writes the edits
+  // larger batches: the keys and kinds lie where k_ingest_emit, once it has read
+  // them, writes the edits and counts
   d.ing_key = reinterpret_cast<unsigned long long*>(d.ins_r);
-  d.ing_na = d.ins_c;
+  d.ing_sorted = reinterpret_cast<unsigned long long*>(d.ins_c);
+  d.ing_na = d.gi;
   AL(d.rec_r_node, nc, 0);
   AL(d.rec_r_is, nc, 0);
   AL(d.rec_r_ic, nc, 0);

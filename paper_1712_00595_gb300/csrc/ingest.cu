@@ -422,17 +422,19 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest(Dev d, const osp_upda
 // CTA spent 760 us on 10,001 ops and 867 us on 15,000: two bitonic sorts (105
 // passes of 16,384 keys through shared memory each), the existence searches
 // (some 14 scattered loads an op from one SM) and 16 ops a thread one after the
-// other. Here the searches and validation run one op a thread, and one CTA sorts
-// by stable 8-bit radix passes over the bits in use.
+// other. Here all but the emission runs one op a thread, and one CTA emits the
+// lists and sorts the edits for the columns by stable 8-bit radix passes over the
+// bits in use.
 //   k_ingest_scan   node count before each op; first deletion, last zeroing
 //   k_ingest_keys   validation; sort keys (u, v, position)
-//   k_ingest_sort   the radix sort (or the report of the first invalid op)
+//   k_ingest_rank   their order (or the report of the first invalid op)
 //   k_ingest_edits  last op of each pair against the current row: net edits
 //   k_ingest_emit   edit lists and records of rows, the same sorted for columns
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr int kSortRows = kMaxBatch / kIngestThreads;  // keys a thread
+constexpr unsigned long long kLastKeys = ~0ull << 14;    // ops without an edge, by position
 
 // Bits of a node id among n nodes, so that no id has all of them set.
 __device__ __forceinline__ int id_bits(int n) { return 32 - __clz(n); }
@@ -658,7 +660,7 @@ __global__ void __launch_bounds__(256) k_ingest_keys(Dev d, const osp_update* __
   const int na = d.ing_na[p];
   const int bits = id_bits(ctl->n + ctl->ing_adds);
   bool ok = false;
-  unsigned long long key = kNoKey;
+  unsigned long long key = kLastKeys | (unsigned)p;
   if (o.op == OSP_OP_INSERT_EDGE || o.op == OSP_OP_DELETE_EDGE) {
     if (o.u >= 0 && o.u < na && o.v >= 0 && o.v < na) {
       const int du = d.del_pos[o.u], dv = d.del_pos[o.v];
@@ -677,44 +679,75 @@ __global__ void __launch_bounds__(256) k_ingest_keys(Dev d, const osp_update* __
   d.ing_key[p] = key;
 }
 
-__global__ void __launch_bounds__(kIngestThreads) k_ingest_sort(Dev d, const osp_update* __restrict__ ops,
-                                                                int U) {
-  extern __shared__ unsigned long long skey[];
+// n -= a < b: the borrow of a - b, three instructions.
+__device__ __forceinline__ void sub_borrow(int& n, unsigned long long a, unsigned long long b) {
+  asm("{\n.reg .u32 t;\nsub.cc.u32 t, %1, %3;\nsubc.cc.u32 t, %2, %4;\nsubc.u32 %0, %0, 0;\n}"
+      : "+r"(n)
+      : "r"((unsigned)a), "r"((unsigned)(a >> 32)), "r"((unsigned)b), "r"((unsigned)(b >> 32)));
+}
+
+// Sorted place of each key = how many keys are smaller (they differ in the position;
+// ops without a key sort last), or the report of the first invalid op. Lane = key,
+// a warp an eighth of the others, which all lanes read together. U^2 comparisons
+// over the whole chip are less than five radix passes in one CTA (15,000 keys 62 ->
+// 52 us, 10,000 46 -> 34).
+__global__ void __launch_bounds__(256) k_ingest_rank(Dev d, const osp_update* __restrict__ ops, int U) {
+  __shared__ int s_cnt[8][32];
+  __shared__ ulonglong2 s_key[8][32];
   Ctl* ctl = d.ctl;
   U = batch_size(d, U);
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int i0 = blockIdx.x * 32;
+  if (i0 >= U && blockIdx.x) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = i0 + lane;
   const int bad = ctl->ing_bad;
   if (bad != kNoPos) {
-    for (int p = tid; p < U; p += kIngestThreads) {
-      const int op = ops[p].op;
+    if (w == 0 && i < U) {
+      const int op = ops[i].op;
       if (op == OSP_OP_DELETE_NODE || op == OSP_OP_ZERO_ROW) {
-        const osp_update o = load_op(ops, p, d);
+        const osp_update o = load_op(ops, i, d);
         if (o.u >= 0 && o.u < d.nc) {
           if (op == OSP_OP_DELETE_NODE) d.del_pos[o.u] = kNoPos;
           else d.clr_pos[o.u] = -1;
         }
       }
     }
-    if (tid == 0) {
+    if (i0 == 0 && threadIdx.x == 0) {
       ctl->status = OSP_EINVAL;
       ctl->bad_op = bad;
       ctl->n_clr = 0;
     }
     return;
   }
-  const int per = sort_rows(U);
-  unsigned long long key[kSortRows];
-#pragma unroll
-  for (int r = 0; r < kSortRows; ++r) {
-    const int i = (w * per + r) * 32 + lane;
-    key[r] = r < per && i < U ? d.ing_key[i] : kNoKey;
+  const unsigned long long key = i < U ? d.ing_key[i] : kNoKey;
+  // 64 keys at a time, a pair a lane, through shared memory; the next ones load
+  // meanwhile
+  const int pairs = U >> 1;
+  const int lo = (int)((long long)pairs * w >> 3), hi = (int)((long long)pairs * (w + 1) >> 3);
+  const ulonglong2* all = reinterpret_cast<const ulonglong2*>(d.ing_key);
+  const ulonglong2 none = make_ulonglong2(~0ull, ~0ull);  // below no key
+  int cnt = 0;
+  ulonglong2 next = lo + lane < hi ? __ldg(all + lo + lane) : none;
+  for (int b = lo; b < hi; b += 32) {
+    __syncwarp();
+    s_key[w][lane] = next;
+    __syncwarp();
+    next = b + 32 + lane < hi ? __ldg(all + b + 32 + lane) : none;
+#pragma unroll 16
+    for (int q = 0; q < 32; ++q) {
+      const ulonglong2 k = s_key[w][q];
+      sub_borrow(cnt, k.x, key);
+      sub_borrow(cnt, k.y, key);
+    }
   }
-  __syncthreads();  // all keys are in registers
-  radix_sort(key, per, 14, 14 + 2 * id_bits(ctl->n + ctl->ing_adds), skey,
-             reinterpret_cast<int*>(skey + per * kIngestThreads));
+  cnt = -cnt;
+  if (w == 0 && (U & 1)) cnt += d.ing_key[U - 1] < key;
+  s_cnt[w][lane] = cnt;
+  __syncthreads();
+  if (w != 0 || i >= U) return;
 #pragma unroll
-  for (int r = 0; r < kSortRows; ++r)
-    if (r < per && (w * per + r) * 32 + lane < U) d.ing_key[(w * per + r) * 32 + lane] = key[r];
+  for (int q = 1; q < 8; ++q) cnt += s_cnt[q][lane];
+  d.ing_sorted[cnt] = key >= kLastKeys ? kNoKey : key;
 }
 
 // One thread per sorted op: the last op of each (u, v) against the current row.
@@ -724,11 +757,11 @@ __global__ void __launch_bounds__(256) k_ingest_edits(Dev d, const osp_update* _
   U = batch_size(d, U);
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= U) return;
-  const unsigned long long key = d.ing_key[i];
+  const unsigned long long key = d.ing_sorted[i];
   const int n_old = ctl->n;
   const int bits = id_bits(n_old + ctl->ing_adds);
   int kind = 0;
-  if (key != kNoKey && (i == U - 1 || (d.ing_key[i + 1] >> 14) != (key >> 14))) {
+  if (key != kNoKey && (i == U - 1 || (d.ing_sorted[i + 1] >> 14) != (key >> 14))) {
     const int p = (int)(key & 0x3FFF);
     const int u = (int)(key >> (14 + bits));
     const int v = (int)((key >> 14) & ((1ull << bits) - 1));
@@ -770,7 +803,7 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp
 #pragma unroll
   for (int r = 0; r < kSortRows; ++r) {
     const int i = (w * per + r) * 32 + lane;
-    key[r] = r < per && i < U ? d.ing_key[i] : kNoKey;
+    key[r] = r < per && i < U ? d.ing_sorted[i] : kNoKey;
     kind[r] = r < per && i < U ? d.ing_na[i] : 0;
     if (r < per) skey[i] = key[r];
   }

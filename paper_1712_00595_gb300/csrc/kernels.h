@@ -10,7 +10,7 @@ __global__ void k_cpi_begin_uniform(Dev d, int n0);
 __global__ void k_ingest(Dev d, const osp_update* __restrict__ ops, int U);
 __global__ void k_ingest_scan(Dev d, const osp_update* __restrict__ ops, int U);
 __global__ void k_ingest_keys(Dev d, const osp_update* __restrict__ ops, int U);
-__global__ void k_ingest_sort(Dev d, const osp_update* __restrict__ ops, int U);
+__global__ void k_ingest_rank(Dev d, const osp_update* __restrict__ ops, int U);
 __global__ void k_ingest_edits(Dev d, const osp_update* __restrict__ ops, int U);
 __global__ void k_ingest_emit(Dev d, const osp_update* __restrict__ ops, int U);
 __global__ void k_expand(Dev d);
