@@ -618,7 +618,7 @@ osp_status enqueue_update(osp_ctx* ctx, const osp_update* ops_dev, int U, int Np
     k_ingest_keys<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
     k_ingest_rank<<<(Np + 31) / 32, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
     k_ingest_edits<<<nb, 256, 0, ctx->stream>>>(ctx->d, ops_dev, U);
-    k_ingest_emit<<<1, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
+    k_ingest_emit<<<2, 1024, sort, ctx->stream>>>(ctx->d, ops_dev, U);
     ctx->launches += 5;
   }
   k_expand<<<g, 256, 0, ctx->stream>>>(ctx->d);

@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest(Dev d, const osp_upda
 // CTA spent 760 us on 10,001 ops and 867 us on 15,000: two bitonic sorts (105
 // passes of 16,384 keys through shared memory each), the existence searches
 // (some 14 scattered loads an op from one SM) and 16 ops a thread one after the
-// other. Here all but the emission runs one op a thread, and one CTA emits the
-// lists and sorts the edits for the columns by stable 8-bit radix passes over the
+// other. Here all but the emission runs one op a thread, and two CTAs emit the
+// lists, one sorting the edits for the columns by stable 8-bit radix passes over the
 // bits in use.
 //   k_ingest_scan   node count before each op; first deletion, last zeroing
 //   k_ingest_keys   validation; sort keys (u, v, position)
@@ -509,15 +509,16 @@ __device__ void radix_sort(unsigned long long (&key)[kSortRows], int per, int lo
 
 // Edit lists and records of one direction from `per` * 1024 sorted edits (key[r]
 // as in radix_sort; kind 0 none, 1 insert, 2 delete; group_of(key) the list's
-// node, member_of(key) the entry). s_a, s_b: 1024 per + 1 ints each.
+// node, member_of(key) the entry). s_key: the keys, and once the groups' heads are
+// known the counts before each group (2 (1024 per + 1) ints, the buffer is longer).
 template <typename GroupF, typename MemberF>
 __device__ void emit_edits(const unsigned long long (&key)[kSortRows], const int (&kind)[kSortRows],
-                           int per, unsigned long long* s_key, int* s_a, int* s_b, GroupF group_of,
-                           MemberF member_of, int* ins_out, int* del_out, int* rec_node, int* rec_is,
+                           int per, unsigned long long* s_key, GroupF group_of, MemberF member_of, int* ins_out, int* del_out, int* rec_node, int* rec_is,
                            int* rec_ic, int* rec_ds, int* rec_dc, int* flag_arr, int* n_rec,
                            int* n_ins, int* n_del) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int N = per * kIngestThreads;
+  int* s_a = reinterpret_cast<int*>(s_key);
+  int* s_b = s_a + per * kIngestThreads + 1;
   // the three running counts (insertions, deletions, groups) by warp: a warp's
   // keys are consecutive
   __shared__ int s_heads;
@@ -600,7 +601,6 @@ __device__ void emit_edits(const unsigned long long (&key)[kSortRows], const int
     *n_del = td;
   }
   __syncthreads();
-  (void)N;
 }
 
 __device__ __forceinline__ int batch_size(const Dev& d, int U) { return U < 0 ? d.ctl->batch_U : U; }
@@ -785,8 +785,12 @@ __global__ void __launch_bounds__(256) k_ingest_edits(Dev d, const osp_update* _
   d.ing_na[i] = kind;
 }
 
-__global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp_update* __restrict__ ops,
-                                                                int U) {
+// A cluster of two CTAs: rows, node deletions and zeroed rows in the first, the
+// columns (with their sort) in the second; one after the other in one CTA they took
+// 98 us for 15,000 ops, 59 so. Both read the keys that the columns' edits
+// replace, so nothing is written before both have them in registers.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kIngestThreads)
+    k_ingest_emit(Dev d, const osp_update* __restrict__ ops, int U) {
   extern __shared__ unsigned long long skey[];
   __shared__ int s_ndel, s_nclr;
   Ctl* ctl = d.ctl;
@@ -796,8 +800,8 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp
   const int per = sort_rows(U);
   const int adds = ctl->ing_adds;
   const int bits = id_bits(ctl->n + adds);
-  int* s_a = reinterpret_cast<int*>(skey + per * kIngestThreads);  // at least 32 x 256 ints
-  int* s_b = d.gi;  // [kMaxBatch + 1]
+  const bool columns = blockIdx.x == 1;
+  int* s_cnt = reinterpret_cast<int*>(skey + per * kIngestThreads);  // 32 x 256 ints
   unsigned long long key[kSortRows];
   int kind[kSortRows];
 #pragma unroll
@@ -808,16 +812,37 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp
     if (r < per) skey[i] = key[r];
   }
   if (tid == 0) s_ndel = s_nclr = 0;
-  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   int n_ins = 0, n_del = 0;
-  emit_edits(
-      key, kind, per, skey, d.gd, s_b, [&](unsigned long long k) { return (int)(k >> (14 + bits)); },
-      [&](unsigned long long k) { return (int)((k >> 14) & ((1ull << bits) - 1)); }, d.ins_r, d.del_r,
-      d.rec_r_node, d.rec_r_is, d.rec_r_ic, d.rec_r_ds, d.rec_r_dc, d.rflag, &ctl->n_rec_r, &n_ins,
-      &n_del);
-  if (tid == 0) {  // summed over the sub-batches of a large batch
-    ctl->net_ins += n_ins - ctl->ing_reins;
-    ctl->net_del += n_del;
+  if (!columns) {
+    emit_edits(
+        key, kind, per, skey, [&](unsigned long long k) { return (int)(k >> (14 + bits)); },
+        [&](unsigned long long k) { return (int)((k >> 14) & ((1ull << bits) - 1)); }, d.ins_r, d.del_r,
+        d.rec_r_node, d.rec_r_is, d.rec_r_ic, d.rec_r_ds, d.rec_r_dc, d.rflag, &ctl->n_rec_r, &n_ins,
+        &n_del);
+    if (tid == 0) {  // summed over the sub-batches of a large batch
+      ctl->net_ins += n_ins - ctl->ing_reins;
+      ctl->net_del += n_del;
+    }
+    // node deletions and zeroed rows
+    for (int p = tid; p < U; p += kIngestThreads) {
+      const int op = ops[p].op;
+      if (op == OSP_OP_DELETE_NODE) {
+        const int u = load_op(ops, p, d).u;
+        d.del_nodes[atomicAdd(&s_ndel, 1)] = u;
+        d.del_pos[u] = kNoPos;
+      } else if (op == OSP_OP_ZERO_ROW) {
+        const int u = load_op(ops, p, d).u;
+        if (d.clr_pos[u] == p) d.clr_nodes[atomicAdd(&s_nclr, 1)] = u;  // once per row
+      }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      ctl->n_del = s_ndel;
+      ctl->n_clr = s_nclr;
+      ctl->n += adds;
+    }
+    return;
   }
   // the same edits by (v, u): they come by u, so a stable sort by v is enough
 #pragma unroll
@@ -830,7 +855,7 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp
     }
   }
   __syncthreads();
-  radix_sort(key, per, bits + 1, 2 * bits + 1, skey, s_a);
+  radix_sort(key, per, bits + 1, 2 * bits + 1, skey, s_cnt);
 #pragma unroll
   for (int r = 0; r < kSortRows; ++r) {
     if (r < per) skey[(w * per + r) * 32 + lane] = key[r];
@@ -838,28 +863,10 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest_emit(Dev d, const osp
   }
   __syncthreads();
   emit_edits(
-      key, kind, per, skey, d.gd, s_b, [&](unsigned long long k) { return (int)(k >> (bits + 1)); },
+      key, kind, per, skey, [&](unsigned long long k) { return (int)(k >> (bits + 1)); },
       [&](unsigned long long k) { return (int)((k >> 1) & ((1ull << bits) - 1)); }, d.ins_c, d.del_c,
       d.rec_c_node, d.rec_c_is, d.rec_c_ic, d.rec_c_ds, d.rec_c_dc, d.cflag, &ctl->n_rec_c, &n_ins,
       &n_del);
-  // node deletions and zeroed rows
-  for (int p = tid; p < U; p += kIngestThreads) {
-    const int op = ops[p].op;
-    if (op == OSP_OP_DELETE_NODE) {
-      const int u = load_op(ops, p, d).u;
-      d.del_nodes[atomicAdd(&s_ndel, 1)] = u;
-      d.del_pos[u] = kNoPos;
-    } else if (op == OSP_OP_ZERO_ROW) {
-      const int u = load_op(ops, p, d).u;
-      if (d.clr_pos[u] == p) d.clr_nodes[atomicAdd(&s_nclr, 1)] = u;  // once per row
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    ctl->n_del = s_ndel;
-    ctl->n_clr = s_nclr;
-    ctl->n += adds;
-  }
 }
 
 // Node deletions: the deleted node's own row and column are cleared, and every
