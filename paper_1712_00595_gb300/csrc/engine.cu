@@ -19,7 +19,6 @@ using namespace osp;
 
 namespace {
 
-constexpr int kIngestSmem = kMaxBatch * 8;
 // shared memory of the batch sorts: keys of whole rows of 1024, digit counts by warp
 constexpr size_t ingest_sort_smem(int U) {
   return (size_t)((U + 1023) / 1024) * 1024 * 8 + 32 * 256 * sizeof(int);
@@ -1016,8 +1015,6 @@ osp_status osp_create(osp_ctx** out, const osp_options* opt) {
   }
   if (e == cudaSuccess) e = cudaMallocHost(&ctx->pinned, kPinnedBytes);
   for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaEventCreate(&ctx->ev[i]);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_ingest, cudaFuncAttributeMaxDynamicSharedMemorySize, kIngestSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_ingest_emit, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)ingest_sort_smem(kMaxBatch));
