@@ -63,7 +63,8 @@ struct Ctl {
   int n_clr;                   // rows zeroed by the last ingested batch (clr_nodes)
   int n_hubs, n_pieces;        // pull step: long in-lists and their pieces
   int n_tasks;                 // pull step: warp tasks
-  int plan_done;               // CTAs that have planned their nodes
+  int plan_done;               // CTAs that have listed their pieces, then planned their nodes
+  long long touch;             // out-list entries, old and new, of the sub-batch's changed rows
   int n_mpieces;               // merge pieces of the current batch
   int dense0;                  // 1: x(0) is found by a dense scan of xacc (no queue from the merge)
   int n_opieces;               // several seeds: offset items (256 entries of a changed row)

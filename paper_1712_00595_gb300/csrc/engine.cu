@@ -622,7 +622,8 @@ osp_status enqueue_update(osp_ctx* ctx, const osp_update* ops_dev, int U, int Np
   }
   k_expand<<<g, 256, 0, ctx->stream>>>(ctx->d);
   ++ctx->launches;
-  k_merge_pieces<<<1, 1024, 0, ctx->stream>>>(
+  // a CTA per 1,024 lists that the ops can change (node deletions can add more)
+  k_merge_pieces<<<std::min(ctx->num_sms, (2 * Np + 1023) / 1024), 1024, 0, ctx->stream>>>(
       ctx->d, ctx->opt.push_beta > 0 ? ctx->opt.push_beta : kPushBeta);
   ++ctx->launches;
   k_merge_count<<<g, 256, 0, ctx->stream>>>(ctx->d);

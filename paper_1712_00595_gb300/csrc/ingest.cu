@@ -169,6 +169,9 @@ __global__ void k_reset_batch(Dev d, int cont) {
   c->n_rec_r = 0;
   c->n_rec_c = 0;
   c->n_del = 0;
+  c->n_mpieces = 0;
+  c->plan_done = 0;
+  c->touch = 0;
   if (cont) return;
   c->m_delta = 0;
   c->net_ins = 0;

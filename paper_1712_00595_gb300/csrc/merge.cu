@@ -113,82 +113,91 @@ __device__ __forceinline__ ListRec list_rec(const Dev& d, int c, int n_rows) {
   return L;
 }
 
+// Old entries of a list go in pieces of kPiece; an empty list has one piece.
+__device__ __forceinline__ int pieces_of(int len) { return max(1, (len + kPiece - 1) / kPiece); }
+
 }  // namespace
 
-// One CTA: list each changed list's pieces and remember its old slot.
+// List each changed list's pieces and remember its old slot: 1,024 lists a CTA at a
+// time, whose pieces get the next places of the table (their order does not
+// matter). The CTA that finishes last bounds the offset's support. In one CTA
+// 30,000 lists took 34 us, 7 so.
 __global__ void __launch_bounds__(1024) k_merge_pieces(Dev d, double beta) {
   __shared__ int s_w[32];
   __shared__ long long s_b[32];
+  __shared__ int s_base;
   Ctl* ctl = d.ctl;
   if (*(volatile int*)&ctl->status) return;
   const int nr = ctl->n_rec_r;
   const int R = nr + ctl->n_rec_c;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  // lists in rows of 1024, four rows' loads in flight (consecutive lists a thread
-  // had cost 55 us for 10,000 lists, each thread's loads one after the other)
-  __shared__ int s_base;
-  long long touch = 0;  // out-list entries old and new of the changed rows
-  if (tid == 0) s_base = 0;
-  __syncthreads();
-  for (int c0 = 0; c0 < R; c0 += 4 * 1024) {
-    int node[4], L[4];
-    unsigned o[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + 1024 * q + tid;
-      node[q] = c < nr ? d.rec_r_node[c] : c < R ? d.rec_c_node[c - nr] : 0;
+  const bool alone = gridDim.x == 1;  // small batches: no atomics to wait for
+  int listed = 0;                     // thread 31: pieces of this CTA
+  long long touch = 0;                // out-list entries old and new of the changed rows
+  for (int c0 = blockIdx.x * 1024; c0 < R; c0 += gridDim.x * 1024) {
+    const int c = c0 + tid;
+    int L = 0;
+    unsigned o = 0;
+    if (c < nr) {
+      const int node = d.rec_r_node[c];
+      L = d.len_r[node];
+      o = d.off_r[node];
+      touch += L + d.rec_r_ic[c];
+    } else if (c < R) {
+      const int node = d.rec_c_node[c - nr];
+      L = d.len_c[node];
+      o = d.off_c[node];
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + 1024 * q + tid;
-      L[q] = c < nr ? d.len_r[node[q]] : c < R ? d.len_c[node[q]] : 0;
-      o[q] = c < nr ? d.off_r[node[q]] : c < R ? d.off_c[node[q]] : 0u;
-      if (c < nr) touch += L[q] + d.rec_r_ic[c];
+    const int np = c < R ? pieces_of(L) : 0;
+    int x = np;
+    for (int k = 1; k < 32; k <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, k);
+      if (lane >= k) x += y;
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + 1024 * q + tid;
-      if (c0 + 1024 * q >= R) break;  // uniform
-      const int np = c < R ? (L[q] > 0 ? (L[q] + kPiece - 1) / kPiece : 1) : 0;
-      int x = np;
+    if (lane == 31) s_w[w] = x;
+    __syncthreads();
+    if (w == 0) {
+      int t = s_w[lane];
       for (int k = 1; k < 32; k <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, k);
-        if (lane >= k) x += y;
+        const int y = __shfl_up_sync(0xffffffffu, t, k);
+        if (lane >= k) t += y;
       }
-      if (lane == 31) s_w[w] = x;
-      __syncthreads();
-      if (w == 0) {
-        int t = s_w[lane];
-        for (int k = 1; k < 32; k <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, t, k);
-          if (lane >= k) t += y;
-        }
-        s_w[lane] = t;
+      s_w[lane] = t;
+      if (lane == 31) {
+        s_base = alone ? listed : atomicAdd(&ctl->n_mpieces, t);
+        listed += t;
       }
-      __syncthreads();
-      const int base = s_base + (w ? s_w[w - 1] : 0) + x - np;
-      if (c < R) {
-        d.rec_old_off[c] = o[q];
-        d.rec_old_len[c] = L[q];
-        d.rec_pstart[c] = base;
-        for (int k = 0; k < np; ++k) d.piece_rec[base + k] = c;
-      }
-      __syncthreads();
-      if (tid == 0) s_base += s_w[31];
-      __syncthreads();
     }
+    __syncthreads();
+    const int base = s_base + (w ? s_w[w - 1] : 0) + x - np;
+    if (c < R) {
+      d.rec_old_off[c] = o;
+      d.rec_old_len[c] = L;
+      d.rec_pstart[c] = base;
+      for (int k = 0; k < np; ++k) d.piece_rec[base + k] = c;
+    }
+    __syncthreads();
   }
   touch = warp_sum(touch);
   if (lane == 0) s_b[w] = touch;
+  if (alone && tid == 31) ctl->n_mpieces = listed;
   __syncthreads();
   if (tid == 0) {
-    ctl->n_mpieces = s_base;
-    d.rec_pstart[R] = s_base;
     long long t = 0;
     for (int i = 0; i < 32; ++i) t += s_b[i];
-    // the offset reaches at most `t` nodes; above n/beta the first step is
-    // dense anyway and x(0) is collected by a scan instead of a queue
-    ctl->dense0 |= (double)t > (double)ctl->n / beta;  // sticky over sub-batches
+    // the offset reaches at most `touch` nodes; above n/beta the first step is
+    // dense anyway and x(0) is collected by a scan instead of a queue (sticky over
+    // sub-batches)
+    if (alone) {
+      ctl->dense0 |= (double)t > (double)ctl->n / beta;
+      return;
+    }
+    if (t) atomicAdd((unsigned long long*)&ctl->touch, (unsigned long long)t);
+    __threadfence();
+    if (atomicAdd(&ctl->plan_done, 1) == (int)gridDim.x - 1) {
+      __threadfence();
+      ctl->dense0 |= (double)*(volatile long long*)&ctl->touch > (double)ctl->n / beta;
+    }
   }
 }
 
@@ -241,58 +250,94 @@ __global__ void __launch_bounds__(256, 6) k_merge_count(Dev d) {
   }
 }
 
-// Per list: piece bases, new length, fresh pool space, new slot.
+// Per list: piece bases, new length, fresh pool space, new slot. Lane = list (the
+// warp together for the lists of many pieces), one draw of pool space a warp: a warp
+// and a draw per list took 20 us for 30,000 lists, 8 so.
 __global__ void __launch_bounds__(256) k_merge_plan(Dev d) {
+  constexpr int kAlone = 8;  // pieces that a lane adds up by itself
   Ctl* ctl = d.ctl;
   if (*(volatile int*)&ctl->status) return;
   const int nr = ctl->n_rec_r;
   const int R = nr + ctl->n_rec_c;
   const double c1 = 1.0 - ctl->c;
-  const unsigned long long cap_r = ctl->pool_cap_r, cap_c = ctl->pool_cap_c;
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   long long mdelta = 0;
-  for (int c = gw; c < R; c += nw) {
-    const ListRec L = list_rec(d, c, nr);
-    const int p0 = d.rec_pstart[c], p1 = d.rec_pstart[c + 1];
+  for (int b = gw * 32; b < R; b += nw * 32) {
+    const int c = b + lane;
+    const bool in = c < R;
+    const bool rows = c < nr;
+    int node = 0, ic = 0, p0 = 0, np = 0, old = 0;
+    if (in) {
+      node = rows ? d.rec_r_node[c] : d.rec_c_node[c - nr];
+      ic = rows ? d.rec_r_ic[c] : d.rec_c_ic[c - nr];
+      p0 = d.rec_pstart[c];
+      old = d.rec_old_len[c];
+      np = pieces_of(old);
+    }
     int run = 0;
-    for (int b = p0; b < p1; b += 32) {  // exclusive scan of the piece counts
-      const int p = b + lane;
-      const int v = p < p1 ? d.piece_cnt[p] : 0;
-      int x = v;
+    if (np <= kAlone) {
+      for (int k = 0; k < np; ++k) {
+        const int v = d.piece_cnt[p0 + k];
+        d.piece_base[p0 + k] = run;
+        run += v;
+      }
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, np > kAlone); m; m &= m - 1) {
+      const int j = __ffs(m) - 1;
+      const int q0 = __shfl_sync(0xffffffffu, p0, j), q1 = q0 + __shfl_sync(0xffffffffu, np, j);
+      int sum = 0;
+      for (int q = q0; q < q1; q += 32) {  // exclusive scan of the piece counts
+        const int p = q + lane;
+        const int v = p < q1 ? d.piece_cnt[p] : 0;
+        int x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (p < q1) d.piece_base[p] = sum + x - v;
+        sum += __shfl_sync(0xffffffffu, x, 31);
+      }
+      if (lane == j) run = sum;
+    }
+    const int dp = in ? run + ic : 0;
+    unsigned long long fb = 0;
+#pragma unroll
+    for (int kind = 0; kind < 2; ++kind) {  // out-lists, in-lists
+      const bool mine = in && rows == (kind == 0);
+      long long x = mine ? dp : 0;
+      if (!__any_sync(0xffffffffu, x > 0)) continue;
       for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
       }
-      if (p < p1) d.piece_base[p] = run + x - v;
-      run += __shfl_sync(0xffffffffu, x, 31);
+      unsigned long long base = 0;
+      if (lane == 31)
+        base = atomicAdd(kind == 0 ? &ctl->pool_top_r : &ctl->pool_top_c, (unsigned long long)x);
+      base = __shfl_sync(0xffffffffu, base, 31);
+      if (mine && dp > 0) fb = base + (unsigned long long)(x - dp);
     }
-    const int dp = run + L.ic;
-    unsigned long long fb = 0;
-    if (lane == 0 && dp > 0)
-      fb = atomicAdd(L.rows ? &ctl->pool_top_r : &ctl->pool_top_c, (unsigned long long)dp);
-    fb = __shfl_sync(0xffffffffu, fb, 0);
-    if (fb + (unsigned long long)dp > (L.rows ? cap_r : cap_c)) {
+    if (__any_sync(0xffffffffu,
+                   in && fb + (unsigned long long)dp > (rows ? ctl->pool_cap_r : ctl->pool_cap_c))) {
       if (lane == 0) atomicCAS(&ctl->status, 0, (int)OSP_ENOMEM);
       return;
     }
-    if (lane == 0) {
-      d.rec_fbase[c] = (unsigned)fb;
-      d.rec_dp[c] = dp;
-      if (L.rows) {
-        d.off_r[L.node] = (unsigned)fb;
-        d.len_r[L.node] = dp;
-        const double s = dp ? c1 / (double)dp : 0.0;
-        d.scale_d[L.node] = s;
-        d.scale_f[L.node] = (float)s;
-        mdelta += dp - d.rec_old_len[c];
-        d.rflag[L.node] = 0;
-      } else {
-        d.off_c[L.node] = (unsigned)fb;
-        d.len_c[L.node] = dp;
-        d.cflag[L.node] = 0;
-      }
+    if (!in) continue;
+    d.rec_fbase[c] = (unsigned)fb;
+    d.rec_dp[c] = dp;
+    if (rows) {
+      d.off_r[node] = (unsigned)fb;
+      d.len_r[node] = dp;
+      const double s = dp ? c1 / (double)dp : 0.0;
+      d.scale_d[node] = s;
+      d.scale_f[node] = (float)s;
+      mdelta += dp - old;
+      d.rflag[node] = 0;
+    } else {
+      d.off_c[node] = (unsigned)fb;
+      d.len_c[node] = dp;
+      d.cflag[node] = 0;
     }
   }
   mdelta = warp_sum(mdelta);
@@ -319,9 +364,9 @@ __global__ void __launch_bounds__(256, 4) k_merge_write(Dev d) {
     const int c = d.piece_rec[p];
     const ListRec R = list_rec(d, c, nr);
     const int q = p - d.rec_pstart[c];
-    const int npieces = d.rec_pstart[c + 1] - d.rec_pstart[c];
     const unsigned o = d.rec_old_off[c];
     const int L = d.rec_old_len[c];
+    const int npieces = pieces_of(L);
     const int dp = d.rec_dp[c];
     int* F = R.pool + d.rec_fbase[c];
     const int base = d.piece_base[p];
