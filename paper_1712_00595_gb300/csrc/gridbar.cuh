@@ -1,7 +1,8 @@
-// Grid-wide barrier of the persistent cooperative kernels: the last CTA to
+// Grid-wide barrier of the persistent cooperative kernels. Seed block: the last CTA to
 // arrive runs the step decision, then opens the barrier; the others wait with
 // a bounded spin (time and iteration limits) and stop on a timeout or an
-// error status, so a lost CTA cannot hang the device.
+// error status, so a lost CTA cannot hang the device. One seed: arrivals are counted
+// up and every CTA waits for the count (grid_wait).
 #pragma once
 #include "common.cuh"
 

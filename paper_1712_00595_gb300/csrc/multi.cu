@@ -13,7 +13,9 @@
 //            the first gather block y(0) = x(0) (1-c) / d; other rows of y(0)
 //            are written as zero.
 //   steps    pull only: x(i)[v] = sum over the in-list of v of y(i-1)[u],
-//            a warp per node, lanes over columns; long in-lists in pieces.
+//            rows through per-warp rings in shared memory (k_propagate_ring) or
+//            a warp per node, lanes over columns (k_propagate_multi); long
+//            in-lists in pieces.
 //   stop     per column (Algorithm 1 loop test, do-while form): a column whose
 //            ||x(i)||_1 <= eps stops adding and propagating; the call ends
 //            when no column is left or at the iteration cap.
