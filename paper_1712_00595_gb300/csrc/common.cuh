@@ -172,7 +172,10 @@ struct Dev {
   int* hubs; int* hub_pstart; double* hub_acc; int* hub_cnt;  // [pool cap / kHubThreshold + 2]
   int* piece_hub;  // [2 pool cap / kMultiHub + 4] the long in-list each piece belongs to
   double* piece_part;  // [as piece_hub] deterministic mode: per-piece partial sums
-  double* hub_l1;      // [as hubs] deterministic mode: |x_v| of each long in-list's node
+  // deterministic mode: |x_v| of each long in-list's node, by step parity (a CTA
+  // that leaves the step barrier first finishes lists of the next step while others
+  // still sum this one's). The second half lies in hub_acc, which that mode leaves idle.
+  double* hub_l1[2];   // [as hubs]
   // push step: pieces of the rows longer than kPushPiece [2 pool cap / kPushPiece + 2],
   // in piece_rec, piece_cnt and piece_part
   unsigned* big_off; int* big_len; double* big_y;

@@ -1207,8 +1207,9 @@ osp_status osp_load_graph(osp_ctx* ctx, int64_t n, int64_t m, const int32_t* src
     // pieces: at most m / piece + (lists) <= 2 cap / kMultiHub, pieces never shorter than kMultiHub
     AL(d.piece_hub, 2 * nh + 4, 0);
     AL(d.piece_part, 2 * nh + 4, 0);
-    AL(d.hub_l1, nh, 0);
+    AL(d.hub_l1[0], nh, 0);
     AL(d.hub_acc, nh, 0);
+    d.hub_l1[1] = d.hub_acc;
     AL(d.hub_cnt, nh, 0);
     // push: a row above kPushPiece entries has at most 2 len / kPushPiece pieces, and
     // the arrays of the merge's pieces and of the pull-only deterministic sums are

@@ -121,7 +121,8 @@ __device__ bool step_barrier(const Dev& d, const PropParams& pp, int step_mode, 
     __syncthreads();
     double a = 0.0;
     const int nh = ctl->n_hubs;
-    for (int i = threadIdx.x; i < nh; i += blockDim.x) a += __ldcg(d.hub_l1 + i);
+    const double* hub_l1 = d.hub_l1[it & 1];  // by parity like the partials
+    for (int i = threadIdx.x; i < nh; i += blockDim.x) a += __ldcg(hub_l1 + i);
     a = warp_sum(a);
     if (lane == 0 && w > 0) s_l1[w] = a;
     __syncthreads();
@@ -505,7 +506,7 @@ __device__ __forceinline__ double stream_lists(const int* __restrict__ pool, con
 template <typename T>
 __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_pieces,
                             int n_tasks, WarpStream<T>& W, int* grab, int hub_thr, int hub_piece,
-                            bool det) {
+                            bool det, double* hub_l1) {
   constexpr bool kF32 = std::is_same<T, float>::value;
   double l1 = 0.0;
   const int lane = threadIdx.x & 31;
@@ -564,7 +565,7 @@ __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_
             d.hub_cnt[h] = 0;
             double hl = 0.0;
             finish_node(d, v, x, yd, kF32, hl);
-            d.hub_l1[h] = hl;
+            hub_l1[h] = hl;
           }
         } else {
           atomicAdd(&d.hub_acc[h], (double)acc);
@@ -819,7 +820,7 @@ __global__ void __launch_bounds__(kOneThreads, 1) k_propagate(Dev d, PropParams 
       l1 = pull_step<T>(d, yb[src], yb[dst], n_hubs, n_pieces, n_tasks,
                         reinterpret_cast<WarpStream<T>*>(dsm)[threadIdx.x >> 5],
                         &ctl->ctr[it & 3], hub_thr, hub_piece,
-                        pp.det != 0);
+                        pp.det != 0, d.hub_l1[it & 1]);
     }
     target += gridDim.x;
     if (!step_barrier(d, pp, mode, n, m, l1, ef, target, cs, s_red, s_l1, s_ef)) return;

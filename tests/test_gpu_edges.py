@@ -293,3 +293,43 @@ def test_topk_of_a_vector_at_any_element(start, n):
         want = np.lexsort((np.arange(n), ~key))[:c]
         assert np.array_equal(ids[:c].cpu().numpy(), want)
         assert np.array_equal(sc[:c].cpu().numpy(), v[want])
+
+
+@pytest.mark.parametrize("prec", [F64, F32])
+def test_deterministic_norms_with_many_lists_in_pieces(prec):
+    """Deterministic mode with 60 in-lists of two to nine pieces, whose |x| joins a
+    step's norm apart from the CTAs' sums and is written again in the next step: the
+    norm of every step agrees with the oracle's, and two contexts agree bit for bit.
+
+    Relative bound of a step's norm, as in the parity tests: an entry rounds the stored
+    value, the scale and the product once each, per-lane chains of at most 1,024 / 32
+    terms, five warp levels and nine pieces (at most 50 u, u = 2^-24 or 2^-53); the
+    oracle adds its in-edges in turn; the two norm sums add 2 n 2^-53."""
+    rng = np.random.default_rng(17)
+    n = 10_000
+    src, dst = [rng.integers(0, n, 8 * n)], [rng.integers(0, n, 8 * n)]
+    for v in range(60):
+        src.append(rng.choice(n, int(rng.integers(1025, 9000)), replace=False))
+        dst.append(np.full(src[-1].size, 3 * v))
+    src, dst = np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+    ops = W.edge_update_stream(src, dst, n, 1, 300, 300, seed=4)[0]
+    runs = []
+    for _ in range(2):
+        eng = N.Engine(precision=prec, device=0, deterministic=True)
+        eng.load_graph(n, src, dst)
+        eng.set_seeds([1], C_RESTART)
+        eng.init_scores(1e-11)
+        runs.append([eng.get_l1_history(), eng.query()])
+        eng.apply_updates(ops, 1e-11)
+        runs[-1] += [eng.get_l1_history(), eng.query()]
+        eng.close()
+    for a, b in zip(*runs):
+        assert a.shape == b.shape and np.array_equal(a.view(np.uint64), b.view(np.uint64))
+    hist = runs[0][0]
+    rp, col = O.Graph(n, src, dst).csr()
+    want = O.cpi(rp, col, 1, C_RESTART, 1e-11, force_iters=hist.size - 1)[2]
+    u = 2.0 ** -53 if prec == F64 else 2.0 ** -24
+    d_in = int(np.bincount(col, minlength=n).max())
+    delta = 50 * u + (d_in + 2) * 2.0 ** -53
+    rtol = (1.0 + delta) ** np.arange(hist.size) - 1.0 + 2 * n * 2.0 ** -53
+    assert np.all(np.abs(hist - want) <= rtol * want)
