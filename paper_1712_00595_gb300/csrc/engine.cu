@@ -768,6 +768,10 @@ osp_status apply_large(osp_ctx* ctx, const osp_update* ops, bool host, int64_t U
     osp_status s = reserve_for_batch(ctx, u);
     if (s != OSP_OK) {
       err = s;
+      if (ci == 0) {  // no sub-batch has reset the counters and the barrier of the propagation below
+        k_reset_batch<<<1, 256, 0, ctx->stream>>>(ctx->d, 0);
+        ++ctx->launches;
+      }
       break;
     }
     const osp_update* p = ops + s0;

@@ -333,3 +333,45 @@ def test_deterministic_norms_with_many_lists_in_pieces(prec):
     delta = 50 * u + (d_in + 2) * 2.0 ** -53
     rtol = (1.0 + delta) ** np.arange(hist.size) - 1.0 + 2 * n * 2.0 ** -53
     assert np.all(np.abs(hist - want) <= rtol * want)
+
+
+@pytest.mark.parametrize("S", [1, 3])
+def test_large_batch_without_node_room_changes_nothing(S):
+    """A batch of several sub-batches whose first one finds no node slots left is
+    refused with OSP_ENOMEM: scores, graph and residual bound stay, bit for bit, the
+    call's steps are those of a zero offset, and later batches go on from there."""
+    n = 200
+    src, dst = W.er_graph(n, 1500, 5)
+    eng = N.Engine(precision=N.OSP_PREC_FP64, device=0, max_nodes=n)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.arange(S, dtype=np.int32), C_RESTART)
+    eng.init_scores(1e-10)
+    grow = np.zeros(300, W.UPDATE_DTYPE)  # room is left for a batch of 16,084 ops only
+    grow["op"] = W.OP_ADD_NODE
+    eng.apply_updates(grow, 1e-9)
+    eng.apply_updates(W.edge_update_stream(src, dst, n, 1, 40, 40, seed=2)[0], 1e-9)
+    rng = np.random.default_rng(4)
+    big = np.zeros(20_000, W.UPDATE_DTYPE)
+    big["u"], big["v"] = rng.integers(0, n, (2, big.size))
+    before = [eng.query(j) for j in range(S)], eng.export_graph(0), eng.get_residual_bounds()
+    for _ in range(20):
+        st = eng.apply_updates(big, 1e-9, allow=(N.OSP_ENOMEM,))
+        assert eng.last_status == N.OSP_ENOMEM
+        assert st["iterations"] == 1 and st["qoff_l1"] == 0.0 and st["last_x_l1"] == 0.0
+        assert np.array_equal(eng.get_l1_history(), [0.0, 0.0])
+        assert np.array_equal(eng.get_residual_bounds(), before[2])
+        for j in range(S):
+            assert np.array_equal(eng.query(j), before[0][j])
+        assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(0), before[1]))
+    g = O.Graph(n, src, dst)
+    g.apply(grow)
+    g.apply(W.edge_update_stream(src, dst, n, 1, 40, 40, seed=2)[0])
+    old = g.csr()
+    ops = big[:3000]
+    st = eng.apply_updates(ops, 1e-9)
+    assert g.apply(ops) == -1
+    it = eng.get_seed_stats()[0] if S > 1 else [st["iterations"]]
+    for j in range(S):
+        r = O.osp(old, g.csr(), before[0][j], C_RESTART, 1e-9, force_iters=int(it[j]))[0]
+        assert np.abs(eng.query(j) - r).sum() <= 1e-10
+    eng.close()
