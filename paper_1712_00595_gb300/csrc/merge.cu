@@ -409,9 +409,10 @@ __global__ void __launch_bounds__(256, 4) k_merge_write(Dev d) {
       const int a0 = q * kPiece;
       const int a1 = min(L, a0 + kPiece);
       const int jlo = q == 0 ? 0 : lower_bound_i(I, ic, A[a0 - 1] + 1);
-      // piece q takes the insertions whose place among the old entries is in [a0, a1)
-      // (the last piece also those above every old entry)
-      const int jhi = q == npieces - 1 ? ic : lower_bound_i(I, ic, A[a1 - 1]);
+      // piece q takes the insertions above the old entry before it, up to its own last
+      // one (the last piece also those above every old entry): an insertion can equal
+      // an old entry of a row that was zeroed before it
+      const int jhi = q == npieces - 1 ? ic : lower_bound_i(I, ic, A[a1 - 1] + 1);
       for (int jb = jlo; jb < jhi; jb += 32) {
         const int j = jb + lane;
         const bool in = j < jhi;

@@ -375,3 +375,49 @@ def test_large_batch_without_node_room_changes_nothing(S):
         r = O.osp(old, g.csr(), before[0][j], C_RESTART, 1e-9, force_iters=int(it[j]))[0]
         assert np.abs(eng.query(j) - r).sum() <= 1e-10
     eng.close()
+
+
+@pytest.mark.parametrize("fill", [0, 600])
+@pytest.mark.parametrize("S", [1, 3])
+def test_zeroed_rows_get_back_the_entries_at_the_edges_of_the_merge_pieces(S, fill):
+    """A row zeroed and given back old entries in one batch, the entries around the
+    256-entry pieces of the old list among them: in its own out-list (node 5) and as
+    an entry of long in-lists (node 7's). Graph equal to the oracle's, scores L1 <=
+    1e-10. fill: other ops, for the ingest over many CTAs."""
+    rng = np.random.default_rng(fill)
+    n = 1500
+    src = [np.full(1100, 5), np.arange(8, 908), rng.integers(8, n, 6000)]
+    dst = [np.arange(20, 1120), np.full(900, 7), rng.integers(8, n, 6000)]
+    e = np.unique(np.stack([np.concatenate(src), np.concatenate(dst)], 1), axis=0).astype(np.int32)
+    src, dst = np.ascontiguousarray(e[:, 0]), np.ascontiguousarray(e[:, 1])
+    eng = N.Engine(precision=N.OSP_PREC_FP64, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.array([5, 0, 300][:S], np.int32), C_RESTART)
+    eng.init_scores(1e-12)
+    g = O.Graph(n, src, dst)
+    old = g.csr()
+    r = [O.cpi(*old, s, C_RESTART, 1e-12)[0] for s in [5, 0, 300][:S]]
+    for turn in range(3):
+        out5 = old[1][old[0][5]:old[0][6]]
+        in7 = np.flatnonzero([7 in old[1][old[0][u]:old[0][u + 1]] for u in range(n)])
+        back5 = out5[[i for i in (0, 254, 255, 256, 511, 512, 767, 1023) if i < out5.size]]
+        ops = [(5, 0, 4)] + [(5, int(v), 0) for v in back5]
+        for i in (254, 255, 256, 511, 512, 767):
+            if i < in7.size and in7[i] != 5:
+                ops += [(int(in7[i]), 0, 4), (int(in7[i]), 7, 0)]
+        # node 5 gets a long row again for the next turn
+        more = [(5, int(v), 0) for v in rng.choice(np.arange(20, n), 700, replace=False)]
+        more += [(int(u), int(v), 0) for u, v in rng.integers(8, n, (fill, 2))]
+        for batch in (ops, more) if turn % 2 else (ops + more[700:], more):
+            batch = np.array(batch, W.UPDATE_DTYPE)
+            st = eng.apply_updates(batch, 1e-12)
+            assert g.apply(batch) == -1
+            new = g.csr()
+            assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(0), new))
+            assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(1), g.csc()))
+            it = eng.get_seed_stats()[0] if S > 1 else [st["iterations"]]
+            for j in range(S):
+                r[j] = O.osp(old, new, r[j], C_RESTART, 1e-12, force_iters=int(it[j]))[0]
+                assert np.abs(eng.query(j) - r[j]).sum() <= 1e-10
+            old = new
+    eng.close()
