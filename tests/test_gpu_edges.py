@@ -421,3 +421,26 @@ def test_zeroed_rows_get_back_the_entries_at_the_edges_of_the_merge_pieces(S, fi
                 assert np.abs(eng.query(j) - r[j]).sum() <= 1e-10
             old = new
     eng.close()
+
+
+@pytest.mark.parametrize("prec,S,kw", [
+    (F64, 17, {}), (F64, 100, dict(seed_group=128)), (F32, 100, {}), (F32, 40, dict(seed_gather=1)),
+    (F32, 40, dict(seed_gather=2)), (BF16, 100, {}), (BF16, 40, dict(seed_gather=2))])
+def test_block_norms_of_a_call_are_the_largest_of_its_seeds(prec, S, kw):
+    """qoff_l1, last_x_l1 and the step history of a seed block are the maxima of the
+    per-seed norms (all below 1), to the bit."""
+    n = 1500
+    src, dst = W.er_graph(n, 12_000, 6)
+    eng = N.Engine(precision=prec, device=0, **kw)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.random.default_rng(1).permutation(n)[:S].astype(np.int32), C_RESTART)
+    sts = [eng.init_scores(1e-6)]
+    for ops in [None] + W.edge_update_stream(src, dst, n, 2, 60, 60, seed=3):
+        if ops is not None:
+            sts.append(eng.apply_updates(ops, 1e-6))
+        it, q, last = eng.get_seed_stats()
+        hist = eng.get_l1_history()
+        assert hist.size == sts[-1]["iterations"] + 1 and np.all(hist > 0) and np.all(hist < 1)
+        assert hist[0] == sts[-1]["qoff_l1"] == q.max()
+        assert hist[-1] == sts[-1]["last_x_l1"] == last[it == it.max()].max()
+    eng.close()
