@@ -991,8 +991,8 @@ __device__ void decide_multi(const Dev& d, const PropParams& pp, int it, long lo
       if (stop) {
         M.active[j] = 0;
         // the untaken tail's residual x(k+1) has norm <= (1-c) ||x(k)||_1; L may
-        // hold float sums of at most 32 nonnegative terms (relative error below
-        // 2^-19), hence the margin
+        // hold float sums of at most 32 nonnegative terms (bf16 rows; relative error
+        // below 2^-19), hence the margin
         M.res_bound[j] += (1.0 - ctl->c) * L * (1.0 + 0x1p-18);
       } else {
         live = 1;
@@ -2159,11 +2159,12 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
           const bool mine = vb + lane < c1t && my_len <= hub_thr;  // hubs go by pieces
           const unsigned fin = __ballot_sync(0xffffffffu, mine && (my_len > 0 || my_s != (A)0));
           if (!fin) continue;
-          // |x| of the run summed in the rows' accumulation type (at most 32
-          // nonnegative terms), then added to the FP64 partial once
-          A l1f[KG];
+          // |x| of the run, added to the FP64 partial once: in double, for bf16 rows in
+          // float (at most 32 nonnegative terms)
+          using L = std::conditional_t<kMma, float, double>;
+          L l1f[KG];
 #pragma unroll
-          for (int k = 0; k < KG; ++k) l1f[k] = (A)0;
+          for (int k = 0; k < KG; ++k) l1f[k] = (L)0;
           if constexpr (kMma) {
             mma_stream<KG>(
                 d.pool_c, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
@@ -2247,8 +2248,9 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
 #pragma unroll
               for (int k = 0; k < KG; ++k)
                 if (((amk >> k) & 1u) && acc[k] != (A)0) {
-                  red_add_once(rp + col[k], widen(acc[k]), pol.once);
-                  l1f[k] += fabs(acc[k]);
+                  const double x = widen(acc[k]);
+                  red_add_once(rp + col[k], x, pol.once);
+                  l1f[k] += fabs(x);
                 }
               if (sj != (A)0) {
                 alignas(16) TY yv[KG];
@@ -2265,7 +2267,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             if (cur != 127u) done(cur);
 #pragma unroll
             for (int k = 0; k < KG; ++k)
-              if (l1f[k] != (A)0) atomicAdd(my_part + col[k], (double)l1f[k]);
+              if (l1f[k] != 0.0) atomicAdd(my_part + col[k], l1f[k]);
           }
         }
       }

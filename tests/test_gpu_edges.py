@@ -444,3 +444,26 @@ def test_block_norms_of_a_call_are_the_largest_of_its_seeds(prec, S, kw):
         assert hist[0] == sts[-1]["qoff_l1"] == q.max()
         assert hist[-1] == sts[-1]["last_x_l1"] == last[it == it.max()].max()
     eng.close()
+
+
+@pytest.mark.parametrize("S,group,gather", [(20, 0, 0), (64, 0, 0), (100, 0, 0), (200, 256, 0), (40, 0, 2)])
+def test_norms_of_float_blocks_are_sums_in_double(S, group, gather):
+    """FP32 seed blocks: ||x(k)||_1 against the double sum of |x(k)|, taken as the
+    difference of the scores after k and after k - 1 steps (no list is long enough to
+    be cut, so both runs add the same floats). Bound: the scores round at most
+    2^-53 ||r||_1 = 2^-53 a step, 2 k of them; the sums of n terms 2 n 2^-53 relative."""
+    n, k = 3000, 4
+    src, dst = W.er_graph(n, 30_000, 9)
+    eng = N.Engine(precision=F32, device=0, seed_group=group, seed_gather=gather)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.random.default_rng(S).permutation(n)[:S].astype(np.int32), C_RESTART)
+    r = []
+    for steps in (k - 1, k):
+        eng.set_fixed_iterations(steps)
+        eng.init_scores(1e-9)
+        r.append([eng.query(j) for j in range(S)])
+    _, _, last = eng.get_seed_stats()
+    for j in range(S):
+        want = np.abs(r[1][j] - r[0][j]).sum()
+        assert abs(last[j] - want) <= 2 * k * 2.0 ** -53 + 2 * n * 2.0 ** -53 * want
+    eng.close()
