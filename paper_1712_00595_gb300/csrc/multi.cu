@@ -296,13 +296,13 @@ __device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
          ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
 }
 
-// (double)x for a normal x in four integer operations: the conversion itself
-// runs at the double rate, 16 cycles of the SM per warp. Step values are finite
-// (|x| <= 2); a subnormal one (below 2^-126) comes out below 2^-125.
+// (double)x for a nonzero x, exact up to 2^63 (step values are at most 2): scaled by 2^64,
+// which makes subnormals normal, and put together in four integer operations. The
+// conversion itself runs at the double rate, 16 cycles of the SM per warp.
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) {
-  const int b = __float_as_int(x);
-  return __hiloint2double(((b >> 3) & 0x8FFFFFFF) + 0x38000000, b << 29);
+  const int b = __float_as_int(x * 0x1p64f);
+  return __hiloint2double(((b >> 3) & 0x8FFFFFFF) + 0x34000000, b << 29);
 }
 
 // K-element slice of a staged row (plain loads from shared memory).

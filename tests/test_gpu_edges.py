@@ -467,3 +467,29 @@ def test_norms_of_float_blocks_are_sums_in_double(S, group, gather):
         want = np.abs(r[1][j] - r[0][j]).sum()
         assert abs(last[j] - want) <= 2 * k * 2.0 ** -53 + 2 * n * 2.0 ** -53 * want
     eng.close()
+
+
+@pytest.mark.parametrize("S,kw", [(5, {}), (64, {}), (100, {}), (5, dict(seed_gather=2))])
+def test_float_blocks_keep_subnormal_steps(S, kw):
+    """A chain of 13 nodes, each with 2,000 out-edges: x falls by 0.85 / 2000 a step,
+    past the smallest normal float (2^-126) at the twelfth. Every score is the oracle's
+    within a step's float rounding: 13 x 4 roundings of 2^-24 relative, and 13 x 2 of
+    the subnormal grid's half unit, 2^-150."""
+    levels, fan = 13, 2000
+    n = levels + fan
+    src, dst = [], []
+    for i in range(levels - 1):
+        src += [i] * fan
+        dst += [i + 1] + list(range(levels, n - 1))
+    src, dst = np.array(src, np.int32), np.array(dst, np.int32)
+    seeds = np.concatenate([[0], levels + np.arange(S - 1)]).astype(np.int32)
+    eng = N.Engine(precision=F32, device=0, **kw)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(seeds, C_RESTART)
+    eng.set_fixed_iterations(levels)
+    eng.init_scores(1e-9)
+    want = O.cpi(*O.Graph(n, src, dst).csr(), 0, C_RESTART, 1e-9, force_iters=levels)[0]
+    assert 0 < want[levels - 1] < 2.0 ** -126
+    got = eng.query(0)
+    assert np.all(np.abs(got - want) <= 4 * levels * 2.0 ** -24 * want + levels * 2.0 ** -149)
+    eng.close()
