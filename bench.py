@@ -603,7 +603,7 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
         "config": dict(config, seed_gather=args.seed_gather, autotune=bool(args.autotune),
                        schedule=list(eng.get_schedule()), node_order="descending out-degree",
                        seed_group=group,
-                       column_groups="packed per batch by offset size" if args.seed_gather != "bulk"
+                       column_groups="packed per batch by offset size" if args.seed_gather == "auto"
                        and S > group and group * by <= 512 else "fixed"),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,

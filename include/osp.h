@@ -119,12 +119,12 @@ typedef struct {
                            2/4/8 with several seeds) on the first CPI steps and keeps the
                            fastest for every later call (osp_get_schedule reports it). */
     int32_t seed_gather; /* seed block (two or more seeds), how pull steps read source rows:
+                            1 = each lane loads its columns of up to eight rows into registers;
                             2 = whole rows are copied into a shared-memory ring by bulk
-                            asynchronous copies (cp.async.bulk, mbarrier); 0 or 1 = through rings
-                            of 16-byte asynchronous copies where a group's row has 64 to 512 bytes
+                            asynchronous copies (cp.async.bulk, mbarrier); 0 = through rings of
+                            16-byte asynchronous copies where a group's row has 64 to 512 bytes
                             (bf16 rows are then summed by the tensor cores with 0 and 1), else
-                            each lane loads its columns of up to eight rows into registers. Results
-                            are the same up to rounding order. */
+                            as 1. Results are the same up to rounding order. */
     int32_t seed_group;  /* seed block: columns per column group of the pull steps (32, 64, 128
                             or 256, at most Sp; 0 = 64 for FP64 gather rows and for bf16 rows of a
                             graph below 2^19 nodes, else 128). A pull step walks the graph

@@ -453,7 +453,7 @@ osp_status finish_call(osp_ctx* ctx, int64_t m_before, osp_batch_stats* st) {
   return OSP_OK;
 }
 
-bool seed_ring(const osp_ctx* ctx, int precision, int KG);
+SeedRows seed_rows(const osp_ctx* ctx, int precision, int KG);
 
 // The pull-step schedule in force: {task items, long-list threshold, piece,
 // node weight}; unset entries take the defaults of the seed count.
@@ -469,7 +469,7 @@ const int* schedule(osp_ctx* ctx) {
   static const int ring[4] = {kTaskItems, 512, 512, kMultiNodeItems};
   static const int mma[4] = {kTaskItems, 1024, 1024, 8};
   if (ctx->sched[0] > 0) return ctx->sched;
-  if (ctx->S > 1 && !seed_ring(ctx, ctx->opt.precision, ctx->d.mu.KG)) return multi;
+  if (ctx->S > 1 && seed_rows(ctx, ctx->opt.precision, ctx->d.mu.KG) != SeedRows::kRing) return multi;
   if (ctx->S > 1) return ctx->opt.precision == OSP_PREC_BF16_ACC64 ? mma : ring;
   return single;
 }
@@ -522,6 +522,10 @@ PropParams prop_params(osp_ctx* ctx, double eps) {
   return pp;
 }
 
+int elem_bytes(int precision) {
+  return precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
+}
+
 // Seed block: gather rows of internal ids below hot_n get L2 priority. With
 // the degree node order those are the most-read rows; the budget is
 // osp_options.l2_hot_bytes (default 60% of L2) over the bytes of one group's
@@ -534,21 +538,17 @@ int hot_rows(const osp_ctx* ctx, int precision, int KG) {
     l2 = 0;
   }
   const int64_t budget = ctx->opt.l2_hot_bytes > 0 ? ctx->opt.l2_hot_bytes : (int64_t)l2 * 6 / 10;
-  const int elem = precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
-  const int64_t rows = budget / (32LL * KG * elem);
+  const int64_t rows = budget / (32LL * KG * elem_bytes(precision));
   return (int)std::min<int64_t>(rows, ctx->nc);
 }
 
-int elem_bytes(int precision) {
-  return precision == OSP_PREC_FP64 ? 8 : precision == OSP_PREC_FP32_ACC64 ? 4 : 2;
-}
-
-// How a seed block's pull steps read source rows: by bulk copies if the options
-// ask for them; else through row rings where a group's row fits (64 to 512
-// bytes), and by lane gathers where not.
-bool seed_bulk(const osp_ctx* ctx) { return ctx->opt.seed_gather == 2; }
-bool seed_ring(const osp_ctx* ctx, int precision, int KG) {
-  return !seed_bulk(ctx) && seed_ring_fits(elem_bytes(precision), KG);
+// How a seed block's pull steps read source rows: by bulk copies or by lane gathers
+// if the options ask for them; else through row rings where a group's row fits (64 to
+// 512 bytes), and by lane gathers where not.
+SeedRows seed_rows(const osp_ctx* ctx, int precision, int KG) {
+  if (ctx->opt.seed_gather == 2) return SeedRows::kBulk;
+  return ctx->opt.seed_gather == 0 && seed_ring_fits(elem_bytes(precision), KG) ? SeedRows::kRing
+                                                                                : SeedRows::kLanes;
 }
 
 // The persistent propagation kernel of one call.
@@ -560,14 +560,14 @@ osp_status enqueue_propagate(osp_ctx* ctx, const PropParams& pp, bool init) {
     const int prec = as_init ? (int)OSP_PREC_FP32_ACC64 : ctx->opt.precision;
     const int KG = as_init ? ctx->d.mu.KG_init : ctx->d.mu.KG;
     PropParams p = pp;
-    p.hot_n = hot_rows(ctx, prec, KG);
-    const bool bulk = seed_bulk(ctx);
+    const SeedRows rows = seed_rows(ctx, prec, KG);
+    if (rows != SeedRows::kRing) p.hot_n = hot_rows(ctx, prec, KG);
     Dev d = ctx->d;
-    // row rings: the columns are packed into groups per call, largest offsets first, so that the columns still running
-    // after the first steps share few groups
-    d.mu.pack = seed_ring(ctx, prec, KG);
+    // row rings: the columns are packed into groups per call, largest offsets first, so
+    // that the columns still running after the first steps share few groups
+    d.mu.pack = rows == SeedRows::kRing;
     CK(launch_propagate_multi(d, p, prec, KG, as_init ? ctx->grid_multi_init : ctx->grid_multi,
-                              bulk, ctx->stream));
+                              rows, ctx->stream));
   }
   else
     CK(launch_propagate(ctx->d, pp, ctx->grid_prop, ctx->stream));
@@ -1402,9 +1402,9 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
     const int prec_init =
         ctx->opt.precision == OSP_PREC_FP64 ? OSP_PREC_FP64 : OSP_PREC_FP32_ACC64;
     ctx->grid_multi = propagate_multi_grid(ctx->opt.precision, M.KG, ctx->num_sms,
-                                           seed_bulk(ctx));
+                                           seed_rows(ctx, ctx->opt.precision, M.KG));
     ctx->grid_multi_init = propagate_multi_grid(prec_init, M.KG_init, ctx->num_sms,
-                                                seed_bulk(ctx));
+                                                seed_rows(ctx, prec_init, M.KG_init));
     if (ctx->grid_multi <= 0 || ctx->grid_multi_init <= 0) {
       free_multi(ctx);
       return fail(ctx, OSP_ECUDA, "no resident grid for the seed-block kernel");

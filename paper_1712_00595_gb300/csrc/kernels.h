@@ -58,11 +58,12 @@ __global__ void k_offset_multi_plan(Dev d);
 __global__ void k_multi_cpi_begin(Dev d);
 // Group rows the row-ring kernel is built for (K columns a lane): 64 to 512 bytes.
 constexpr bool seed_ring_fits(int elem, int KG) { return KG <= 4 && 32 * KG * elem <= 512; }
-// bulk: the variant that stages source rows in shared memory by bulk copies;
-// else the row ring where its rows fit, lane gathers into registers where not.
-int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk);
+// How a pull step reads source rows: through row rings, by lane gathers into registers, or
+// staged whole in shared memory by bulk copies.
+enum class SeedRows { kRing, kLanes, kBulk };
+int propagate_multi_grid(int precision, int KG, int num_sms, SeedRows rows);
 cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int precision, int KG,
-                                   int grid, bool bulk, cudaStream_t s);
+                                   int grid, SeedRows rows, cudaStream_t s);
 cudaError_t launch_offset_multi(const Dev& d, int grid, cudaStream_t s);
 // Failure-detection self-test: which 0 = grid barrier, 1 = staged-row mbarrier;
 // lose != 0 makes the wait run out (src: 64 floats on the device).

@@ -2288,35 +2288,35 @@ struct MultiFn {
 };
 
 template <typename TY, int KG>
-MultiFn multi_fn_k(bool bulk) {
-  if (bulk) return {(const void*)k_propagate_multi<TY, KG, true>, RingCfg<TY, KG>::kSmem};
+MultiFn multi_fn_k(SeedRows rows) {
+  if (rows == SeedRows::kBulk) return {(const void*)k_propagate_multi<TY, KG, true>, RingCfg<TY, KG>::kSmem};
   if constexpr (seed_ring_fits((int)sizeof(TY), KG))
-    return {(const void*)k_propagate_ring<TY, KG>,
-            RingWarp<TY, KG>::kWarps * (int)sizeof(RingWarp<TY, KG>), 32 * RingWarp<TY, KG>::kWarps};
-  else
-    return {(const void*)k_propagate_multi<TY, KG, false>, 0};
+    if (rows == SeedRows::kRing)
+      return {(const void*)k_propagate_ring<TY, KG>,
+              RingWarp<TY, KG>::kWarps * (int)sizeof(RingWarp<TY, KG>), 32 * RingWarp<TY, KG>::kWarps};
+  return {(const void*)k_propagate_multi<TY, KG, false>, 0};
 }
 
 template <typename TY>
-MultiFn multi_fn(int KG, bool bulk) {
+MultiFn multi_fn(int KG, SeedRows rows) {
   switch (KG) {
-    case 1: return multi_fn_k<TY, 1>(bulk);
-    case 2: return multi_fn_k<TY, 2>(bulk);
-    case 4: return multi_fn_k<TY, 4>(bulk);
-    default: return multi_fn_k<TY, 8>(bulk);
+    case 1: return multi_fn_k<TY, 1>(rows);
+    case 2: return multi_fn_k<TY, 2>(rows);
+    case 4: return multi_fn_k<TY, 4>(rows);
+    default: return multi_fn_k<TY, 8>(rows);
   }
 }
 
-MultiFn pick_multi(int precision, int KG, bool bulk) {
-  if (precision == OSP_PREC_FP64) return multi_fn<double>(KG, bulk);
-  if (precision == OSP_PREC_FP32_ACC64) return multi_fn<float>(KG, bulk);
-  return multi_fn<__nv_bfloat16>(KG, bulk);
+MultiFn pick_multi(int precision, int KG, SeedRows rows) {
+  if (precision == OSP_PREC_FP64) return multi_fn<double>(KG, rows);
+  if (precision == OSP_PREC_FP32_ACC64) return multi_fn<float>(KG, rows);
+  return multi_fn<__nv_bfloat16>(KG, rows);
 }
 
 }  // namespace
 
-int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk) {
-  const MultiFn f = pick_multi(precision, KG, bulk);
+int propagate_multi_grid(int precision, int KG, int num_sms, SeedRows rows) {
+  const MultiFn f = pick_multi(precision, KG, rows);
   if (f.smem > 0 &&
       cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem) != cudaSuccess)
     return 0;
@@ -2330,11 +2330,11 @@ int propagate_multi_grid(int precision, int KG, int num_sms, bool bulk) {
 }
 
 cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int precision, int KG,
-                                   int grid, bool bulk, cudaStream_t s) {
+                                   int grid, SeedRows rows, cudaStream_t s) {
   Dev dd = d;
   PropParams p = pp;
   void* args[] = {&dd, &p};
-  const MultiFn f = pick_multi(precision, KG, bulk);
+  const MultiFn f = pick_multi(precision, KG, rows);
   return cudaLaunchCooperativeKernel(f.fn, dim3(grid), dim3(f.threads), args, (size_t)f.smem, s);
 }
 

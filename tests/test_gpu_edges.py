@@ -493,3 +493,36 @@ def test_float_blocks_keep_subnormal_steps(S, kw):
     got = eng.query(0)
     assert np.all(np.abs(got - want) <= 4 * levels * 2.0 ** -24 * want + levels * 2.0 ** -149)
     eng.close()
+
+
+@pytest.mark.parametrize("prec,S,group", [
+    (F64, 20, 0), (F64, 60, 0), (F32, 20, 0), (F32, 40, 64), (F32, 100, 0), (BF16, 20, 0), (BF16, 64, 0),
+    (BF16, 200, 128)])
+def test_register_gathers_are_taken_where_asked_for(prec, S, group):
+    """seed_gather 1 in the group widths that the row rings serve by default: its own
+    schedule is in force, and the scores follow the oracle's lock-step, L1 <= 1e-10
+    (double) and 1e-5 a seed (the bounds of the seed-block tests)."""
+    n = 2300
+    rng = np.random.default_rng(S)
+    src, dst = edge_graph(rng, n, 0)
+    seeds = rng.permutation(n)[:S].astype(np.int32)
+    eng = N.Engine(precision=prec, device=0, seed_gather=N.SEED_GATHER_REGISTERS, seed_group=group)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(seeds, C_RESTART)
+    assert eng.get_schedule() == (1024, 256, 256, 4)
+    eng.init_scores(1e-11)
+    it, _, _ = eng.get_seed_stats()
+    tol = 1e-10 if prec == F64 else 1e-5
+    g = O.Graph(n, src, dst)
+    old = g.csr()
+    pick = list(range(0, S, max(1, S // 8)))
+    r = {j: O.cpi(*old, int(seeds[j]), C_RESTART, 1e-11, force_iters=int(it[j]))[0] for j in pick}
+    for ops in W.edge_update_stream(src, dst, n, 2, 300, 300, seed=S):
+        eng.apply_updates(ops, 1e-9)
+        assert g.apply(ops) == -1
+        it, _, _ = eng.get_seed_stats()
+        for j in pick:
+            r[j], _, _, _ = O.osp(old, g.csr(), r[j], C_RESTART, 1e-9, force_iters=int(it[j]))
+            assert np.abs(eng.query(j) - r[j]).sum() <= tol
+        old = g.csr()
+    eng.close()
