@@ -253,6 +253,12 @@ struct PropParams {
 #define OSP_GUARD(ctl, cond, what, a, b, c) true
 #endif
 
+// Id u of a list entry whose value or row is gathered; in a checked build a bad one is
+// reported and node 0 taken in its place.
+__device__ __forceinline__ int list_id(const Dev& d, int u, int at) {
+  return OSP_GUARD(d.ctl, u >= 0 && u < d.nc, "list id", u, at, d.nc) ? u : 0;
+}
+
 // ---------------------------------------------------------------------------
 // small device helpers
 // ---------------------------------------------------------------------------

@@ -181,16 +181,16 @@ struct ColGroup {
 // KG columns; ys points at the lane's first column of row 0 of the group, rows
 // Sp elements apart): 32 ids per coalesced load, then kDepth rows in flight.
 template <typename TY, int KG, typename A>
-__device__ __forceinline__ void sum_rows(const int* p, int len, const TY* ys, int Sp, A (&acc)[KG],
-                                         int idx0, const L2Pol& pol, unsigned long long cold,
+__device__ __forceinline__ void sum_rows(const Dev& d, const int* p, int len, const TY* ys, int Sp,
+                                         A (&acc)[KG], int idx0, const L2Pol& pol, unsigned long long cold,
                                          int hot_n, bool on) {
   constexpr int D = ColGroup<TY, KG>::kDepth;
   const int lane = threadIdx.x & 31;
   for (int b = 0; b < len; b += 32) {
     const int cnt = min(32, len - b);
     // ids of the first block may come preloaded (idx0 >= 0 on every lane)
-    const int idx = (b == 0 && __all_sync(0xffffffffu, idx0 >= 0)) ? idx0
-                    : (lane < cnt ? __ldg(p + b + lane) : 0);
+    const int idx = list_id(d, (b == 0 && __all_sync(0xffffffffu, idx0 >= 0)) ? idx0
+                               : (lane < cnt ? __ldg(p + b + lane) : 0), b + lane);
     int j = 0;
     for (; j + D <= cnt; j += D) {
       alignas(16) TY a[D][KG];
@@ -492,9 +492,9 @@ __device__ __forceinline__ void ring_stream(int E, RingWarp<TY, KG>& W, const ch
 }
 
 // The words of a piece of a long in-list (ids p[0 .. L), L >= 1): node 0.
-__device__ __forceinline__ unsigned piece_word(const int* p, int L, int w) {
+__device__ __forceinline__ unsigned piece_word(const Dev& d, const int* p, int L, int w) {
   const int q = 32 * w + (threadIdx.x & 31);
-  return (unsigned)__ldg(p + min(q, L - 1)) | (q < L ? 0u : 127u << 25);
+  return (unsigned)list_id(d, __ldg(p + min(q, L - 1)), q) | (q < L ? 0u : 127u << 25);
 }
 
 // The in-lists of a run of up to 32 nodes as one edge stream: lane j holds node
@@ -502,11 +502,11 @@ __device__ __forceinline__ unsigned piece_word(const int* p, int L, int w) {
 // windows' words, in order.
 template <typename TY, int KG>
 struct RunWords {
-  const int* pool;
+  const Dev& d;
   int P, E, started;  // first position of the lane's list, edges of the run, last list's rank
   int ll;
-  __device__ __forceinline__ RunWords(const int* pl, int l, unsigned off, int incl, RingWarp<TY, KG>& W)
-      : pool(pl), P(incl - l), E(__shfl_sync(0xffffffffu, incl, 31)), started(-1), ll(l) {
+  __device__ __forceinline__ RunWords(const Dev& dev, int l, unsigned off, int incl, RingWarp<TY, KG>& W)
+      : d(dev), P(incl - l), E(__shfl_sync(0xffffffffu, incl, 31)), started(-1), ll(l) {
     const int lane = threadIdx.x & 31;
     __syncwarp();  // the last run's list table has been read
     const unsigned full = __ballot_sync(0xffffffffu, ll > 0);
@@ -521,8 +521,8 @@ struct RunWords {
     const uint2 l = W.lists[started + __popc(hm & (lanemask_lt() | (1u << lane)))];
     started += __popc(hm);
     // the sum wraps back; positions past the end repeat the last edge, for no node
-    const unsigned u = (unsigned)__ldg(pool + (l.x + (unsigned)min(q, E - 1)));
-    return u | (q < E ? l.y : 127u << 25);
+    const int u = __ldg(d.pool_c + (l.x + (unsigned)min(q, E - 1)));
+    return (unsigned)list_id(d, u, q) | (q < E ? l.y : 127u << 25);
   }
 };
 
@@ -539,13 +539,13 @@ __device__ __forceinline__ int warp_inclusive(int x) {
 // bf16: sum of the rows of one piece of a long in-list: in the lanes with t = 0,
 // d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
 template <int KG>
-__device__ __forceinline__ void mma_piece(const int* p, int L, const char* src, bool on, int parts,
+__device__ __forceinline__ void mma_piece(const Dev& dev, const int* p, int L, const char* src, bool on, int parts,
                                           RingWarp<__nv_bfloat16, KG>& W, float (&d)[8 * KG]) {
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
   ring_stream<__nv_bfloat16, KG>(
-      L, W, src, on, [&](int w) { return piece_word(p, L, w); },
+      L, W, src, on, [&](int w) { return piece_word(dev, p, L, w); },
       [&](int, const unsigned* w, unsigned stage) {
         const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
         const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
@@ -557,7 +557,7 @@ __device__ __forceinline__ void mma_piece(const int* p, int L, const char* src, 
 // bf16: a run's lists. The nodes are taken eight at a time: finish(c, d) gets the
 // sums of nodes 8 c .. 8 c + 7 (fragments as in mma_stage), in order, once each.
 template <int KG, typename F>
-__device__ __forceinline__ void mma_stream(const int* pool, int ll, unsigned off, const char* src,
+__device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off, const char* src,
                                            bool on, int parts, RingWarp<__nv_bfloat16, KG>& W, F finish) {
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
   const int incl = warp_inclusive(ll);
@@ -566,7 +566,7 @@ __device__ __forceinline__ void mma_stream(const int* pool, int ll, unsigned off
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
   int c = 0;  // eight nodes being summed, and the stream position after them
   int Ec = __shfl_sync(0xffffffffu, incl, 7);
-  RunWords<__nv_bfloat16, KG> R(pool, ll, off, incl, W);
+  RunWords<__nv_bfloat16, KG> R(dev, ll, off, incl, W);
   if (R.E > 0) {
     ring_stream<__nv_bfloat16, KG>(
         R.E, W, src, on, [&](int w) { return R.word(w, W); },
@@ -764,8 +764,8 @@ __device__ __forceinline__ void narrow_finish(const Narrow<W>& N, const Multi& M
 // lists summed in pieces, at pool offset off) into acc_s[j * W + column]
 // (this warp's shared memory, zeroed by the caller).
 template <int W>
-__device__ __forceinline__ void narrow_stream(const Narrow<W>& N, const int* pool, int ll,
-                                              unsigned off, float* acc_s) {
+__device__ __forceinline__ void narrow_stream(const Dev& d, const Narrow<W>& N, int ll, unsigned off,
+                                              float* acc_s) {
   const int lane = threadIdx.x & 31;
   int incl = ll;
 #pragma unroll
@@ -794,7 +794,8 @@ __device__ __forceinline__ void narrow_stream(const Narrow<W>& N, const int* poo
       const unsigned oj = __shfl_sync(0xffffffffu, off, j);
       node[r] = q < E ? j : -1;
       row[r].zero();
-      if (q < E) row[r].load(N.src + (size_t)__ldg(pool + oj + (unsigned)(q - Pj)) * N.stride);
+      if (q < E)
+        row[r].load(N.src + (size_t)list_id(d, __ldg(d.pool_c + oj + (unsigned)(q - Pj)), q) * N.stride);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -860,7 +861,7 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
         for (int r = 0; r < 4; ++r) {
           const int e = b + 32 * r + lane;
           rw[r].zero();
-          if (e < Lp) rw[r].load(N.src + (size_t)__ldg(pl + e) * N.stride);
+          if (e < Lp) rw[r].load(N.src + (size_t)list_id(d, __ldg(pl + e), e) * N.stride);
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -913,7 +914,7 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
       for (int c = 0; c < W; c += 4)
         reinterpret_cast<float4*>(acc_s)[(lane * W + c) / 4] = make_float4(0.f, 0.f, 0.f, 0.f);
       __syncwarp();
-      narrow_stream<W>(N, d.pool_c, mine ? len : 0, off, acc_s);
+      narrow_stream<W>(d, N, mine ? len : 0, off, acc_s);
       __syncwarp();
       if (fin) {
         float x[W];
@@ -1613,7 +1614,7 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
 #pragma unroll
         for (int k = 0; k < KG; ++k) acc[k] = (A)0;
         if constexpr (kBulk) ring_sum_list<TY, KG, A>(rg, d, p, L, ysg, acc, pol, cold, hot_n);
-        else sum_rows<TY, KG, A>(p, L, ysl, G, acc, -1, pol, cold, hot_n, act != 0);
+        else sum_rows<TY, KG, A>(d, p, L, ysl, G, acc, -1, pol, cold, hot_n, act != 0);
         A* ha = hub_acc + (size_t)h * Sp + c0;
 #pragma unroll
         for (int k = 0; k < KG; ++k) atomicAdd(ha + k, acc[k]);
@@ -1814,7 +1815,7 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
 #pragma unroll
           for (int k = 0; k < KG; ++k) acc[k] = (A)0;
           if (len > 0)
-            sum_rows<TY, KG, A>(d.pool_c + off, len, ysl, G, acc, idx, pol, cold, hot_n, act != 0);
+            sum_rows<TY, KG, A>(d, d.pool_c + off, len, ysl, G, acc, idx, pol, cold, hot_n, act != 0);
           finish_slice<TY, KG, A>(M, rbase_of(v), ybase_of(v), acc, s, len > 0, rr, eo, act, yd, l1, pol);
           if (!more) break;
         }
@@ -2058,7 +2059,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
           A* ha = hub_acc + (size_t)h * Sp + g * G;
           if constexpr (kMma) {
             float D[8 * KG];
-            mma_piece<KG>(p, L, src, on, running_parts<KG>(am), W, D);
+            mma_piece<KG>(d, p, L, src, on, running_parts<KG>(am), W, D);
             if ((lane & 3) == 0) {
               const int fg = lane >> 2;
 #pragma unroll
@@ -2071,7 +2072,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             for (int k = 0; k < KG; ++k) acc[k] = (A)0;
             unsigned cur = 0u;
             ring_stream<TY, KG>(
-                L, W, src, on, [&](int w) { return piece_word(p, L, w); },
+                L, W, src, on, [&](int w) { return piece_word(d, p, L, w); },
                 [&](int, const unsigned* w, unsigned stage) {
                   // rows past the end begin "no node": the list's sum is put aside there
                   add_stage<TY, KG>(w, W.rows + (stage - smem_u32(W.rows)), acc, cur, [&](unsigned) {
@@ -2167,7 +2168,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
           for (int k = 0; k < KG; ++k) l1f[k] = (L)0;
           if constexpr (kMma) {
             mma_stream<KG>(
-                d.pool_c, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
+                d, mine ? my_len : 0, my_off, src, on, parts, W, [&](int c, const float (&D)[8 * KG]) {
                   if (!((fin >> (8 * c)) & 0xFFu)) return;  // warp-uniform
                   // the sums by node and slot (conflict-free: banks 8 t + g)
                   const int fg = lane >> 2, t2 = 2 * (lane & 3);
@@ -2236,7 +2237,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
               store_k<TY, KG>(yd + g * gs + (size_t)(vb + __ffs(z) - 1) * G + lane * KG, zero);
             }
             const int ll = mine ? my_len : 0;
-            RunWords<TY, KG> R(d.pool_c, ll, my_off, warp_inclusive(ll), W);
+            RunWords<TY, KG> R(d, ll, my_off, warp_inclusive(ll), W);
             if (R.E == 0) continue;
             A acc[KG];
 #pragma unroll

@@ -374,8 +374,8 @@ __device__ __forceinline__ unsigned stream_starts(int ll, int P, int eb) {
 }
 
 // Sums of the lists of a chunk; returns lane j's.
-__device__ __forceinline__ float stream_lists(const int* __restrict__ pool, const float* ys, int ll,
-                                              unsigned o, WarpStream<float>& W) {
+__device__ __forceinline__ float stream_lists(const Dev& d, const float* ys, int ll, unsigned o,
+                                              WarpStream<float>& W) {
   constexpr int R = WarpStream<float>::kRounds;
   const int lane = threadIdx.x & 31;
   const unsigned le = lanemask_lt() | (1u << lane);
@@ -390,7 +390,8 @@ __device__ __forceinline__ float stream_lists(const int* __restrict__ pool, cons
       hm[r] = stream_starts(ll, P, eb + 32 * r);
       const int e = eb + 32 * r + lane;
       k[r] = started + __popc(hm[r] & le);
-      id[r] = e < total ? __ldg(pool + (W.delta[k[r]] + (unsigned)e)) : -1;  // the sum wraps back
+      // the sum wraps back
+      id[r] = e < total ? list_id(d, __ldg(d.pool_c + (W.delta[k[r]] + (unsigned)e)), e) : -1;
       started += __popc(hm[r]);
     }
     float v[R];
@@ -414,8 +415,8 @@ __device__ __forceinline__ float stream_lists(const int* __restrict__ pool, cons
   return ll > 0 ? W.sum[rank] : 0.f;
 }
 
-__device__ __forceinline__ double stream_lists(const int* __restrict__ pool, const double* ys, int ll,
-                                               unsigned o, WarpStream<double>& W) {
+__device__ __forceinline__ double stream_lists(const Dev& d, const double* ys, int ll, unsigned o,
+                                               WarpStream<double>& W) {
   constexpr int R = WarpStream<double>::kRounds;
   const int lane = threadIdx.x & 31;
   int P, rank;
@@ -435,7 +436,7 @@ __device__ __forceinline__ double stream_lists(const int* __restrict__ pool, con
       }
       const int e = eb + 32 * r + lane;
       const int k = started + __popc(hm & (lanemask_lt() | (1u << lane))) - 1;
-      if (e < total) id[r] = __ldg(pool + (W.delta[k] + (unsigned)e));  // the sum wraps back
+      if (e < total) id[r] = list_id(d, __ldg(d.pool_c + (W.delta[k] + (unsigned)e)), e);  // wraps back
       started += __popc(hm);
     }
   };
@@ -544,11 +545,11 @@ __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_
       T acc = (T)0;
       int j = lane;
       for (; j + 96 < L; j += 128) {
-        const int a0 = __ldg(p + j), a1 = __ldg(p + j + 32), a2 = __ldg(p + j + 64),
-                  a3 = __ldg(p + j + 96);
+        const int a0 = list_id(d, __ldg(p + j), j), a1 = list_id(d, __ldg(p + j + 32), j),
+                  a2 = list_id(d, __ldg(p + j + 64), j), a3 = list_id(d, __ldg(p + j + 96), j);
         acc += (ys[a0] + ys[a1]) + (ys[a2] + ys[a3]);
       }
-      for (; j < L; j += 32) acc += ys[__ldg(p + j)];
+      for (; j < L; j += 32) acc += ys[list_id(d, __ldg(p + j), j)];
       acc = warp_sum(acc);
       if (lane == 0) {
         const int np = (full + hub_piece - 1) / hub_piece;
@@ -594,7 +595,7 @@ __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_
       }
       const bool hub = len > hub_thr;
       const bool light = len <= kStreamMax<T>;
-      T s = stream_lists(d.pool_c, ys, light ? len : 0, o, W);
+      T s = stream_lists(d, ys, light ? len : 0, o, W);
       // longer lists: the whole warp, blocks of 256 entries (eight coalesced id
       // loads and gathers per lane); the ids of the next block (of this list or
       // the next one) load while the current block's gathers are in flight
@@ -607,7 +608,8 @@ __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_
         int jb = 0;
         int a[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = 32 * q + lane < hl ? __ldg(p + 32 * q + lane) : -1;
+        for (int q = 0; q < 8; ++q)
+          a[q] = 32 * q + lane < hl ? list_id(d, __ldg(p + 32 * q + lane), q) : -1;
         T acc = (T)0;
         for (;;) {
           T t[8];
@@ -629,7 +631,7 @@ __device__ double pull_step(const Dev& d, const T* ys, T* yd, int n_hubs, int n_
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
               const int j = njb + 32 * q + lane;
-              a[q] = j < nhl ? __ldg(np + j) : -1;
+              a[q] = j < nhl ? list_id(d, __ldg(np + j), j) : -1;
             }
           }
           if (kF32) {
