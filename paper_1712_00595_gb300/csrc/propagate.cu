@@ -39,10 +39,12 @@ struct CallState {
 };
 
 // One grid barrier, run by warp 0 between two __syncthreads (the caller's):
-// arrive, wait, and true if the call goes on. All lanes return the same value.
+// arrive, wait, and true if the call goes on. All lanes return the same value
+// and see what lane 0's wait has acquired (the shuffle alone orders no memory).
 __device__ __forceinline__ bool warp0_barrier(const Dev& d, unsigned target) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0) ok = grid_wait(d.bar, target, d.ctl);
+  __syncwarp();
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
