@@ -1619,6 +1619,7 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
 #pragma unroll
         for (int k = 0; k < KG; ++k) atomicAdd(ha + k, acc[k]);
         __threadfence();
+        __syncwarp();  // every lane's additions come before lane 0's count
         int last = 0;
         if (lane == 0) {
           const int np = (full + hub_piece - 1) / hub_piece;
@@ -1627,6 +1628,7 @@ __global__ void __launch_bounds__(kPropThreads, MultiOcc<TY, KG>::value)
         last = __shfl_sync(0xffffffffu, last, 0);
         if (last) {
           __threadfence();
+          __syncwarp();  // ... and its count before every lane's reads
 #pragma unroll
           for (int k = 0; k < KG; ++k) {
             acc[k] = __ldcg(ha + k);
@@ -2086,11 +2088,13 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             }
           }
           __threadfence();
+          __syncwarp();  // every lane's additions come before lane 0's count
           int last = 0;
           if (lane == 0) last = atomicAdd(&M.hub_cnt[h * 8 + g], 1) == np - 1;
           last = __shfl_sync(0xffffffffu, last, 0);
           if (last) {
             __threadfence();
+            __syncwarp();  // ... and its count before every lane's reads
             if (lane == 0) M.hub_cnt[h * 8 + g] = 0;
             const A sv = scale_of<A>(d, v);
 #pragma unroll
