@@ -966,16 +966,18 @@ osp_status osp_selftest_wait(int32_t device, int32_t which, int32_t lose) {
   std::vector<float> h(64);
   for (int i = 0; i < 64; ++i) h[i] = 1.0f + (float)i;
   if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess &&
-      cudaMalloc(&ctl, sizeof(Ctl)) == cudaSuccess &&
+      cudaMalloc(&ctl, 2 * sizeof(Ctl)) == cudaSuccess &&
       cudaMalloc(&src, sizeof(float) * 64) == cudaSuccess &&
-      cudaMemsetAsync(ctl, 0, sizeof(Ctl), st) == cudaSuccess &&
+      cudaMemsetAsync(ctl, 0, 2 * sizeof(Ctl), st) == cudaSuccess &&
       cudaMemcpyAsync(src, h.data(), sizeof(float) * 64, cudaMemcpyHostToDevice, st) == cudaSuccess &&
       launch_selftest(ctl, src, which, lose ? 1 : 0, st) == cudaSuccess &&
       cudaStreamSynchronize(st) == cudaSuccess) {
-    Ctl c;
-    if (cudaMemcpy(&c, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost) == cudaSuccess) {
-      if (c.status != 0) r = (osp_status)c.status;
-      else r = c.iter == 1 ? OSP_OK : OSP_ECUDA;  // completed, and (staging) the rows intact
+    Ctl c[2];
+    if (cudaMemcpy(c, ctl, sizeof(c), cudaMemcpyDeviceToHost) == cudaSuccess) {
+      // completed, and (staging) the rows intact
+      const auto result = [](const Ctl& w) { return w.status != 0 ? w.status : w.iter == 1 ? OSP_OK : OSP_ECUDA; };
+      r = (osp_status)result(c[0]);
+      if (which == 0 && result(c[1]) != r) r = OSP_ECUDA;  // one barrier gave up, the other did not
     }
   }
   cudaGetLastError();

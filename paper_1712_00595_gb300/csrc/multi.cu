@@ -2348,11 +2348,14 @@ cudaError_t launch_propagate_multi(const Dev& d, const PropParams& pp, int preci
 // are made to run out on purpose (a CTA that never arrives; an mbarrier whose
 // announced bytes never all land), and the status word must report it.
 // ---------------------------------------------------------------------------
+// Both grid barriers one after the other: the seed block's on ctl[0], the one-seed
+// kernel's on ctl[1] (its arrivals in bar_count).
 __global__ void k_selftest_barrier(Ctl* ctl, int lose) {
   __shared__ BarShared sh;
   if (lose && blockIdx.x == 0) return;  // this CTA never arrives
   if (bar_arrive(ctl, sh) && threadIdx.x == 0) ctl->iter = 1;
   bar_release(ctl, sh);
+  if (threadIdx.x == 0 && grid_wait(&ctl[1].bar_count, gridDim.x, ctl + 1)) ctl[1].iter = 1;
 }
 
 __global__ void k_selftest_stage(Ctl* ctl, const float* src, int lose) {

@@ -142,7 +142,7 @@ def _ptr(a) -> C.c_void_p:
 
 def selftest_wait(which, lose, device=0):
     """osp_selftest_wait: run one bounded wait of the persistent kernels
-    (which 0 = grid barrier, 1 = staged-row mbarrier), made to run out when
+    (which 0 = the two grid barriers, 1 = staged-row mbarrier), made to run out when
     lose is true. Returns the status code (OSP_OK or OSP_ETIMEOUT)."""
     return load_library().osp_selftest_wait(int(device), int(which), int(bool(lose)))
 

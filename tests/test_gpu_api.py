@@ -140,3 +140,14 @@ def test_bounded_waits_run_out_and_report_timeout(which):
     r = eng.query(0)
     assert np.all(np.isfinite(r)) and 0.5 < r.sum() <= 1 + 1e-9 and r[0] >= 0.15
     eng.close()
+
+
+def test_both_grid_barriers_run_out_one_after_the_other():
+    # the seed block's barrier and the one-seed kernel's have a limit of 2 s each: a CTA
+    # that reaches neither keeps the self-test busy for both
+    import time
+    assert N.selftest_wait(0, False) == N.OSP_OK
+    t0 = time.perf_counter()
+    assert N.selftest_wait(0, True) == N.OSP_ETIMEOUT
+    assert 3.5 < time.perf_counter() - t0 < 20.0
+    assert N.selftest_wait(0, False) == N.OSP_OK
