@@ -526,3 +526,48 @@ def test_register_gathers_are_taken_where_asked_for(prec, S, group):
             assert np.abs(eng.query(j) - r[j]).sum() <= tol
         old = g.csr()
     eng.close()
+
+
+@pytest.mark.parametrize("graphs", [0, 1])
+@pytest.mark.parametrize("n_ops", [512, 513, 16383, 16384])
+def test_batches_at_the_limits_of_the_ingest_routes(n_ops, graphs):
+    """The last batch size of the one-CTA ingest and the first of the one over many
+    CTAs, and the largest batches, whose last op (a node op at position 16,383) has the
+    highest key of all: graph equal to the oracle's; each kind of invalid op, an unknown
+    code among them, at the first, a middle and the last position is the one reported
+    and leaves the graph as it was."""
+    rng = np.random.default_rng(n_ops)
+    n = 900
+    src, dst = W.er_graph(n, 8000, 3)
+    seed = 5
+    eng = N.Engine(precision=F64, device=0, max_nodes=n + 60_000, use_graphs=graphs)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds([seed], C_RESTART)
+    eng.init_scores(1e-8)
+    g = O.Graph(n, src, dst)
+    nn = n
+    for last in (2, 3, 4):
+        ops = np.zeros(n_ops, W.UPDATE_DTYPE)
+        ops["op"] = rng.choice([0, 1, 2, 4], n_ops, p=[0.49, 0.49, 0.01, 0.01])
+        count = nn + np.cumsum(ops["op"] == 2) - (ops["op"] == 2)  # nodes before each op
+        ops["u"] = 10 + (rng.random(n_ops) * (count - 10)).astype(np.int32)
+        ops["v"] = 10 + (rng.random(n_ops) * (count - 10)).astype(np.int32)
+        few = rng.random(n_ops) < 0.2  # a few rows get many ops
+        ops["u"][few] = rng.integers(10, 20, few.sum())
+        ops[-1] = (6 + last % 2, 0, last)  # ids below 10 take no other op
+        before = eng.export_graph(0)
+        for k, (at, op) in enumerate([(0, (nn + 70_000, 0, 0)), (n_ops // 2, (0, -1, 1)),
+                                      (n_ops - 1, (seed, 0, 3)), (n_ops - 1, (0, 0, 9)),
+                                      (n_ops // 3, (0, 0, -1))]):
+            bad = ops.copy()
+            bad[at] = op
+            st = eng.apply_updates(bad, 1e-6, allow=(N.OSP_EINVAL,))
+            assert eng.last_status == N.OSP_EINVAL and st["bad_op"] == at, (k, at)
+        assert all(np.array_equal(a, b) for a, b in zip(before, eng.export_graph(0)))
+        eng.apply_updates(ops, 1e-6)
+        assert g.apply(ops, protect=(seed,)) == -1
+        nn += int((ops["op"] == 2).sum())
+        assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(0), g.csr()))
+        assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(1), g.csc()))
+        # node 7 was deleted in the second turn, node 6 is emptied in the third
+    eng.close()
