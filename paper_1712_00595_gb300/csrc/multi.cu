@@ -595,11 +595,15 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
 // float and double rows go through the same ring and are added by the lanes,
 // lane l the slots [KG l, KG (l + 1)) of each row: one shared load and KG (float:
 // KG / 2 packed) additions a row, a node's sum staying in registers from its
-// first row to its last. A stage's rows are summed in two chains of their own and
-// then added to the node's sum, so that a float sum's depth is rows / kRs + kRs / 2.
-// (Double rows are bound by their additions, 16 cycles of the SM per row of 32
-// columns, and take one chain.)
+// first row to its last (NodeSum). A node's rows within a stage are summed by themselves
+// (float: in two chains) and then added to the node's sum, which is put aside every
+// kSumStages stages, so that the depth of a sum of k rows is kRs + kSumStages +
+// k / (kRs kSumStages): one chain of 500 doubles was off by 3 to 8 units of 2^-53, now by
+// 1, as the lane gathers. Double rows are bound by their additions, 16 cycles of the SM
+// per row of 32 columns: a stage's first row starts its chain without one, which pays for
+// the addition to the node's sum.
 // ---------------------------------------------------------------------------
+constexpr int kSumStages = 16;
 template <int KG>
 __device__ __forceinline__ void add_row(float (&a)[KG], const float (&x)[KG]) {
   if constexpr (KG == 1) {
@@ -621,19 +625,40 @@ __device__ __forceinline__ void add_row(double (&a)[KG], const double (&x)[KG]) 
   for (int k = 0; k < KG; ++k) a[k] += x[k];
 }
 
-// Rows of a stage, each added to its node's sum acc; done(node) is called after a
-// node's last row (then acc starts again from zero). cur: the node being summed
-// (127: none yet).
-template <typename TY, int KG, typename F>
-__device__ __forceinline__ void add_stage(const unsigned* w, const unsigned char* stage, TY (&acc)[KG],
-                                          unsigned& cur, F done) {
+// A node's sum: acc, and what was put aside of a long list.
+template <typename TY, int KG>
+struct NodeSum {
+  TY acc[KG], aside[KG];
+  unsigned cur;  // the node being summed (127: none yet)
+  __device__ __forceinline__ explicit NodeSum(unsigned node) : cur(node) { clear(); }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < KG; ++k) acc[k] = aside[k] = (TY)0;
+  }
+  __device__ __forceinline__ void put_aside() {
+    add_row<KG>(aside, acc);
+#pragma unroll
+    for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
+  }
+  __device__ __forceinline__ void complete() { add_row<KG>(acc, aside); }
+};
+
+// Rows of stage h, each added to its node's sum; done(node) is called after a node's last
+// row, with the sum in S.acc (which then starts again from zero). kLong: the stream holds a
+// list of more than kSumStages stages; without one nothing is put aside (double: an addition
+// a node. 17 seeds at 65,537 nodes there and back 11.26 ms, 11.9 with it; one form with a
+// test of a flag is no better. Float rows always take it: 256 columns from scratch 23.6 ms
+// against 23.1 with one chain, 23.8 with two forms of the loop).
+template <typename TY, int KG, bool kLong, typename F>
+__device__ __forceinline__ void add_stage(int h, const unsigned* w, const unsigned char* stage,
+                                          NodeSum<TY, KG>& S, F done) {
   using RW = RingWarp<TY, KG>;
   constexpr int RS = RW::kRs;
   const int lane = threadIdx.x & 31;
   const unsigned node = w[lane & (RS - 1)] >> 25;
   const unsigned prev = __shfl_up_sync(0xffffffffu, node, 1);
   // bit r: row r begins another node than the row before it
-  const unsigned heads = __ballot_sync(0xffffffffu, lane < RS && node != (lane ? prev : cur));
+  const unsigned heads = __ballot_sync(0xffffffffu, lane < RS && node != (lane ? prev : S.cur));
   // the lane's slots of every row first: between the rows' additions a node may
   // end, and each load would come after what that stores and be waited for (the
   // wait for shared memory was the largest stall)
@@ -647,29 +672,40 @@ __device__ __forceinline__ void add_stage(const unsigned* w, const unsigned char
   for (int c = 0; c < kChains; ++c)
 #pragma unroll
     for (int k = 0; k < KG; ++k) part[c][k] = (TY)0;
-  auto gather = [&]() {  // the chains into the node's sum
-    if constexpr (kChains == 2) {
-      add_row<KG>(part[0], part[1]);
-      add_row<KG>(acc, part[0]);
-#pragma unroll
-      for (int c = 0; c < kChains; ++c)
-#pragma unroll
-        for (int k = 0; k < KG; ++k) part[c][k] = (TY)0;
-    }
+  auto gather = [&]() {  // the stage's chains into the node's sum
+    if constexpr (kChains == 2) add_row<KG>(part[0], part[1]);
+    add_row<KG>(S.acc, part[0]);
   };
 #pragma unroll
   for (int r = 0; r < RS; ++r) {
     if ((heads >> r) & 1u) {  // warp-uniform
-      gather();
-      if (cur != 127u) done(cur);
+      if (r > 0) gather();
+      if (S.cur != 127u) {
+        if constexpr (kLong) S.complete();
+        done(S.cur);
+      }
+      S.clear();
+      S.cur = __shfl_sync(0xffffffffu, node, r);
+      if constexpr (kChains == 2) {
 #pragma unroll
-      for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
-      cur = __shfl_sync(0xffffffffu, node, r);
+        for (int k = 0; k < KG; ++k) part[0][k] = part[1][k] = (TY)0;
+        add_row<KG>(part[r & 1], x[r]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < KG; ++k) part[0][k] = x[r][k];
+      }
+    } else if constexpr (kChains == 2) {
+      add_row<KG>(part[r & 1], x[r]);
+    } else if (r == 0) {
+#pragma unroll
+      for (int k = 0; k < KG; ++k) part[0][k] = x[0][k];
+    } else {
+      add_row<KG>(part[0], x[r]);
     }
-    if constexpr (kChains == 2) add_row<KG>(part[r & 1], x[r]);
-    else add_row<KG>(acc, x[r]);
   }
   gather();
+  if constexpr (kLong)
+    if (h % kSumStages == kSumStages - 1) S.put_aside();
 }
 
 // ---------------------------------------------------------------------------
@@ -2069,22 +2105,20 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
                 if ((am[f >> 2] >> (8 * (f & 3) + fg)) & 1u) atomicAdd(ha + 8 * f + fg, D[2 * f]);
             }
           } else {
-            A acc[KG];
+            NodeSum<A, KG> sum(0u);
+            auto add = [&](unsigned) {
 #pragma unroll
-            for (int k = 0; k < KG; ++k) acc[k] = (A)0;
-            unsigned cur = 0u;
+              for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, sum.acc[k]);
+            };
             ring_stream<TY, KG>(
                 L, W, src, on, [&](int w) { return piece_word(d, p, L, w); },
-                [&](int, const unsigned* w, unsigned stage) {
-                  // rows past the end begin "no node": the list's sum is put aside there
-                  add_stage<TY, KG>(w, W.rows + (stage - smem_u32(W.rows)), acc, cur, [&](unsigned) {
-#pragma unroll
-                    for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, acc[k]);
-                  });
+                [&](int h, const unsigned* w, unsigned stage) {
+                  // rows past the end begin "no node": the piece's sum is complete there
+                  add_stage<TY, KG, true>(h, w, W.rows + (stage - smem_u32(W.rows)), sum, add);
                 });
-            if (cur == 0u) {
-#pragma unroll
-              for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, acc[k]);
+            if (sum.cur == 0u) {
+              sum.complete();
+              add(0u);
             }
           }
           __threadfence();
@@ -2243,10 +2277,8 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             const int ll = mine ? my_len : 0;
             RunWords<TY, KG> R(d, ll, my_off, warp_inclusive(ll), W);
             if (R.E == 0) continue;
-            A acc[KG];
-#pragma unroll
-            for (int k = 0; k < KG; ++k) acc[k] = (A)0;
-            unsigned cur = 127u;
+            NodeSum<A, KG> sum(127u);
+            const A(&acc)[KG] = sum.acc;
             auto done = [&](unsigned j) {  // node vb + j: x = acc
               const A sj = __shfl_sync(0xffffffffu, my_s, (int)j);
               double* rp = M.r + (size_t)(vb + j) * Sp;
@@ -2264,12 +2296,24 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
                 store_k<TY, KG>(yd + g * gs + (size_t)(vb + j) * G + lane * KG, yv);
               }
             };
-            ring_stream<TY, KG>(
-                R.E, W, src, on, [&](int w) { return R.word(w, W); },
-                [&](int, const unsigned* w, unsigned stage) {
-                  add_stage<TY, KG>(w, W.rows + (stage - smem_u32(W.rows)), acc, cur, done);
-                });
-            if (cur != 127u) done(cur);
+            auto stream = [&](auto longs) {
+              ring_stream<TY, KG>(
+                  R.E, W, src, on, [&](int w) { return R.word(w, W); },
+                  [&](int h, const unsigned* w, unsigned stage) {
+                    add_stage<TY, KG, decltype(longs)::value>(h, w, W.rows + (stage - smem_u32(W.rows)),
+                                                              sum, done);
+                  });
+            };
+            if constexpr (std::is_same<TY, float>::value) {
+              stream(std::true_type{});
+            } else {
+              if (__reduce_max_sync(0xffffffffu, ll) > RW::kRs * kSumStages) stream(std::true_type{});
+              else stream(std::false_type{});
+            }
+            if (sum.cur != 127u) {
+              sum.complete();
+              done(sum.cur);
+            }
 #pragma unroll
             for (int k = 0; k < KG; ++k)
               if (l1f[k] != 0.0) atomicAdd(my_part + col[k], l1f[k]);

@@ -571,3 +571,97 @@ def test_batches_at_the_limits_of_the_ingest_routes(n_ops, graphs):
         assert all(np.array_equal(a, b) for a, b in zip(eng.export_graph(1), g.csc()))
         # node 7 was deleted in the second turn, node 6 is emptied in the third
     eng.close()
+
+
+def sum_graph(rng, S, lengths, reps, row, max_degree, n):
+    """S seeds with `row` out-edges each into a pool of nodes, lists of the given lengths
+    drawn from the pool, pool nodes with out-degrees up to max_degree (spread over their
+    logarithm). Returns the edges and {length: nodes}."""
+    pool0 = S + reps * len(lengths)
+    pool = np.arange(pool0, n)
+    src = [np.repeat(np.arange(S), row)]
+    dst = [np.concatenate([rng.choice(pool, row, replace=False) for _ in range(S)])]
+    lists, v = {}, S
+    for k in lengths:
+        for _ in range(reps):
+            src.append(rng.choice(pool, k, replace=False))
+            dst.append(np.full(k, v))
+            lists.setdefault(k, []).append(v)
+            v += 1
+    deg = np.exp(rng.uniform(0, np.log(max_degree), pool.size)).astype(int)
+    src.append(np.repeat(pool, deg))
+    dst.append(rng.choice(pool, deg.sum()))
+    e = np.unique(np.stack([np.concatenate(src), np.concatenate(dst)], 1), axis=0).astype(np.int32)
+    return np.ascontiguousarray(e[:, 0]), np.ascontiguousarray(e[:, 1]), lists
+
+
+def row_sum_errors(got, y, src, dst, nodes):
+    """(got - sum of the in-list's y) / sum |y|, signed so that a sum too small in size is
+    negative, for every seed and node; the sums exact enough at twice the precision."""
+    out = []
+    for v in nodes:
+        part = y[:, src[dst == v]].astype(np.longdouble)
+        s, m = part.sum(1), np.abs(part).sum(1)
+        ok = m > 0
+        out.append(((got[ok, v] - s[ok]) / m[ok] * np.sign(s[ok])).astype(np.float64))
+    return np.concatenate(out)
+
+
+@pytest.mark.parametrize("S", [20, 40])
+def test_double_row_sums_are_not_one_chain(S):
+    """Lists of equal values 2^-12 fl(0.75 / 7), whose additions to a long sum all round the
+    same way: one chain of 500 is off by 86 units of 2^-53. Sums by stages of at most 16
+    rows, 16 stages a part, four parts, two pieces: at most 16 + 16 + 4 + 3 additions deep,
+    half a unit in the last place (2^-53 relative) each."""
+    from fractions import Fraction
+    n, row = 1800, 768
+    src, dst = [np.repeat(np.arange(S), row)], [np.tile(np.arange(900, 900 + row), S)]
+    lists = (300, 500, 512, 767)
+    for i, k in enumerate(lists):
+        src.append(np.arange(900, 900 + k))
+        dst.append(np.full(k, 100 + i))
+    for u in range(900, 900 + row):  # every pool node: seven out-edges
+        have = sum(u < 900 + k for k in lists)
+        src.append(np.full(7 - have, u))
+        dst.append(200 + (u + np.arange(7 - have)) % 300)
+    src, dst = np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+    eng = N.Engine(precision=F64, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.arange(S, dtype=np.int32), 0.25)
+    eng.set_fixed_iterations(2)
+    eng.init_scores(1e-9)
+    y = Fraction(0.75 / 7) / 2 ** 12  # 0.25 x (0.75 / 768), exact, times fl(0.75 / 7)
+    for j in (0, S - 1):
+        r = eng.query(j)
+        for i, k in enumerate(lists):
+            assert abs(Fraction(float(r[100 + i])) / (k * y) - 1) <= Fraction(39, 2 ** 53), (j, k)
+    eng.close()
+
+
+@pytest.mark.parametrize("prec,S", [(F32, 40), (F32, 100), (BF16, 100)])
+def test_float_row_sums_of_long_lists(prec, S):
+    """Second step from scratch (float rows, also of a bf16 block): lists of 1,000 and 1,024
+    rows against the double sum. An addition to a partial sum s rounds by at most 2^-24 s,
+    as a random variable with a deviation of 2^-24 s / sqrt(3). Sums by stages of 8 or 16
+    rows, 16 stages a part: the parts' sums, (2/8)^2 + .. + (8/8)^2 = 3.2, the stages within
+    the parts 0.7 more, rows within stages and pieces less than 0.6: a deviation of
+    sqrt(4.5 / 3) = 1.2 units of 2^-24, a mean size of 0.8 times that, 1.0. (A chain of 125
+    stage sums: 3.0.)"""
+    rng = np.random.default_rng(S)
+    n = 6000
+    src, dst, lists = sum_graph(rng, S, (1000, 1024), 8, 3000, 400, n)
+    eng = N.Engine(precision=prec, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.arange(S, dtype=np.int32), C_RESTART)
+    eng.set_fixed_iterations(2)
+    eng.init_scores(1e-9)
+    got = np.stack([eng.query(j) for j in range(S)])
+    eng.close()
+    d = np.bincount(src, minlength=n)
+    scale = np.where(d > 0, (1 - C_RESTART) / np.maximum(d, 1), 0.0).astype(np.float32)
+    x = np.zeros((S, n), np.float32)
+    for j in range(S):
+        x[j, dst[src == j]] = np.float32(C_RESTART) * scale[j]
+    for k, nodes in lists.items():
+        err = row_sum_errors(got, x * scale, src, dst, nodes) * 2.0 ** 24
+        assert np.abs(err).mean() <= 1.0, (k, np.abs(err).mean())
