@@ -329,8 +329,8 @@ __device__ __forceinline__ void load_k(const T* p, T (&out)[K]) {
 //   A = rows transposed (m = columns, G / 16 tiles; k = edges),
 //   B = membership      (k = edges, n = nodes, entries 1.0 or 0.0),
 //   D = sums            (m = columns, n = nodes, float accumulation).
-// Products with 1.0 and 0.0 are exact, the sums are float sums. A warp keeps a
-// ring of kStages stages of 16 rows in shared memory: cp.async brings the rows
+// Products with 1.0 and 0.0 are exact; the sums are float sums, truncated, and so kept to
+// short chains (mma_put). A warp keeps a ring of kStages stages of 16 rows in shared memory: cp.async brings the rows
 // in (16 bytes a lane, no registers held), ldmatrix.trans takes them out as A
 // fragments, and a membership entry is one comparison of the edge's node number.
 // Adding the rows in lanes took 13 warp instructions per edge and 32 columns
@@ -536,6 +536,45 @@ __device__ __forceinline__ int warp_inclusive(int x) {
   return x;
 }
 
+// The tensor cores' float accumulator drops the bits that do not fit instead of rounding
+// them, so a chain ends after kMmaChain stages of 16 rows: its sums are added, rounded to
+// nearest, to those put aside in shared memory (`put`), each lane its own entries. Against
+// the double sums of the same rows, lists of 1,000 came out 1.5 to 1.9 units of 2^-24 small
+// on average, 0.03 so (0.35 in size; one lane addition after the other in pieces of 256,
+// 0.3), lists of 64 exact either way; a step takes as long as without it (2^21 nodes, 256
+// seeds there and back 161.4 ms, 160.7 so; only runs with a longer list put anything aside).
+constexpr int kMmaChain = 8;
+template <int KG>
+__device__ __forceinline__ void mma_put(float (&d)[8 * KG], RingWarp<__nv_bfloat16, KG>& W, int parts,
+                                        bool& put) {
+  const int fg = (threadIdx.x & 31) >> 2, t2 = 2 * (threadIdx.x & 3);
+#pragma unroll
+  for (int f = 0; f < 4 * KG; ++f) {
+    if (f >= 4 * parts) break;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float* a = &W.acc[t2 + q][8 * f + fg];
+      *a = put ? *a + d[2 * f + q] : d[2 * f + q];
+      d[2 * f + q] = 0.f;
+    }
+  }
+  put = true;
+}
+// d += the sums put aside.
+template <int KG>
+__device__ __forceinline__ void mma_take(float (&d)[8 * KG], const RingWarp<__nv_bfloat16, KG>& W, int parts,
+                                         bool& put) {
+  if (!put) return;  // warp-uniform
+  const int fg = (threadIdx.x & 31) >> 2, t2 = 2 * (threadIdx.x & 3);
+#pragma unroll
+  for (int f = 0; f < 4 * KG; ++f) {
+    if (f >= 4 * parts) break;
+    d[2 * f] += W.acc[t2][8 * f + fg];
+    d[2 * f + 1] += W.acc[t2 + 1][8 * f + fg];
+  }
+  put = false;
+}
+
 // bf16: sum of the rows of one piece of a long in-list: in the lanes with t = 0,
 // d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
 template <int KG>
@@ -544,14 +583,17 @@ __device__ __forceinline__ void mma_piece(const Dev& dev, const int* p, int L, c
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
+  bool put = false;
   ring_stream<__nv_bfloat16, KG>(
       L, W, src, on, [&](int w) { return piece_word(dev, p, L, w); },
-      [&](int, const unsigned* w, unsigned stage) {
+      [&](int h, const unsigned* w, unsigned stage) {
         const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
         const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
         mma_stage<KG>(d, stage, member2(u0, (unsigned)(lane >> 2)), member2(u1, (unsigned)(lane >> 2)),
                       parts);
+        if (h % kMmaChain == kMmaChain - 1) mma_put<KG>(d, W, parts, put);
       });
+  mma_take<KG>(d, W, parts, put);
 }
 
 // bf16: a run's lists. The nodes are taken eight at a time: finish(c, d) gets the
@@ -566,6 +608,8 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
   int c = 0;  // eight nodes being summed, and the stream position after them
   int Ec = __shfl_sync(0xffffffffu, incl, 7);
+  const bool longs = __reduce_max_sync(0xffffffffu, ll) > 16 * kMmaChain;
+  bool put = false;
   RunWords<__nv_bfloat16, KG> R(dev, ll, off, incl, W);
   if (R.E > 0) {
     ring_stream<__nv_bfloat16, KG>(
@@ -578,7 +622,11 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
               const unsigned node = (unsigned)(8 * c + (lane >> 2));
               mma_stage<KG>(d, stage, member2(u0, node), member2(u1, node), parts);
             }
-            if (Ec > 16 * h + 16) break;  // goes on in the next half window
+            if (Ec > 16 * h + 16) {  // goes on in the next half window
+              if (longs && h % kMmaChain == kMmaChain - 1) mma_put<KG>(d, W, parts, put);
+              break;
+            }
+            mma_take<KG>(d, W, parts, put);
             finish(c, d);
 #pragma unroll
             for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;

@@ -665,3 +665,40 @@ def test_float_row_sums_of_long_lists(prec, S):
     for k, nodes in lists.items():
         err = row_sum_errors(got, x * scale, src, dst, nodes) * 2.0 ** 24
         assert np.abs(err).mean() <= 1.0, (k, np.abs(err).mean())
+
+
+@pytest.mark.parametrize("S", [20, 40, 100])
+def test_bf16_row_sums_of_long_lists_are_not_truncated(S):
+    """First step of a batch, bf16 rows over many decades: sums of 500 to 1,024 rows against
+    the double sum of the stored rows. Sums that round to nearest have a mean error of zero;
+    half a unit of 2^-24 is allowed. (Chains of up to 64 tensor-core additions, which drop
+    what does not fit, came out 1.5 to 2.2 units small.)"""
+    rng = np.random.default_rng(S)
+    n = 5000
+    src, dst, lists = sum_graph(rng, S, (500, 1000, 1024), 12, 2500, 1000, n)
+    eng = N.Engine(precision=BF16, device=0)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(np.arange(S, dtype=np.int32), C_RESTART)
+    eng.init_scores(1e-10)
+    r0 = np.stack([eng.query(j) for j in range(S)])
+    rows = np.concatenate([np.arange(S), rng.choice(np.arange(n // 2, n), 600, replace=False)])
+    out = {u: dst[src == u] for u in rows.tolist()}
+    ops = np.zeros(rows.size, W.UPDATE_DTYPE)  # one new edge a row, into the upper half
+    for i, (u, t) in enumerate(out.items()):
+        ops[i] = (u, rng.choice(np.setdiff1d(np.arange(n // 2, n), t)), 0)
+    eng.set_fixed_iterations(1)
+    eng.apply_updates(ops, 1e-9)
+    got = np.stack([eng.query(j) for j in range(S)])
+    eng.close()
+    x = np.zeros((S, n))
+    for op, (u, t) in zip(ops, out.items()):
+        x[:, t] += (0.85 / (t.size + 1) - 0.85 / t.size) * r0[:, u:u + 1]
+        x[:, op["v"]] += 0.85 / (t.size + 1) * r0[:, u]
+    src, dst = np.concatenate([src, ops["u"]]), np.concatenate([dst, ops["v"]])
+    d = np.bincount(src, minlength=n)
+    scale = np.where(d > 0, 0.85 / np.maximum(d, 1), 0.0).astype(np.float32)
+    b = (x.astype(np.float32) * scale).view(np.uint32).astype(np.uint64)
+    y = (((b + 0x7FFF + ((b >> 16) & 1)) >> 16) << 16).astype(np.uint32).view(np.float32)  # to bf16
+    for k, nodes in lists.items():
+        err = row_sum_errors(got - r0 - x, y, src, dst, nodes) * 2.0 ** 24
+        assert abs(err.mean()) <= 0.5, (k, err.mean())
