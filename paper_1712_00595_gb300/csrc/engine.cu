@@ -465,7 +465,9 @@ const int* schedule(osp_ctx* ctx) {
   // 40.6 with 1,024; float, 2^18 nodes, 64 seeds: 181 us a step with 256, 173
   // with 512), but not so long that their chain of double additions is the step
   // (65,537 nodes, 17 seeds: 97 us with 512, 137 with 1,024). A bf16 node's
-  // finish weighs as much as 8 edges.
+  // finish weighs as much as 8 edges. A bf16 block's start from scratch, in float rows,
+  // goes by the bf16 schedule too: 23.5 ms for 256 columns of 2^18 nodes, 24.4 by that of
+  // float blocks.
   static const int ring[4] = {kTaskItems, 512, 512, kMultiNodeItems};
   static const int mma[4] = {kTaskItems, 1024, 1024, 8};
   if (ctx->sched[0] > 0) return ctx->sched;
@@ -1399,7 +1401,9 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
                   : ctx->opt.precision == OSP_PREC_BF16_ACC64 ? (ctx->n >= (1 << 19) ? 128 : 64)
                   : ctx->opt.precision == OSP_PREC_FP32_ACC64 ? 128 : 64;
     M.KG = std::max(1, std::min(K, g / 32));
-    M.KG_init = ctx->opt.seed_group > 0 ? M.KG : std::min(K, 4);
+    // a bf16 block starts from scratch in float, whose rows hold 128 columns in 512 bytes
+    const bool bf16 = ctx->opt.precision == OSP_PREC_BF16_ACC64;
+    M.KG_init = ctx->opt.seed_group == 0 && bf16 ? std::min(K, 4) : M.KG;
     CK(cudaMemcpyAsync(M.seeds, by_col.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, ctx->stream));
     const int prec_init =
         ctx->opt.precision == OSP_PREC_FP64 ? OSP_PREC_FP64 : OSP_PREC_FP32_ACC64;
