@@ -58,7 +58,8 @@ typedef enum {
  *              accumulation and the ||x||_1 stopping test in double.
  * BF16_ACC64:  batches store the gather vector as bfloat16 (rounded to
  *              nearest), products and in-row sums in float, r / offset /
- *              stopping test in double; osp_init_scores runs as FP32_ACC64.
+ *              stopping test in double (|x| of up to 32 nodes at a time is
+ *              added in float first); osp_init_scores runs as FP32_ACC64.
  *              Each stored value's rounding residual is carried into the
  *              rounding of the same entry at the next step (error feedback),
  *              so the stored values' rounding errors telescope instead of

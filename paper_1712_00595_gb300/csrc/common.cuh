@@ -104,7 +104,7 @@ struct Multi {
   int S, Sp, K;
   int KG;              // columns per lane in a column group of the batch kernel
   int KG_init;         // ... of a bf16 block's initial CPI, in float rows
-  int pack;            // 1: bf16 32-column groups take their columns through slot_col (set per launch)
+  int pack;            // 1: groups take their columns through slot_col (row rings; set per launch)
   int* slot_col;       // [Sp] packed groups: column held by group slot q (chosen at each x(0))
   int* col_slot;       // [Sp] its inverse
   int* seeds;          // [S] internal ids, by column

@@ -1,5 +1,6 @@
-// Batch ingest: validation, canonical ordering and net edits (one CTA), then
-// the expansion of node deletions to the rows and columns they touch.
+// Batch ingest: validation, canonical ordering and net edits (one CTA up to kIngestOne
+// ops, many above), then the expansion of node deletions to the rows and columns they
+// touch.
 //
 // Semantics (osp.h): ops apply in order; the net effect on an edge (u,v) is
 // the last edge op naming it, unless u or v is deleted by the batch, in which
@@ -220,6 +221,8 @@ __global__ void k_cpi_begin(Dev d) {
   c->q_size[0] = 1;
 }
 
+// At most kIngestOne ops: one a thread.
+static_assert(kIngestOne <= kIngestThreads, "k_ingest's keys and flags");
 __global__ void __launch_bounds__(kIngestThreads) k_ingest(Dev d, const osp_update* __restrict__ ops,
                                                            int U) {
   extern __shared__ unsigned long long skey[];

@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(256, 4) k_merge_write(Dev d) {
 // f(v) = (in-list entries below v) + node_w v >= t task_items (so a task holds
 // about task_items items, an edge counting 1 and a node node_w, and never
 // splits a list); in-lists longer than hub_thr are listed and cut into pieces.
-// Two launches over kPlanCtas consecutive ranges of nodes: sums of the ranges,
+// Two launches, a range of consecutive nodes a CTA: sums of the ranges,
 // then every CTA scans its own range from the sum of those before it. A prefix
 // over all nodes in memory, the task starts from it and the pieces were six
 // launches, with two 64-bit divisions a node; an update phase of 1,000 edge ops
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(256, 4) k_merge_write(Dev d) {
 namespace {
 constexpr int kPlanThreads = 1024;
 
-// Nodes [lo, hi) of CTA b of nb: a multiple of four each, but for the last.
+// Nodes [lo, hi) of this CTA: a multiple of four each, but for the last.
 __device__ __forceinline__ void plan_range(int n, int& lo, int& hi) {
   const long long per = (((long long)n + gridDim.x - 1) / gridDim.x + 3) & ~3ll;
   lo = (int)min((long long)n, per * blockIdx.x);

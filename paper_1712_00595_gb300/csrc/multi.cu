@@ -761,7 +761,7 @@ __device__ __forceinline__ void add_stage(int h, const unsigned* w, const unsign
 // group slots 0..W-1 (W = 4 or 8), a step gathers W-value rows (8 or 16
 // bytes) from a compact [node][W] block, whose rows of the nodes with
 // out-edges (ids first in the degree order) mostly stay in L2, instead of the
-// 64-byte slices of the 32-column group. Lane = position of the in-list
+// rows of a whole group (64 to 256 bytes). Lane = position of the in-list
 // stream of 32 nodes: each lane loads one row, a segmented warp scan per
 // column sums each node's run, and the run's last lane adds it to the node's
 // sums in shared memory; then lane = node finishes. A step reads the rows the

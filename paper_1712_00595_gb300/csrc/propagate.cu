@@ -72,7 +72,7 @@ __device__ __forceinline__ bool mid_barrier(const Dev& d, unsigned target, CallS
 // from all partials summed in one fixed order. Against one CTA deciding for
 // all this saves the release hop and the re-read of its verdict, and one CTA
 // per SM quarters the arrivals: a step of a 10,000-node graph in double went
-// from 17.8 to 14.9 us, and to 9.6 us with the cheaper double sums above.
+// from 17.8 to 14.9 us, and to 9.6 us with the cheaper double sums of stream_lists.
 __device__ bool step_barrier(const Dev& d, const PropParams& pp, int step_mode, int n, long long m,
                              double l1, long long ef, unsigned target, CallState& cs, double* s_red,
                              double* s_l1, long long* s_ef) {
