@@ -804,16 +804,18 @@ struct NRow<8> {
 };
 
 // Node v's sums x: R += x (running columns), |x| into l1, next compact row and
-// residual w = x s + e_old (when v has out-edges).
+// residual w = x s + e_old (when v has out-edges). The score reductions are marked
+// evict-first as in the group steps (2^23 nodes, 4 of 256 columns running: 2,040 -> 1,780
+// us a step, 8: 2,670 -> 2,190).
 template <int W>
 __device__ __forceinline__ void narrow_finish(const Narrow<W>& N, const Multi& M, int v,
                                               const float (&x)[W], float s, bool has_in,
-                                              double (&l1)[W]) {
+                                              unsigned long long once, double (&l1)[W]) {
   if (has_in) {
 #pragma unroll
     for (int c = 0; c < W; ++c)
       if ((N.act >> c) & 1u) {
-        atomicAdd(M.r + (size_t)v * M.Sp + N.col[c], (double)x[c]);
+        red_add_once(M.r + (size_t)v * M.Sp + N.col[c], (double)x[c], once);
         l1[c] += fabs((double)x[c]);
       }
   }
@@ -859,9 +861,10 @@ __device__ __forceinline__ void narrow_stream(const Dev& d, const Narrow<W>& N, 
   }
   const int P = incl - ll;
   const int E = __shfl_sync(0xffffffffu, incl, 31);
-  // windows of 32 positions with their loads in flight together (narrower
-  // rows leave registers for more)
-  constexpr int R = W == 4 ? 8 : 6;
+  // windows of 32 positions with their loads in flight together; of eight (rows of 4) or
+  // six the last ones of a run often lie past its end (the same steps 1,750 -> 1,720 and
+  // 2,155 -> 2,080 us)
+  constexpr int R = 4;
   for (int w0 = 0; w0 < E; w0 += 32 * R) {
     int node[R];
     NRow<W> row[R];
@@ -912,7 +915,8 @@ __device__ __forceinline__ void narrow_stream(const Dev& d, const Narrow<W>& N, 
 template <int W>
 __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow<W>& N, int n_items,
                                             int n_pieces, int hub_thr, int hub_piece, float* hub_acc,
-                                            float* acc_s, double* my_part, Ctl* ctl) {
+                                            float* acc_s, double* my_part, Ctl* ctl,
+                                            unsigned long long once) {
   const int lane = threadIdx.x & 31;
   const int Sp = M.Sp;
   double l1n[W];
@@ -973,7 +977,7 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
             ha[c] = 0.f;
           }
           M.hub_cnt[h * 8] = 0;
-          narrow_finish<W>(N, M, v, x, scale_of<float>(d, v), true, l1n);
+          narrow_finish<W>(N, M, v, x, scale_of<float>(d, v), true, once, l1n);
         }
       }
       __syncwarp();
@@ -1004,7 +1008,7 @@ __device__ __forceinline__ void narrow_step(const Dev& d, const Multi& M, Narrow
         float x[W];
 #pragma unroll
         for (int c = 0; c < W; ++c) x[c] = acc_s[lane * W + c];
-        narrow_finish<W>(N, M, vl, x, sc, len > 0, l1n);
+        narrow_finish<W>(N, M, vl, x, sc, len > 0, once, l1n);
       }
       __syncwarp();
     }
@@ -2101,7 +2105,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
           }
           narrow_step<4>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
-                         my_part, ctl);
+                         my_part, ctl, pol.once);
         } else {
           Narrow<8> N{src, stride, yn[it & 1], eb, G, {}, 0u};
   #pragma unroll
@@ -2110,7 +2114,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             if (*(volatile int*)&M.active[N.col[c]]) N.act |= 1u << c;
           }
           narrow_step<8>(d, M, N, n_items, n_pieces, hub_thr, hub_piece, hub_acc, acc_s,
-                         my_part, ctl);
+                         my_part, ctl, pol.once);
         }
       }
     }
