@@ -70,6 +70,7 @@ struct osp_ctx {
   osp_options opt{};
   int device = 0;
   int num_sms = 0;
+  int l2_bytes = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::string err;
@@ -534,12 +535,8 @@ int elem_bytes(int precision) {
 // row slice.
 int hot_rows(const osp_ctx* ctx, int precision, int KG) {
   if (ctx->opt.node_order != 1 || ctx->opt.l2_hot_bytes < 0) return 0;
-  int l2 = 0;
-  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device) != cudaSuccess) {
-    cudaGetLastError();
-    l2 = 0;
-  }
-  const int64_t budget = ctx->opt.l2_hot_bytes > 0 ? ctx->opt.l2_hot_bytes : (int64_t)l2 * 6 / 10;
+  const int64_t budget =
+      ctx->opt.l2_hot_bytes > 0 ? ctx->opt.l2_hot_bytes : (int64_t)ctx->l2_bytes * 6 / 10;
   const int64_t rows = budget / (32LL * KG * elem_bytes(precision));
   return (int)std::min<int64_t>(rows, ctx->nc);
 }
@@ -883,8 +880,8 @@ osp_status enqueue_gather(osp_ctx* ctx, cudaStream_t st, const int* cols, double
       ++ctx->launches;
     }
     for (int i = 0; i < m && m < 4; ++i) {
-      k_gather_col<<<ctx->num_sms * 8, 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, cols[i], ctx->d.int2ext,
-                                                     n, dsts[i]);
+      launch_gather_col(ctx->d.mu.r, ctx->d.mu.Sp, cols[i], ctx->d.int2ext, n, dsts[i], ctx->num_sms,
+                        ctx->l2_bytes, st);
       ++ctx->launches;
     }
   } else {
@@ -1014,6 +1011,7 @@ osp_status osp_create(osp_ctx** out, const osp_options* opt) {
   ctx->device = ctx->opt.device;
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->l2_bytes, cudaDevAttrL2CacheSize, ctx->device);
   if (e == cudaSuccess) {
     if (ctx->opt.stream) {
       ctx->stream = (cudaStream_t)ctx->opt.stream;
@@ -1550,7 +1548,7 @@ osp_status scores_in_caller_order(osp_ctx* ctx, int col, int normalize, double* 
   const int n = (int)ctx->n;
   cudaStream_t st = ctx->stream;
   if (ctx->S > 1)
-    k_gather_col<<<ctx->num_sms * 8, 256, 0, st>>>(ctx->d.mu.r, ctx->d.mu.Sp, col, ctx->d.int2ext, n, dst);
+    launch_gather_col(ctx->d.mu.r, ctx->d.mu.Sp, col, ctx->d.int2ext, n, dst, ctx->num_sms, ctx->l2_bytes, st);
   else
     k_gather_ext<<<ctx->num_sms * 4, 256, 0, st>>>(ctx->d.r, ctx->d.ext2int, n, dst);
   if (normalize) {

@@ -40,8 +40,8 @@ __global__ void k_scale_copy(const double* r, int n, const double* __restrict__ 
 __global__ void k_topk_sort(TopkJobs J, int cap);
 __global__ void k_gather_cols(const double* __restrict__ r, int Sp, const int* __restrict__ int2ext,
                               int n, int m, GatherJobs G);
-__global__ void k_gather_col(const double* __restrict__ r, int Sp, int col,
-                             const int* __restrict__ int2ext, int n, double* out);
+void launch_gather_col(const double* r, int Sp, int col, const int* int2ext, int n, double* out,
+                       int num_sms, int64_t l2_bytes, cudaStream_t st);
 int enqueue_topk_select(const TopkJobs& J, int num_sms, cudaStream_t st);
 int enqueue_topk_sort(const TopkJobs& J, cudaStream_t st);
 constexpr int kTopkMaxK = 4096;

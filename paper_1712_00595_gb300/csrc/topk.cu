@@ -581,16 +581,6 @@ __global__ void __launch_bounds__(1024) k_topk_sort(TopkJobs J, int cap) {
   if (threadIdx.x == 0) *jb.out_k = kk;
 }
 
-// One score of a row: the line is not wanted again, and the fetch hint keeps the
-// L2 from pulling more of the row (a device query of one column at 2^21 nodes: 43
-// against 67 us with 64 columns, 64 against 70 with 256, where the DRAM still reads
-// 128 bytes a row; 17.5 against 19 at 131,072 nodes).
-__device__ __forceinline__ double ld_score(const double* p) {
-  double x;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::64B.f64 %0, [%1];" : "=d"(x) : "l"(p));
-  return x;
-}
-
 // Seed-block columns in caller order: dst_j[int2ext[v]] = r[v Sp + col_j],
 // walked in internal order, so that rows come in address order (the scattered
 // writes land in L2). A warp takes 32 rows: lane = job reads one value of each
@@ -618,28 +608,46 @@ __global__ void __launch_bounds__(32 * kGatherWarps) k_gather_cols(const double*
   }
 }
 
-// One column of the seed block in caller order, walked in internal order: four
-// rows a thread in flight. (Read in caller order, the rows came from all over
-// the block: 70 us a column of 2^21 nodes and 256 columns, TLB misses included.)
+// One column of the seed block in caller order, walked in internal order. kFar: the lines
+// it touches do not stay in L2: four rows a thread in flight, past the L1, with a hint that
+// keeps the L2 from fetching more of the row; else plain loads, whose 128-byte lines serve
+// the next fifteen columns.
+template <bool kFar>
 __global__ void __launch_bounds__(256) k_gather_col(const double* __restrict__ r, int Sp, int col,
                                                     const int* __restrict__ int2ext, int n, double* out) {
   const int stride = gridDim.x * blockDim.x;
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n; b += 4 * stride) {
-    double x[4];
-    int to[4];
+  constexpr int R = kFar ? 4 : 1;
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n; b += R * stride) {
+    double x[R];
+    int to[R];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < R; ++q) {
       const long long v = (long long)b + (long long)q * stride;
       to[q] = -1;
       if (v < n) {
-        x[q] = ld_score(r + (size_t)v * Sp + col);
+        const double* p = r + (size_t)v * Sp + col;
+        if constexpr (kFar)
+          asm volatile("ld.global.nc.L1::no_allocate.L2::64B.f64 %0, [%1];" : "=d"(x[q]) : "l"(p));
+        else
+          x[q] = __ldg(p);
         to[q] = int2ext[v];
       }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < R; ++q)
       if (to[q] >= 0) out[to[q]] = x[q];
   }
+}
+
+// Far when a column's 128-byte lines fill more than 60% of L2. Columns queried in turn,
+// us each, far and near: 64 columns of 400,000 nodes 16.5 and 15.6, 700,000 19.5 and 22.4,
+// 2^20 23 and 31, 2^21 36 and 57; near everywhere below, with the steps between: 100
+// columns of 131,071 nodes there and back 5.6 and 5.3 ms, 256 of 2^18 from scratch 23.5 and
+// 22.5.
+void launch_gather_col(const double* r, int Sp, int col, const int* int2ext, int n, double* out,
+                       int num_sms, int64_t l2_bytes, cudaStream_t st) {
+  const bool far = (int64_t)n * 128 > l2_bytes * 6 / 10;
+  (far ? k_gather_col<true> : k_gather_col<false>)<<<num_sms * 8, 256, 0, st>>>(r, Sp, col, int2ext, n, out);
 }
 
 int enqueue_topk_select(const TopkJobs& J, int num_sms, cudaStream_t st) {

@@ -702,3 +702,30 @@ def test_bf16_row_sums_of_long_lists_are_not_truncated(S):
     for k, nodes in lists.items():
         err = row_sum_errors(got - r0 - x, y, src, dst, nodes) * 2.0 ** 24
         assert abs(err.mean()) <= 0.5, (k, err.mean())
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("n", [2, 40_001, 900_001])
+def test_columns_of_a_block_in_either_form_of_the_query(n, order):
+    """A seed block's columns, small ones and those whose lines exceed the L2: the query of
+    each column equals the rankings' scores (gathered by another kernel), to the bit, and
+    the device query the host query."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    S = min(n, 5)
+    src, dst = rng.integers(0, n, (2, 2 * n)).astype(np.int32)
+    eng = N.Engine(precision=F32, device=0, node_order=order)
+    eng.load_graph(n, src, dst)
+    eng.set_seeds(rng.choice(n, S, replace=False).astype(np.int32), C_RESTART)
+    eng.init_scores(1e-4)
+    eng.query_slots(S)
+    eng.topk_async_many(range(S), range(S), 500)
+    out = torch.empty(n, dtype=torch.float64, device="cuda")
+    for j in range(S):
+        ids, sc = eng.topk_wait(j)
+        r = eng.query(j)
+        want_ids, want_sc = O.topk(r, 500)
+        assert np.array_equal(ids, want_ids) and np.array_equal(sc, want_sc)
+        eng.query_device(out, j)
+        assert np.array_equal(out.cpu().numpy(), r)
+    eng.close()
