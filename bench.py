@@ -187,10 +187,13 @@ def traffic_record(kernel="k_propagate<float>"):
         return None
 
 
-def column_group(asked, elem, n, S):
+def column_group(asked, elem, n, S, ring=True):
     """Columns per group of a seed block's gather rows of `elem`-byte values: as asked, else
-    the engine's default (osp_options.seed_group), at most the block's columns."""
+    the engine's default (osp_options.seed_group), at most the block's columns. ring: rows
+    gathered as seed_gather 0 does."""
     default = 64 if elem == 8 or (elem == 2 and n < 1 << 19) else 128
+    if elem == 2 and not ring:
+        default = 32
     return min(asked or default, next(32 * k for k in (1, 2, 4, 8) if 32 * k >= S))
 
 
@@ -593,7 +596,7 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
     achieved = ab / (prop_ms / 1e3) / 1e9
     dense_step = multi_alg_bytes(dict(stats[-1], iterations=1), stats[-1]["m_edges"], S, by)
     hist = np.bincount(np.concatenate(counts[Wm + 1:]).astype(np.int64))
-    group = column_group(args.seed_group, by, n, S)
+    group = column_group(args.seed_group, by, n, S, args.seed_gather == "auto")
     rec = traffic_record("k_propagate_multi")
     traffic = None
     if rec and config["workload"] == HEADLINE:

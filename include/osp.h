@@ -128,7 +128,8 @@ typedef struct {
                             as 1. Results are the same up to rounding order. */
     int32_t seed_group;  /* seed block: columns per column group of the pull steps (32, 64, 128
                             or 256, at most Sp; 0 = 64 for FP64 gather rows and for bf16 rows of a
-                            graph below 2^19 nodes, else 128). A pull step walks the graph
+                            graph below 2^19 nodes, else 128; bf16 rows with seed_gather
+                            1 or 2: 32). A pull step walks the graph
                             once per group that still has a running column, so groups whose
                             seeds have all stopped cost nothing; inside a group, a lane whose
                             columns have all stopped loads and stores nothing. With row rings

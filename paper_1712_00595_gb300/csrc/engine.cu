@@ -1394,9 +1394,12 @@ osp_status osp_set_seeds(osp_ctx* ctx, const int32_t* seeds, int32_t S, double c
     // 128 columns share the ids and memberships of an edge among more values, but
     // keep only two row stages in flight a warp: 2^21 nodes, 256 seeds 1,624
     // against 1,930 us a step, 2^20 nodes, 128 seeds 634 against 727; 131,071
-    // nodes, 100 seeds 60 against 48), unless the options say
+    // nodes, 100 seeds 60 against 48) and 32 for lane gathers and bulk copies (300,000
+    // nodes, 64 seeds there and back 1.77 and 1.66 ms, 2.25 and 2.32 with 64), unless
+    // the options say
     const int g = ctx->opt.seed_group > 0 ? ctx->opt.seed_group
-                  : ctx->opt.precision == OSP_PREC_BF16_ACC64 ? (ctx->n >= (1 << 19) ? 128 : 64)
+                  : ctx->opt.precision == OSP_PREC_BF16_ACC64
+                      ? (ctx->opt.seed_gather != 0 ? 32 : ctx->n >= (1 << 19) ? 128 : 64)
                   : ctx->opt.precision == OSP_PREC_FP32_ACC64 ? 128 : 64;
     M.KG = std::max(1, std::min(K, g / 32));
     // a bf16 block starts from scratch in float, whose rows hold 128 columns in 512 bytes

@@ -116,8 +116,10 @@ def test_l1_lookup_roofline():
 
 def test_reported_column_group_is_the_engines_default():
     """osp_options.seed_group 0: 64 for FP64 rows and for bf16 rows below 2^19 nodes, else
-    128; at most the block's columns."""
+    128 (bf16 rows not in rings: 32); at most the block's columns."""
     assert [bench.column_group(0, e, n, 256) for e in (8, 4, 2) for n in (1 << 18, 1 << 19)] == [
         64, 64, 128, 128, 64, 128]
     assert bench.column_group(0, 4, 1000, 33) == 64 and bench.column_group(256, 8, 1000, 20) == 32
     assert bench.column_group(32, 2, 1 << 24, 256) == 32
+    assert bench.column_group(0, 2, 1 << 24, 256, ring=False) == 32
+    assert bench.column_group(0, 4, 1 << 24, 256, ring=False) == 128
