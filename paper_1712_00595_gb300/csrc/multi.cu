@@ -329,10 +329,11 @@ __device__ __forceinline__ void load_k(const T* p, T (&out)[K]) {
 //   A = rows transposed (m = columns, G / 16 tiles; k = edges),
 //   B = membership      (k = edges, n = nodes, entries 1.0 or 0.0),
 //   D = sums            (m = columns, n = nodes, float accumulation).
-// Products with 1.0 and 0.0 are exact; the sums are float sums, truncated, and so kept to
-// short chains (mma_put). A warp keeps a ring of kStages stages of 16 rows in shared memory: cp.async brings the rows
-// in (16 bytes a lane, no registers held), ldmatrix.trans takes them out as A
-// fragments, and a membership entry is one comparison of the edge's node number.
+// Products with 1.0 and 0.0 are exact; the sums are float sums, truncated, and so kept
+// to short chains (mma_put). A warp keeps a ring of kStages stages of 16 rows in shared
+// memory: cp.async brings the rows in (16 bytes a lane, no registers held),
+// ldmatrix.trans takes them out as A fragments, and a membership entry is one
+// comparison of the edge's node number.
 // Adding the rows in lanes took 13 warp instructions per edge and 32 columns
 // (four conversions and two packed additions a row and lane, a node test, a
 // flush per run); this form takes about 2. The kernel had been bound by
@@ -578,8 +579,8 @@ __device__ __forceinline__ void mma_take(float (&d)[8 * KG], const RingWarp<__nv
 // bf16: sum of the rows of one piece of a long in-list: in the lanes with t = 0,
 // d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
 template <int KG>
-__device__ __forceinline__ void mma_piece(const Dev& dev, const int* p, int L, const char* src, bool on, int parts,
-                                          RingWarp<__nv_bfloat16, KG>& W, float (&d)[8 * KG]) {
+__device__ __forceinline__ void mma_piece(const Dev& dev, const int* p, int L, const char* src, bool on,
+                                          int parts, RingWarp<__nv_bfloat16, KG>& W, float (&d)[8 * KG]) {
   const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
@@ -646,8 +647,8 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
 // first row to its last (NodeSum). A node's rows within a stage are summed by themselves
 // (float: in two chains) and then added to the node's sum, which is put aside every
 // kSumStages stages, so that the depth of a sum of k rows is kRs + kSumStages +
-// k / (kRs kSumStages): one chain of 500 doubles was off by 3 to 8 units of 2^-53, now by
-// 1, as the lane gathers. Double rows are bound by their additions, 16 cycles of the SM
+// k / (kRs kSumStages): one chain of 500 doubles was off by 3 to 8 units of 2^-53, these
+// sums by 0.7 (lane gathers 0.9). Double rows are bound by their additions, 16 cycles of the SM
 // per row of 32 columns: a stage's first row starts its chain without one, which pays for
 // the addition to the node's sum.
 // ---------------------------------------------------------------------------
