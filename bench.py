@@ -155,7 +155,7 @@ def alg_bytes(st, n, m, bx, bs, S=1):
 # capture, valid only for the kernel sources they were taken on.
 TRAFFIC_RECORDS = {
     "k_propagate<float>": ("propagate_rmat20_traffic.txt", ("propagate.cu", "common.cuh")),
-    "k_propagate_multi": ("propagate_multi_rmat24_s256_traffic.txt", ("multi.cu", "common.cuh")),
+    "k_propagate_ring": ("propagate_ring_rmat24_s256_traffic.txt", ("multi.cu", "common.cuh")),
 }
 TRAFFIC_SOURCES = TRAFFIC_RECORDS["k_propagate<float>"][1]
 
@@ -597,9 +597,10 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
     dense_step = multi_alg_bytes(dict(stats[-1], iterations=1), stats[-1]["m_edges"], S, by)
     hist = np.bincount(np.concatenate(counts[Wm + 1:]).astype(np.int64))
     group = column_group(args.seed_group, by, n, S, args.seed_gather == "auto")
-    rec = traffic_record("k_propagate_multi")
+    rec = traffic_record("k_propagate_ring")
     traffic = None
-    if rec and config["workload"] == HEADLINE:
+    ring = args.seed_gather == "auto" and group * by <= 512
+    if rec and ring and config["workload"] == HEADLINE:
         # DRAM bytes per algorithmic byte of the small-case capture, times this run's bytes
         traffic = float(rec["dram_bytes_per_alg_byte"]) * ab / K
     out = {
@@ -611,14 +612,15 @@ def run_multi(args, rank, world, name=None, steps=None, warmup=None, extras=True
         "config": dict(config, seed_gather=args.seed_gather, autotune=bool(args.autotune),
                        schedule=list(eng.get_schedule()), node_order="descending out-degree",
                        seed_group=group,
-                       column_groups="packed per batch by offset size" if args.seed_gather == "auto"
-                       and S > group and group * by <= 512 else "fixed"),
+                       column_groups="packed per batch by offset size" if ring and S > group
+                       else "fixed"),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_per_alg_byte": float(rec["dram_bytes_per_alg_byte"])
                      if traffic is not None else None,
                      "traffic_source": rec.get("source") if traffic is not None else None,
-                     "kernel": "k_propagate_ring", "peak_kind": peak_kind + " (hbm_gbs copy)",
+                     "kernel": "k_propagate_ring" if ring else "k_propagate_multi",
+                     "peak_kind": peak_kind + " (hbm_gbs copy)",
                      "alg_bytes_per_launch": ab / K, "ms_per_launch": prop_ms / K,
                      "dense_step_alg_bytes": dense_step},
         "phases_ms_per_step": {"update_merge_offset": sum(s["ms_update"] for s in stats) / K,

@@ -1,6 +1,7 @@
 """Host-side logic of the benchmark: algorithmic byte counts, the committed
 traffic record, and the replica timing reduction over two gloo ranks."""
 import os
+import re
 import socket
 
 import pytest
@@ -123,3 +124,14 @@ def test_reported_column_group_is_the_engines_default():
     assert bench.column_group(32, 2, 1 << 24, 256) == 32
     assert bench.column_group(0, 2, 1 << 24, 256, ring=False) == 32
     assert bench.column_group(0, 4, 1 << 24, 256, ring=False) == 128
+
+
+def test_traffic_records_name_kernels_of_their_sources():
+    """Each committed DRAM record parses and belongs to a kernel that its sources define."""
+    for kernel, (name, sources) in bench.TRAFFIC_RECORDS.items():
+        with open(os.path.join(bench.ROOT, "profiles", name)) as f:
+            keys = {line.split("=", 1)[0].strip() for line in f if "=" in line and line[0] != "#"}
+        assert "source_sha256_16" in keys and any(k.startswith("dram_bytes_per_") for k in keys)
+        src = "".join(open(os.path.join(bench.ROOT, "paper_1712_00595_gb300", "csrc", s)).read()
+                      for s in sources)
+        assert re.search(r"__global__[^;{]*\b%s\(" % re.escape(kernel.split("<")[0]), src)
