@@ -458,7 +458,7 @@ SeedRows seed_rows(const osp_ctx* ctx, int precision, int KG);
 
 // The pull-step schedule in force: {task items, long-list threshold, piece,
 // node weight}; unset entries take the defaults of the seed count.
-const int* schedule(osp_ctx* ctx) {
+const int* schedule(osp_ctx* ctx, bool init = false) {
   static const int single[4] = {kTaskItems, kHubThreshold, kHubPiece, 1};
   static const int multi[4] = {kTaskItems, kMultiHub, kMultiHub, kMultiNodeItems};
   // row rings: a piece costs atomics, a fence and a dozen dependent loads, so
@@ -467,13 +467,14 @@ const int* schedule(osp_ctx* ctx) {
   // with 512), but not so long that their chain of double additions is the step
   // (65,537 nodes, 17 seeds: 97 us with 512, 137 with 1,024). A bf16 node's
   // finish weighs as much as 8 edges. A bf16 block's start from scratch, in float rows,
-  // goes by the bf16 schedule too: 23.5 ms for 256 columns of 2^18 nodes, 24.4 by that of
-  // float blocks.
+  // goes by the bf16 schedule too, but for its pieces: 23.5 ms for 256 columns of 2^18
+  // nodes, 24.4 by that of float blocks.
   static const int ring[4] = {kTaskItems, 512, 512, kMultiNodeItems};
   static const int mma[4] = {kTaskItems, 1024, 1024, 8};
+  static const int mma_init[4] = {kTaskItems, 512, 512, 8};
   if (ctx->sched[0] > 0) return ctx->sched;
   if (ctx->S > 1 && seed_rows(ctx, ctx->opt.precision, ctx->d.mu.KG) != SeedRows::kRing) return multi;
-  if (ctx->S > 1) return ctx->opt.precision == OSP_PREC_BF16_ACC64 ? mma : ring;
+  if (ctx->S > 1) return ctx->opt.precision != OSP_PREC_BF16_ACC64 ? ring : init ? mma_init : mma;
   return single;
 }
 
@@ -481,14 +482,14 @@ const int* schedule(osp_ctx* ctx) {
 int64_t small_tasks(const osp_ctx* ctx) { return std::min<int64_t>(kMaxSmallTasks, ctx->nc); }
 
 // Pull-step plan for the graph as it is after the merge.
-osp_status plan_pull(osp_ctx* ctx) {
+osp_status plan_pull(osp_ctx* ctx, bool init = false) {
   cudaStream_t st = ctx->stream;
   static_assert(kMaxBatch * sizeof(osp_update) >= kMaxGrid * sizeof(unsigned), "a sum per CTA");
   unsigned* sums = reinterpret_cast<unsigned*>(ctx->ops_stage);  // the batch has been merged
   const int plan_grid = std::min(ctx->num_sms, kMaxGrid);
   k_plan_sums<<<plan_grid, 1024, 0, st>>>(ctx->d, sums);
   ++ctx->launches;
-  const int* sc = schedule(ctx);
+  const int* sc = schedule(ctx, init);
   // A graph whose tasks of sc[0] items would leave warps idle is cut finer:
   // two tasks a warp with one seed (down to 32 items: 10,000 nodes and 100,000
   // edges in double ran 82 us a step in 107 tasks of 1,024, 9.6 us in 3,437 of
@@ -576,7 +577,7 @@ osp_status enqueue_propagate(osp_ctx* ctx, const PropParams& pp, bool init) {
 
 osp_status run_propagation(osp_ctx* ctx, double eps, bool init = false) {
   const PropParams pp = prop_params(ctx, eps);
-  osp_status s = plan_pull(ctx);
+  osp_status s = plan_pull(ctx, init);
   if (s != OSP_OK) return s;
   // queries in flight read the scores this kernel changes
   if (!ctx->qslots.empty()) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_queries, 0));

@@ -368,7 +368,9 @@ struct RingWarp {
   static constexpr int kCtas = 2;   // per SM
   static_assert(kChunks <= 32 && kRow * kRs <= 4096, "a stage is one chunk a lane, up to eight times");
   alignas(128) unsigned char rows[kStages * kStageBytes];
-  alignas(16) float acc[kMma ? 8 : 1][G + 4];  // bf16: sums of eight nodes, by node and slot
+  alignas(16) float acc[kMma ? 8 : 1][kMma ? G + 4 : 4];  // bf16: sums of eight nodes, by node and slot
+  static constexpr bool kDouble = std::is_same<TY, double>::value;
+  alignas(16) TY aside[kDouble ? G : 8];  // double: what was put aside of a long list's sum
   alignas(16) unsigned words[4][32];  // edges of four windows: row | node of the run << 25
   alignas(8) uint2 lists[32];       // nonempty lists of a run: pool offset - position, node << 25
 };
@@ -645,10 +647,12 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
 // lane l the slots [KG l, KG (l + 1)) of each row: one shared load and KG (float:
 // KG / 2 packed) additions a row, a node's sum staying in registers from its
 // first row to its last (NodeSum). A node's rows within a stage are summed by themselves
-// (float: in two chains) and then added to the node's sum, which is put aside every
-// kSumStages stages, so that the depth of a sum of k rows is kRs + kSumStages +
-// k / (kRs kSumStages): one chain of 500 doubles was off by 3 to 8 units of 2^-53, these
-// sums by 0.7 (lane gathers 0.9). Double rows are bound by their additions, 16 cycles of the SM
+// (float: in two chains) and then added to the node's sum, which double rows and float
+// rows of 128 columns put aside every kSumStages stages, so that the depth of their sum of
+// k rows is kRs + kSumStages + k / (kRs kSumStages): one chain of 500 doubles was off by 3
+// to 8 units of 2^-53, these sums by 0.7 (lane gathers 0.9), stages of 8 floats in one
+// chain by 1.6 of 2^-24, so by 0.7 (lane gathers 0.95); stages of 16 floats (512 rows at
+// most to a piece) by 1.2, bulk copies by 1.3. Double rows are bound by their additions, 16 cycles of the SM
 // per row of 32 columns: a stage's first row starts its chain without one, which pays for
 // the addition to the node's sum.
 // ---------------------------------------------------------------------------
@@ -674,30 +678,62 @@ __device__ __forceinline__ void add_row(double (&a)[KG], const double (&x)[KG]) 
   for (int k = 0; k < KG; ++k) a[k] += x[k];
 }
 
-// A node's sum: acc, and what was put aside of a long list.
+// A node's sum: acc, and what was put aside of a long list: double rows in shared memory,
+// each lane its own slots, if anything (`put`, warp-uniform); float rows of 128 columns
+// (stages of 8) in registers; narrower float rows put nothing aside.
 template <typename TY, int KG>
 struct NodeSum {
-  TY acc[KG], aside[KG];
+  static constexpr bool kDouble = RingWarp<TY, KG>::kDouble;
+  static constexpr bool kAside = kDouble || KG == 4;
+  alignas(16) TY acc[KG];
+  TY regs[kDouble ? 1 : KG];
+  TY* mem;
+  bool put;
   unsigned cur;  // the node being summed (127: none yet)
-  __device__ __forceinline__ explicit NodeSum(unsigned node) : cur(node) { clear(); }
+  __device__ __forceinline__ NodeSum(unsigned node, RingWarp<TY, KG>& W)
+      : mem(W.aside + (kDouble ? (threadIdx.x & 31) * KG : 0)), cur(node) {
+    clear();
+  }
   __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int k = 0; k < KG; ++k) acc[k] = aside[k] = (TY)0;
+    for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
+    put = false;
+    if constexpr (kAside && !kDouble) {
+#pragma unroll
+      for (int k = 0; k < KG; ++k) regs[k] = (TY)0;
+    }
   }
   __device__ __forceinline__ void put_aside() {
-    add_row<KG>(aside, acc);
+    if constexpr (kDouble) {
+      complete();
+      store_k<TY, KG>(mem, acc);
+      clear();
+      put = true;
+    } else if constexpr (kAside) {
+      add_row<KG>(regs, acc);
 #pragma unroll
-    for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
+      for (int k = 0; k < KG; ++k) acc[k] = (TY)0;
+    }
   }
-  __device__ __forceinline__ void complete() { add_row<KG>(acc, aside); }
+  __device__ __forceinline__ void complete() {
+    if constexpr (kDouble) {
+      if (put) {
+        alignas(16) TY a[KG];
+        load_k<TY, KG>(mem, a);
+        add_row<KG>(acc, a);
+      }
+    } else if constexpr (kAside) {
+      add_row<KG>(acc, regs);
+    }
+  }
 };
 
 // Rows of stage h, each added to its node's sum; done(node) is called after a node's last
 // row, with the sum in S.acc (which then starts again from zero). kLong: the stream holds a
-// list of more than kSumStages stages; without one nothing is put aside (double: an addition
-// a node. 17 seeds at 65,537 nodes there and back 11.26 ms, 11.9 with it; one form with a
-// test of a flag is no better. Float rows always take it: 256 columns from scratch 23.6 ms
-// against 23.1 with one chain, 23.8 with two forms of the loop).
+// list of more than kSumStages stages; without one nothing is put aside (double only; 64
+// seeds at 65,537 nodes 182 us a step, 192 with the sums put aside in registers and always
+// added. Float rows of 128 columns take one form: 256 columns of 2^18 nodes 509 us against
+// 494 with one chain, 510 with two forms, 514 through shared memory).
 template <typename TY, int KG, bool kLong, typename F>
 __device__ __forceinline__ void add_stage(int h, const unsigned* w, const unsigned char* stage,
                                           NodeSum<TY, KG>& S, F done) {
@@ -735,22 +771,19 @@ __device__ __forceinline__ void add_stage(int h, const unsigned* w, const unsign
       }
       S.clear();
       S.cur = __shfl_sync(0xffffffffu, node, r);
-      if constexpr (kChains == 2) {
 #pragma unroll
-        for (int k = 0; k < KG; ++k) part[0][k] = part[1][k] = (TY)0;
-        add_row<KG>(part[r & 1], x[r]);
+      for (int c = 0; c < kChains; ++c)
+#pragma unroll
+        for (int k = 0; k < KG; ++k) part[c][k] = kChains == 2 ? (TY)0 : x[r][k];
+    } else if (kChains == 1) {
+      if (r == 0) {
+#pragma unroll
+        for (int k = 0; k < KG; ++k) part[0][k] = x[0][k];
       } else {
-#pragma unroll
-        for (int k = 0; k < KG; ++k) part[0][k] = x[r][k];
+        add_row<KG>(part[0], x[r]);
       }
-    } else if constexpr (kChains == 2) {
-      add_row<KG>(part[r & 1], x[r]);
-    } else if (r == 0) {
-#pragma unroll
-      for (int k = 0; k < KG; ++k) part[0][k] = x[0][k];
-    } else {
-      add_row<KG>(part[0], x[r]);
     }
+    if constexpr (kChains == 2) add_row<KG>(part[r & 1], x[r]);
   }
   gather();
   if constexpr (kLong)
@@ -2158,7 +2191,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
                 if ((am[f >> 2] >> (8 * (f & 3) + fg)) & 1u) atomicAdd(ha + 8 * f + fg, D[2 * f]);
             }
           } else {
-            NodeSum<A, KG> sum(0u);
+            NodeSum<A, KG> sum(0u, W);
             auto add = [&](unsigned) {
 #pragma unroll
               for (int k = 0; k < KG; ++k) atomicAdd(ha + lane * KG + k, sum.acc[k]);
@@ -2330,7 +2363,7 @@ __global__ void __launch_bounds__(32 * RingWarp<TY, KG>::kWarps, RingWarp<TY, KG
             const int ll = mine ? my_len : 0;
             RunWords<TY, KG> R(d, ll, my_off, warp_inclusive(ll), W);
             if (R.E == 0) continue;
-            NodeSum<A, KG> sum(127u);
+            NodeSum<A, KG> sum(127u, W);
             const A(&acc)[KG] = sum.acc;
             auto done = [&](unsigned j) {  // node vb + j: x = acc
               const A sj = __shfl_sync(0xffffffffu, my_s, (int)j);
