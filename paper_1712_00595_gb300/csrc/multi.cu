@@ -543,9 +543,10 @@ __device__ __forceinline__ int warp_inclusive(int x) {
 // them, so a chain ends after kMmaChain stages of 16 rows: its sums are added, rounded to
 // nearest, to those put aside in shared memory (`put`), each lane its own entries. Against
 // the double sums of the same rows, lists of 1,000 came out 1.5 to 1.9 units of 2^-24 small
-// on average, 0.03 so (0.35 in size; one lane addition after the other in pieces of 256,
-// 0.3), lists of 64 exact either way; a step takes as long as without it (2^21 nodes, 256
-// seeds there and back 161.4 ms, 160.7 so; only runs with a longer list put anything aside).
+// on average, 0.03 to 0.05 so (0.35 in size; one lane addition after the other in pieces of
+// 256, 0.3; with chains of 12 half a unit small); lists of 64 are exact either way. Only
+// eight nodes with more than a chain's rows put anything aside: steps take 1 to 2% longer
+// (131,071 nodes, 256 seeds 196 -> 201 us, 2^21 nodes 2,812 -> 2,841).
 constexpr int kMmaChain = 8;
 template <int KG>
 __device__ __forceinline__ void mma_put(float (&d)[8 * KG], RingWarp<__nv_bfloat16, KG>& W, int parts,
@@ -579,24 +580,31 @@ __device__ __forceinline__ void mma_take(float (&d)[8 * KG], const RingWarp<__nv
 }
 
 // bf16: sum of the rows of one piece of a long in-list: in the lanes with t = 0,
-// d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g.
+// d[4 f] and d[4 f + 2] hold slots 16 f + g and 16 f + 8 + g. Row r adds to node r mod 8,
+// eight sums of an eighth of the rows, which need three bits less; they are added up at
+// the end.
 template <int KG>
 __device__ __forceinline__ void mma_piece(const Dev& dev, const int* p, int L, const char* src, bool on,
                                           int parts, RingWarp<__nv_bfloat16, KG>& W, float (&d)[8 * KG]) {
-  const int lane = threadIdx.x & 31, t2 = 2 * (lane & 3);
+  const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
+  const unsigned mine = (t2 == g ? 0xFFFFu : 0u) | (t2 + 1 == g ? 0xFFFF0000u : 0u);
 #pragma unroll
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
-  bool put = false;
   ring_stream<__nv_bfloat16, KG>(
       L, W, src, on, [&](int w) { return piece_word(dev, p, L, w); },
-      [&](int h, const unsigned* w, unsigned stage) {
+      [&](int, const unsigned* w, unsigned stage) {
         const uint2 u0 = *reinterpret_cast<const uint2*>(w + t2);
         const uint2 u1 = *reinterpret_cast<const uint2*>(w + 8 + t2);
-        mma_stage<KG>(d, stage, member2(u0, (unsigned)(lane >> 2)), member2(u1, (unsigned)(lane >> 2)),
-                      parts);
-        if (h % kMmaChain == kMmaChain - 1) mma_put<KG>(d, W, parts, put);
+        mma_stage<KG>(d, stage, member2(u0, 0u) & mine, member2(u1, 0u) & mine, parts);
       });
-  mma_take<KG>(d, W, parts, put);
+#pragma unroll
+  for (int f = 0; f < 4 * KG; ++f) {
+    if (f >= 4 * parts) break;  // warp-uniform
+    float x = d[2 * f] + d[2 * f + 1];
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    d[2 * f] = x;
+  }
 }
 
 // bf16: a run's lists. The nodes are taken eight at a time: finish(c, d) gets the
@@ -611,8 +619,8 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
   for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
   int c = 0;  // eight nodes being summed, and the stream position after them
   int Ec = __shfl_sync(0xffffffffu, incl, 7);
-  const bool longs = __reduce_max_sync(0xffffffffu, ll) > 16 * kMmaChain;
-  bool put = false;
+  int since = 0;     // stage from which those nodes' sums are in d
+  bool put = false;  // what came before lies aside
   RunWords<__nv_bfloat16, KG> R(dev, ll, off, incl, W);
   if (R.E > 0) {
     ring_stream<__nv_bfloat16, KG>(
@@ -626,13 +634,17 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
               mma_stage<KG>(d, stage, member2(u0, node), member2(u1, node), parts);
             }
             if (Ec > 16 * h + 16) {  // goes on in the next half window
-              if (longs && h % kMmaChain == kMmaChain - 1) mma_put<KG>(d, W, parts, put);
+              if (h - since >= kMmaChain - 1) {
+                mma_put<KG>(d, W, parts, put);
+                since = h + 1;
+              }
               break;
             }
             mma_take<KG>(d, W, parts, put);
             finish(c, d);
 #pragma unroll
             for (int k = 0; k < 8 * KG; ++k) d[k] = 0.f;
+            since = h;
             if (++c == 4) break;
             Ec = __shfl_sync(0xffffffffu, incl, 8 * c + 7);
           }
