@@ -664,9 +664,9 @@ __device__ __forceinline__ void mma_stream(const Dev& dev, int ll, unsigned off,
 // k rows is kRs + kSumStages + k / (kRs kSumStages): one chain of 500 doubles was off by 3
 // to 8 units of 2^-53, these sums by 0.7 (lane gathers 0.9), stages of 8 floats in one
 // chain by 1.6 of 2^-24, so by 0.7 (lane gathers 0.95); stages of 16 floats (512 rows at
-// most to a piece) by 1.2, bulk copies by 1.3. Double rows are bound by their additions, 16 cycles of the SM
-// per row of 32 columns: a stage's first row starts its chain without one, which pays for
-// the addition to the node's sum.
+// most to a piece) by 1.2, bulk copies by 1.3. Double rows are bound by their additions,
+// 16 cycles of the SM per row of 32 columns: a stage's first row starts its chain without
+// one, which pays for the addition to the node's sum.
 // ---------------------------------------------------------------------------
 constexpr int kSumStages = 16;
 template <int KG>

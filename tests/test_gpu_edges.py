@@ -646,7 +646,9 @@ def test_float_row_sums_of_long_lists(prec, S):
     rows, 16 stages a part: the parts' sums, (2/8)^2 + .. + (8/8)^2 = 3.2, the stages within
     the parts 0.7 more, rows within stages and pieces less than 0.6: a deviation of
     sqrt(4.5 / 3) = 1.2 units of 2^-24, a mean size of 0.8 times that, 1.0. (A chain of 125
-    stage sums: 3.0.)"""
+    stage sums: 3.0.) Rows of at most 64 columns take one chain of 32 stages of 16 rows in
+    each piece of 512: 2 (1/2)^2 (11.3) = 5.7 and 1.3 for the rest, of which half is left when
+    s counts with its place between two powers of two: sqrt(3.5 / 3) times 0.8, 0.9."""
     rng = np.random.default_rng(S)
     n = 6000
     src, dst, lists = sum_graph(rng, S, (1000, 1024), 8, 3000, 400, n)
